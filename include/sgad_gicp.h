@@ -69,7 +69,8 @@ typedef struct {
     int32_t status;       /* bit 0: a set overflowed its capacity (cleared by
                              sgad_gicp_frame, set by it or by sgad_gicp_insert);
                              bit 1: fewer than 6 correspondences or a singular system
-                             ended the last sgad_gicp_track */
+                             ended the last sgad_gicp_track; bit 2: a wait between the
+                             tracking kernel's blocks gave up */
     double cost;          /* Eq. 2 at the start of the last iteration */
     double step;          /* |xi| of the last iteration */
 } sgad_gicp_stats;
@@ -93,7 +94,7 @@ sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_camera *cam, c
                             const sgad_gaussian_set *out, int32_t *pix_out, int32_t *knn_out, void *workspace,
                             size_t ws_bytes, void *stream);
 
-/* The map's spatial hash grid (cells of max(r_max, d_overlap) / 3; searches visit rings
+/* The map's spatial hash grid (cells of max(r_max, d_overlap) / 2; searches visit rings
  * of cells until their result is proven). Required after the caller changes the map;
  * sgad_gicp_insert rebuilds it itself. */
 sgad_status sgad_gicp_index(const sgad_gicp_params *p, const sgad_gaussian_set *map, void *workspace,
@@ -119,9 +120,9 @@ sgad_status sgad_gicp_set_pose(const double pose[12], void *workspace, size_t ws
  * initial pose, or from the workspace's pose (sgad_gicp_set_pose, or the last estimate)
  * when pose0 is NULL, so that a frame's calls can be captured once in a CUDA graph and
  * replayed with a new starting pose; the estimate stays in the workspace (read by
- * sgad_gicp_result, used by sgad_gicp_insert). 1 + max_iters kernel launches (the last block of each iteration
- * solves and updates the pose); iterations after convergence exit
- * at once. Capturable in a CUDA graph. */
+ * sgad_gicp_result, used by sgad_gicp_insert). Two kernel launches: the second, a cooperative one, runs every
+ * iteration (the last block of each solves and updates the pose, the others wait for it
+ * with a limit). Capturable in a CUDA graph. */
 sgad_status sgad_gicp_track(const sgad_gicp_params *p, const sgad_gaussian_set *src,
                             const sgad_gaussian_set *map, const double pose0[12], void *workspace,
                             size_t ws_bytes, void *stream);

@@ -27,8 +27,11 @@ using sgad::report_error;
 constexpr int kSys = 29;                 // H upper triangle (21), g (6), cost, count
 constexpr int kSelBlock = 1024;          // cells per selection block (4 per thread)
 constexpr int kMaxSelBlocks = 16384;     // selection grids of up to 16.7 M cells
-constexpr int kStepThreads = 128;        // correspondence step: 16 teams of 8 lanes per block
+constexpr int kRowPts = 16;              // source points of one row of partial sums
+constexpr int kStepThreads = 32 * kRowPts;   // correspondence step: one warp per point of a row
+constexpr int kMaxRows = 4 * 152;        // rows of partial sums; more points share the rows
 constexpr int kInsThreads = 256;         // map-update kernels
+constexpr int kInsPts = 64;              // source points per block of the overlap test
 constexpr int kKMatchMax = 8;
 
 struct GicpState {
@@ -39,16 +42,13 @@ struct GicpState {
     float tol;
     int32_t map_old, ins_total;
     int32_t blocks_done;     // step blocks finished in the current iteration
+    uint32_t sync;           // grid-wide steps completed (the tracking kernel waits on it)
 };
 
 struct GLayout {
-    size_t state, sel_counts, tile_sums, hash_cnt, hash_off, hash_pts, knn_cnt, knn_off, knn_pts, partial, ins_flags,
-        ins_counts, total;
-    int32_t table, knn_table, max_blocks, step_blocks;
+    size_t state, sel_counts, hash_head, hash_pts, knn_head, knn_pts, partial, ins_flags, ins_counts, total;
+    int32_t table, knn_table, max_blocks, rows;
 };
-
-constexpr int kScanTile = 4096;          // buckets per tile of the parallel scan
-constexpr int kMaxTiles = 4096;          // tables of up to 2^24 buckets
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -66,10 +66,9 @@ GLayout glayout(const sgad_gicp_params &p)
     L.table = table_for(p.map_capacity);
     L.knn_table = table_for(p.src_capacity);
     L.max_blocks = (p.src_capacity + kInsThreads - 1) / kInsThreads;
-    // the correspondence step: one team of 8 lanes per source point, 16 per block (blocks
-    // small enough to spread a few thousand points evenly over the SMs), grid-stride over
-    // at most 4 blocks per SM of a 152-SM part (the solve sums one partial row per block)
-    L.step_blocks = std::min((p.src_capacity + 15) / 16, 4 * 152);
+    // rows of 16 points each; points beyond kMaxRows rows are added to the rows in turn (the
+    // solve sums one partial row per 16 points)
+    L.rows = std::min((p.src_capacity + kRowPts - 1) / kRowPts, kMaxRows);
     size_t o = 0;
     const auto take = [&o](size_t bytes) {
         const size_t at = o;
@@ -78,16 +77,13 @@ GLayout glayout(const sgad_gicp_params &p)
     };
     L.state = take(sizeof(GicpState));
     L.sel_counts = take((size_t)kMaxSelBlocks * sizeof(int32_t));
-    L.tile_sums = take((size_t)kMaxTiles * sizeof(int32_t));
-    L.hash_cnt = take((size_t)L.table * sizeof(int32_t));
-    L.hash_off = take((size_t)(L.table + 1) * sizeof(int32_t));
+    L.hash_head = take((size_t)L.table * sizeof(int32_t));
     L.hash_pts = take((size_t)p.map_capacity * sizeof(float4));
-    L.knn_cnt = take((size_t)L.knn_table * sizeof(int32_t));
-    L.knn_off = take((size_t)(L.knn_table + 1) * sizeof(int32_t));
+    L.knn_head = take((size_t)L.knn_table * sizeof(int32_t));
     L.knn_pts = take((size_t)p.src_capacity * sizeof(float4));
-    L.partial = take((size_t)std::max(L.max_blocks, L.step_blocks) * 32 * sizeof(float));
+    L.partial = take((size_t)L.rows * 32 * sizeof(float));
     L.ins_flags = take((size_t)p.src_capacity * sizeof(int32_t));
-    L.ins_counts = take((size_t)(L.max_blocks + 1) * sizeof(int32_t));
+    L.ins_counts = take(((size_t)p.src_capacity / kInsPts + 2) * sizeof(int32_t));
     L.total = o;
     return L;
 }
@@ -255,6 +251,8 @@ struct SelArgs {
     int32_t *count;
     int32_t capacity;
     int32_t *blk;
+    int32_t *cell_point;     // [ncells] point of a cell or -1, or null
+    int32_t *point_cell;     // [capacity] cell of a point (with cell_point)
     GicpState *state;
 };
 
@@ -302,6 +300,8 @@ __global__ void __launch_bounds__(256) k_select_write(const __grid_constant__ Se
     bool over = false;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+        const int c = blockIdx.x * kSelBlock + threadIdx.x * 4 + k;
+        if (a.cell_point && c < a.ncells) a.cell_point[c] = ok[k] && o < a.capacity ? o : -1;
         if (!ok[k]) continue;
         if (o < a.capacity) {
             // p = d ((u - cx) / fx, (v - cy) / fy, 1), each step rounded as written
@@ -309,6 +309,7 @@ __global__ void __launch_bounds__(256) k_select_write(const __grid_constant__ Se
             const float y = __fmul_rn(d[k], __fdiv_rn(__fsub_rn((float)v[k], a.cy), a.fy));
             a.pos[o] = make_float4(x, y, d[k], 0.f);
             if (a.pix) a.pix[o] = v[k] * a.W + u[k];
+            if (a.cell_point) a.point_cell[o] = c;
         } else {
             over = true;
         }
@@ -318,244 +319,361 @@ __global__ void __launch_bounds__(256) k_select_write(const __grid_constant__ Se
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *a.count = min(prefix + total, a.capacity);
 }
 
-// ------------------------------------------------------------------ team search
-// Neighbour searches run one query per team of kTeam lanes of a warp: the lanes share the
-// cells of each ring, keep their own sorted candidate lists, and rank their candidates
-// among the team's through shared memory, which gives the exact team-wide k-th candidate
-// after every ring (for the stopping proof) and the final sorted list.
-constexpr int kTeam = 8;
-constexpr int kRings = 6;                // rings searched before the exhaustive fallback
+// ------------------------------------------------------------------ neighbour search
+// A search runs one query per warp. Its result is the list of the nearest points as 64-bit
+// keys (bits of the squared distance << 32 | index), ascending over the lanes: lane k holds
+// the (k + 1)-th nearest, ~0 past the last found, so the order is by distance, then index.
+// A search is a chain of dependent loads, so a warp's 32 lanes load as many cells at once
+// as they can; with 8 lanes per query and the cells of a ring in turn the first step of a
+// track took 103 us at 8,160 points, half of it a tail of a few slow queries.
+constexpr unsigned kFull = 0xffffffffu;
+constexpr uint64_t kNone = ~0ull;
+constexpr int kRings = 6;                // rings searched before the exhaustive pass
 
 struct Grid {
-    const int32_t *off;       // [table + 1] bucket offsets
-    const float4 *pts;        // [indexed count] points sorted by bucket: x, y, z, index bits
+    const int32_t *head;      // [table] first point of a bucket's chain + 1, 0: empty
+    const float4 *pts;        // [cap] x, y, z, next point of the chain + 1 (bits)
     float inv_cell, cell;
     uint32_t mask;
+    int32_t cap;
 };
 
-__device__ __forceinline__ bool lex_less(float d1, int j1, float d2, int j2)
+__device__ __forceinline__ uint64_t pack_key(float d, int j)
 {
-    return d1 < d2 || (d1 == d2 && j1 < j2);
+    return ((uint64_t)__float_as_uint(d) << 32) | (uint32_t)j;
+}
+__device__ __forceinline__ float key_dist(uint64_t k) { return __uint_as_float((uint32_t)(k >> 32)); }
+
+// Compare-exchange with the lane `o` away: the lane keeps the smaller key if `low`.
+__device__ __forceinline__ uint64_t exchange(uint64_t k, int o, bool low)
+{
+    const uint64_t y = __shfl_xor_sync(kFull, k, o);
+    return (k < y) == low ? k : y;
 }
 
-__device__ __forceinline__ unsigned team_mask() { return 0xFFu << (threadIdx.x & 24); }
-
-// Sorted insert into a lane's list (entries are unique: every point is seen once);
-// (wd, wj) tracks the list's K-th entry for the early rejection.
-template <int KMAX>
-__device__ __forceinline__ void lane_insert(float d, int j, int K, float (&bd)[KMAX], int (&bj)[KMAX], float &wd,
-                                            int &wj)
+// Takes the lanes' new keys c (kNone: none) into the sorted list `best`, of which the
+// `keep` smallest are wanted. Keys are unique (every point is seen once). A few keys are
+// shifted in one by one (~100 cycles each); more are sorted across the lanes (a bitonic
+// network, 15 exchanges) and merged (the smaller of the list and the reversed keys is
+// bitonic and holds the 32 smallest: 5 exchanges).
+__device__ __forceinline__ void warp_insert(uint64_t &best, uint64_t c, int keep)
 {
-    if (!lex_less(d, j, wd, wj)) return;
-    float cd = d;
-    int cj = j;
+    const int lane = threadIdx.x & 31;
+    const uint64_t worst = __shfl_sync(kFull, best, keep - 1);
+    unsigned m = __ballot_sync(kFull, c < worst);
+    if (__popc(m) > 8) {
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        if (k < K && lex_less(cd, cj, bd[k], bj[k])) {
-            const float td = bd[k];
-            const int tj = bj[k];
-            bd[k] = cd;
-            bj[k] = cj;
-            cd = td;
-            cj = tj;
-        }
-        if (k == K - 1) {
-            wd = bd[k];
-            wj = bj[k];
-        }
+        for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+            for (int o = size >> 1; o > 0; o >>= 1) c = exchange(c, o, ((lane & size) == 0) == ((lane & o) == 0));
+        const uint64_t r = __shfl_xor_sync(kFull, c, 31);
+        best = r < best ? r : best;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = exchange(best, o, (lane & o) == 0);
+        return;
+    }
+    while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        const uint64_t v = __shfl_sync(kFull, c, src);
+        const int p = __popc(__ballot_sync(kFull, best < v));
+        const uint64_t up = __shfl_up_sync(kFull, best, 1);
+        best = lane < p ? best : (lane == p ? v : up);
     }
 }
 
-// Calls f(q) for every point of the cells of ring r around (ix, iy, iz) that this lane
-// owns (cube cells c = tl, tl + kTeam, ... with Chebyshev distance r). Points stored in
-// a visited bucket but belonging to another cell (hash collisions) are skipped, so each
-// point is seen once, in its own cell.
+// Walks the chains of the lanes' buckets (first point + 1 = e) in step and calls
+// f(point, index), index -1 for a lane whose point is none or lies in another cell than
+// (cx, cy, cz), with the whole warp. Indexes are checked and the steps bounded by the
+// capacity.
 template <typename F>
-__device__ __forceinline__ void team_ring(const Grid &g, int ix, int iy, int iz, int r, int tl, F &&f)
+__device__ __forceinline__ void walk_chain(const Grid &g, int e, float4 q, int cx, int cy, int cz, F &&f)
 {
-    const int side = 2 * r + 1, ncube = side * side * side;
-#pragma unroll 1
-    for (int c = tl; c < ncube; c += kTeam) {
-        const int dx = c % side - r, dy = (c / side) % side - r, dz = c / (side * side) - r;
-        if (max(abs(dx), max(abs(dy), abs(dz))) != r) continue;
-        const int cx = ix + dx, cy = iy + dy, cz = iz + dz;
-        const uint32_t h = cell_hash(cx, cy, cz, g.mask);
-        const int e1 = g.off[h + 1];
-#pragma unroll 1
-        for (int e = g.off[h]; e < e1; ++e) {
-            const float4 q = g.pts[e];
+    for (int t = 0; t <= g.cap && __any_sync(kFull, e > 0); ++t) {
+        int i = -1, next = 0;
+        if (e > 0) {
             if (cell_of(q.x, g.inv_cell) == cx && cell_of(q.y, g.inv_cell) == cy && cell_of(q.z, g.inv_cell) == cz)
-                f(q);
+                i = e - 1;
+            next = __float_as_int(q.w);
+        }
+        next = next > 0 && next <= g.cap ? next : 0;
+        float4 qn = q;
+        if (next) qn = g.pts[next - 1];                        // on its way during f
+        f(q, i);
+        e = next;
+        q = qn;
+    }
+}
+
+// The cells at Chebyshev distance R around x's cell (BALL: at most R), 32 at a time; four
+// of a lane's bucket heads are loaded together, then their first points. f(point, index, -1
+// for a lane without one) is called by the whole warp.
+template <int R, bool BALL, typename F>
+__device__ __forceinline__ void ring_walk(const Grid &g, float3 x, F &&f)
+{
+    constexpr int side = 2 * R + 1, ncube = side * side * side;
+    constexpr int kAhead = ncube > 32 ? 4 : 1;
+    const int lane = threadIdx.x & 31;
+    const int ix = cell_of(x.x, g.inv_cell), iy = cell_of(x.y, g.inv_cell), iz = cell_of(x.z, g.inv_cell);
+#pragma unroll 1
+    for (int c0 = 0; c0 < ncube; c0 += 32 * kAhead) {
+        int e[kAhead];
+        float4 q[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int c = c0 + 32 * u + lane;
+            const int dx = c % side - R, dy = (c / side) % side - R, dz = c / (side * side) - R;
+            const bool on = c < ncube && (BALL || max(abs(dx), max(abs(dy), abs(dz))) == R);
+            const int h = on ? g.head[cell_hash(ix + dx, iy + dy, iz + dz, g.mask)] : 0;
+            e[u] = h > 0 && h <= g.cap ? h : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) q[u] = e[u] ? g.pts[e[u] - 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int c = c0 + 32 * u + lane;
+            const int dx = c % side - R, dy = (c / side) % side - R, dz = c / (side * side) - R;
+            walk_chain(g, e[u], q[u], ix + dx, iy + dy, iz + dz, f);
         }
     }
 }
 
-// The team's K smallest (d, j) entries in order, merged from the lanes' sorted lists
-// (copied to the team's shared-memory slots sd/sj [kTeam][KMAX]): K rounds of a team
-// argmin over the lanes' heads. Writes out/outd [0, found) and returns found.
-template <int KMAX>
-__device__ __forceinline__ int team_select(const float (&bd)[KMAX], const int (&bj)[KMAX], int K, float *sd, int *sj,
-                                           int tl, int *out, float *outd)
+template <int R, bool BALL, typename F>
+__device__ __forceinline__ void ring_cells(const Grid &g, float3 x, F &&f)
 {
-    const unsigned m = team_mask();
-#pragma unroll
-    for (int k = 0; k < KMAX; ++k)
-        if (k < K) {
-            sd[tl * KMAX + k] = bd[k];
-            sj[tl * KMAX + k] = bj[k];
-        }
-    __syncwarp(m);
-    int head = 0;
-    float hd = sd[tl * KMAX];
-    int hj = sj[tl * KMAX];
-    int found = 0;
-#pragma unroll 1
-    for (; found < K; ++found) {
-        float md = hd;
-        int mj = hj, ml = tl;
-#pragma unroll
-        for (int o = kTeam / 2; o > 0; o >>= 1) {
-            const float od = __shfl_xor_sync(m, md, o, kTeam);
-            const int oj = __shfl_xor_sync(m, mj, o, kTeam), ol = __shfl_xor_sync(m, ml, o, kTeam);
-            if (lex_less(od, oj, md, mj) || (od == md && oj == mj && ol < ml)) {
-                md = od;
-                mj = oj;
-                ml = ol;
-            }
-        }
-        if (mj == INT_MAX) break;                             // the lanes hold no more entries
-        if (tl == 0) {
-            out[found] = mj;
-            outd[found] = md;
-        }
-        if (tl == ml) {
-            ++head;
-            hd = head < K ? sd[tl * KMAX + head] : FLT_MAX;
-            hj = head < K ? sj[tl * KMAX + head] : INT_MAX;
-        }
-    }
-    __syncwarp(m);
-    return found;
+    ring_walk<R, BALL>(g, x, [&](float4 q, int i) {
+        if (i >= 0) f(q);
+    });
 }
 
-// K nearest points of `me` among the indexed ones (optionally within r_max): on return
-// out[0 .. K) (team shared memory) holds their indices nearest first, -1 past the last
-// found; returns the number found. `pos`/`n` serve the exhaustive fallback.
-template <int KMAX>
-__device__ int team_nearest(const Grid &g, float3 me, int K, float r_max, int max_rings, const float4 *pos, int n,
-                            float *sd, int *sj, int *out, float *outd)
+// Ring r (r = 1: with the cell itself) into the sorted list. The points found are gathered
+// in `buf` (64 keys of shared memory of the warp) and taken 32 at a time: a step along the
+// chains finds a few points, and taking them in step by step was most of the search.
+__device__ __forceinline__ void search_ring(const Grid &g, float3 x, int r, int keep, uint64_t &best, uint64_t *buf)
 {
-    const int tl = threadIdx.x & (kTeam - 1);
-    float bd[KMAX];
-    int bj[KMAX];
-#pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        bd[k] = FLT_MAX;
-        bj[k] = INT_MAX;
-    }
-    float wd = FLT_MAX;
-    int wj = INT_MAX;
-    const float r2 = r_max * r_max;
-    const int ix = cell_of(me.x, g.inv_cell), iy = cell_of(me.y, g.inv_cell), iz = cell_of(me.z, g.inv_cell);
-    int found = 0;
-    bool proven = false;
-#pragma unroll 1
-    for (int r = 0; r <= max_rings && !proven; ++r) {
-        team_ring(g, ix, iy, iz, r, tl, [&](float4 q) {
-            const float d = sqdist(q.x, q.y, q.z, me.x, me.y, me.z);
-            if (d <= r2) lane_insert<KMAX>(d, __float_as_int(q.w), K, bd, bj, wd, wj);
-        });
-        if (r == 0) continue;                               // nothing is proven at radius 0
-        found = team_select<KMAX>(bd, bj, K, sd, sj, tl, out, outd);
-        const float reach = (float)r * g.cell * (1.f - 1e-4f);
-        // every point outside the searched rings lies at least `reach` away
-        proven = reach >= r_max || (found == K && outd[K - 1] < reach * reach);
-    }
-    if (!proven) {                                          // exhaustive over the set, from scratch
-#pragma unroll
-        for (int k = 0; k < KMAX; ++k) {
-            bd[k] = FLT_MAX;
-            bj[k] = INT_MAX;
+    const int lane = threadIdx.x & 31;
+    uint64_t worst = __shfl_sync(kFull, best, keep - 1);
+    int cnt = 0;
+    const auto take = [&](float4 q, int i) {
+        uint64_t c = kNone;
+        if (i >= 0) {
+            const float d = sqdist(q.x, q.y, q.z, x.x, x.y, x.z);
+            if (d <= FLT_MAX) c = pack_key(d, i);
         }
-        wd = FLT_MAX;
-        wj = INT_MAX;
-#pragma unroll 1
-        for (int j = tl; j < n; j += kTeam) {
-            const float4 q = pos[j];
-            const float d = sqdist(q.x, q.y, q.z, me.x, me.y, me.z);
-            if (d <= r2) lane_insert<KMAX>(d, j, K, bd, bj, wd, wj);
+        const unsigned m = __ballot_sync(kFull, c < worst);
+        if (m == 0u) return;
+        if (c < worst) buf[cnt + __popc(m & ((1u << lane) - 1u))] = c;
+        cnt += __popc(m);
+        if (cnt >= 32) {
+            __syncwarp();
+            const uint64_t k = buf[lane], rest = buf[32 + lane];
+            __syncwarp();
+            cnt -= 32;
+            if (lane < cnt) buf[lane] = rest;
+            warp_insert(best, k, keep);
+            worst = __shfl_sync(kFull, best, keep - 1);
         }
-        found = team_select<KMAX>(bd, bj, K, sd, sj, tl, out, outd);
+    };
+    switch (r) {
+    case 1: ring_walk<1, true>(g, x, take); break;
+    case 2: ring_walk<2, false>(g, x, take); break;
+    case 3: ring_walk<3, false>(g, x, take); break;
+    case 4: ring_walk<4, false>(g, x, take); break;
+    case 5: ring_walk<5, false>(g, x, take); break;
+    default: ring_walk<6, false>(g, x, take); break;
     }
-    return found;
+    __syncwarp();
+    const uint64_t k = lane < cnt ? buf[lane] : kNone;
+    __syncwarp();
+    warp_insert(best, k, keep);
 }
 
 // ------------------------------------------------------------------ shapes
-// One team per selected point: its K_c nearest selected points (FP32 squared distance,
-// ties by index) from a ring search of the points' own hash grid, then (lane 0) the
-// covariance, its eigen-decomposition and the normalised shape.
-template <int KMAX>
-__global__ void __launch_bounds__(128) k_shape(const float4 *__restrict__ pos, const int32_t *count, int K, float eps,
-                                               Grid g, float4 *cov, float4 *normal, int32_t *knn_out)
+// One warp per selected point: its K_c nearest selected points (FP32 squared distance,
+// ties by index) and their covariance, kShapeRounds points in turn; then the block's first
+// warp, a point per lane, takes the eigen-decompositions and writes the normalised shapes
+// (a decomposition is ~1,400 dependent instructions, the same for a warp of one point or
+// of 32).
+constexpr int kShapeRounds = 2;
+constexpr int kShapeThreads = 512;
+constexpr int kShapePts = kShapeThreads / 32 * kShapeRounds;
+static_assert(kShapePts == 32, "one point per lane of the block's first warp");
+
+// The selection grid: cell (cu, cv) is the pixel (cu R, cv R), whose ray is
+// (x0 + cu step_x, y0 + cv step_y, 1).
+struct Window {
+    const int32_t *point_cell, *cell_point;
+    int32_t ncx, ncy;
+    float step_x, step_y, x0, y0;
+};
+
+struct ShapeArgs {
+    const float4 *pos;
+    const int32_t *count;
+    float4 *cov, *normal;
+    int32_t *knn_out;
+    int32_t K;
+    float eps;
+    Window w;
+    Grid g;
+};
+
+// Distance from the point at depth d on the ray slope r to the nearest ray with a slope
+// between r + a and r + b (both on one side of r): a point of such a ray lies in the plane
+// through the centre with its slope s, at d |s - r| / sqrt(1 + s^2), which has no minimum
+// inside the interval (it rises while 1 + r s > 0 and falls after).
+__device__ __forceinline__ float slope_gap(float d, float r, float a, float b)
 {
-    __shared__ float s_d[128 / kTeam][kTeam * KMAX];
-    __shared__ int s_j[128 / kTeam][kTeam * KMAX];
-    __shared__ int s_out[128 / kTeam][KMAX];
-    __shared__ float s_outd[128 / kTeam][KMAX];
-    const int kcov = K;
-    const int n = *count;
-    const int team = threadIdx.x / kTeam, tl = threadIdx.x & (kTeam - 1);
-    const int i = blockIdx.x * (128 / kTeam) + team;
-    if (i >= n) return;                                       // whole team
-    K = min(K, n);                                            // fewer points than K_c: all of them
-    const float4 me4 = pos[i];
-    const float3 me = make_float3(me4.x, me4.y, me4.z);
-    team_nearest<KMAX>(g, me, K, FLT_MAX, kRings, pos, n, s_d[team], s_j[team], s_out[team], s_outd[team]);
-    const int *nb = s_out[team];
-    if (knn_out)
-        for (int k = tl; k < kcov; k += kTeam) knn_out[(size_t)i * kcov + k] = k < K ? nb[k] : -1;
-    if (tl != 0) return;
-    // covariance of the K neighbours (FP32): mean, then centred second moments
-    float mx = 0.f, my = 0.f, mz = 0.f;
+    return d * fminf(fabsf(a) * rsqrtf(1.f + (r + a) * (r + a)), fabsf(b) * rsqrtf(1.f + (r + b) * (r + b)));
+}
+
+// K nearest points by windows of the selection grid around the point's cell: the points
+// outside the window lie on rays at least one window edge away, so the search ends once the
+// K-th distance is below the smallest distance to such a ray. No hash grid is built (its
+// build was 6 launches) and a window's 25 cells are one step of the warp.
+__device__ __forceinline__ uint64_t window_nearest(const ShapeArgs &a, int i, float4 me, int K)
+{
+    const Window &w = a.w;
+    const int lane = threadIdx.x & 31;
+    const int c = w.point_cell[i], cv = c / w.ncx, cu = c - cv * w.ncx;
+    const float rx = w.x0 + (float)cu * w.step_x, ry = w.y0 + (float)cv * w.step_y;
+    // the points' FP32 coordinates are off their rays by a few units in the last place
+    const float off_ray = 1e-6f * me.z * (1.f + fabsf(rx) + fabsf(ry));
+    uint64_t best = kNone;
+    const auto take = [&](int u, int v, bool on) {
+        uint64_t k = kNone;
+        if (on && u >= 0 && u < w.ncx && v >= 0 && v < w.ncy) {
+            const int j = w.cell_point[(size_t)v * w.ncx + u];
+            if (j >= 0) {
+                const float4 q = a.pos[j];
+                const float d = sqdist(q.x, q.y, q.z, me.x, me.y, me.z);
+                if (d <= FLT_MAX) k = pack_key(d, j);
+            }
+        }
+        warp_insert(best, k, K);
+    };
+    take(cu - 2 + lane % 5, cv - 2 + lane / 5, lane < 25);
 #pragma unroll 1
-    for (int k = 0; k < K; ++k) {
-        const float4 q = pos[nb[k]];
-        mx += q.x;
-        my += q.y;
-        mz += q.z;
-    }
-    const float invk = 1.f / (float)K;
-    mx *= invk;
-    my *= invk;
-    mz *= invk;
-    float A[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+    for (int m = 2;; ++m) {
+        const bool l = cu - m > 0, r = cu + m < w.ncx - 1, t = cv - m > 0, b = cv + m < w.ncy - 1;
+        if (!(l || r || t || b)) break;                          // every cell was seen
+        float gap = FLT_MAX;
+        const float mx = (float)(m + 1) * w.step_x, my = (float)(m + 1) * w.step_y;
+        if (l) gap = fminf(gap, slope_gap(me.z, rx, -mx, -(float)cu * w.step_x));
+        if (r) gap = fminf(gap, slope_gap(me.z, rx, mx, (float)(w.ncx - 1 - cu) * w.step_x));
+        if (t) gap = fminf(gap, slope_gap(me.z, ry, -my, -(float)cv * w.step_y));
+        if (b) gap = fminf(gap, slope_gap(me.z, ry, my, (float)(w.ncy - 1 - cv) * w.step_y));
+        const uint64_t kth = __shfl_sync(kFull, best, K - 1);
+        gap = gap * (1.f - 1e-4f) - off_ray;
+        if (gap > 0.f && kth != kNone && key_dist(kth) < gap * gap) break;
+        // the next frame of cells: 8 (m + 1) of them, side by side
+        const int m1 = m + 1, edge = 2 * m1;
 #pragma unroll 1
-    for (int k = 0; k < K; ++k) {
-        const float4 q = pos[nb[k]];
-        const float dx = q.x - mx, dy = q.y - my, dz = q.z - mz;
-        A[0][0] += dx * dx;
-        A[0][1] += dx * dy;
-        A[0][2] += dx * dz;
-        A[1][1] += dy * dy;
-        A[1][2] += dy * dz;
-        A[2][2] += dz * dz;
+        for (int c0 = 0; c0 < 4 * edge; c0 += 32) {
+            const int k = c0 + lane, s = k / edge, o = k - s * edge;
+            const int du = s == 0 ? o - m1 : (s == 1 ? m1 : (s == 2 ? m1 - o : -m1));
+            const int dv = s == 0 ? -m1 : (s == 1 ? o - m1 : (s == 2 ? m1 : m1 - o));
+            take(cu + du, cv + dv, k < 4 * edge);
+        }
     }
-    A[0][0] *= invk;
-    A[0][1] *= invk;
-    A[0][2] *= invk;
-    A[1][1] *= invk;
-    A[1][2] *= invk;
-    A[2][2] *= invk;
-    A[1][0] = A[0][1];
-    A[2][0] = A[0][2];
-    A[2][1] = A[1][2];
+    return best;
+}
+
+// The same from the points' hash grid: rings of cells until the K-th distance is below the
+// searched radius, else every point.
+__device__ __forceinline__ uint64_t hash_nearest(const ShapeArgs &a, float4 me, int n, int K, uint64_t *buf)
+{
+    const int lane = threadIdx.x & 31;
+    const float3 x = make_float3(me.x, me.y, me.z);
+    uint64_t best = kNone;
+#pragma unroll 1
+    for (int r = 1; r <= kRings; ++r) {
+        search_ring(a.g, x, r, K, best, buf);
+        const float reach = (float)r * a.g.cell * (1.f - 1e-4f);
+        const uint64_t kth = __shfl_sync(kFull, best, K - 1);
+        if (kth != kNone && key_dist(kth) < reach * reach) return best;
+    }
+    best = kNone;
+#pragma unroll 1
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane;
+        uint64_t k = kNone;
+        if (j < n) {
+            const float4 q = a.pos[j];
+            const float d = sqdist(q.x, q.y, q.z, x.x, x.y, x.z);
+            if (d <= FLT_MAX) k = pack_key(d, j);
+        }
+        warp_insert(best, k, K);
+    }
+    return best;
+}
+
+template <bool WINDOW>
+__global__ void __launch_bounds__(kShapeThreads) k_shape(const __grid_constant__ ShapeArgs a)
+{
+    __shared__ float s_cov[kShapePts][7];
+    __shared__ uint64_t s_buf[WINDOW ? 1 : kShapeThreads / 32][64];
+    const int n = *a.count;
+    const int i0 = blockIdx.x * kShapePts;
+    if (i0 >= n) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int K = min(a.K, n);                                // fewer points than K_c: all of them
+#pragma unroll 1
+    for (int t = 0; t < kShapeRounds; ++t) {
+        const int slot = t * (kShapeThreads / 32) + warp, i = i0 + slot;
+        if (i >= n) break;
+        const float4 me = a.pos[i];
+        const uint64_t best = WINDOW ? window_nearest(a, i, me, K) : hash_nearest(a, me, n, K, s_buf[WINDOW ? 0 : warp]);
+        const int nb = best != kNone ? (int)(uint32_t)best : -1;
+        if (a.knn_out && lane < a.K) a.knn_out[(size_t)i * a.K + lane] = lane < K ? nb : -1;
+        const float4 q = lane < K && nb >= 0 ? a.pos[nb] : me;
+        // covariance of the K neighbours (FP32), nearest first: mean, then centred second
+        // moments
+        float mx = 0.f, my = 0.f, mz = 0.f;
+#pragma unroll 1
+        for (int k = 0; k < K; ++k) {
+            mx += __shfl_sync(kFull, q.x, k);
+            my += __shfl_sync(kFull, q.y, k);
+            mz += __shfl_sync(kFull, q.z, k);
+        }
+        const float invk = 1.f / (float)K;
+        mx = __fmul_rn(mx, invk);
+        my = __fmul_rn(my, invk);
+        mz = __fmul_rn(mz, invk);
+        const float qx = q.x - mx, qy = q.y - my, qz = q.z - mz;
+        float A[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int k = 0; k < K; ++k) {
+            const float dx = __shfl_sync(kFull, qx, k), dy = __shfl_sync(kFull, qy, k), dz = __shfl_sync(kFull, qz, k);
+            A[0] += dx * dx;
+            A[1] += dx * dy;
+            A[2] += dx * dz;
+            A[3] += dy * dy;
+            A[4] += dy * dz;
+            A[5] += dz * dz;
+        }
+        if (lane == 0) {
+#pragma unroll
+            for (int e = 0; e < 6; ++e) s_cov[slot][e] = A[e] * invk;
+        }
+    }
+    __syncthreads();
+    const int i = i0 + lane;
+    if (warp != 0 || i >= n) return;
+    float A[3][3];
+    A[0][0] = s_cov[lane][0];
+    A[0][1] = A[1][0] = s_cov[lane][1];
+    A[0][2] = A[2][0] = s_cov[lane][2];
+    A[1][1] = s_cov[lane][3];
+    A[1][2] = A[2][1] = s_cov[lane][4];
+    A[2][2] = s_cov[lane][5];
     float w[3], V[3][3];
     eig3(A, w, V);
     float sc[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) sc[k] = sqrtf(fmaxf(w[k], 0.f));
     const float smax = sc[2];
-    const float floor_s = sqrtf(eps);
+    const float floor_s = sqrtf(a.eps);
 #pragma unroll
     for (int k = 0; k < 3; ++k) sc[k] = fmaxf(smax > 0.f ? sc[k] / smax : 1.f, floor_s);
     float C[6];
@@ -567,88 +685,28 @@ __global__ void __launch_bounds__(128) k_shape(const float4 *__restrict__ pos, c
         for (int k = 0; k < 3; ++k) acc += V[rr[e]][k] * (sc[k] * sc[k]) * V[cc[e]][k];
         C[e] = acc;
     }
-    cov[2 * i] = make_float4(C[0], C[1], C[2], C[3]);
-    cov[2 * i + 1] = make_float4(C[4], C[5], 0.f, 0.f);
-    normal[i] = make_float4(V[0][0], V[1][0], V[2][0], 0.f);
+    a.cov[2 * i] = make_float4(C[0], C[1], C[2], C[3]);
+    a.cov[2 * i + 1] = make_float4(C[4], C[5], 0.f, 0.f);
+    a.normal[i] = make_float4(V[0][0], V[1][0], V[2][0], 0.f);
 }
 
 // ------------------------------------------------------------------ hash grid
-
-
-__global__ void k_hash_count(const float4 *pos, const int32_t *count, float inv_cell, uint32_t mask, int32_t *cnt)
+// Links every point into its bucket's chain (any order: a search's result does not depend
+// on it). The chains replace a counting sort of the buckets (a count, three scans and a
+// fill). `commit`: the points are the map after an update, whose count becomes
+// min(old + inserted, capacity).
+__global__ void __launch_bounds__(256) k_hash_link(const float4 *pos, int32_t *count, int32_t cap, float inv_cell,
+                                                   uint32_t mask, int32_t *head, float4 *pts,
+                                                   const GicpState *commit)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= *count) return;
-    const float4 p = pos[i];
-    atomicAdd(&cnt[cell_hash(cell_of(p.x, inv_cell), cell_of(p.y, inv_cell), cell_of(p.z, inv_cell), mask)], 1);
-}
-
-// Exclusive offsets of the bucket counts in three parallel passes (tile sums, a scan of
-// the tile sums, offsets within each tile); the counts are reset to 0 for use as fill
-// cursors.
-__global__ void __launch_bounds__(256) k_scan_tiles(const int32_t *cnt, int table, int32_t *tile_sums)
-{
-    __shared__ int red[8];
-    const int b0 = blockIdx.x * kScanTile;
-    int s = 0;
-    for (int t = threadIdx.x; t < kScanTile; t += 256)
-        if (b0 + t < table) s += cnt[b0 + t];
-    int total;
-    block_exclusive_scan(s, red, &total);
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_top(int32_t *tile_sums, int ntiles)
-{
-    __shared__ int red[32];
-    int v[4], s = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.x * 4 + k;
-        v[k] = i < ntiles ? tile_sums[i] : 0;
-        s += v[k];
+    const int n = min(commit ? commit->map_old + commit->ins_total : *count, cap);
+    if (commit && blockIdx.x == 0 && threadIdx.x == 0) *count = n;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const float4 p = pos[i];
+        const uint32_t h = cell_hash(cell_of(p.x, inv_cell), cell_of(p.y, inv_cell), cell_of(p.z, inv_cell), mask);
+        const int next = atomicExch(&head[h], i + 1);
+        pts[i] = make_float4(p.x, p.y, p.z, __int_as_float(next));
     }
-    int total;
-    int o = block_exclusive_scan(s, red, &total);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.x * 4 + k;
-        if (i < ntiles) tile_sums[i] = o;
-        o += v[k];
-    }
-}
-
-__global__ void __launch_bounds__(256) k_scan_write(int32_t *cnt, int32_t *off, int table, const int32_t *tile_sums)
-{
-    __shared__ int red[8];
-    const int b0 = blockIdx.x * kScanTile + threadIdx.x * 16;
-    int v[16], s = 0;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        v[k] = b0 + k < table ? cnt[b0 + k] : 0;
-        s += v[k];
-    }
-    int total;
-    int o = tile_sums[blockIdx.x] + block_exclusive_scan(s, red, &total);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        if (b0 + k < table) {
-            off[b0 + k] = o;
-            cnt[b0 + k] = 0;
-        }
-        o += v[k];
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 255) off[table] = o;
-}
-
-__global__ void k_hash_fill(const float4 *pos, const int32_t *count, float inv_cell, uint32_t mask,
-                            const int32_t *off, int32_t *cnt, float4 *pts)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= *count) return;
-    const float4 p = pos[i];
-    const uint32_t h = cell_hash(cell_of(p.x, inv_cell), cell_of(p.y, inv_cell), cell_of(p.z, inv_cell), mask);
-    pts[off[h] + atomicAdd(&cnt[h], 1)] = make_float4(p.x, p.y, p.z, __int_as_float(i));
 }
 
 // ------------------------------------------------------------------ Gauss-Newton step
@@ -661,22 +719,20 @@ struct StepArgs {
     float r_max;
     int32_t kmatch;
     int32_t system;          // accumulate the Gauss-Newton system
-    int32_t use_state;       // pose from the state (tracking) instead of `pose`
+    int32_t rows;            // rows of partial sums
     GicpState *state;
-    Pose12 pose;
+    Pose12 pose;             // of a single step (tracking takes the state's)
     int32_t *idx_out;
-    float *partial;          // [gridDim.x][32]
+    float *partial;          // [rows][32]
 };
 
-constexpr int kStepTeams = kStepThreads / kTeam;         // source points per block and round
-
-__device__ void sum_partials(const float *partial, int nblocks, double *sys);
-__device__ void solve_state(GicpState *st, const double *sys);
+// Rows of partial sums that hold points: row v sums points 16 (v + k rows) .. + 15.
+__device__ __forceinline__ int rows_used(int n, int rows) { return max(1, min(rows, (n + kRowPts - 1) / kRowPts)); }
 
 // The contribution of one correspondence to the Gauss-Newton system (H upper triangle,
 // g = J^T M e, cost, count) in FP32.
 __device__ __forceinline__ void gn_terms(const float *P, float3 x, float4 b, float4 cb0, float4 cb1, float4 ca0,
-                                         float4 ca1, float (&acc)[kSys])
+                                         float4 ca1, float *acc)
 {
     const float Ca[3][3] = {{ca0.x, ca0.y, ca0.z}, {ca0.y, ca0.w, ca1.x}, {ca0.z, ca1.x, ca1.y}};
     const float R[3][3] = {{P[0], P[1], P[2]}, {P[4], P[5], P[6]}, {P[8], P[9], P[10]}};
@@ -717,220 +773,423 @@ __device__ __forceinline__ void gn_terms(const float *P, float3 x, float4 b, flo
     acc[28] += 1.f;
 }
 
-// One team per source point (grid-stride over the points): the k_match nearest map
-// Gaussians within r_max by a ring search of the map's grid (cells of r_max / 3, at most
-// 3 rings), the smallest point-to-surface distance among them (ties by squared
-// distance, then index), and that correspondence's Gauss-Newton terms, reduced per block.
-__global__ void __launch_bounds__(kStepThreads) k_gicp_step(const __grid_constant__ StepArgs a)
+
+// A tracked point's candidates, kept between the iterations of one track in shared memory:
+// the 32 nearest map points of x0 with their normals, and a radius rho: every map point
+// nearer than rho to x0 is among them. So at x, with delta = |x - x0|, every map point
+// nearer than rho - delta is, and the k_match nearest within r_max are exact as long as
+// they lie inside that radius (a margin covers the rounding of the distances). As the pose
+// converges delta shrinks, and an iteration reads 32 kept points instead of searching the
+// grid.
+struct Kept {
+    float4 src;               // the source point
+    float4 x0;                // x0, rho (0: no candidates)
+    float4 pos[32];           // x, y, z, index (-1: none)
+    float nx[32], ny[32], nz[32];
+};
+constexpr int kKeptPts = 4;               // points per warp with candidates; further ones search each time
+constexpr size_t kTrackSmem = (size_t)kKeptPts * kRowPts * sizeof(Kept);
+constexpr int kBatchRows = 2;             // rows whose points' terms are taken together
+constexpr float kMargin = 1.f - 1e-4f;
+
+// Correspondence of x, or -1; whole warp. kept: the point's candidates (null: none kept).
+// first: the first step of a track, which moves the points most: its search ends as soon as
+// its result is proven and keeps nothing; a later one goes on until the candidates allow a
+// move of `slack` (0.3 of a cell, 1.5 cm at the default radius: with half of that, single
+// points outran theirs in each of the next ten iterations, and one search delays the
+// iteration of all by 10-15 us).
+__device__ __forceinline__ int match_point(const StepArgs &a, float3 x, Kept *kept, bool first, uint64_t *buf)
 {
-    __shared__ float red[kStepThreads / 32][kSys + 3];
-    __shared__ float s_d[kStepTeams][kTeam * kKMatchMax];
-    __shared__ int s_j[kStepTeams][kTeam * kKMatchMax];
-    __shared__ int s_out[kStepTeams][kKMatchMax];
-    __shared__ float s_outd[kStepTeams][kKMatchMax];
-    if (a.use_state && a.state->done) return;                  // uniform across the grid
-    float P[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) P[k] = a.use_state ? a.state->posef[k] : a.pose.p[k];
-    const int team = threadIdx.x / kTeam, tl = threadIdx.x & (kTeam - 1);
-    const int n = *a.scount, nm = *a.mcount;
-    const unsigned m = team_mask();
-    float acc[kSys];
-#pragma unroll
-    for (int k = 0; k < kSys; ++k) acc[k] = 0.f;
+    const int lane = threadIdx.x & 31;
+    const int K = a.kmatch;
+    const float r2 = a.r_max * a.r_max;
+    bool member = false;
+    float d = FLT_MAX, nx = 0.f, ny = 0.f, nz = 0.f;
+    int j = INT_MAX;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool ok = false;
+    if (kept && !first && kept->x0.w > 0.f) {
+        const float4 h = kept->x0;
+        q = kept->pos[lane];
+        nx = kept->nx[lane];
+        ny = kept->ny[lane];
+        nz = kept->nz[lane];
+        j = __float_as_int(q.w);
+        const float s2 = sqdist(h.x, h.y, h.z, x.x, x.y, x.z);
+        const float delta = s2 > 0.f ? s2 * rsqrtf(s2) : 0.f;
+        const float lim = h.w * kMargin - delta * (2.f - kMargin);
+        d = sqdist(q.x, q.y, q.z, x.x, x.y, x.z);
+        member = j >= 0 && d <= r2;
+        // the K nearest are known if K lie inside the radius, or all within r_max do
+        ok = lim > 0.f && (__popc(__ballot_sync(kFull, member && d < lim * lim)) >= K || a.r_max < lim);
+        // the first K were the nearest to x0: the farthest of them bounds the K-th distance
+        const unsigned far = __reduce_max_sync(kFull, lane >= K ? 0u : (member ? __float_as_uint(d) : 0xffffffffu));
+        member = member && __float_as_uint(d) <= far;
+    }
+    if (!ok) {
+        const bool keep = kept && !first;
+        const float slack = 0.3f * a.grid.cell;
+        uint64_t best = kNone;
+        float rho = 0.f;
+        // rings of cells of half of r_max or more: two prove any result
 #pragma unroll 1
-    for (int base = blockIdx.x * kStepTeams; base < n; base += gridDim.x * kStepTeams) {
-        const int i = base + team;
-        if (i >= n) continue;                                  // whole team
-        const float3 x = transform(P, a.spos[i]);
-        const int found = team_nearest<kKMatchMax>(a.grid, x, a.kmatch, a.r_max, 3, a.mpos, nm, s_d[team], s_j[team],
-                                                  s_out[team], s_outd[team]);
-        // point-to-surface choice among the found candidates (lane k takes candidate k)
-        float bm = FLT_MAX, bd2 = FLT_MAX;
-        int bj = INT_MAX;
-        if (tl < found) {
-            const int j = s_out[team][tl];
-            const float4 b = a.mpos[j], nr = a.mnorm[j];
-            const float dx = __fsub_rn(b.x, x.x), dy = __fsub_rn(b.y, x.y), dz = __fsub_rn(b.z, x.z);
-            bm = fabsf(__fadd_rn(__fadd_rn(__fmul_rn(nr.x, dx), __fmul_rn(nr.y, dy)), __fmul_rn(nr.z, dz)));
-            bd2 = s_outd[team][tl];
-            bj = j;
+        for (int r = 1; r <= 3; ++r) {
+            search_ring(a.grid, x, r, keep ? 32 : K, best, buf);
+            const float reach = (float)r * a.grid.cell * (1.f - 1e-4f);
+            const uint64_t kth = __shfl_sync(kFull, best, K - 1), end = __shfl_sync(kFull, best, 31);
+            const bool have = kth != kNone && key_dist(kth) <= r2;
+            const bool proven = reach >= a.r_max || (kth != kNone && key_dist(kth) < reach * reach);
+            const bool full = end != kNone && sqrtf(key_dist(end)) < reach;
+            rho = full ? sqrtf(key_dist(end)) : reach;
+            const float need = have ? sqrtf(key_dist(kth)) : a.r_max;
+            if (proven && (!keep || full || rho - need >= slack)) break;
         }
-#pragma unroll
-        for (int o = kTeam / 2; o > 0; o >>= 1) {
-            const float om = __shfl_xor_sync(m, bm, o, kTeam), od = __shfl_xor_sync(m, bd2, o, kTeam);
-            const int oj = __shfl_xor_sync(m, bj, o, kTeam);
-            if (om < bm || (om == bm && (od < bd2 || (od == bd2 && oj < bj)))) {
-                bm = om;
-                bd2 = od;
-                bj = oj;
+        d = best != kNone ? key_dist(best) : FLT_MAX;
+        j = best != kNone ? (int)(uint32_t)best : -1;
+        member = lane < K && j >= 0 && d <= r2;
+        if (keep ? j >= 0 : member) {
+            q = a.grid.pts[j];
+            const float4 nr = a.mnorm[j];
+            nx = nr.x;
+            ny = nr.y;
+            nz = nr.z;
+        }
+        if (keep) {
+            q.w = __int_as_float(j);
+            kept->pos[lane] = q;
+            kept->nx[lane] = nx;
+            kept->ny[lane] = ny;
+            kept->nz[lane] = nz;
+            if (lane == 0) kept->x0 = make_float4(x.x, x.y, x.z, rho);
+            __syncwarp();
+        }
+    }
+    // The smallest point-to-surface distance among the K nearest members (ties by distance,
+    // index): the members in the order of that distance, until one is among the K nearest.
+    unsigned bm = 0xffffffffu;
+    if (member) {
+        const float dx = __fsub_rn(q.x, x.x), dy = __fsub_rn(q.y, x.y), dz = __fsub_rn(q.z, x.z);
+        bm = __float_as_uint(fabsf(__fadd_rn(__fadd_rn(__fmul_rn(nx, dx), __fmul_rn(ny, dy)), __fmul_rn(nz, dz))));
+    }
+    const uint64_t key = pack_key(d, j);
+#pragma unroll 1
+    for (;;) {
+        const unsigned m1 = __reduce_min_sync(kFull, bm);
+        if (m1 == 0xffffffffu) return -1;
+        const unsigned eq = __ballot_sync(kFull, bm == m1);
+        uint64_t k = __shfl_sync(kFull, key, __ffs(eq) - 1);
+        if (eq & (eq - 1)) {                                     // equal distances to the surface
+            for (unsigned rest = eq & (eq - 1); rest; rest &= rest - 1) {
+                const uint64_t o = __shfl_sync(kFull, key, __ffs(rest) - 1);
+                k = o < k ? o : k;
             }
         }
-        const int jbest = found > 0 ? bj : -1;
-        if (tl == 0) {
-            if (a.idx_out) a.idx_out[i] = jbest;
-            if (a.system && jbest >= 0)
-                gn_terms(P, x, a.mpos[jbest], a.mcov[2 * jbest], a.mcov[2 * jbest + 1], a.scov[2 * i],
-                         a.scov[2 * i + 1], acc);
-        }
-    }
-    if (!a.system) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kSys; ++k) {
-        float v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kSys) {
-        float s = 0.f;
-#pragma unroll
-        for (int w = 0; w < kStepThreads / 32; ++w) s += red[w][threadIdx.x];
-        a.partial[blockIdx.x * 32 + threadIdx.x] = s;
-    }
-    if (!a.use_state) return;
-    // tracking: the last block to finish sums the partials and takes the step
-    __shared__ int s_last;
-    __shared__ double sys[kSys];
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&a.state->blocks_done, 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    sum_partials(a.partial, gridDim.x, sys);
-    if (threadIdx.x == 0) {
-        solve_state(a.state, sys);
-        a.state->blocks_done = 0;
+        if (__popc(__ballot_sync(kFull, member && key < k)) < K) return (int)(uint32_t)k;
+        if (bm == m1) bm = 0xffffffffu;
     }
 }
 
-// Sum of the per-block partials in FP64 in a fixed order (warp w takes rows w, w + nw,
-// ...; the warps' sums are added in warp order), so the result does not depend on
-// scheduling. Partials are read through L2 (written by other blocks of the same grid).
-__device__ void sum_partials(const float *partial, int nblocks, double *sys)
+__device__ void sum_partials(const float *partial, int nrows, double *sys);
+__device__ bool solve_state(GicpState *st, const double *sys, double &step2);
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
 {
-    __shared__ double part[8][kSys];                    // blocks of up to 256 threads
-    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, k = threadIdx.x & 31;
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_release(uint32_t *p, uint32_t v)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+constexpr uint32_t kSyncSpins = 1u << 22;   // a wait on the other blocks gives up after a few seconds
+
+// Correspondences and partial sums of the Gauss-Newton system. A block takes rows of 16
+// points, one warp per point. TRACK: the whole of a track in one cooperative launch: after
+// each iteration the last block to finish sums the rows, solves and updates the pose, and
+// the others wait for it. One launch per iteration, with a search for every point, took
+// 100-200 us each (8,160-12,288 points, 15-25 iterations); here the first two iterations,
+// which search, take 45-65 us and the others 13-16 us: 3-5 us for the kept candidates, 1 for
+// the terms, 3 for the sum, 4.5 for the solve (dependent FP64 operations) and 2-3 for the
+// blocks to meet. A track of 25 iterations of 8,160 points: 0.41 ms, one of 15 iterations of
+// 12,288: 0.32 ms.
+template <bool TRACK>
+__global__ void __launch_bounds__(kStepThreads, 2) k_gicp_step(const __grid_constant__ StepArgs a)
+{
+    extern __shared__ float4 track_smem[];                     // TRACK: Kept [kKeptPts][16 warps]
+    Kept *const cache = reinterpret_cast<Kept *>(track_smem);
+    __shared__ float s_acc[kBatchRows][kRowPts][33];
+    __shared__ int s_match[kBatchRows][kRowPts];
+    __shared__ uint64_t s_buf[kRowPts][64];
+    __shared__ float s_pose[12];
+    __shared__ double s_sys[kSys];
+    __shared__ int s_last, s_done;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n = *a.scount;
+    const int used = rows_used(n, a.rows);
+    const uint32_t epoch = TRACK && threadIdx.x == 0 ? ld_acquire(&a.state->sync) : 0u;
+#pragma unroll 1
+    for (uint32_t it = 0;; ++it) {
+        if (threadIdx.x < 12) s_pose[threadIdx.x] = TRACK ? __ldcg(&a.state->posef[threadIdx.x]) : a.pose.p[threadIdx.x];
+        __syncthreads();
+        int slot = 0;
+#pragma unroll 1
+        for (int v0 = blockIdx.x; v0 < used; v0 += kBatchRows * gridDim.x) {
+#pragma unroll
+            for (int b = 0; b < kBatchRows; ++b) s_acc[b][warp][lane] = 0.f;
+#pragma unroll 1
+            for (int base = 0; base + v0 * kRowPts < n; base += a.rows * kRowPts) {
+#pragma unroll 1
+                for (int b = 0; b < kBatchRows; ++b, ++slot) {
+                    const int v = v0 + b * (int)gridDim.x, i = base + v * kRowPts + warp;
+                    int j = -1;
+                    if (v < used && i < n) {                   // whole warp
+                        Kept *kept = TRACK && slot < kKeptPts ? cache + slot * kRowPts + warp : nullptr;
+                        float4 src;
+                        if (kept && it > 0) {
+                            src = kept->src;
+                        } else {
+                            src = a.spos[i];
+                            if (kept && lane == 0) {
+                                kept->src = src;
+                                kept->x0 = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+                        }
+                        j = match_point(a, transform(s_pose, src), kept, it == 0, s_buf[warp]);
+                        if (!TRACK && a.idx_out && lane == 0) a.idx_out[i] = j;
+                    }
+                    if (lane == 0) s_match[b][warp] = j;
+                }
+                if (!a.system) continue;
+                __syncthreads();
+                // the terms of the batch's points, one per thread (a point's ~300 operations
+                // are one dependent chain, paid once for the batch)
+                if (threadIdx.x < kBatchRows * kRowPts) {
+                    const int b = threadIdx.x / kRowPts, w = threadIdx.x % kRowPts, j = s_match[b][w];
+                    const int i = base + (v0 + b * (int)gridDim.x) * kRowPts + w;
+                    if (j >= 0)
+                        gn_terms(s_pose, transform(s_pose, a.spos[i]), a.mpos[j], a.mcov[2 * j], a.mcov[2 * j + 1],
+                                 a.scov[2 * i], a.scov[2 * i + 1], s_acc[b][w]);
+                }
+                __syncthreads();
+            }
+            if (!a.system) continue;
+            if (threadIdx.x < kBatchRows * 32 && lane < kSys) {
+                // the 16 points in a fixed order: pairs two apart, then neighbours, then fours
+                const int b = threadIdx.x >> 5, v = v0 + b * (int)gridDim.x;
+                float s = 0.f;
+#pragma unroll
+                for (int w = 0; w < kRowPts; w += 4) {
+                    const float(*r)[33] = &s_acc[b][w];
+                    s += (r[0][lane] + r[2][lane]) + (r[1][lane] + r[3][lane]);
+                }
+                if (v < used) a.partial[v * 32 + lane] = s;
+            }
+            __syncthreads();
+        }
+        if (!TRACK) return;
+        // (the barrier and thread 0's fence order every thread's rows before the count)
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(&a.state->blocks_done, 1) == (int)gridDim.x - 1;
+            __threadfence();
+        }
+        __syncthreads();
+        if (s_last) {
+            sum_partials(a.partial, used, s_sys);
+            if (warp == 0) {
+                double step2 = 0.0;
+                const bool done = solve_state(a.state, s_sys, step2);
+                if (lane == 0) {
+                    a.state->blocks_done = 0;
+                    s_done = done;
+                    __threadfence();
+                    st_release(&a.state->sync, epoch + it + 1u);
+                    // (stored before this block is counted in the next iteration)
+                    if (step2 >= 0.0) a.state->step = sqrt(step2);
+                }
+            }
+        } else if (threadIdx.x == 0) {
+            uint32_t t = 0;
+            while (ld_acquire(&a.state->sync) != epoch + it + 1u && ++t < kSyncSpins) {
+            }
+            if (t >= kSyncSpins) {                             // recorded; the block ends
+                atomicOr(&a.state->status, 4);
+                s_done = 1;
+            } else {
+                s_done = __ldcg(&a.state->done);
+            }
+        }
+        __syncthreads();
+        if (s_done) return;
+    }
+}
+
+// Sum of the rows of partials in a fixed order: warp w takes rows w, w + nw, ..., one
+// column per lane, and adds them without a rounding that matters: with sigma a power of two
+// above the sum of their magnitudes, (v + sigma) - sigma is v's part in multiples of
+// sigma's last place, whose sum is exact (Rump, Ogita and Oishi 2008); the rests are split
+// and added the same way once more, which leaves 2^-34 of the largest row to a plain sum.
+// The warps' three parts are then added in FP64 in warp order. FP64 adds and conversions
+// run at 2 lanes per cycle and SM on this chip: adding 510 rows in FP64 took one block
+// about 9 us, this 2-3 us. Partials are read through L2 (written by other blocks of the
+// same grid).
+__device__ void sum_partials(const float *partial, int nrows, double *sys)
+{
+    constexpr int kWarps = kStepThreads / 32, kPer = (kMaxRows + kWarps - 1) / kWarps;
+    __shared__ double part[kWarps][kSys];
+    const int w = threadIdx.x >> 5, k = threadIdx.x & 31;
     if (k < kSys) {
-        // eight independent sums keep eight row loads in flight; added in a fixed order
-        double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        int b = w;
-        for (; b + 7 * nw < nblocks; b += 8 * nw) {
+        float v[kPer], top = 0.f;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) s[u] += (double)__ldcg(partial + (b + u * nw) * 32 + k);
+        for (int u = 0; u < kPer; ++u)
+            v[u] = w + u * kWarps < nrows ? __ldcg(partial + (w + u * kWarps) * 32 + k) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) top = fmaxf(top, fabsf(v[u]));
+        // the power of two above 64 times the largest (kPer < 64 rows)
+        const int e = (int)(__float_as_uint(top) >> 23) + 7;
+        double total = 0.0;
+        if (e < 254 && e > 32) {
+            const float s1 = __uint_as_float((uint32_t)e << 23), s2 = __uint_as_float((uint32_t)(e - 17) << 23);
+            float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                const float h = __fsub_rn(__fadd_rn(v[u], s1), s1), r = __fsub_rn(v[u], h);
+                const float m = __fsub_rn(__fadd_rn(r, s2), s2);
+                a1 = __fadd_rn(a1, h);
+                a2 = __fadd_rn(a2, m);
+                a3 = __fadd_rn(a3, __fsub_rn(r, m));
+            }
+            total = ((double)a1 + (double)a2) + (double)a3;
+        } else {                                                // infinities, NaN, subnormals
+            for (int u = 0; u < kPer; ++u) total += (double)v[u];
         }
-        for (int u = 0; b < nblocks; b += nw, ++u) s[u & 7] += (double)__ldcg(partial + b * 32 + k);
-        part[w][k] = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+        part[w][k] = total;
     }
     __syncthreads();
     if (threadIdx.x < kSys) {
-        double s = 0.0;
-        for (int q = 0; q < nw; ++q) s += part[q][threadIdx.x];
-        sys[threadIdx.x] = s;
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < kStepThreads / 32; ++q) s[q & 3] += part[q][threadIdx.x];
+        sys[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
     }
     __syncthreads();
 }
 
-__global__ void k_gicp_sum(const float *partial, int nblocks, double *out)
+__global__ void __launch_bounds__(kStepThreads) k_gicp_sum(const float *partial, const int32_t *count, int rows,
+                                                           double *out)
 {
     __shared__ double sys[kSys];
-    sum_partials(partial, nblocks, sys);
+    sum_partials(partial, rows_used(*count, rows), sys);
     if (threadIdx.x < kSys) out[threadIdx.x] = sys[threadIdx.x];
 }
 
-__device__ void exp_so3(const double w[3], double E[3][3])
+// Reciprocal of a positive, normal d: the hardware's approximation (error e0 ~ 2^-20) and one
+// step of the third-order Newton iteration r (1 + e + e^2), e = 1 - d r, which leaves e0^3.
+__device__ __forceinline__ double reciprocal(double d)
 {
-    const double th = sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
-    const double K[3][3] = {{0.0, -w[2], w[1]}, {w[2], 0.0, -w[0]}, {-w[1], w[0], 0.0}};
-    double a, b;
-    if (th < 1e-12) {
-        a = 1.0;
-        b = 0.5;
-    } else {
-        a = sin(th) / th;
-        b = (1.0 - cos(th)) / (th * th);
-    }
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) {
-            double kk = 0.0;
-            for (int m = 0; m < 3; ++m) kk += K[r][m] * K[m][c];
-            E[r][c] = (r == c ? 1.0 : 0.0) + a * K[r][c] + b * kk;
-        }
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
-// One thread: from the summed system, a Cholesky solve of H xi = -g in FP64 and the
-// pose update (R, t) <- (Exp(omega) R, Exp(omega) t + v).
-__device__ void solve_state(GicpState *st, const double *sys)
+// One warp: from the summed system, an L D L^T solve of H xi = -g in FP64 and the pose
+// update (R, t) <- (Exp(omega) R, Exp(omega) t + v); returns whether the track is over, and
+// |xi|^2 (-1: no step) in step2.
+// Lane r < 6 holds row r of H and lane 6 the row -g, whose factor is the forward
+// substitution; FP64 operations are slow and dependent here, so the rows go side by side,
+// with reciprocals instead of square roots (one thread with a Cholesky factor took ~20 us,
+// this ~3 us).
+__device__ bool solve_state(GicpState *st, const double *sys, double &step2)
 {
-    st->n = (int)sys[28];
-    st->cost = sys[27];
-    if (sys[28] < 6.0) {
-        st->status |= 2;
-        st->done = 1;
-        return;
+    const int lane = threadIdx.x & 31;
+    double old[3] = {0.0, 0.0, 0.0};                           // the column of the old pose that a lane needs
+    if (lane < 12) {
+#pragma unroll
+        for (int m = 0; m < 3; ++m) old[m] = st->pose[4 * m + (lane & 3)];
     }
-    double H[6][6], g[6];
-    int t = 0;
-    for (int r = 0; r < 6; ++r)
-        for (int c = r; c < 6; ++c) {
-            H[r][c] = sys[t];
-            H[c][r] = sys[t];
-            ++t;
-        }
-    for (int c = 0; c < 6; ++c) g[c] = sys[21 + c];
-    // Cholesky H = L L^T
-    double L[6][6] = {};
+    const int iters = st->iters + 1, max_iters = st->max_iters;
+    const double tol = (double)st->tol;
+    if (lane == 0) {
+        st->n = (int)sys[28];
+        st->cost = sys[27];
+    }
+    bool good = sys[28] >= 6.0;
+    const int row = min(lane, 6);
+    double A[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const int lo = min(row, c), hi = max(row, c);          // upper triangle, row by row
+        A[c] = row < 6 ? sys[lo * 6 - lo * (lo - 1) / 2 + hi - lo] : -sys[21 + c];
+    }
+    // column by column; A becomes the rows of L (unit diagonal), of lane 6 D^-1 L^-1 (-g)
+#pragma unroll
     for (int j = 0; j < 6; ++j) {
-        double d = H[j][j];
-        for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
-        if (!(d > 0.0)) {
+        const double d = __shfl_sync(kFull, A[j], j);
+        good = good && d > 0.0;
+        const double u = A[j];
+        A[j] = u * reciprocal(d);
+#pragma unroll
+        for (int c = j + 1; c < 6; ++c) A[c] -= A[j] * __shfl_sync(kFull, u, c);
+    }
+    if (!good) {                                               // uniform: too few points, or not positive definite
+        if (lane == 0) {
             st->status |= 2;
             st->done = 1;
-            return;
         }
-        L[j][j] = sqrt(d);
-        for (int i = j + 1; i < 6; ++i) {
-            double s = H[i][j];
-            for (int k = 0; k < j; ++k) s -= L[i][k] * L[j][k];
-            L[i][j] = s / L[j][j];
+        step2 = -1.0;
+        return true;
+    }
+    // back substitution
+    double xi[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) xi[c] = __shfl_sync(kFull, A[c], 6);
+#pragma unroll
+    for (int i = 5; i >= 1; --i)
+#pragma unroll
+        for (int c = 0; c < i; ++c) xi[c] -= __shfl_sync(kFull, A[c], i) * xi[i];
+    // Exp(omega) = I + a K + b K^2 with a = sin(th) / th, b = (1 - cos(th)) / th^2: their
+    // Taylor series for a small angle (the terms after the last are below 1e-17 of the sum)
+    const double t2 = xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2];
+    double ea, eb;
+    if (t2 < 0.01) {
+        ea = 1.0 + t2 * (-1.0 / 6 + t2 * (1.0 / 120 + t2 * (-1.0 / 5040 + t2 * (1.0 / 362880 - t2 * (1.0 / 39916800)))));
+        eb = 0.5 + t2 * (-1.0 / 24 + t2 * (1.0 / 720 + t2 * (-1.0 / 40320 + t2 * (1.0 / 3628800 - t2 * (1.0 / 479001600)))));
+    } else {
+        const double th = sqrt(t2);
+        ea = sin(th) / th;
+        eb = (1.0 - cos(th)) / t2;
+    }
+    // lane e < 12: element (e / 4, e % 4) of the new pose. K^2 = w w^T - th^2 I
+    if (lane < 12) {
+        const int r = lane >> 2, c = lane & 3;
+        const double w[3] = {xi[0], xi[1], xi[2]};
+        const double wr = r == 0 ? w[0] : (r == 1 ? w[1] : w[2]);
+        const double K[3] = {r == 0 ? 0.0 : (r == 1 ? w[2] : -w[1]), r == 0 ? -w[2] : (r == 1 ? 0.0 : w[0]),
+                             r == 0 ? w[1] : (r == 1 ? -w[0] : 0.0)};
+        double v = c == 3 ? (r == 0 ? xi[3] : (r == 1 ? xi[4] : xi[5])) : 0.0;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const double E = (r == m ? 1.0 - eb * t2 : 0.0) + ea * K[m] + eb * (wr * w[m]);
+            v += E * old[m];
         }
+        st->pose[lane] = v;
+        st->posef[lane] = (float)v;
     }
-    double y[6], xi[6];
-    for (int i = 0; i < 6; ++i) {
-        double s = -g[i];
-        for (int k = 0; k < i; ++k) s -= L[i][k] * y[k];
-        y[i] = s / L[i][i];
+    step2 = (t2 + xi[3] * xi[3]) + (xi[4] * xi[4] + xi[5] * xi[5]);
+    const bool conv = step2 < tol * tol;                       // |xi| < tol
+    const bool done = conv || iters >= max_iters;
+    if (lane == 0) {
+        st->iters = iters;
+        if (conv) st->converged = 1;
+        if (done) st->done = 1;
     }
-    for (int i = 5; i >= 0; --i) {
-        double s = y[i];
-        for (int k = i + 1; k < 6; ++k) s -= L[k][i] * xi[k];
-        xi[i] = s / L[i][i];
-    }
-    double E[3][3];
-    exp_so3(xi, E);
-    double Pn[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c)
-            Pn[4 * r + c] = E[r][0] * st->pose[c] + E[r][1] * st->pose[4 + c] + E[r][2] * st->pose[8 + c];
-        Pn[4 * r + 3] = E[r][0] * st->pose[3] + E[r][1] * st->pose[7] + E[r][2] * st->pose[11] + xi[3 + r];
-    }
-    for (int k = 0; k < 12; ++k) {
-        st->pose[k] = Pn[k];
-        st->posef[k] = (float)Pn[k];
-    }
-    double nrm = 0.0;
-    for (int k = 0; k < 6; ++k) nrm += xi[k] * xi[k];
-    st->step = sqrt(nrm);
-    st->iters += 1;
-    if (st->step < (double)st->tol) {
-        st->converged = 1;
-        st->done = 1;
-    } else if (st->iters >= st->max_iters) {
-        st->done = 1;
-    }
+    __syncwarp();
+    return done;
 }
 
 __global__ void k_gicp_init(GicpState *st, PoseD p0, int keep_pose, int max_iters, float tol, int done)
@@ -964,48 +1223,51 @@ struct InsArgs {
     int32_t *blk;
 };
 
+// Whether an indexed point lies within d_ov of x; whole warp.
 __device__ __forceinline__ bool overlaps(float3 x, const Grid &g, float d_ov)
 {
     const float d2ov = d_ov * d_ov;
-    const int ix = cell_of(x.x, g.inv_cell), iy = cell_of(x.y, g.inv_cell), iz = cell_of(x.z, g.inv_cell);
-    // cells of a third of max(r_max, d_ov) >= d_ov / 3: the three rings reach d_ov
-#pragma unroll 1
-    for (int r = 0; r <= 3; ++r) {
-        const int side = 2 * r + 1, ncube = side * side * side;
-#pragma unroll 1
-        for (int c = 0; c < ncube; ++c) {
-            const int dx = c % side - r, dy = (c / side) % side - r, dz = c / (side * side) - r;
-            if (max(abs(dx), max(abs(dy), abs(dz))) != r) continue;
-            const uint32_t h = cell_hash(ix + dx, iy + dy, iz + dz, g.mask);
-            const int e1 = g.off[h + 1];
-#pragma unroll 1
-            for (int e = g.off[h]; e < e1; ++e) {
-                const float4 b = g.pts[e];
-                if (sqdist(b.x, b.y, b.z, x.x, x.y, x.z) <= d2ov) return true;
-            }
-        }
-        if ((float)r * g.cell * (1.f - 1e-4f) >= d_ov) break;
-    }
-    return false;
+    bool hit = false;
+    const auto near = [&](float4 b) {
+        if (sqdist(b.x, b.y, b.z, x.x, x.y, x.z) <= d2ov) hit = true;
+    };
+    // cells of half of max(r_max, d_ov) >= d_ov / 2: two rings reach d_ov
+    ring_cells<1, true>(g, x, near);
+    if (__any_sync(kFull, hit)) return true;
+    if (g.cell * (1.f - 1e-4f) >= d_ov) return false;
+    ring_cells<2, false>(g, x, near);
+    return __any_sync(kFull, hit);
 }
 
-__global__ void __launch_bounds__(256) k_insert_flag(const __grid_constant__ InsArgs a)
+// One warp per source point, kInsPts points per block: the search is a chain of dependent
+// loads, so it takes a warp's lanes for the 27 nearest cells at once.
+__global__ void __launch_bounds__(1024) k_insert_flag(const __grid_constant__ InsArgs a)
 {
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    bool keep = false;
-    if (i < *a.scount) {
-        const float3 x = transform(a.state->posef, a.spos[i]);
-        keep = *a.mcount == 0 || !overlaps(x, a.grid, a.d_ov);
-        a.flags[i] = keep ? 1 : 0;
+    __shared__ int s_keep[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n = *a.scount;
+    const bool empty = *a.mcount == 0;
+    int kept = 0;
+#pragma unroll 1
+    for (int k = 0; k < kInsPts / 32; ++k) {
+        const int i = blockIdx.x * kInsPts + k * 32 + warp;
+        if (i >= n) break;
+        const bool keep = empty || !overlaps(transform(a.state->posef, a.spos[i]), a.grid, a.d_ov);
+        if (lane == 0) a.flags[i] = keep ? 1 : 0;
+        kept += keep ? 1 : 0;
     }
-    const int n = __syncthreads_count(keep);
-    if (threadIdx.x == 0) a.blk[blockIdx.x] = n;
+    if (lane == 0) s_keep[warp] = kept;
+    __syncthreads();
+    if (warp == 0) {
+        const int tot = __reduce_add_sync(kFull, s_keep[lane]);
+        if (lane == 0) a.blk[blockIdx.x] = tot;
+    }
 }
 
 __global__ void __launch_bounds__(256) k_insert_write(const __grid_constant__ InsArgs a)
 {
     __shared__ int red[8];
-    const int prefix = block_prefix(a.blk, blockIdx.x, red);
+    const int prefix = block_prefix(a.blk, blockIdx.x * (256 / kInsPts), red);
     const int i = blockIdx.x * 256 + threadIdx.x;
     const int n = *a.scount;
     const bool keep = i < n && a.flags[i] != 0;
@@ -1043,11 +1305,6 @@ __global__ void __launch_bounds__(256) k_insert_write(const __grid_constant__ In
         a.state->map_old = old;
         a.state->ins_total = prefix + total;
     }
-}
-
-__global__ void k_insert_commit(GicpState *st, int32_t *mcount, int32_t mcap)
-{
-    *mcount = min(st->map_old + st->ins_total, mcap);
 }
 
 }  // namespace
@@ -1089,15 +1346,18 @@ sgad_status check_ws(void *ws, size_t bytes, size_t need)
 template <typename T>
 T *at(void *ws, size_t off) { return reinterpret_cast<T *>(static_cast<char *>(ws) + off); }
 
-// Map grid cells of a third of the larger search radius: correspondence and overlap
-// searches visit rings of cells until their result is proven (at most 3 rings).
-float cell_size(const sgad_gicp_params *p) { return fmaxf(p->r_max, p->d_overlap) * (1.001f / 3.f); }
+// Map grid cells of half the larger search radius: correspondence and overlap searches
+// visit rings of cells until their result is proven (at most 2 rings, 125 cells; cells of a
+// third took 343 to reach as far, most of them empty at the 2-8 cm spacing of a map's
+// points).
+float cell_size(const sgad_gicp_params *p) { return fmaxf(p->r_max, p->d_overlap) * (1.001f / 2.f); }
 
 Grid grid_of(const sgad_gicp_params *p, void *ws, const GLayout &L)
 {
     Grid g;
-    g.off = at<int32_t>(ws, L.hash_off);
+    g.head = at<int32_t>(ws, L.hash_head);
     g.pts = at<float4>(ws, L.hash_pts);
+    g.cap = p->map_capacity;
     g.cell = cell_size(p);
     g.inv_cell = 1.f / g.cell;
     g.mask = (uint32_t)L.table - 1u;
@@ -1110,30 +1370,23 @@ sgad_status launched(const char *what)
     return e == cudaSuccess ? SGAD_OK : report_error(SGAD_ERR_CUDA, what);
 }
 
-// Counting sort of a set's indices by the hash of their cells: counts, parallel scan,
-// fill (entries within a bucket in arbitrary order; queries do not depend on it).
-sgad_status hash_build(const float4 *pos, const int32_t *count, int32_t capacity, float inv_cell, int32_t table,
-                       int32_t *cnt, int32_t *off, float4 *pts, int32_t *tile_sums, cudaStream_t st)
+// Index of a set: empty chains, then every point linked into its cell's chain. `commit`:
+// the map update's state, whose new count is written to *count (see k_hash_link).
+sgad_status hash_build(const float4 *pos, int32_t *count, int32_t capacity, float inv_cell, int32_t table,
+                       int32_t *head, float4 *pts, const GicpState *commit, cudaStream_t st)
 {
-    if (cudaMemsetAsync(cnt, 0, (size_t)table * sizeof(int32_t), st) != cudaSuccess)
+    if (cudaMemsetAsync(head, 0, (size_t)table * sizeof(int32_t), st) != cudaSuccess)
         return report_error(SGAD_ERR_CUDA, "sgad_gicp: memset failed");
-    const uint32_t mask = (uint32_t)table - 1u;
-    const int blocks = (capacity + 255) / 256;
-    const int tiles = (table + kScanTile - 1) / kScanTile;
-    k_hash_count<<<blocks, 256, 0, st>>>(pos, count, inv_cell, mask, cnt);
-    k_scan_tiles<<<tiles, 256, 0, st>>>(cnt, table, tile_sums);
-    k_scan_top<<<1, 1024, 0, st>>>(tile_sums, tiles);
-    k_scan_write<<<tiles, 256, 0, st>>>(cnt, off, table, tile_sums);
-    k_hash_fill<<<blocks, 256, 0, st>>>(pos, count, inv_cell, mask, off, cnt, pts);
+    const int blocks = std::min((capacity + 255) / 256, 4 * 152);
+    k_hash_link<<<blocks, 256, 0, st>>>(pos, count, capacity, inv_cell, (uint32_t)table - 1u, head, pts, commit);
     return launched("sgad_gicp: index launch failed");
 }
 
 sgad_status build_index(const sgad_gicp_params *p, const sgad_gaussian_set *map, void *ws, const GLayout &L,
-                        cudaStream_t st)
+                        const GicpState *commit, cudaStream_t st)
 {
     return hash_build(reinterpret_cast<const float4 *>(map->pos), map->count, map->capacity, 1.f / cell_size(p),
-                      L.table, at<int32_t>(ws, L.hash_cnt), at<int32_t>(ws, L.hash_off), at<float4>(ws, L.hash_pts),
-                      at<int32_t>(ws, L.tile_sums), st);
+                      L.table, at<int32_t>(ws, L.hash_head), at<float4>(ws, L.hash_pts), commit, st);
 }
 
 StepArgs step_args(const sgad_gicp_params *p, const sgad_gaussian_set *src, const sgad_gaussian_set *map, void *ws,
@@ -1153,6 +1406,7 @@ StepArgs step_args(const sgad_gicp_params *p, const sgad_gaussian_set *src, cons
     a.kmatch = p->k_match;
     a.state = at<GicpState>(ws, L.state);
     a.partial = at<float>(ws, L.partial);
+    a.rows = L.rows;
     return a;
 }
 
@@ -1213,34 +1467,51 @@ extern "C" sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_cam
     a.capacity = out->capacity;
     a.blk = at<int32_t>(workspace, L.sel_counts);
     a.state = at<GicpState>(workspace, L.state);
+    // The neighbour search scans the selection grid around a point's cell, which needs the
+    // maps between cells and points (in the room of the hash grid's points, four words per
+    // point). A set of far fewer points than cells takes the hash grid instead.
+    const bool window = ncells <= 3ll * p->src_capacity;
+    a.point_cell = at<int32_t>(workspace, L.knn_pts);
+    a.cell_point = window ? a.point_cell + p->src_capacity : nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nb = (int)((ncells + kSelBlock - 1) / kSelBlock);
     k_select_count<<<nb, 256, 0, st>>>(a);
     k_select_write<<<nb, 256, 0, st>>>(a);
-    const float4 *pos = reinterpret_cast<const float4 *>(out->pos);
-    // the points' own hash grid for the neighbour search; its cells are about twice the
-    // selection spacing at 2 m (a performance choice only: the search proves its result)
-    const float cell = fmaxf(5e-3f, 2.f * (float)p->stride * 2.f / cam->fx);
-    Grid g;
-    g.off = at<int32_t>(workspace, L.knn_off);
-    g.pts = at<float4>(workspace, L.knn_pts);
-    g.cell = cell;
-    g.inv_cell = 1.f / cell;
-    g.mask = (uint32_t)L.knn_table - 1u;
-    if ((s = hash_build(pos, out->count, out->capacity, g.inv_cell, L.knn_table, at<int32_t>(workspace, L.knn_cnt),
-                        at<int32_t>(workspace, L.knn_off), at<float4>(workspace, L.knn_pts),
-                        at<int32_t>(workspace, L.tile_sums), st)))
-        return s;
-    const int sb = (out->capacity + (128 / kTeam) - 1) / (128 / kTeam);
-    float4 *cov = reinterpret_cast<float4 *>(out->cov), *nrm = reinterpret_cast<float4 *>(out->normal);
-    if (p->k_cov <= 8)
-        k_shape<8><<<sb, 128, 0, st>>>(pos, out->count, p->k_cov, p->eps, g, cov, nrm, knn_out);
-    else if (p->k_cov <= 16)
-        k_shape<16><<<sb, 128, 0, st>>>(pos, out->count, p->k_cov, p->eps, g, cov, nrm, knn_out);
-    else if (p->k_cov <= 24)
-        k_shape<24><<<sb, 128, 0, st>>>(pos, out->count, p->k_cov, p->eps, g, cov, nrm, knn_out);
-    else
-        k_shape<32><<<sb, 128, 0, st>>>(pos, out->count, p->k_cov, p->eps, g, cov, nrm, knn_out);
+    ShapeArgs sa;
+    std::memset(&sa, 0, sizeof(sa));
+    sa.pos = reinterpret_cast<const float4 *>(out->pos);
+    sa.count = out->count;
+    sa.K = p->k_cov;
+    sa.eps = p->eps;
+    sa.cov = reinterpret_cast<float4 *>(out->cov);
+    sa.normal = reinterpret_cast<float4 *>(out->normal);
+    sa.knn_out = knn_out;
+    const int sb = (out->capacity + kShapePts - 1) / kShapePts;
+    if (window) {
+        sa.w.point_cell = a.point_cell;
+        sa.w.cell_point = a.cell_point;
+        sa.w.ncx = a.ncx;
+        sa.w.ncy = (cam->height + p->stride - 1) / p->stride;
+        sa.w.step_x = (float)p->stride / cam->fx;
+        sa.w.step_y = (float)p->stride / cam->fy;
+        sa.w.x0 = -cam->cx / cam->fx;
+        sa.w.y0 = -cam->cy / cam->fy;
+        k_shape<true><<<sb, kShapeThreads, 0, st>>>(sa);
+    } else {
+        // cells of about twice the selection spacing at 2 m (a performance choice only: the
+        // search proves its result)
+        Grid &g = sa.g;
+        g.head = at<int32_t>(workspace, L.knn_head);
+        g.pts = at<float4>(workspace, L.knn_pts);
+        g.cell = fmaxf(5e-3f, 2.f * (float)p->stride * 2.f / cam->fx);
+        g.inv_cell = 1.f / g.cell;
+        g.mask = (uint32_t)L.knn_table - 1u;
+        g.cap = p->src_capacity;
+        if ((s = hash_build(sa.pos, out->count, out->capacity, g.inv_cell, L.knn_table,
+                            at<int32_t>(workspace, L.knn_head), at<float4>(workspace, L.knn_pts), nullptr, st)))
+            return s;
+        k_shape<false><<<sb, kShapeThreads, 0, st>>>(sa);
+    }
     return launched("sgad_gicp_frame: launch failed");
 }
 
@@ -1252,7 +1523,7 @@ extern "C" sgad_status sgad_gicp_index(const sgad_gicp_params *p, const sgad_gau
     if ((s = check_set(map, p->map_capacity, "sgad_gicp_index: bad map set"))) return s;
     const GLayout L = glayout(*p);
     if ((s = check_ws(workspace, ws_bytes, L.total))) return s;
-    return build_index(p, map, workspace, L, static_cast<cudaStream_t>(stream));
+    return build_index(p, map, workspace, L, nullptr, static_cast<cudaStream_t>(stream));
 }
 
 namespace {
@@ -1286,7 +1557,7 @@ extern "C" sgad_status sgad_gicp_correspond(const sgad_gicp_params *p, const sga
     StepArgs a = step_args(p, src, map, workspace, L);
     std::memcpy(a.pose.p, pose, sizeof(a.pose.p));
     a.idx_out = idx_out;
-    k_gicp_step<<<L.step_blocks, kStepThreads, 0, static_cast<cudaStream_t>(stream)>>>(a);
+    k_gicp_step<false><<<L.rows, kStepThreads, 0, static_cast<cudaStream_t>(stream)>>>(a);
     return launched("sgad_gicp_correspond: launch failed");
 }
 
@@ -1302,8 +1573,8 @@ extern "C" sgad_status sgad_gicp_linearize(const sgad_gicp_params *p, const sgad
     std::memcpy(a.pose.p, pose, sizeof(a.pose.p));
     a.system = 1;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    k_gicp_step<<<L.step_blocks, kStepThreads, 0, st>>>(a);
-    k_gicp_sum<<<1, 32, 0, st>>>(a.partial, L.step_blocks, system_out);
+    k_gicp_step<false><<<L.rows, kStepThreads, 0, st>>>(a);
+    k_gicp_sum<<<1, kStepThreads, 0, st>>>(a.partial, a.scount, L.rows, system_out);
     return launched("sgad_gicp_linearize: launch failed");
 }
 
@@ -1337,12 +1608,28 @@ extern "C" sgad_status sgad_gicp_track(const sgad_gicp_params *p, const sgad_gau
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     StepArgs a = step_args(p, src, map, workspace, L);
     a.system = 1;
-    a.use_state = 1;
-    k_gicp_init<<<1, 1, 0, st>>>(a.state, p0, pose0 ? 0 : 1, p->max_iters, p->tol, 0);
-    // one launch per iteration: each step's last block solves and updates the pose
-    for (int it = 0; it < p->max_iters; ++it) {
-        k_gicp_step<<<L.step_blocks, kStepThreads, 0, st>>>(a);
+    // every block of the tracking kernel waits for the others once an iteration, so its grid
+    // is what the device holds at once (a cooperative launch), at most a block per row
+    static int resident[64] = {};
+    constexpr size_t smem = kTrackSmem;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    int blocks = e == cudaSuccess && dev >= 0 && dev < 64 ? resident[dev] : 0;
+    if (e == cudaSuccess && blocks == 0) {
+        int per_sm = 0, sms = 0;
+        e = cudaFuncSetAttribute(k_gicp_step<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gicp_step<true>, kStepThreads, smem);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        blocks = per_sm * sms;
+        if (e == cudaSuccess && dev >= 0 && dev < 64) resident[dev] = blocks;
     }
+    if (e != cudaSuccess || blocks < 1) return report_error(SGAD_ERR_CUDA, "sgad_gicp_track: no resident blocks");
+    k_gicp_init<<<1, 1, 0, st>>>(a.state, p0, pose0 ? 0 : 1, p->max_iters, p->tol, 0);
+    void *args[] = {&a};
+    e = cudaLaunchCooperativeKernel((const void *)k_gicp_step<true>, dim3(std::min(blocks, L.rows)),
+                                    dim3(kStepThreads), args, smem, st);
+    if (e != cudaSuccess) return report_error(SGAD_ERR_CUDA, "sgad_gicp_track: cooperative launch failed");
     return launched("sgad_gicp_track: launch failed");
 }
 
@@ -1368,11 +1655,10 @@ extern "C" sgad_status sgad_gicp_insert(const sgad_gicp_params *p, const sgad_ga
     a.state = at<GicpState>(workspace, L.state);
     a.flags = at<int32_t>(workspace, L.ins_flags);
     a.blk = at<int32_t>(workspace, L.ins_counts);
-    k_insert_flag<<<L.max_blocks, 256, 0, st>>>(a);
+    k_insert_flag<<<(p->src_capacity + kInsPts - 1) / kInsPts, 1024, 0, st>>>(a);
     k_insert_write<<<L.max_blocks, 256, 0, st>>>(a);
-    k_insert_commit<<<1, 1, 0, st>>>(a.state, map->count, map->capacity);
     if ((s = launched("sgad_gicp_insert: launch failed"))) return s;
-    return build_index(p, map, workspace, L, st);
+    return build_index(p, map, workspace, L, a.state, st);
 }
 
 extern "C" sgad_status sgad_gicp_result(void *workspace, size_t ws_bytes, double pose[12], sgad_gicp_stats *stats,
