@@ -135,11 +135,13 @@ typedef struct {
 
 /* Backward compositing algorithm (default WARP_LOCAL). All give the same gradients up
  * to the order of floating-point additions.
- *   WARP_LOCAL: every warp independently takes (tile, 8x4 pixel block) units from a queue
- *     (heaviest tile first under the persistent schedule) and walks only the entries the
- *     forward's per-warp masks mark for its block, 32 per round with no block-wide
- *     barrier; per (entry, pixel) pair it keeps two numbers in shared memory, and one lane
- *     per entry sums them (bwd_batch does not apply).
+ *   WARP_LOCAL: in both passes every warp independently takes (tile, 8x4 pixel block) units
+ *     from a queue (heaviest tile first under the persistent schedule), with no block-wide
+ *     barrier. The forward walks only the entries whose alpha >= 1/255 box may touch the
+ *     block (up to 2^24 Gaussians the lists carry that as a mask) and lists the ones that
+ *     reached one of its pixels; the backward walks those, 32 per round; per (entry, pixel)
+ *     pair it keeps two numbers in shared memory, and one lane per entry sums them
+ *     (fwd_batch and bwd_batch do not apply).
  *   WARP_REDUCE: thread blocks walk the masked entries of a tile in batches of bwd_batch
  *     staged entries per block-wide barrier, evaluate each at all 32 pixels of a warp's
  *     block and reduce the per-pair moments over the warp.
@@ -162,7 +164,7 @@ typedef struct {
                                     written as zeros */
     int32_t fwd_batch;           /* list entries staged per thread-block barrier in forward
                                     compositing: 128, 192, 256, 384, 512, 768 or 1024;
-                                    0 = default (512) */
+                                    0 = default (512); not used with WARP_LOCAL */
     int32_t bwd_batch;           /* the same for the warp-reduced backward; 0 = default (256) */
     int32_t fwd_schedule;        /* SGAD_SCHEDULE_* of forward compositing (default TILES) */
     int32_t bwd_schedule;        /* SGAD_SCHEDULE_* of backward compositing (default TILES) */
@@ -192,9 +194,10 @@ const char *sgad_last_error(void);
  * every (Gaussian, view) pair (8 B each), per-tile offsets, counters, heavy-first order and the list of tiles sorted exactly (16 B per tile), the
  * per-pixel state kept for the backward pass (8 B per view pixel), two key arrays
  * (16 B per key), the per-pixel
- * contribution words of the pair-parallel backward (32 B per key + 1 KB per tile) and
- * the per-warp contribution masks the forward leaves for the warp-local and
- * warp-reduced backwards (1 B per key + 64 B per tile). */
+ * contribution words of the pair-parallel backward or the per-block lists of the warp-local
+ * one (32 B per key + 1 KB per tile) and the per-warp contribution masks the forward leaves
+ * for the warp-reduced backward or the block masks of the warp-local forward (1 B per key +
+ * 64 B per tile). */
 sgad_status sgad_workspace_size(const sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
                                 const sgad_camera *views, int32_t n_views, int64_t key_capacity,
                                 size_t *bytes);
@@ -211,10 +214,8 @@ sgad_status sgad_count_keys(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_k
  * projection and tile binning of every (Gaussian, view) pair, a per-tile sort by
  * (depth, index), and front-to-back compositing of colour, depth and alpha.
  * out[k] receives view k. The per-pixel final transmittance and contributor count, the
- * sorted tile lists and, per warp of 8x4 pixels and chunk of 32 list entries, the mask
- * of entries that reached one of those pixels are kept in the workspace for
- * sgad_backward(). If the keys do
- * not fit in key_capacity the outputs are left untouched and sgad_check() reports
+ * sorted tile lists and, per 8x4 pixel block, which entries reached one of its pixels are
+ * kept in the workspace for sgad_backward(). If the keys do not fit in key_capacity the outputs are left untouched and sgad_check() reports
  * SGAD_ERR_KEY_OVERFLOW together with the count needed. */
 sgad_status sgad_forward(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
                          const sgad_camera *views, int32_t n_views, sgad_images *out,
@@ -234,14 +235,14 @@ sgad_status sgad_backward(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
  * Sweeps the tile shapes {16x16, 8x32, 32x8}, the batch sizes {128, 192, 256, 384, 512}
  * (forward also 768 and 1024)
  * and the schedules {TILES, PERSISTENT} of both compositing passes (and, for the
- * backward, the warp-local algorithm, reported with batch -1, and the pair-parallel
- * algorithm, reported with batch 0 and charged with the cost of the contribution words
- * its forward writes), timing each candidate
+ * backward, the warp-local algorithm, reported with batch -1 and chosen with the time of
+ * its own forward, and the pair-parallel algorithm, reported with batch 0 and charged with
+ * the cost of the contribution words its forward writes), timing each candidate
  * with CUDA events on `stream` (median of `reps` runs after one warm-up), and stores the
  * fastest combination in ctx's options: per tile shape, binning + emission + sort is
  * timed once, then each (batch, schedule) of forward compositing, then of backward
  * compositing (including the clearing of the gradient accumulators) on the gradients
- * grad_in; the shape with the smallest sum of the three best times wins.
+ * grad_in; the combination with the smallest sum of the three times wins.
  *
  * kfs, views, out, grad_in and grads_out are as for sgad_forward() / sgad_backward();
  * the workspace must hold the keys of every tile shape tried (a shape whose keys do not

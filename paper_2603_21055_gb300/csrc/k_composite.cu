@@ -53,12 +53,13 @@ cudaError_t persistent_blocks(bool fwd, int batch, const Scene &sc, int max_bloc
 cudaError_t launch_composite(bool fwd, int batch, int schedule, int max_blocks, const Scene &sc, const World *world,
                              const uint32_t *off, const uint64_t *entries, float *pix_t, uint32_t *pix_n, float4 *gacc,
                              WsHeader *hdr, const uint32_t *order, uint32_t *contrib, uint32_t *wmask,
-                             cudaStream_t st)
+                             const uint8_t *bmask, cudaStream_t st)
 {
     if (sc.n_tiles <= 0) return cudaSuccess;
     CompositeArgs a = {};
     a.contrib = contrib;
     a.wmask = wmask;
+    a.bmask = bmask;
     for (int i = 0; i < sc.n_views && !fwd; ++i)
         if (sc.view[i].d_pose) a.pose = 1;
     a.world = world;
@@ -68,20 +69,20 @@ cudaError_t launch_composite(bool fwd, int batch, int schedule, int max_blocks, 
     a.pix_n = pix_n;
     a.gacc = gacc;
     a.hdr = hdr;
-    if (!fwd && batch < 0) {
-        // warp-local backward: resident warps take (tile, block) units from a queue, in
-        // the heavy-first tile order (persistent), in tile order, or view by view
+    if (batch < 0) {
+        // warp-local pass: resident warps take (tile, block) units from a queue, in the
+        // heavy-first tile order (persistent), in tile order, or view by view
         int blocks = 0;
-        cudaError_t e = persistent_blocks(false, batch, sc, max_blocks, &blocks);
+        cudaError_t e = persistent_blocks(fwd, batch, sc, max_blocks, &blocks);
         if (e != cudaSuccess) return e;
-        a.queue = &hdr->queue_bwd;
+        a.queue = fwd ? &hdr->queue_fwd : &hdr->queue_bwd;
         auto run = [&](int tile0, int n_tiles, const uint32_t *ord) {
             a.tile0 = tile0;
             a.n_launch_tiles = n_tiles;
             a.order = ord;
             cudaError_t r = cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), st);
             if (r != cudaSuccess) return r;
-            return dispatch(false, batch, sc, a, blocks < n_tiles ? blocks : n_tiles, nullptr, st);
+            return dispatch(fwd, batch, sc, a, blocks < n_tiles ? blocks : n_tiles, nullptr, st);
         };
         if (schedule == SGAD_SCHEDULE_PER_VIEW) {
             for (int i = 0; i < sc.n_views; ++i) {

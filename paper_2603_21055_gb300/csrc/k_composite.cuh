@@ -36,9 +36,9 @@
 // Gaussian atomic conflicts between neighbouring pixels), so the warp-reduced one above
 // is the default.
 //
-// A third backward, the warp-local one (k_composite_bwdl, the default), has no block-wide
-// barrier at all: every warp takes (tile, 8x4 pixel block) units from a queue and walks
-// only the entries its forward mask marks, 32 at a time. Each lane keeps its pixel's
+// A third backward, the warp-local one (k_composite_bwdl, the default) with a forward of its
+// own (k_composite_fwdl), has no block-wide barrier at all: every warp takes (tile, 8x4 pixel block) units from a queue and walks
+// only the entries its forward listed, 32 at a time. Each lane keeps its pixel's
 // reverse-walk state; per (entry, contributing pixel) it leaves two numbers in the warp's
 // shared memory (dL/dpower and the blend weight), and then one lane per entry sums its
 // pixels' moments and applies the chain rule. No (entry, lane) slot of a warp-wide
@@ -91,12 +91,18 @@ struct CompositeArgs {
     // for tile t, list chunk c (entries 32c .. 32c + 31) and forward thread i (its
     // pixel), word contrib[8 off[t] + 256 t + 256 c + i] has bit j set iff entry 32c + j
     // contributed to that pixel. Written for every chunk the pixel's warp walked.
+    // For the warp-local pair of passes the same room holds lists instead: of tile t with n
+    // entries, block wb's list of contributing list positions, ascending, starts at word
+    // 8 off[t] + 256 t + wb n, and its length is word 8 off[t] + 256 t + 8 n + wb.
     uint32_t *contrib;
     // Per-warp contribution masks (forward writes, warp-reduced backward reads): for tile
     // t, list chunk c and forward warp w (its 8x4 pixel block), word
     // wmask[(off[t] >> 2) + 16 t + 8 c + w] has bit j set iff entry 32c + j contributed to
     // a pixel of that block. Written for every chunk the warp walked.
     uint32_t *wmask;
+    // Block masks (warp-local forward; may be null): bit wb of byte i is clear when list
+    // entry i's alpha >= 1/255 box touches no pixel of block wb of its tile.
+    const uint8_t *bmask;
     int32_t pose;                 // some view wants its pose gradient (selects the kernel variant)
 };
 
@@ -365,6 +371,309 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks<B>())
     }
     const uint32_t wp = __reduce_add_sync(kFull, n_pairs), we = __reduce_add_sync(kFull, n_evals);
     if ((threadIdx.x & 31) == 0 && we) {
+        atomicAdd(&a.hdr->n_pairs, (unsigned long long)wp);
+        atomicAdd(&a.hdr->n_evals, (unsigned long long)we);
+    }
+}
+
+// ------------------------------------------------------------------ warp-local forward
+//
+// The forward of the warp-local backward. Work unit: one 8x4 pixel block of one tile, lane
+// = pixel, taken from an atomic queue by single warps (heaviest tile first when the tile
+// order is given), so that no warp waits for another: in the block-staged forward the eight
+// warps of a tile meet at a barrier per batch, stop at different depths and wait for the
+// deepest one, and for its tile to end. A unit walks its tile's list from the front:
+//   1. gather: the list positions whose block mask (a byte per entry, formed where the
+//      entries are emitted) has the block's bit, about 8 of 32, are appended to a ring in
+//      shared memory, 128 list entries per load;
+//   2. when the ring holds 32 (or the list ends), lane j projects and stages the ring's
+//      entry j and forms its box mask over the block, a bit transpose gives every lane the
+//      entries whose box covers its pixel, and each lane walks only those, in order, with
+//      the block-staged forward's arithmetic (bit-identical images);
+//   3. the entries that reached a pixel of the block are appended to the block's list for the
+//      backward.
+// Rounds of 32 entries that touch the block, instead of 32 consecutive ones, take the walk's
+// steps (the most candidates of any lane) per list chunk from 4.6 to 3.6 and the transposes
+// from one to a quarter. Without masks (more than 2^24 Gaussians) step 1 projects every
+// entry for each block: the L1 wavefronts of those gathers (16 B and 4 B from 32 lines per
+// chunk) were then as many as all others of the kernel (L1 at 80 %).
+// Measured on the room workload (8 keyframes of 640x480 into 8 views, 34 M entries, 130 M
+// contributing pairs): 1.08 ms in tile order, 1.01 ms heaviest first, against 1.85 and
+// 1.68 ms for the block-staged forward and 1.41 and 1.33 ms without masks; the masks cost
+// the count and the emission 0.08 ms. 4 blocks per SM (59 registers): 5 (48 registers)
+// take 1.14 and 1.07 ms. The two packed multiplies and adds, the exact halves and the
+// flushed exponential take the walk's step from about 60 to 48 instructions.
+constexpr int kFwdlThreads = 256;           // 8 independent warps per block
+#ifndef SGAD_FWDL_MINBLOCKS
+#define SGAD_FWDL_MINBLOCKS 4
+#endif
+
+// Two FP32 values in one 64-bit register, added, multiplied and fused by one instruction
+// each (sm_100 and later): the same rounding of each half as the scalar operations, at one
+// issue slot instead of two.
+typedef unsigned long long float2x;
+__device__ __forceinline__ float2x pack2(float x, float y)
+{
+    float2x r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void unpack2(float2x v, float &x, float &y)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ float2x add2(float2x a, float2x b)
+{
+    float2x r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float2x mul2(float2x a, float2x b)
+{
+    float2x r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float2x fma2(float2x a, float2x b, float2x c)
+{
+    float2x r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// e^x for x <= 0 as 2^(x log2 e), subnormal results flushed to zero (alphas below 1/255 are
+// skipped, so no result near them is used).
+__device__ __forceinline__ float exp_walk(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__fmul_rn(x, 1.44269504f)));
+    return r;
+}
+
+// A staged Gaussian as the warp-local passes keep it in shared memory:
+//   a = (px, py, -conic_a / 2, -conic_c / 2), b = (conic_b, opacity), c = (r, g, b, z)
+// The halves are exact, so the exponent -(conic_a dx^2 + conic_c dy^2) / 2 - conic_b dx dy
+// has the bits of gauss_alpha(). Its skip below kPowerSkip is left out: the alpha test takes
+// the same entries (alpha < 1/255 there for any opacity).
+struct __align__(16) WalkEntry {
+    float4 a, c;
+    float2 b, pad;
+};
+
+__device__ __forceinline__ void to_walk(const Staged &g, WalkEntry &e)
+{
+    e.a = make_float4(g.a.x, g.a.y, -0.5f * g.b.x, -0.5f * g.b.z);
+    e.c = g.c;
+    e.b = make_float2(g.b.y, g.b.w);
+}
+
+// Alpha of a staged Gaussian at the pixel whose negated coordinates are nq (its offset from
+// the mean in dx, dy); false when the entry is skipped.
+__device__ __forceinline__ bool walk_alpha(const float4 a, const float2 b, float2x nq, float &alpha, float &raw)
+{
+    const float2x d = add2(pack2(a.x, a.y), nq), d2 = mul2(d, d);
+    float dx, dy, xx, yy;
+    unpack2(d, dx, dy);
+    unpack2(d2, xx, yy);
+    const float power = __fsub_rn(__fmaf_rn(a.z, xx, __fmul_rn(a.w, yy)), __fmul_rn(b.x, __fmul_rn(dx, dy)));
+    raw = __fmul_rn(b.y, exp_walk(power));
+    alpha = fminf(kAlphaCap, raw);
+    return !(power > 0.0f) && alpha >= kAlphaFloor;
+}
+
+constexpr int kRing = 256;                  // >= 31 + 128, a power of two
+struct FwdlWarpSmem {
+    WalkEntry e[32];                // the round's entries
+    uint32_t pos[kRing];            // ring: list positions of entries that may touch the block
+};
+constexpr size_t kFwdlSmemBytes = (kFwdlThreads / 32) * sizeof(FwdlWarpSmem);
+
+// Whether the alpha >= 1/255 box of a Gaussian (world record w0, opacity o) may touch the
+// pixels [bx, bx + 7] x [by, by + 3]. Never false when the exact box (stage()) does: the
+// mean's error from the approximate reciprocal is below 1e-6 of its terms, the half extents'
+// below 1e-5 of them.
+__device__ __forceinline__ bool may_touch(const float4 w0, float o, const ViewDev &v, float bxf, float byf)
+{
+    const float tx = __fmaf_rn(v.R[0], w0.x, __fmaf_rn(v.R[1], w0.y, __fmaf_rn(v.R[2], w0.z, v.t[0])));
+    const float ty = __fmaf_rn(v.R[3], w0.x, __fmaf_rn(v.R[4], w0.y, __fmaf_rn(v.R[5], w0.z, v.t[1])));
+    const float tz = __fmaf_rn(v.R[6], w0.x, __fmaf_rn(v.R[7], w0.y, __fmaf_rn(v.R[8], w0.z, v.t[2])));
+    const float iz = __fdividef(1.0f, tz);
+    const float ux = tx * iz, uy = ty * iz;
+    const float px = fmaf(v.fx, ux, v.cx), py = fmaf(v.fy, uy, v.cy);
+    const float l = __logf(255.0f * o) + 2e-6f;        // as in stage()
+    const float e = 2.0003f * l;                        // 2 l x 1.0001, raised
+    const float sz = w0.w * iz, jx = sz * v.fx, jy = sz * v.fy;
+    const float ex = e * fmaf(jx * jx, fmaf(ux, ux, 1.0f), kDilation);
+    const float ey = e * fmaf(jy * jy, fmaf(uy, uy, 1.0f), kDilation);
+    const float hx = fmaf(ex, rsqrtf(ex), fmaf(1e-6f, fabsf(px) + fabsf(v.cx), 0.03f));
+    const float hy = fmaf(ey, rsqrtf(ey), fmaf(1e-6f, fabsf(py) + fabsf(v.cy), 0.03f));
+    const float dx = px - (bxf + 3.5f), dy = py - (byf + 1.5f);
+    return l > 0.0f && fabsf(dx) <= hx + 3.5f && fabsf(dy) <= hy + 1.5f;
+}
+
+template <int TW, int TH, bool MASKS>
+__device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &a, int tile, int wb, FwdlWarpSmem &S,
+                                          int lane, uint32_t &n_pairs, uint32_t &n_evals)
+{
+    const ViewDev &v = sc.view[find_view_of_tile(sc, tile)];
+    const int local = tile - v.tile_base;
+    const int tx = local % v.tiles_x, ty = local / v.tiles_x;
+    const int bx = tx * TW + (wb % (TW / 8)) * 8, by = ty * TH + (wb / (TW / 8)) * 4;
+    const float bxf = (float)bx, byf = (float)by;
+    const int px = bx + (lane & 7), py = by + (lane >> 3);
+    const bool inside = px < v.W && py < v.H;
+    if (!__any_sync(kFull, inside)) return;
+    const float qx = (float)px, qy = (float)py;
+    const uint32_t s = a.off[tile], len = a.off[tile + 1] - s;
+    uint32_t *const room = a.contrib + contrib_base(a, tile, s);
+    uint32_t *const list = room + (size_t)wb * len;
+    const uint64_t *const ents = a.entries + s;
+
+    // the pixel's state: transmittance, colour and depth, alpha, last contributor
+    float T = 1.0f, aa = 0.f;
+    float2x acc_rg = pack2(0.f, 0.f), acc_bd = pack2(0.f, 0.f);
+    int last = -1;
+    bool done = !inside;
+    const float2x nq = pack2(-qx, -qy);
+    uint32_t n_list = 0;
+    uint32_t head = 0;                                 // ring: first entry
+    int cnt = 0;                                       // and how many
+    // masks: four list entries per lane and load, from the 4-byte boundary at or before the
+    // list's first (positions below 0 are dropped); one load ahead
+    const int lead = (int)(s & 3u);
+    const uint32_t *const words = reinterpret_cast<const uint32_t *>(a.bmask + (s - lead));
+    int next = MASKS ? -lead : 0;                      // first position not gathered
+    const auto load_masks = [&](int p) {
+        return MASKS && p + 4 * lane < (int)len ? words[(p + lead) / 4 + lane] : 0u;
+    };
+    uint32_t word = load_masks(next);
+    for (;;) {
+        // 1. gather
+        while (cnt < 32 && next < (int)len) {
+            if (MASKS) {
+                const int p = next + 4 * lane;
+                uint32_t m = (word >> wb) & 0x01010101u;
+                if (p < 0) m &= 0xffffffffu << (8 * -p);
+                if (p + 4 > (int)len) m = p < (int)len ? m & (0xffffffffu >> (8 * (p + 4 - (int)len))) : 0u;
+                next += 128;
+                word = load_masks(next);
+                // place of the lane's entries: those of the lanes before it, in list order
+                int place = 0, total = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t bal = __ballot_sync(kFull, m >> (8 * k) & 1u);
+                    place += __popc(bal & lane_mask_lt(lane));
+                    total += __popc(bal);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (m >> (8 * k) & 1u) S.pos[(head + cnt + place++) & (kRing - 1)] = (uint32_t)(p + k);
+                cnt += total;
+            } else {
+                const int p = next + lane;
+                bool hit = false;
+                if (p < (int)len) {
+                    const uint32_t g = (uint32_t)ents[p];
+                    if (g < sc.n_gauss) hit = may_touch(a.world[g].w0, a.world[g].w1.x, v, bxf, byf);
+                }
+                const uint32_t hits = __ballot_sync(kFull, hit);
+                if (hit) S.pos[(head + cnt + __popc(hits & lane_mask_lt(lane))) & (kRing - 1)] = (uint32_t)p;
+                cnt += __popc(hits);
+                next += 32;
+            }
+        }
+        if (cnt == 0) break;
+        __syncwarp();
+        // 2. a round: the first 32 of the ring
+        const int n = min(cnt, 32);
+        uint32_t row = 0u;
+        uint32_t my_pos = 0u;
+        if (lane < n) {
+            my_pos = S.pos[(head + lane) & (kRing - 1)];
+            Staged g;
+            stage_entry(sc, a, v, ents[my_pos], g);
+            to_walk(g, S.e[lane]);
+            row = box_block_mask(g.a, bxf, byf);
+        }
+        uint32_t mine = warp_transpose32(row, lane);
+        __syncwarp();
+        if (done) mine = 0u;
+        n_evals += __popc(mine);                       // less the candidates left when the pixel stops
+        uint32_t bits = 0u;
+        while (__any_sync(kFull, mine != 0u)) {
+            if (mine) {
+                const uint32_t low = mine & (0u - mine);
+                mine ^= low;
+                const WalkEntry &g = S.e[31 - __clz(low)];
+                const float4 ga = g.a, gc = g.c;
+                const float2 gb = g.b;
+                float alpha, raw;
+                if (walk_alpha(ga, gb, nq, alpha, raw)) {
+                    const float test = __fmul_rn(T, __fsub_rn(1.0f, alpha));
+                    if (test < kTStop) {
+                        done = true;
+                        n_evals -= __popc(mine);
+                        mine = 0u;
+                    } else {
+                        bits |= low;
+                        const float w = __fmul_rn(alpha, T);
+                        const float2x ww = pack2(w, w);
+                        acc_rg = fma2(ww, pack2(gc.x, gc.y), acc_rg);
+                        acc_bd = fma2(ww, pack2(gc.z, gc.w), acc_bd);
+                        aa = __fadd_rn(aa, w);
+                        T = test;
+                    }
+                }
+            }
+        }
+        n_pairs += __popc(bits);
+        if (bits) last = (int)S.pos[(head + 31 - __clz(bits)) & (kRing - 1)];
+        // 3. the block's list
+        const uint32_t reached = __reduce_or_sync(kFull, bits);
+        if (reached >> lane & 1u) list[n_list + __popc(reached & lane_mask_lt(lane))] = my_pos;
+        n_list += __popc(reached);
+        head += n;
+        cnt -= n;
+        __syncwarp();                                  // the ring's and the entries' readers are done
+        if (__all_sync(kFull, done)) break;
+    }
+    if (lane == 0) room[8 * (size_t)len + wb] = n_list;
+    if (inside) {
+        float cr, cg, cb, dd;
+        unpack2(acc_rg, cr, cg);
+        unpack2(acc_bd, cb, dd);
+        const size_t hw = (size_t)v.W * v.H, p = (size_t)py * v.W + px;
+        v.rgb[p] = cr + T * sc.bg[0];
+        v.rgb[hw + p] = cg + T * sc.bg[1];
+        v.rgb[2 * hw + p] = cb + T * sc.bg[2];
+        v.depth[p] = dd;
+        v.alpha[p] = aa;
+        a.pix_t[v.pix_base + p] = T;
+        a.pix_n[v.pix_base + p] = (uint32_t)(last + 1);
+    }
+}
+
+template <int TW, int TH, bool MASKS>
+__global__ void __launch_bounds__(kFwdlThreads, SGAD_FWDL_MINBLOCKS)
+    k_composite_fwdl(const __grid_constant__ Scene sc, const CompositeArgs a)
+{
+    static_assert(TW * TH == 256 && TW % 8 == 0 && TH % 4 == 0, "tile must hold eight 8x4 blocks");
+    __shared__ FwdlWarpSmem smem[kFwdlThreads / 32];
+    FwdlWarpSmem &S = smem[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    if (a.hdr->overflow) return;
+    const uint32_t n_units = (uint32_t)a.n_launch_tiles * 8u;
+    uint32_t n_pairs = 0, n_evals = 0;
+    for (;;) {
+        uint32_t u = 0u;
+        if (lane == 0) u = atomicAdd(a.queue, 1u);
+        u = __shfl_sync(kFull, u, 0);
+        if (u >= n_units) break;
+        const int tile = a.order ? (int)a.order[u >> 3] : a.tile0 + (int)(u >> 3);
+        fwdl_unit<TW, TH, MASKS>(sc, a, tile, (int)(u & 7u), S, lane, n_pairs, n_evals);
+    }
+    const uint32_t wp = __reduce_add_sync(kFull, n_pairs), we = __reduce_add_sync(kFull, n_evals);
+    if (lane == 0 && we) {
         atomicAdd(&a.hdr->n_pairs, (unsigned long long)wp);
         atomicAdd(&a.hdr->n_evals, (unsigned long long)we);
     }
@@ -937,12 +1246,12 @@ __global__ void __launch_bounds__(kPairThreads, 4) k_composite_bwdp(const __grid
 
 // ------------------------------------------------------------------ warp-local backward
 //
-// Work unit: one 8x4 pixel block of one tile, lane = pixel (the block of forward warp wb,
-// whose contribution masks mark the entries that reached one of these pixels). Units are
+// Work unit: one 8x4 pixel block of one tile, lane = pixel (the block wb of the warp-local
+// forward, whose list holds the entries that reached one of these pixels). Units are
 // taken from an atomic queue by single warps, heaviest tile first when the tile order is
-// given, so warps never wait for one another. A unit walks its marked entries from the
-// largest contributor count down in rounds of up to 32:
-//   1. gather: the next (lower) marked positions, highest first, one per lane;
+// given, so warps never wait for one another. A unit walks its list from the end in rounds
+// of up to 32:
+//   1. the next (lower) list positions, highest first, one per lane;
 //   2. stage: lane j projects entry j into the warp's shared memory and forms its box
 //      mask, the pixels of the block inside the entry's alpha >= 1/255 box;
 //   3. transpose the 32 x 32 bit matrix of box masks (five xor-shuffle steps), so that
@@ -1090,44 +1399,16 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
 #pragma unroll
     for (int q = 0; q < 12; ++q) pose[q] = 0.f;
 
-    // chunk c of the tile list (entries 32c .. 32c + 31) has this block's mask at wm[8 c];
-    // a window of 32 chunks is held one per lane, lane L the chunk cw - L
-    const uint32_t *wm = a.wmask + wmask_base(tile, s) + wb;
-    int cw = (fnc - 1) >> 5;
-    uint32_t wl = cw - lane >= 0 ? wm[8 * (cw - lane)] : 0u;     // bits of chunk cw - lane not yet taken
+    // the block's contributing list positions, as the forward left them
+    const uint32_t *const room = a.contrib + contrib_base(a, tile, s);
+    const uint32_t *const list = room + (size_t)wb * (uint32_t)len;
+    int left = min((int)room[8 * (size_t)len + wb], len);
     for (;;) {
-        // 1. gather up to 32 marked positions, highest first, into S.pos: a scan of the
-        // lanes' remaining bit counts orders the window's chunks, and each lane writes the
-        // highest bits of its chunk that still fit the round
-        int n = 0;
-        while (n < 32) {
-            const int cnt = __popc(wl);
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const int total = __shfl_sync(kFull, incl, 31);
-            if (total == 0) {
-                cw -= 32;
-                if (cw < 0) break;
-                wl = cw - lane >= 0 ? wm[8 * (cw - lane)] : 0u;
-                continue;
-            }
-            const int excl = incl - cnt;
-            int take = 32 - n - excl;
-            take = take < 0 ? 0 : (take > cnt ? cnt : take);
-            for (int t = 0; t < take; ++t) {
-                const int bit = 31 - __clz(wl);
-                wl &= ~(1u << bit);
-                S.pos[n + excl + t] = 32 * (cw - lane) + bit;
-            }
-            n += total < 32 - n ? total : 32 - n;
-        }
+        // 1. the next 32 positions from the end of the list
+        const int n = min(left, 32);
         if (n == 0) break;
-        __syncwarp();
-        const int my_pos = lane < n ? S.pos[lane] : 0;
+        const int my_pos = lane < n ? min((int)list[left - 1 - lane], len - 1) : 0;
+        left -= n;
         // 2. stage (lane j: entry j) and the box masks
         uint32_t my_g = 0u, row = 0u;
         float4 my_w0 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1369,15 +1650,31 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
     return cudaGetLastError();
 }
 
+template <int TW, int TH>
+cudaError_t launch_fwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks, int *occupancy, cudaStream_t st)
+{
+    if (occupancy)
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_fwdl<TW, TH, true>, kFwdlThreads, 0);
+    if (grid_blocks <= 0) return cudaSuccess;
+    if (a.bmask)
+        k_composite_fwdl<TW, TH, true><<<grid_blocks, kFwdlThreads, 0, st>>>(sc, a);
+    else
+        k_composite_fwdl<TW, TH, false><<<grid_blocks, kFwdlThreads, 0, st>>>(sc, a);
+    return cudaGetLastError();
+}
+
 // Dispatch on the batch size for one tile shape (instantiated in one translation unit per
-// shape); in the backward, batch 0 selects the pair-parallel kernel and a negative batch
-// the warp-local one. occupancy != nullptr: only report the resident blocks per SM.
+// shape); in the backward, batch 0 selects the pair-parallel kernel; a negative batch
+// selects the warp-local kernel of either pass. occupancy != nullptr: only report the
+// resident blocks per SM.
 template <int TW, int TH>
 cudaError_t launch_composite_shape(bool fwd, int batch, const Scene &sc, const CompositeArgs &a, int grid_blocks,
                                    int *occupancy, cudaStream_t st)
 {
     if (!fwd && batch == 0) return launch_bwdp<TW, TH>(sc, a, grid_blocks, occupancy, st);
-    if (!fwd && batch < 0) return launch_bwdl<TW, TH>(sc, a, grid_blocks, occupancy, st);
+    if (batch < 0)
+        return fwd ? launch_fwdl<TW, TH>(sc, a, grid_blocks, occupancy, st)
+                   : launch_bwdl<TW, TH>(sc, a, grid_blocks, occupancy, st);
 #define SGAD_BATCH_CASE(Bv)                                                                     \
     case Bv:                                                                                    \
         return occupancy ? occupancy_tb<TW, TH, Bv>(fwd, occupancy)                            \

@@ -29,9 +29,19 @@
 // exact 64-bit LSD order instead: passes on the index field, then on the depth field.
 // Larger buckets are sorted in cap-sized chunks the same way and then merged through
 // global memory, ping-ponging with a scratch key array.
+//
+// For the warp-local passes (PACK) an entry arrives with its index in 24 bits and the tile's
+// block mask in the low 8: the order is the same (a Gaussian is listed once per tile), and
+// the last write separates the plain entry from the mask, kept as one byte per entry.
 #include "sgad_device.cuh"
 
 namespace sgad {
+
+// The plain entry and the block mask of a packed one.
+__device__ __forceinline__ uint64_t plain_entry(uint64_t k)
+{
+    return (k & 0xffffffff00000000ull) | (uint32_t)((uint32_t)k >> 8);
+}
 
 constexpr unsigned kFull32 = 0xffffffffu;
 constexpr int kSortThreads = 512;
@@ -283,10 +293,10 @@ __device__ __forceinline__ void sort_tile_exact(const uint32_t *__restrict__ off
 
 // The tiles the bucket sort listed (hdr->n_sort_exact of them in `list`), taken by the
 // blocks of a fixed grid in turn.
-template <int kPer>
+template <int kPer, bool PACK>
 __global__ void __launch_bounds__(kSortThreads, kPer <= 12 ? 2 : 1)
     k_sort_tiles(const uint32_t *__restrict__ off, uint64_t *__restrict__ entries, uint64_t *__restrict__ alt, int cap,
-                 const WsHeader *hdr, const uint32_t *__restrict__ list)
+                 const WsHeader *hdr, const uint32_t *__restrict__ list, uint8_t *__restrict__ masks)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem &s = *reinterpret_cast<SortSmem *>(smem_raw);
@@ -294,8 +304,15 @@ __global__ void __launch_bounds__(kSortThreads, kPer <= 12 ? 2 : 1)
     if (hdr->overflow) return;
     const uint32_t n_list = hdr->n_sort_exact;
     for (uint32_t k = blockIdx.x; k < n_list; k += gridDim.x) {
-        sort_tile_exact<kPer>(off, entries, alt, cap, (int)list[k], s, ks);
+        const uint32_t t = list[k];
+        sort_tile_exact<kPer>(off, entries, alt, cap, (int)t, s, ks);
         __syncthreads();
+        if (PACK)
+            for (uint32_t i = off[t] + threadIdx.x; i < off[t + 1]; i += kSortThreads) {
+                const uint64_t key = entries[i];
+                entries[i] = plain_entry(key);
+                masks[i] = (uint8_t)key;
+            }
     }
 }
 
@@ -347,9 +364,10 @@ constexpr int kBucketEntries = kBucketThreads * kBucketPer;
 constexpr int kBucketBinsLog2 = 12;                     // at most 4,096 buckets
 constexpr int kBucketMax = 64;                          // larger buckets: exact path
 
+template <bool PACK>
 __global__ void __launch_bounds__(kBucketThreads, 3)
     k_sort_tiles_bucket(const uint32_t *__restrict__ off, uint64_t *__restrict__ entries, int cap, WsHeader *hdr,
-                        uint32_t *__restrict__ list)
+                        uint32_t *__restrict__ list, uint8_t *__restrict__ masks)
 {
     __shared__ __align__(16) uint32_t start[1 << kBucketBinsLog2];    // bucket counts, then bucket starts
     __shared__ uint32_t red[2][kBucketThreads / 32];
@@ -359,7 +377,14 @@ __global__ void __launch_bounds__(kBucketThreads, 3)
     const int t = blockIdx.x;
     const uint32_t s0 = off[t];
     const int n = (int)(off[t + 1] - s0);
-    if (n <= 1) return;
+    if (n <= 1) {
+        if (PACK && n == 1 && threadIdx.x == 0) {
+            const uint64_t key = entries[s0];
+            entries[s0] = plain_entry(key);
+            masks[s0] = (uint8_t)key;
+        }
+        return;
+    }
     if (n > cap || n > kBucketEntries) {
         if (threadIdx.x == 0) list[atomicAdd(&hdr->n_sort_exact, 1u)] = (uint32_t)t;
         return;
@@ -482,13 +507,14 @@ __global__ void __launch_bounds__(kBucketThreads, 3)
         int r = lo;
 #pragma unroll 4
         for (int j = lo; j < hi; ++j) r += ks[j] < key ? 1 : 0;
-        out[r] = key;
+        out[r] = PACK ? plain_entry(key) : key;
+        if (PACK) masks[s0 + r] = (uint8_t)key;
     }
 }
 
-template <int kPer>
+template <int kPer, bool PACK>
 static cudaError_t launch_sort(const uint32_t *off, uint64_t *entries, uint64_t *alt, int n_tiles, int cap,
-                               WsHeader *hdr, uint32_t *list, cudaStream_t st)
+                               WsHeader *hdr, uint32_t *list, uint8_t *masks, cudaStream_t st)
 {
     // Raise the kernel's dynamic shared-memory limit once per device and size (outside
     // any stream capture, which only replays launches).
@@ -498,36 +524,40 @@ static cudaError_t launch_sort(const uint32_t *off, uint64_t *entries, uint64_t 
     if (e != cudaSuccess) return e;
     const size_t smem = ((sizeof(SortSmem) + 15) & ~size_t(15)) + (size_t)cap * sizeof(uint64_t);
     if (dev < 0 || dev >= 64 || configured[dev] < (int)smem) {
-        e = cudaFuncSetAttribute(k_sort_tiles<kPer>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_sort_tiles<kPer, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = (int)smem;
     }
     static int bucket_configured[64] = {};
     constexpr int bucket_smem = kBucketEntries * (int)sizeof(uint64_t);
     if (dev < 0 || dev >= 64 || !bucket_configured[dev]) {
-        e = cudaFuncSetAttribute(k_sort_tiles_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize, bucket_smem);
+        e = cudaFuncSetAttribute(k_sort_tiles_bucket<PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, bucket_smem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) bucket_configured[dev] = 1;
     }
     if (n_tiles <= 0) return cudaSuccess;
-    k_sort_tiles_bucket<<<n_tiles, kBucketThreads, bucket_smem, st>>>(off, entries, cap, hdr, list);
+    k_sort_tiles_bucket<PACK><<<n_tiles, kBucketThreads, bucket_smem, st>>>(off, entries, cap, hdr, list, masks);
     // the listed tiles: a fixed grid (two blocks per SM) so the launch can be captured
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int grid = n_tiles < 2 * sms ? n_tiles : 2 * sms;
-    k_sort_tiles<kPer><<<grid, kSortThreads, smem, st>>>(off, entries, alt, cap, hdr, list);
+    k_sort_tiles<kPer, PACK><<<grid, kSortThreads, smem, st>>>(off, entries, alt, cap, hdr, list, masks);
     return cudaSuccess;
 }
 
 // cap in [64, 12288] (checked by the caller). list: n_tiles words of workspace for the
 // tiles the bucket sort hands to the exact radix sort (counted in hdr->n_sort_exact,
-// which the forward clears).
+// which the forward clears). masks: one byte per key for the block masks of packed entries,
+// null when the entries are plain.
 cudaError_t launch_sort_tiles(const uint32_t *off, uint64_t *entries, uint64_t *alt, int n_tiles, int cap,
-                              WsHeader *hdr, uint32_t *list, cudaStream_t st)
+                              WsHeader *hdr, uint32_t *list, uint8_t *masks, cudaStream_t st)
 {
-    if (cap <= kSortThreads * 12) return launch_sort<12>(off, entries, alt, n_tiles, cap, hdr, list, st);
-    return launch_sort<24>(off, entries, alt, n_tiles, cap, hdr, list, st);
+    if (cap <= kSortThreads * 12)
+        return masks ? launch_sort<12, true>(off, entries, alt, n_tiles, cap, hdr, list, masks, st)
+                     : launch_sort<12, false>(off, entries, alt, n_tiles, cap, hdr, list, masks, st);
+    return masks ? launch_sort<24, true>(off, entries, alt, n_tiles, cap, hdr, list, masks, st)
+                 : launch_sort<24, false>(off, entries, alt, n_tiles, cap, hdr, list, masks, st);
 }
 
 }  // namespace sgad

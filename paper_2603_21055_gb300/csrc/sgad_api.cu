@@ -9,13 +9,14 @@
 #include "sgad_device.cuh"
 
 namespace sgad {
-void launch_project_count(const Scene &, World *, uint32_t *, uint2 *, cudaStream_t);
+void launch_project_count(const Scene &, World *, uint32_t *, uint2 *, bool, cudaStream_t);
 void launch_scan_tiles(uint32_t *, uint32_t *, int, uint64_t, WsHeader *, uint32_t *, cudaStream_t);
-void launch_emit(const Scene &, const uint2 *, const uint32_t *, uint32_t *, uint64_t *, WsHeader *, cudaStream_t);
-cudaError_t launch_sort_tiles(const uint32_t *, uint64_t *, uint64_t *, int, int, WsHeader *, uint32_t *, cudaStream_t);
+void launch_emit(const Scene &, const uint2 *, const uint32_t *, uint32_t *, uint64_t *, WsHeader *, bool, cudaStream_t);
+cudaError_t launch_sort_tiles(const uint32_t *, uint64_t *, uint64_t *, int, int, WsHeader *, uint32_t *, uint8_t *,
+                              cudaStream_t);
 cudaError_t launch_composite(bool, int, int, int, const Scene &, const World *, const uint32_t *, const uint64_t *,
                              float *, uint32_t *, float4 *, WsHeader *, const uint32_t *, uint32_t *, uint32_t *,
-                             cudaStream_t);
+                             const uint8_t *, cudaStream_t);
 bool valid_batch(int, bool);
 void launch_finalize(const Scene &, const World *, const float4 *, cudaStream_t);
 void launch_l1_batch(int, const float *const *, const float *const *, const float *const *, const float *const *,
@@ -184,6 +185,9 @@ struct Ws {
     uint64_t *keys_alt() const { return reinterpret_cast<uint64_t *>(base + L.keys_alt); }
     uint32_t *contrib() const { return reinterpret_cast<uint32_t *>(base + L.contrib); }
     uint32_t *wmask() const { return reinterpret_cast<uint32_t *>(base + L.wmask); }
+    // the warp-local forward's block masks (1 B per key), in the room of the contribution
+    // masks, which it does not write
+    uint8_t *bmask() const { return reinterpret_cast<uint8_t *>(base + L.wmask); }
 };
 
 sgad_status get_ws(const Scene &sc, uint64_t n_pix, void *workspace, size_t ws_bytes, int64_t key_cap, Ws &ws)
@@ -218,6 +222,13 @@ bool uses_order(const sgad_options &o)
     return o.fwd_schedule == SGAD_SCHEDULE_PERSISTENT || o.bwd_schedule == SGAD_SCHEDULE_PERSISTENT;
 }
 
+// Whether the lists carry block masks for the warp-local forward: its entries' indices then
+// share 32 bits with the 8-bit mask until they are sorted.
+bool uses_masks(const sgad_options &o, const Scene &sc)
+{
+    return o.bwd_algorithm == SGAD_BWD_WARP_LOCAL && sc.n_gauss <= (1u << 24);
+}
+
 // Projection, binning count and scan: the part shared by sgad_count_keys and sgad_forward.
 sgad_status run_binning_count(const sgad_options &o, const Scene &sc, const Ws &ws, int64_t key_cap,
                               bool clear_sticky, cudaStream_t st)
@@ -225,7 +236,7 @@ sgad_status run_binning_count(const sgad_options &o, const Scene &sc, const Ws &
     cudaError_t e = cudaMemsetAsync(ws.hdr(), 0, clear_sticky ? sizeof(WsHeader) : kHeaderPerCall, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.tile_cnt(), 0, ((size_t)sc.n_tiles + 1) * 4, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-    launch_project_count(sc, ws.world(), ws.tile_cnt(), ws.rects(), st);
+    launch_project_count(sc, ws.world(), ws.tile_cnt(), ws.rects(), uses_masks(o, sc), st);
     launch_scan_tiles(ws.tile_cnt(), ws.tile_off(), sc.n_tiles, (uint64_t)key_cap, ws.hdr(),
                       uses_order(o) ? ws.tile_order() : nullptr, st);
     return last_launch("binning");
@@ -238,24 +249,26 @@ sgad_status run_forward_prep(sgad_ctx *ctx, const Scene &sc, const Ws &ws, int64
     sgad_status s = run_binning_count(ctx->opt, sc, ws, key_cap, false, st);
     if (s) return s;
     mark(ctx, 1, st);
-    launch_emit(sc, ws.rects(), ws.tile_off(), ws.tile_cnt(), ws.keys(), ws.hdr(), st);
+    const bool pack = uses_masks(ctx->opt, sc);
+    launch_emit(sc, ws.rects(), ws.tile_off(), ws.tile_cnt(), ws.keys(), ws.hdr(), pack, st);
     mark(ctx, 2, st);
     cudaError_t e = launch_sort_tiles(ws.tile_off(), ws.keys(), ws.keys_alt(), sc.n_tiles, ctx->sort_cap, ws.hdr(),
-                                      ws.sort_list(), st);
+                                      ws.sort_list(), pack ? ws.bmask() : nullptr, st);
     if (e != cudaSuccess) return cuda_fail(e, "sort launch");
     mark(ctx, 3, st);
     return last_launch("binning / emission / sort");
 }
 
-// One compositing pass. batch 0 in the backward selects the pair-parallel kernel; the
-// forward records contribution words when the context's backward is pair-parallel.
+// One compositing pass. batch 0 in the backward selects the pair-parallel kernel, a negative
+// batch the warp-local kernel of either pass; the block-staged forward records contribution
+// words when the context's backward is pair-parallel.
 sgad_status run_composite(const sgad_ctx *ctx, bool fwd, int batch, int schedule, const Scene &sc, const Ws &ws,
                           cudaStream_t st)
 {
-    uint32_t *contrib = (!fwd || ctx->opt.bwd_algorithm == SGAD_BWD_PAIRS) ? ws.contrib() : nullptr;
+    uint32_t *contrib = (!fwd || batch < 0 || ctx->opt.bwd_algorithm == SGAD_BWD_PAIRS) ? ws.contrib() : nullptr;
     const cudaError_t e = launch_composite(fwd, batch, schedule, ctx->opt.max_blocks, sc, ws.world(), ws.tile_off(), ws.keys(), ws.pix_t(),
                                            ws.pix_n(), fwd ? nullptr : ws.gacc(), ws.hdr(), ws.tile_order(), contrib,
-                                           ws.wmask(), st);
+                                           ws.wmask(), batch < 0 && uses_masks(ctx->opt, sc) ? ws.bmask() : nullptr, st);
     return e == cudaSuccess ? SGAD_OK : cuda_fail(e, fwd ? "forward compositing launch" : "backward compositing launch");
 }
 
@@ -267,6 +280,10 @@ int bwd_batch_of(const sgad_options &o)
     if (o.bwd_algorithm == SGAD_BWD_WARP_LOCAL) return -1;
     return o.bwd_batch;
 }
+
+// The batch argument of the forward launch: the warp-local backward reads the lists that the
+// warp-local forward leaves.
+int fwd_batch_of(const sgad_options &o) { return o.bwd_algorithm == SGAD_BWD_WARP_LOCAL ? -1 : o.fwd_batch; }
 
 // Output images of sgad_forward into the launch parameters.
 sgad_status bind_images(Scene &sc, const sgad_images *out, int n_views)
@@ -528,7 +545,7 @@ sgad_status sgad_forward(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf, 
     if (s) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     s = run_forward_prep(ctx, sc, ws, key_capacity, st);
-    if (!s) s = run_composite(ctx, true, ctx->opt.fwd_batch, ctx->opt.fwd_schedule, sc, ws, st);
+    if (!s) s = run_composite(ctx, true, fwd_batch_of(ctx->opt), ctx->opt.fwd_schedule, sc, ws, st);
     if (s) return s;
     mark(ctx, 4, st);
     ctx->fwd_recorded = ctx->profile;
@@ -744,11 +761,13 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
             continue;
         }
         float prep = 0.f;
+        trial.opt.bwd_algorithm = SGAD_BWD_WARP_LOCAL;
         s = timer.median(reps, st, [&] { return run_forward_prep(&trial, sc, ws, keys, st); }, &prep);
         if (s) return s;
         log.add(shape[0], shape[1], SGAD_TUNE_PREP, 0, 0, prep);
-        float best_f = -1.f, best_b = -1.f;
-        int fb = 0, fs = 0, bb = 0, bs = 0;
+        // Block-staged forwards (the warp-reduced and pair-parallel backwards' ones).
+        float best_f = -1.f;
+        int fb = 0, fs = 0;
         trial.opt.bwd_algorithm = SGAD_BWD_WARP_REDUCE;     // forwards without contribution words
         for (int sched : kScheds)
             for (int batch : kBatches) {
@@ -762,16 +781,33 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
                     fs = sched;
                 }
             }
-        // The pair-parallel backward needs the best forward to record contribution words;
-        // that extra forward cost is charged to the pair-parallel candidates.
-        trial.opt.bwd_algorithm = SGAD_BWD_PAIRS;
-        float fwd_words = 0.f;
-        s = timer.median(reps, st, [&] { return run_composite(&trial, true, fb, fs, sc, ws, st); }, &fwd_words);
-        if (s) return s;
-        const float words_cost = fwd_words > best_f ? fwd_words - best_f : 0.f;
+        // Each backward is timed after a forward that leaves what it reads: the warp-local
+        // pair of passes first, then the pair-parallel backward, whose forward also records
+        // contribution words, and the warp-reduced ones. A candidate's total takes the time
+        // of its own forward.
         static const int kBwdBatches[7] = {-1, 0, 128, 192, 256, 384, 512};  // -1: warp-local, 0: pair-parallel
-        for (int sched : kScheds)
-            for (int batch : kBwdBatches) {
+        for (int batch : kBwdBatches) {
+            float fwd_ms = best_f;
+            int fwd_sched = fs;
+            if (batch <= 0) {
+                trial.opt.bwd_algorithm = batch < 0 ? SGAD_BWD_WARP_LOCAL : SGAD_BWD_PAIRS;
+                fwd_ms = -1.f;
+                // (the block-staged forwards wrote over the block masks)
+                if (batch < 0 && (s = run_forward_prep(&trial, sc, ws, keys, st))) return s;
+                for (int sched : kScheds) {
+                    if (batch == 0 && sched != fs) continue;
+                    float ms = 0.f;
+                    s = timer.median(reps, st, [&] {
+                        return run_composite(&trial, true, batch < 0 ? -1 : fb, sched, sc, ws, st);
+                    }, &ms);
+                    if (s) return s;
+                    if (fwd_ms < 0.f || ms < fwd_ms) {
+                        fwd_ms = ms;
+                        fwd_sched = sched;
+                    }
+                }
+            }
+            for (int sched : kScheds) {
                 float ms = 0.f;
                 auto run = [&] {
                     const cudaError_t e = cudaMemsetAsync(ws.gacc(), 0, (size_t)sc.n_gauss * 32, st);
@@ -780,24 +816,19 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
                 };
                 s = timer.median(reps, st, run, &ms);
                 if (s) return s;
-                if (batch == 0) ms += words_cost;
+                if (batch == 0 && fwd_ms > best_f) ms += fwd_ms - best_f;      // the words' cost
                 log.add(shape[0], shape[1], SGAD_TUNE_BWD, batch, sched, ms);
-                if (best_b < 0.f || ms < best_b) {
-                    best_b = ms;
-                    bb = batch;
-                    bs = sched;
-                }
+                const float total = prep + (batch < 0 ? fwd_ms : best_f) + ms;
+                if (best_total >= 0.f && total >= best_total) continue;
+                best_total = total;
+                best.tile_w = shape[0];
+                best.tile_h = shape[1];
+                best.fwd_batch = fb;
+                best.fwd_schedule = fwd_sched;
+                best.bwd_algorithm = batch == 0 ? SGAD_BWD_PAIRS : (batch < 0 ? SGAD_BWD_WARP_LOCAL : SGAD_BWD_WARP_REDUCE);
+                best.bwd_batch = batch <= 0 ? ctx->opt.bwd_batch : batch;
+                best.bwd_schedule = sched;
             }
-        const float total = prep + best_f + best_b;
-        if (best_total < 0.f || total < best_total) {
-            best_total = total;
-            best.tile_w = shape[0];
-            best.tile_h = shape[1];
-            best.fwd_batch = fb;
-            best.fwd_schedule = fs;
-            best.bwd_algorithm = bb == 0 ? SGAD_BWD_PAIRS : (bb < 0 ? SGAD_BWD_WARP_LOCAL : SGAD_BWD_WARP_REDUCE);
-            best.bwd_batch = bb <= 0 ? ctx->opt.bwd_batch : bb;
-            best.bwd_schedule = bs;
         }
     }
     if (n_entries) *n_entries = log.n;

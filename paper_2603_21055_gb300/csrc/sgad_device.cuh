@@ -177,20 +177,45 @@ __device__ __forceinline__ int bin_rect(const Proj &p, const ViewDev &v, int tw_
 }
 
 // Tile rectangle of a (Gaussian, view) pair as the binning count leaves it for the key
-// emission: (tx0 | ty0 << 16, nx | ny << 16); nx = ny = 0 when it lists no tile.
-__device__ __forceinline__ uint2 pack_rect(const Rect &r, int n)
+// emission, a word per axis: first tile (11 bits: 16,384 pixels in tiles of 8), tile count
+// (12 bits, 0 when it lists no tile), and how many columns (rows) of 8x4 pixel blocks at
+// either end of the rectangle the Gaussian's alpha >= 1/255 box does not touch (4 bits each).
+struct Trim {
+    int lo, hi;
+};
+
+__device__ __forceinline__ uint32_t pack_span(int first, int n, Trim t)
 {
-    return n > 0 ? make_uint2((uint32_t)r.tx0 | ((uint32_t)r.ty0 << 16), (uint32_t)r.nx | ((uint32_t)r.ny << 16))
-                 : make_uint2(0u, 0u);
+    return (uint32_t)first | ((uint32_t)n << 11) | ((uint32_t)t.lo << 23) | ((uint32_t)t.hi << 27);
+}
+
+__device__ __forceinline__ uint2 pack_rect(const Rect &r, int n, Trim tx, Trim ty)
+{
+    return n > 0 ? make_uint2(pack_span(r.tx0, r.nx, tx), pack_span(r.ty0, r.ny, ty)) : make_uint2(0u, 0u);
 }
 
 __device__ __forceinline__ int unpack_rect(const uint2 q, Rect &r)
 {
-    r.tx0 = (int)(q.x & 0xffffu);
-    r.ty0 = (int)(q.x >> 16);
-    r.nx = (int)(q.y & 0xffffu);
-    r.ny = (int)(q.y >> 16);
+    r.tx0 = (int)(q.x & 0x7ffu);
+    r.ty0 = (int)(q.y & 0x7ffu);
+    r.nx = (int)(q.x >> 11 & 0xfffu);
+    r.ny = (int)(q.y >> 11 & 0xfffu);
     return r.nx * r.ny;
+}
+
+__device__ __forceinline__ Trim unpack_trim(uint32_t span)
+{
+    return {(int)(span >> 23 & 15u), (int)(span >> 27 & 15u)};
+}
+
+// Blocks of `size` pixels of [first, first + n) that [p - h, p + h] does not touch at either
+// end, at most 15 each (fewer trimmed is always allowed).
+__device__ __forceinline__ Trim block_trim(float p, float h, float inv_size, int first, int n)
+{
+    // block k holds the pixels size k .. size (k + 1) - 1
+    const int lo = __float2int_ru((fmaxf(p - h, -1e6f) + 1.0f) * inv_size) - 1;
+    const int hi = __float2int_rd(fminf(p + h, 1e6f) * inv_size);
+    return {min(max(lo - first, 0), 15), min(max(first + n - 1 - hi, 0), 15)};
 }
 
 // ------------------------------------------- double-float (Dekker/Knuth) arithmetic
