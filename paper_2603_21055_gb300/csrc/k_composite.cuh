@@ -92,8 +92,10 @@ struct CompositeArgs {
     // pixel), word contrib[8 off[t] + 256 t + 256 c + i] has bit j set iff entry 32c + j
     // contributed to that pixel. Written for every chunk the pixel's warp walked.
     // For the warp-local pair of passes the same room holds lists instead: of tile t with n
-    // entries, block wb's list of contributing list positions, ascending, starts at word
-    // 8 off[t] + 256 t + wb n, and its length is word 8 off[t] + 256 t + 8 n + wb.
+    // entries, block wb's list of the k contributing list positions, ascending, starts at
+    // word 8 off[t] + 256 t + wb n; entry i's mask of the pixels it reached (i < n - k: the
+    // others gave way to positions) is word n - 1 - i of the same n words; k is word
+    // 8 off[t] + 256 t + 8 n + wb.
     uint32_t *contrib;
     // Per-warp contribution masks (forward writes, warp-reduced backward reads): for tile
     // t, list chunk c and forward warp w (its 8x4 pixel block), word
@@ -628,10 +630,17 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
         }
         n_pairs += __popc(bits);
         if (bits) last = (int)S.pos[(head + 31 - __clz(bits)) & (kRing - 1)];
-        // 3. the block's list
-        const uint32_t reached = __reduce_or_sync(kFull, bits);
-        if (reached >> lane & 1u) list[n_list + __popc(reached & lane_mask_lt(lane))] = my_pos;
-        n_list += __popc(reached);
+        // 3. the block's list, and the pixels its entries reached from the other end of its
+        // room as long as the two do not meet
+        const uint32_t cm = warp_transpose32(bits, lane);
+        const uint32_t reached = __ballot_sync(kFull, cm != 0u);
+        const uint32_t end = n_list + __popc(reached);
+        if (cm) {
+            const uint32_t i = n_list + __popc(reached & lane_mask_lt(lane));
+            list[i] = my_pos;
+            if (i < len - end) list[len - 1 - i] = cm;
+        }
+        n_list = end;
         head += n;
         cnt -= n;
         __syncwarp();                                  // the ring's and the entries' readers are done
@@ -812,11 +821,22 @@ __device__ __forceinline__ Proj project_chain(const float4 w0, const ViewDev &v)
     return p;
 }
 
+// a / b to within an ulp, b not subnormal: the approximate reciprocal and one correction.
+__device__ __forceinline__ float quotient(float a, float b)
+{
+    const float r = __fdividef(1.0f, b), q = a * r;
+    return fmaf(fmaf(-q, b, a), r, q);
+}
+
 // Chain rule of one staged Gaussian from its ten accumulated pair moments (colour (3),
-// depth, G, G dx, G dy, G dx^2, G dx dy, G dy^2 with G = dL/dpower) down to d mu, d s,
-// d opacity and d colour, added to its accumulator.
+// depth, G, G dx, G dy, G dx^2, G dx dy, G dy^2 with G = dL/dpower) down to the depth
+// |D + delta| along its keyframe ray, s, opacity and colour, added to its accumulator when
+// its keyframe is learnable; returns d L / d t of its view-space centre. The centre's
+// gradient is taken along the ray here, per (block, Gaussian): a nearby view's gradient is
+// mostly across the ray, and sums of its three components, projected at the end, carried
+// their rounding (and its order) into a result 100 times smaller.
 __device__ __forceinline__ float3 chain_and_accumulate(const float *A, const Staged &st, const Proj &pr, float s_,
-                                                       const ViewDev &v, float4 *gacc, uint32_t g)
+                                                       const KfDev &k, const ViewDev &v, float4 *gacc, uint32_t g)
 {
     const float ca = st.b.x, cbb = st.b.y, cc = st.b.z, o = st.b.w;
     const float G = A[4], Gx = A[5], Gy = A[6], Gxx = A[7], Gxy = A[8], Gyy = A[9];
@@ -845,11 +865,21 @@ __device__ __forceinline__ float3 chain_and_accumulate(const float *A, const Sta
     const float gtz = gj00 * (-v.fx * iz2) + gj02 * (2.0f * v.fx * pr.tx * iz2 * iz) + gj11 * (-v.fy * iz2) +
                       gj12 * (2.0f * v.fy * pr.ty * iz2 * iz) + dpx * (-v.fx * pr.tx * iz2) +
                       dpy * (-v.fy * pr.ty * iz2) + A[3];
-    // t = R mu + t_k  ->  d mu = R^T d t
-    const float4 ga = make_float4(v.R[0] * gtx + v.R[3] * gty + v.R[6] * gtz, v.R[1] * gtx + v.R[4] * gty + v.R[7] * gtz,
-                                  v.R[2] * gtx + v.R[5] * gty + v.R[8] * gtz, ds);
-    atomicAdd(&gacc[2 * (size_t)g], ga);
-    atomicAdd(&gacc[2 * (size_t)g + 1], make_float4(d_o, A[0], A[1], A[2]));
+    if (k.learnable) {
+        // t = R mu + t_k, d mu / d |D + delta| = R_i r
+        const int j = (int)(g - k.gbase);
+        int row = (int)__fdividef((float)j, (float)k.W), col = j - row * k.W;   // one off at most
+        if (col < 0) --row, col += k.W;
+        if (col >= k.W) ++row, col -= k.W;
+        const float rx = quotient((float)col - k.cx, k.fx), ry = quotient((float)row - k.cy, k.fy);
+        const float ex = k.R[0] * rx + k.R[1] * ry + k.R[2], ey = k.R[3] * rx + k.R[4] * ry + k.R[5];
+        const float ez = k.R[6] * rx + k.R[7] * ry + k.R[8];
+        const float d_ray = gtx * (v.R[0] * ex + v.R[1] * ey + v.R[2] * ez) +
+                            gty * (v.R[3] * ex + v.R[4] * ey + v.R[5] * ez) +
+                            gtz * (v.R[6] * ex + v.R[7] * ey + v.R[8] * ez);
+        atomicAdd(&gacc[2 * (size_t)g], make_float4(d_ray, ds, d_o, A[0]));
+        atomicAdd(reinterpret_cast<float2 *>(&gacc[2 * (size_t)g + 1]), make_float2(A[1], A[2]));
+    }
     return make_float3(gtx, gty, gtz);
 }
 
@@ -1051,7 +1081,7 @@ __device__ __forceinline__ void bwd_tile(const Scene &sc, const CompositeArgs &a
                 for (int q = 0; q < 10; ++q) any |= A[q] != 0.f;
                 if (any) {
                     w0 = a.world[sg[k]].w0;
-                    gt = chain_and_accumulate(A, sm[k], project_chain(w0, v), w0.w, v, a.gacc, sg[k]);
+                    gt = chain_and_accumulate(A, sm[k], project_chain(w0, v), w0.w, sc.kf[find_kf(sc, sg[k])], v, a.gacc, sg[k]);
                 }
             }
             if (POSE && v.d_pose) pose_reduce(gt, w0, s_pose);
@@ -1215,7 +1245,7 @@ __device__ __forceinline__ void bwdp_tile(const Scene &sc, const CompositeArgs &
                 for (int q = 0; q < 10; ++q) any |= A[q] != 0.f;
                 if (any) {
                     w0 = a.world[sg[k]].w0;
-                    gt = chain_and_accumulate(A, sm[k], project_chain(w0, v), w0.w, v, a.gacc, sg[k]);
+                    gt = chain_and_accumulate(A, sm[k], project_chain(w0, v), w0.w, sc.kf[find_kf(sc, sg[k])], v, a.gacc, sg[k]);
                 }
             }
             if (POSE && v.d_pose) pose_reduce(gt, w0, s_pose);
@@ -1247,128 +1277,168 @@ __global__ void __launch_bounds__(kPairThreads, 4) k_composite_bwdp(const __grid
 // ------------------------------------------------------------------ warp-local backward
 //
 // Work unit: one 8x4 pixel block of one tile, lane = pixel (the block wb of the warp-local
-// forward, whose list holds the entries that reached one of these pixels). Units are
-// taken from an atomic queue by single warps, heaviest tile first when the tile order is
-// given, so warps never wait for one another. A unit walks its list from the end in rounds
-// of up to 32:
-//   1. the next (lower) list positions, highest first, one per lane;
-//   2. stage: lane j projects entry j into the warp's shared memory and forms its box
-//      mask, the pixels of the block inside the entry's alpha >= 1/255 box;
-//   3. transpose the 32 x 32 bit matrix of box masks (five xor-shuffle steps), so that
-//      each lane holds the entries whose box covers its pixel, and drop those at or past
-//      the pixel's contributor count;
-//   4. walk: each lane visits only its own entries, in order, recovers the transmittance
-//      by division, forms dL/dalpha from its suffix sums and, where the entry contributes,
-//      stores (G = alpha dL/dalpha, zero at the alpha cap; w = alpha T) in the entry's
-//      slot range of a per-warp pair buffer (a slot per box pixel);
-//   5. reduce: the lanes' contribution bits are transposed back, and lane j sums the ten
-//      moments of entry j over the pixels it reached (colour and depth: w times the
-//      pixel's image gradients; G, G dx, G dy, G dx^2, G dx dy, G dy^2), applies the chain
-//      rule and adds the result with two vector atomics.
-// Entries whose box slots do not fit the pair buffer together are walked and reduced in
-// consecutive sub-ranges. The per-pair arithmetic is the warp-reduced backward's; no
-// lane steps through an entry whose box misses its pixel.
+// forward, whose list holds the entries that reached one of these pixels and, per entry, the
+// mask of those pixels). Units are taken from an atomic queue by single warps, heaviest tile
+// first when the tile order is given, so warps never wait for one another. A unit walks its
+// list from the end in rounds of up to 32:
+//   1. stage: lane j projects entry j into the warp's shared memory; the transpose of the 32
+//      pixel masks gives every lane the entries that contributed to its pixel, exactly;
+//   2. walk, 16 entries at a time: each lane visits its own entries, in order, recovers the
+//      transmittance by division, forms dL/dalpha from its suffix sums and stores
+//      (G = alpha dL/dalpha, zero at the alpha cap; w = alpha T) at [entry][pixel] of a
+//      zeroed 16 x 32 buffer;
+//   3. moments: the ten sums of an entry over the pixels (colour and depth: w times the
+//      pixel's image gradients; G times 1, x, y, x^2, xy, y^2 of the pixel relative to the
+//      block's centre) are two 16 x 32 by 32 x 8 products on the tensor cores. Each FP32
+//      operand enters as the sum of two TF32 numbers (split_tf32), the coordinates' monomials
+//      are exact, and the products accumulate in FP32;
+//   4. chain: lane j moves entry j's moments to its mean, applies the chain rule down to the
+//      depth along the keyframe's ray and adds the result with two vector atomics.
+// A round's list words, entries and world records are loaded during the round before it.
+// Bound by issue (68 % of the slots at 24 warps per SM) and L1 wavefronts (70 %) together.
+// Room workload (8 x 640x480, 130 M contributing pairs): 1.34 ms against 1.56 ms with box
+// masks, candidates that miss and one lane per entry summing its pixels (a loop as long as
+// the entry with the most, 21.5 against a mean of 7.5). Of it (parts left out in copies) the
+// walk takes 0.56, the moments 0.41, the chain rule 0.12 and staging, masks and loads 0.35.
+// 4 blocks per SM (64 registers): 1.37 ms, 2: 1.64; the rounds loaded when needed: +0.04.
 constexpr int kLocalThreads = 256;          // 8 independent warps per block
-constexpr int kLocalPairCap = 512;          // (G, w) slots per warp
+constexpr int kHalf = 16;                   // entries per walk and product
+constexpr int kPairStride = 36;             // float2 per entry row: 32 pixels, conflict-free fragments
 #ifndef SGAD_BWDL_MINBLOCKS
-#define SGAD_BWDL_MINBLOCKS 4
+#define SGAD_BWDL_MINBLOCKS 3
 #endif
 
-struct LocalWarpSmem {
-    float4 sa[32], sb[32], sc[32];  // the round's entries (Staged a, b, c)
-    float4 pg[32];                  // image gradients (r, g, b, depth) of the unit's pixels
-    float2 pq[32];                  // their coordinates (x, y)
-    float2 pairs[kLocalPairCap];    // (G, w) per box pixel of each entry
-    uint32_t row[32];               // box mask of entry j over the block's pixels
-    int32_t base[32];               // first pair slot of entry j
-    int32_t pos[32];                // list position of entry j (descending in j)
+struct BwdlWarpSmem {
+    WalkEntry e[32];                        // the round's entries
+    float2 pairs[kHalf][kPairStride];       // (G, w) per entry and pixel
+    float mom[32][12];                      // ten moments per entry
 };
-constexpr size_t kLocalSmemBytes = (kLocalThreads / 32) * sizeof(LocalWarpSmem);
+constexpr size_t kLocalSmemBytes = (kLocalThreads / 32) * sizeof(BwdlWarpSmem);
 
-// Moments of the entries [j0, j1) of a round (lane j holds entry j: the pixels it
-// contributed to, cm, its Gaussian g and world record w0; its pair slots start at
-// base_j - b0), the chain rule, and the pose terms accumulated per lane. When the range
-// holds at most 16 entries, the lane 16 away from entry j's lane sums the moments of the
-// entry's bottom two pixel rows and hands them over with one shuffle per moment, so no
-// lane is idle and each walks at most half of an entry's pixels. Whole warp.
-template <bool POSE>
-__device__ __forceinline__ void bwdl_reduce(const ViewDev &v, const CompositeArgs &a, const LocalWarpSmem &S, int j0,
-                                            int j1, int lane, uint32_t cm, uint32_t g, float4 w0, int b0,
-                                            float (&pose)[12])
+// x as the sum of two TF32 operands: x itself, of which the product takes the leading 11
+// bits, and the rest (13 bits, of which it takes 11). Rounding both (two integer operations
+// more) measured the same gradient errors against FP64 (median 1.3e-5 relative on three
+// windows, from the FP32 means, as without tensor cores) and 2 % of the kernel's time; the
+// conversion instruction, at a fraction of the others' rate, 8 %.
+__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo)
 {
-    const bool split = j1 - j0 <= 16;
-    const uint32_t cm_x = __shfl_xor_sync(kFull, cm, 16);
-    const bool own = lane >= j0 && lane < j1;
-    int e = -1;
-    uint32_t m = 0u;
-    if (own) {
-        e = lane;
-        m = split ? (cm & 0xffffu) : cm;
-    } else if (split && (lane ^ 16) >= j0 && (lane ^ 16) < j1) {
-        e = lane ^ 16;
-        m = cm_x & 0xffff0000u;
-    }
-    float A[10];
+    hi = __float_as_uint(x);
+    lo = __float_as_uint(x - __uint_as_float(hi & 0xffffe000u));
+}
+
+// D += A B for a 16 x 8 (row-major) and an 8 x 8 (column-major) TF32 fragment.
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ float reciprocal_walk(float x)     // x in [0.01, 1]
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Fragment B of the colour and depth product: rows (pixels) 8 s + t and 8 s + t + 4, column
+// g = lane / 4 (t = lane % 4): the image gradients' high parts in columns 0 .. 3, their low
+// parts in 4 .. 7.
+struct GradFrags {
+    uint32_t b[4][2];
+};
+
+// Moments of the sixteen rows of S.pairs into rows h .. h + 15 of S.mom. Whole warp.
+__device__ __forceinline__ void bwdl_moments(BwdlWarpSmem &S, int h, int lane, const GradFrags &gf)
+{
+    const int g = lane >> 2, t = lane & 3;
+    float dw[4] = {0.f, 0.f, 0.f, 0.f}, dg[4] = {0.f, 0.f, 0.f, 0.f};
+    // column g of the monomials 1, x, y, x^2, x y, y^2 is al + be y + ga y^2 at the pixels
+    // x = t - 3.5 (row t) and x = t + 0.5 (row t + 4); y = s - 1.5
+    const float x0 = (float)t - 3.5f, x1 = (float)t + 0.5f;
+    const float ga = g == 5 ? 1.f : 0.f;
+    const float al0 = g == 0 ? 1.f : (g == 1 ? x0 : (g == 3 ? x0 * x0 : 0.f));
+    const float al1 = g == 0 ? 1.f : (g == 1 ? x1 : (g == 3 ? x1 * x1 : 0.f));
+    const float be0 = g == 2 ? 1.f : (g == 4 ? x0 : 0.f), be1 = g == 2 ? 1.f : (g == 4 ? x1 : 0.f);
 #pragma unroll
-    for (int q = 0; q < 10; ++q) A[q] = 0.f;
-    if (m) {
-        const float4 sa = S.sa[e];
-        const uint32_t row = S.row[e];
-        const int base = S.base[e] - b0;
-        while (m) {
-            const int p = __ffs(m) - 1;
-            m &= m - 1u;
-            const float2 gw = S.pairs[base + __popc(row & lane_mask_lt(p))];
-            const float4 pg = S.pg[p];
-            const float2 pq = S.pq[p];
-            const float dx = __fsub_rn(sa.x, pq.x);
-            const float dy = __fsub_rn(sa.y, pq.y);
-            A[0] += gw.y * pg.x;
-            A[1] += gw.y * pg.y;
-            A[2] += gw.y * pg.z;
-            A[3] += gw.y * pg.w;
-            const float G = gw.x;
-            A[4] += G;
-            A[5] += G * dx;
-            A[6] += G * dy;
-            A[7] += G * dx * dx;
-            A[8] += G * dx * dy;
-            A[9] += G * dy * dy;
-        }
-    }
-    if (split) {
+    for (int s = 0; s < 4; ++s) {
+        const float y = (float)s - 1.5f;
+        const float2 v[4] = {S.pairs[g][8 * s + t], S.pairs[g + 8][8 * s + t], S.pairs[g][8 * s + t + 4],
+                             S.pairs[g + 8][8 * s + t + 4]};
+        uint32_t hi[4], lo[4];
 #pragma unroll
-        for (int q = 0; q < 10; ++q) A[q] += __shfl_xor_sync(kFull, A[q], 16);
-    }
-    if (!own || cm == 0u) return;
-    Staged st;
-    st.a = S.sa[lane];
-    st.b = S.sb[lane];
-    st.c = S.sc[lane];
-    const float3 gt = chain_and_accumulate(A, st, project_chain(w0, v), w0.w, v, a.gacc, g);
-    if (POSE) {
+        for (int q = 0; q < 4; ++q) split_tf32(v[q].y, hi[q], lo[q]);
+        mma_tf32(dw, hi, gf.b[s][0], gf.b[s][1]);
+        mma_tf32(dw, lo, gf.b[s][0], gf.b[s][1]);
+        const uint32_t m0 = __float_as_uint(fmaf(y, fmaf(y, ga, be0), al0));
+        const uint32_t m1 = __float_as_uint(fmaf(y, fmaf(y, ga, be1), al1));
 #pragma unroll
-        for (int q = 0; q < 12; ++q) {
-            const float gq = (q >> 2) == 0 ? gt.x : ((q >> 2) == 1 ? gt.y : gt.z);
-            const int c = q & 3;
-            pose[q] += c == 3 ? gq : gq * (c == 0 ? w0.x : (c == 1 ? w0.y : w0.z));
-        }
+        for (int q = 0; q < 4; ++q) split_tf32(v[q].x, hi[q], lo[q]);
+        mma_tf32(dg, hi, m0, m1);
+        mma_tf32(dg, lo, m0, m1);
+    }
+    // columns 2 t, 2 t + 1 of rows g and g + 8; the low parts' columns join the high parts'
+#pragma unroll
+    for (int q = 0; q < 4; ++q) dw[q] += __shfl_xor_sync(kFull, dw[q], 2);
+    float *r0 = S.mom[h + g], *r1 = S.mom[h + g + 8];
+    if (t < 2) {
+        *reinterpret_cast<float2 *>(r0 + 2 * t) = make_float2(dw[0], dw[1]);
+        *reinterpret_cast<float2 *>(r1 + 2 * t) = make_float2(dw[2], dw[3]);
+    }
+    if (t < 3) {
+        *reinterpret_cast<float2 *>(r0 + 4 + 2 * t) = make_float2(dg[0], dg[1]);
+        *reinterpret_cast<float2 *>(r1 + 4 + 2 * t) = make_float2(dg[2], dg[3]);
     }
 }
 
-template <int TW, int TH, bool POSE, bool PLAIN>
-__device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &a, int tile, int wb, LocalWarpSmem &S,
+// Colour and depth moments of the pixels left out of the product: w times the gradients for
+// the entries that contributed there (mine: the lane's own), in FP32. Whole warp; slot: the
+// lane's entry's row of S.pairs, -1 for none in this product.
+static __device__ __noinline__ void add_not_finite(BwdlWarpSmem &S, int h, int slot, uint32_t bad, uint32_t mine,
+                                                   float gr, float gg, float gb, float gD)
+{
+    const int lane = threadIdx.x & 31;
+    while (bad) {
+        const int p = __ffs(bad) - 1;
+        bad &= bad - 1u;
+        const uint32_t theirs = __shfl_sync(kFull, mine, p);
+        const float g[4] = {__shfl_sync(kFull, gr, p), __shfl_sync(kFull, gg, p), __shfl_sync(kFull, gb, p),
+                            __shfl_sync(kFull, gD, p)};
+        if (slot >= 0 && (theirs >> lane & 1u)) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) S.mom[h + slot][c] += S.pairs[slot][p].y * g[c];
+        }
+    }
+    __syncwarp();
+}
+
+// FIXED: some keyframe is fixed. Its entries are walked (they take part in the pixels'
+// transmittance and suffix sums) but have no moments, unless the view's pose wants them: a
+// round whose other entries are at most 16 is one walk and one product, and nothing is added
+// for the fixed ones. 5 x 1200x680 with four of five keyframes fixed: 1.48 ms against 1.92
+// with all entries' moments (2.23 before the products). Without a fixed keyframe its checks
+// cost 45 us of 1.34 ms, so that case has its own instance.
+template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED>
+__device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &a, int tile, int wb, BwdlWarpSmem &S,
                                           int lane)
 {
     const ViewDev &v = sc.view[find_view_of_tile(sc, tile)];
     const int local = tile - v.tile_base;
     const int tx = local % v.tiles_x, ty = local / v.tiles_x;
     const int bx = tx * TW + (wb % (TW / 8)) * 8, by = ty * TH + (wb / (TW / 8)) * 4;
+    if (bx >= v.W || by >= v.H) return;                // (the forward skipped the block)
     const float bxf = (float)bx, byf = (float)by;
     const int px = bx + (lane & 7), py = by + (lane >> 3);
     const float qx = (float)px, qy = (float)py;
     const uint32_t s = a.off[tile];
     const int len = (int)(a.off[tile + 1] - s);
+    // the block's contributing list positions and their pixels, as the forward left them
+    const uint32_t *const room = a.contrib + contrib_base(a, tile, s);
+    const uint32_t *const list = room + (size_t)wb * (uint32_t)len;
+    const int total = min((int)room[8 * (size_t)len + wb], len);
+    if (total == 0) return;
+    const uint64_t *const ents = a.entries + s;
     const size_t hw = (size_t)v.W * v.H;
 
     float Tf = 1.0f, gr = 0.f, gg = 0.f, gb = 0.f, gD = 0.f, gA = 0.f;
@@ -1376,7 +1446,7 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
     if (px < v.W && py < v.H) {
         const size_t q = (size_t)py * v.W + px;
         Tf = a.pix_t[v.pix_base + q];
-        nc = min((int)a.pix_n[v.pix_base + q], len);
+        nc = (int)a.pix_n[v.pix_base + q];
         if (v.g_rgb) {
             gr = v.g_rgb[q];
             gg = v.g_rgb[hw + q];
@@ -1385,115 +1455,178 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
         if (v.g_depth) gD = v.g_depth[q];
         if (v.g_alpha) gA = v.g_alpha[q];
     }
-    const int fnc = (int)__reduce_max_sync(kFull, (unsigned)nc);
-    if (fnc == 0) return;
+    // the image gradients as fragments, through the moment rows
+    // (a pixel with a gradient that is not finite stays out of the product, where it would
+    // reach every entry of a round as 0 x inf; see add_not_finite)
+    GradFrags gf;
+    const bool fine = fabsf(gr) < 1e38f && fabsf(gg) < 1e38f && fabsf(gb) < 1e38f && fabsf(gD) < 1e38f;
+    const uint32_t bad = ~__ballot_sync(kFull, fine);
     __syncwarp();                       // the previous unit's readers of S are done
-    S.pg[lane] = make_float4(gr, gg, gb, gD);
-    S.pq[lane] = make_float2(qx, qy);
+    {
+        uint32_t hi[4], lo[4];
+        split_tf32(fine ? gr : 0.f, hi[0], lo[0]);
+        split_tf32(fine ? gg : 0.f, hi[1], lo[1]);
+        split_tf32(fine ? gb : 0.f, hi[2], lo[2]);
+        split_tf32(fine ? gD : 0.f, hi[3], lo[3]);
+        uint32_t *row = reinterpret_cast<uint32_t *>(S.mom[lane]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            row[c] = hi[c];
+            row[4 + c] = lo[c];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            gf.b[k][0] = __float_as_uint(S.mom[8 * k + (lane & 3)][lane >> 2]);
+            gf.b[k][1] = __float_as_uint(S.mom[8 * k + (lane & 3) + 4][lane >> 2]);
+        }
+    }
     const float bgdot = sc.bg[0] * gr + sc.bg[1] * gg + sc.bg[2] * gb;
     // Reverse-walk state: transmittance, and the suffix sums of colour and depth behind
     // the current entry already dotted with this pixel's image gradients (Sg = S_C . g_C
     // + S_D g_D, updated as Sg <- alpha (c . g) + (1 - alpha) Sg) plus the alpha suffix.
     float T = Tf, Sg = 0.f, SA = 0.f;
+    const float2x nq = pack2(-qx, -qy), g_rg = pack2(gr, gg), g_bd = pack2(gb, gD);
     float pose[12];
 #pragma unroll
     for (int q = 0; q < 12; ++q) pose[q] = 0.f;
 
-    // the block's contributing list positions, as the forward left them
-    const uint32_t *const room = a.contrib + contrib_base(a, tile, s);
-    const uint32_t *const list = room + (size_t)wb * (uint32_t)len;
-    int left = min((int)room[8 * (size_t)len + wb], len);
-    for (;;) {
-        // 1. the next 32 positions from the end of the list
+    // Lane j takes entry left - 1 - j of a round, so positions descend. A round's list words,
+    // entry and world record are loaded during the round before it.
+    const auto load_list = [&](int i, int &pos, uint32_t &row) {
+        pos = i >= 0 ? min((int)list[i], len - 1) : 0;
+        row = i >= 0 && i < len - total ? list[len - 1 - i] : 0u;
+    };
+    int pos;
+    uint32_t row;
+    load_list(total - 1 - lane, pos, row);
+    uint64_t ent = total - 1 - lane >= 0 ? ents[pos] : 0ull;
+    World w = a.world[(uint32_t)ent];
+    for (int left = total; left > 0;) {
+        // 1. stage
         const int n = min(left, 32);
-        if (n == 0) break;
-        const int my_pos = lane < n ? min((int)list[left - 1 - lane], len - 1) : 0;
-        left -= n;
-        // 2. stage (lane j: entry j) and the box masks
-        uint32_t my_g = 0u, row = 0u;
-        float4 my_w0 = make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool masked = left - 1 < len - total;    // the round's entries have their masks
+        const uint32_t my_g = (uint32_t)ent;
+        const float4 my_w0 = w.w0;
         if (lane < n) {
-            const uint64_t ent = a.entries[s + my_pos];
-            my_g = (uint32_t)ent;
-            const World w = a.world[my_g];
-            my_w0 = w.w0;
+            const Proj pr = project(w.w0, v);
             Staged st;
-            stage(project(w.w0, v), w.w1, __uint_as_float((uint32_t)(ent >> 32)), st);
-            S.sa[lane] = st.a;
-            S.sb[lane] = st.b;
-            S.sc[lane] = st.c;
-            row = box_block_mask(st.a, bxf, byf);
-        }
-        S.pos[lane] = lane < n ? my_pos : -1;
-        // 3. the entries whose box covers this pixel, before its contributor count
-        uint32_t mine = warp_transpose32(row, lane);
-        __syncwarp();
-        {
-            int lo = 0, hi = n;                 // first j with pos_j < nc (positions descend)
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (S.pos[mid] >= nc) lo = mid + 1; else hi = mid;
+            if (masked)
+                stage_conic(pr, w.w1, __uint_as_float((uint32_t)(ent >> 32)), st);
+            else {
+                stage(pr, w.w1, __uint_as_float((uint32_t)(ent >> 32)), st);
+                row = box_block_mask(st.a, bxf, byf);
             }
-            mine &= lo >= 32 ? 0u : (~0u << lo);
+            to_walk(st, S.e[lane]);
+            if (!masked) S.mom[lane][0] = __int_as_float(pos);
         }
-        // pair slots: entry j owns one slot per pixel it may reach (inside its box, before
-        // the pixel's contributor count), popc(row_j) slots from base_j (exclusive prefix)
-        row = warp_transpose32(mine, lane);
-        const int cnt = __popc(row);
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        S.row[lane] = row;
-        S.base[lane] = incl - cnt;
+        const uint32_t my_mask = row;
+        left -= n;
+        load_list(left - 1 - lane, pos, row);
+        uint32_t mine = warp_transpose32(my_mask, lane);
         __syncwarp();
-        // 4./5. walk and reduce, in sub-ranges whose box slots fit the pair buffer
-        int j0 = 0;
-        while (j0 < n) {
-            const int b0 = __shfl_sync(kFull, incl - cnt, j0);
-            const uint32_t fit = __ballot_sync(kFull, lane >= j0 && lane < n && incl - b0 <= kLocalPairCap);
-            const int j1 = fit ? 32 - __clz(fit) : j0 + 1;   // fit is a run of lanes from j0
-            const uint32_t range = (j1 >= 32 ? ~0u : ((1u << j1) - 1u)) & (~0u << j0);
-            uint32_t todo = mine & range, done = 0u;
+        if (!masked) {
+            // the entries of the box that contributed: alpha >= 1/255, before the pixel's stop
+            uint32_t cand = mine;
+            mine = 0u;
+            while (cand) {
+                const uint32_t low = cand & (0u - cand);
+                cand ^= low;
+                const int j = 31 - __clz(low);
+                float alpha, raw;
+                if (__float_as_int(S.mom[j][0]) < nc && walk_alpha(S.e[j].a, S.e[j].b, nq, alpha, raw)) mine |= low;
+            }
+            __syncwarp();
+        }
+        // the entries with moments, and the walks: 16 entries, or all with at most 16 moments
+        const int kf = FIXED ? find_kf(sc, my_g) : 0;
+        const bool own = lane < n && (!FIXED || POSE || sc.kf[kf].learnable);
+        const uint32_t with = FIXED ? __ballot_sync(kFull, own) : 0u;
+        const int span = FIXED && __popc(with) <= kHalf ? 32 : kHalf;
+        int my_row = lane;                             // this lane's entry's row of S.mom
+#pragma unroll 1
+        for (int h = 0; h < n; h += span) {
+            // 2. walk the entries h .. h + span - 1
+#pragma unroll
+            for (int k = 0; k < kHalf * 32 / 64; ++k) {
+                const int q = lane + 32 * k;             // 16 float4 per row
+                *reinterpret_cast<float4 *>(&S.pairs[q >> 4][2 * (q & 15)]) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            __syncwarp();
+            const uint32_t range = span == 32 ? kFull : 0xffffu << h;
+            uint32_t todo = mine & range;
             while (__any_sync(kFull, todo != 0u)) {
                 if (todo) {
-                    const int j = __ffs(todo) - 1;
-                    todo &= todo - 1u;
-                    Staged st;
-                    st.a = S.sa[j];
-                    st.b = S.sb[j];
-                    st.c = S.sc[j];
-                    float dx, dy, ep, alpha;
-                    const bool hit = gauss_alpha(st, qx, qy, dx, dy, ep, alpha);
-                    // evaluated for every candidate and kept by selects (no branch): a
-                    // candidate that misses writes its own pair slot, which the moment
-                    // loop never reads (it takes the hits only)
-                    {
-                        const float om = __fsub_rn(1.0f, alpha);
-                        const float rom = __fdividef(1.0f, om);     // om >= 0.01: fast reciprocal
-                        const float Ti = T * rom;
-                        const float cg = st.c.x * gr + st.c.y * gg + st.c.z * gb + st.c.w * gD;
-                        // PLAIN: no alpha gradient and no background (the terms are zero)
-                        const float dal = PLAIN ? Ti * (cg - Sg)
-                                                : Ti * ((cg - Sg) + (1.0f - SA) * gA) - (Tf * rom) * bgdot;
-                        Sg = hit ? alpha * cg + om * Sg : Sg;
-                        if (!PLAIN) SA = hit ? alpha + om * SA : SA;
-                        const float G = (st.b.w * ep > kAlphaCap) ? 0.f : dal * alpha;
-                        S.pairs[S.base[j] - b0 + __popc(S.row[j] & lane_mask_lt(lane))] = make_float2(G, alpha * Ti);
-                        T = hit ? Ti : T;
-                        done |= (hit ? 1u : 0u) << j;
-                    }
+                    const uint32_t low = todo & (0u - todo);
+                    todo ^= low;
+                    const int j = 31 - __clz(low);
+                    const WalkEntry &e = S.e[j];
+                    const float4 ea = e.a, ec = e.c;
+                    const float2 eb = e.b;
+                    float alpha, raw;
+                    walk_alpha(ea, eb, nq, alpha, raw);
+                    const float om = __fsub_rn(1.0f, alpha);
+                    const float rom = reciprocal_walk(om);
+                    const float Ti = T * rom;
+                    float ca, cb;
+                    unpack2(fma2(pack2(ec.z, ec.w), g_bd, mul2(pack2(ec.x, ec.y), g_rg)), ca, cb);
+                    const float cg = ca + cb;
+                    // PLAIN: no alpha gradient and no background (the terms are zero)
+                    const float dal = PLAIN ? Ti * (cg - Sg)
+                                            : Ti * ((cg - Sg) + (1.0f - SA) * gA) - (Tf * rom) * bgdot;
+                    Sg = alpha * cg + om * Sg;
+                    if (!PLAIN) SA = alpha + om * SA;
+                    const float2 pair = make_float2(raw > kAlphaCap ? 0.f : dal * alpha, alpha * Ti);
+                    if (!FIXED)
+                        S.pairs[j - h][lane] = pair;
+                    else if (with & low)
+                        S.pairs[__popc(with & range & (low - 1u))][lane] = pair;
+                    T = Ti;
                 }
             }
-            const uint32_t cm = warp_transpose32(done, lane);
             __syncwarp();
-            bwdl_reduce<POSE>(v, a, S, j0, j1, lane, cm, my_g, my_w0, b0, pose);
-            __syncwarp();               // the next sub-range overwrites the pair slots
-            j0 = j1;
+            // 3. their moments
+            if (!FIXED || (with & range)) {
+                bwdl_moments(S, h, lane, gf);
+                __syncwarp();
+                const bool here = FIXED ? own && (range >> lane & 1u) : lane >= h && lane < h + kHalf;
+                const int slot = FIXED ? __popc(with & range & lane_mask_lt(lane)) : lane - h;
+                if (FIXED && here) my_row = h + slot;
+                if (bad) add_not_finite(S, h, here ? slot : -1, bad, mine, gr, gg, gb, gD);
+            }
+            if (h == 0) ent = left - 1 - lane >= 0 ? ents[pos] : 0ull;
         }
-        if (n < 32) break;
+        w = a.world[(uint32_t)ent];
+        // 4. chain rule of entry `lane`
+        if (own) {
+            const float4 ea = S.e[lane].a;
+            const float2 eb = S.e[lane].b;
+            Staged st;
+            st.b = make_float4(-2.f * ea.z, eb.x, -2.f * ea.w, eb.y);
+            float A[10];
+#pragma unroll
+            for (int q = 0; q < 10; ++q) A[q] = S.mom[my_row][q];
+            // sums over the offsets (dx, dy) = (X, Y) - (x, y) of the pixels from the mean
+            const float X = ea.x - (bxf + 3.5f), Y = ea.y - (byf + 1.5f);
+            const float S0 = A[4], Sx = A[5], Sy = A[6];
+            const float Gx = fmaf(X, S0, -Sx), Gy = fmaf(Y, S0, -Sy);
+            A[7] = fmaf(X, Gx - Sx, A[7]);                               // X^2 S0 - 2 X Sx + Sxx
+            A[8] = fmaf(X, Gy, fmaf(-Y, Sx, A[8]));                      // X Y S0 - X Sy - Y Sx + Sxy
+            A[9] = fmaf(Y, Gy - Sy, A[9]);
+            A[5] = Gx;
+            A[6] = Gy;
+            const float3 gt = chain_and_accumulate(A, st, project_chain(my_w0, v), my_w0.w, sc.kf[FIXED ? kf : find_kf(sc, my_g)], v, a.gacc,
+                                                   my_g);
+            if (POSE) {
+#pragma unroll
+                for (int q = 0; q < 12; ++q) {
+                    const float gq = (q >> 2) == 0 ? gt.x : ((q >> 2) == 1 ? gt.y : gt.z);
+                    const int c = q & 3;
+                    pose[q] += c == 3 ? gq : gq * (c == 0 ? my_w0.x : (c == 1 ? my_w0.y : my_w0.z));
+                }
+            }
+        }
+        __syncwarp();                   // the next round's entries and moments
     }
     if (POSE && v.d_pose) {
 #pragma unroll
@@ -1506,13 +1639,13 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
     }
 }
 
-template <int TW, int TH, bool POSE, bool PLAIN>
+template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED>
 __global__ void __launch_bounds__(kLocalThreads, SGAD_BWDL_MINBLOCKS)
     k_composite_bwdl(const __grid_constant__ Scene sc, const CompositeArgs a)
 {
     static_assert(TW * TH == 256 && TW % 8 == 0 && TH % 4 == 0, "tile must hold eight 8x4 blocks");
     extern __shared__ float4 bwdl_smem[];
-    LocalWarpSmem &S = reinterpret_cast<LocalWarpSmem *>(bwdl_smem)[threadIdx.x >> 5];
+    BwdlWarpSmem &S = reinterpret_cast<BwdlWarpSmem *>(bwdl_smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     if (a.hdr->overflow) return;
     const uint32_t n_units = (uint32_t)a.n_launch_tiles * 8u;
@@ -1522,7 +1655,7 @@ __global__ void __launch_bounds__(kLocalThreads, SGAD_BWDL_MINBLOCKS)
         u = __shfl_sync(kFull, u, 0);
         if (u >= n_units) break;
         const int tile = a.order ? (int)a.order[u >> 3] : a.tile0 + (int)(u >> 3);
-        bwdl_unit<TW, TH, POSE, PLAIN>(sc, a, tile, (int)(u & 7u), S, lane);
+        bwdl_unit<TW, TH, POSE, PLAIN, FIXED>(sc, a, tile, (int)(u & 7u), S, lane);
     }
 }
 
@@ -1623,30 +1756,32 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        e = cudaFuncSetAttribute(k_composite_bwdl<TW, TH, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kLocalSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_composite_bwdl<TW, TH, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kLocalSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_composite_bwdl<TW, TH, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kLocalSmemBytes);
+        const void *all[] = {(const void *)k_composite_bwdl<TW, TH, false, false, true>,
+                             (const void *)k_composite_bwdl<TW, TH, false, true, false>,
+                             (const void *)k_composite_bwdl<TW, TH, false, true, true>,
+                             (const void *)k_composite_bwdl<TW, TH, true, false, true>};
+        for (const void *f : all)
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmemBytes);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = 1;
     }
     if (occupancy)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_bwdl<TW, TH, false, false>,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_bwdl<TW, TH, false, true, false>,
                                                              kLocalThreads, kLocalSmemBytes);
     if (grid_blocks <= 0) return cudaSuccess;
     // without an alpha gradient and with a black background the walk drops those terms
-    bool plain = sc.bg[0] == 0.0f && sc.bg[1] == 0.0f && sc.bg[2] == 0.0f;
+    bool plain = sc.bg[0] == 0.0f && sc.bg[1] == 0.0f && sc.bg[2] == 0.0f, fixed = false;
     for (int i = 0; i < sc.n_views && plain; ++i) plain = sc.view[i].g_alpha == nullptr;
+    for (int i = 0; i < sc.n_kf && !fixed; ++i) fixed = sc.kf[i].learnable == 0;
     if (a.pose)
-        k_composite_bwdl<TW, TH, true, false><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
-    else if (plain)
-        k_composite_bwdl<TW, TH, false, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+        k_composite_bwdl<TW, TH, true, false, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+    else if (!plain)
+        k_composite_bwdl<TW, TH, false, false, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+    else if (fixed)
+        k_composite_bwdl<TW, TH, false, true, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
     else
-        k_composite_bwdl<TW, TH, false, false><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+        k_composite_bwdl<TW, TH, false, true, false><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
     return cudaGetLastError();
 }
 

@@ -1,15 +1,14 @@
 // Per-Gaussian and per-pixel elementwise kernels:
-//   k_finalize   : last link of the adjoint (a10): d mu -> d delta through
-//                  mu = R_i |D + delta| r + t_i, d opacity -> d logit, written into the
-//                  caller's gradient planes of learnable keyframes.
+//   k_finalize   : last link of the adjoint (a10): d |D + delta| -> d delta,
+//                  d opacity -> d logit, written into the caller's gradient planes of
+//                  learnable keyframes.
 //   k_l1_grad    : L1 terms of Eq. 1 and their image gradients (a8).
 //   k_adam       : bias-corrected Adam step (a11).
 #include "sgad_device.cuh"
 
 namespace sgad {
 
-__global__ void __launch_bounds__(256) k_finalize(const __grid_constant__ Scene sc, const World *__restrict__ world,
-                                                  const float4 *__restrict__ gacc)
+__global__ void __launch_bounds__(256) k_finalize(const __grid_constant__ Scene sc, const float4 *__restrict__ gacc)
 {
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= sc.n_gauss) return;
@@ -17,30 +16,26 @@ __global__ void __launch_bounds__(256) k_finalize(const __grid_constant__ Scene 
     if (!k.learnable) return;
     const uint32_t j = g - k.gbase;
     const size_t hw = (size_t)k.W * k.H;
-    const float4 a = gacc[2 * (size_t)g], b = gacc[2 * (size_t)g + 1];
-    const float u = (float)(j % (uint32_t)k.W), v = (float)(j / (uint32_t)k.W);
-    const float rx = (u - k.cx) / k.fx, ry = (v - k.cy) / k.fy;
-    // d mu / d |D + delta| = R_i r
-    const float dir_x = k.R[0] * rx + k.R[1] * ry + k.R[2];
-    const float dir_y = k.R[3] * rx + k.R[4] * ry + k.R[5];
-    const float dir_z = k.R[6] * rx + k.R[7] * ry + k.R[8];
+    // (d |D + delta|, d s, d o, d r), (d g, d b)
+    const float4 a = gacc[2 * (size_t)g];
+    const float2 b = *reinterpret_cast<const float2 *>(&gacc[2 * (size_t)g + 1]);
     const float sum = k.depth[j] + k.offset[j];
     const float sgn = sum > 0.0f ? 1.0f : (sum < 0.0f ? -1.0f : 0.0f);
     // the opacity as the projection computed it (same expression: bit-identical), from the
     // 4-byte logit instead of the 32-byte world record
     const float o = 1.0f / (1.0f + expf(-k.logit[j]));
-    k.d_offset[j] = sc.freeze_offset ? 0.0f : sgn * (dir_x * a.x + dir_y * a.y + dir_z * a.z);
-    k.d_scale[j] = a.w;
-    k.d_logit[j] = b.x * o * (1.0f - o);
-    k.d_rgb[j] = b.y;
-    k.d_rgb[hw + j] = b.z;
-    k.d_rgb[2 * hw + j] = b.w;
+    k.d_offset[j] = sc.freeze_offset ? 0.0f : sgn * a.x;
+    k.d_scale[j] = a.y;
+    k.d_logit[j] = a.z * o * (1.0f - o);
+    k.d_rgb[j] = a.w;
+    k.d_rgb[hw + j] = b.x;
+    k.d_rgb[2 * hw + j] = b.y;
 }
 
-void launch_finalize(const Scene &sc, const World *world, const float4 *gacc, cudaStream_t st)
+void launch_finalize(const Scene &sc, const float4 *gacc, cudaStream_t st)
 {
     const unsigned blocks = (sc.n_gauss + 255) / 256;
-    if (blocks) k_finalize<<<blocks, 256, 0, st>>>(sc, world, gacc);
+    if (blocks) k_finalize<<<blocks, 256, 0, st>>>(sc, gacc);
 }
 
 __device__ __forceinline__ float sgnf(float x) { return x > 0.0f ? 1.0f : (x < 0.0f ? -1.0f : 0.0f); }

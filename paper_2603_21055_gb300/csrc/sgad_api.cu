@@ -18,7 +18,7 @@ cudaError_t launch_composite(bool, int, int, int, const Scene &, const World *, 
                              float *, uint32_t *, float4 *, WsHeader *, const uint32_t *, uint32_t *, uint32_t *,
                              const uint8_t *, cudaStream_t);
 bool valid_batch(int, bool);
-void launch_finalize(const Scene &, const World *, const float4 *, cudaStream_t);
+void launch_finalize(const Scene &, const float4 *, cudaStream_t);
 void launch_l1_batch(int, const float *const *, const float *const *, const float *const *, const float *const *,
                      const float *const *, float *const *, float *const *, uint32_t *, const uint32_t *, float, float,
                      float, float *, cudaStream_t);
@@ -257,6 +257,22 @@ sgad_status run_forward_prep(sgad_ctx *ctx, const Scene &sc, const Ws &ws, int64
     if (e != cudaSuccess) return cuda_fail(e, "sort launch");
     mark(ctx, 3, st);
     return last_launch("binning / emission / sort");
+}
+
+// Zeroes the gradient accumulators of the learnable keyframes (the others' are not used),
+// neighbours in one call.
+cudaError_t clear_accumulators(const Scene &sc, const Ws &ws, cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < sc.n_kf && e == cudaSuccess;) {
+        int j = i;
+        while (j < sc.n_kf && (sc.kf[j].learnable != 0) == (sc.kf[i].learnable != 0)) ++j;
+        const uint32_t from = sc.kf[i].gbase, to = j < sc.n_kf ? sc.kf[j].gbase : sc.n_gauss;
+        if (sc.kf[i].learnable)
+            e = cudaMemsetAsync(ws.gacc() + 2 * (size_t)from, 0, (size_t)(to - from) * 32, st);
+        i = j;
+    }
+    return e;
 }
 
 // One compositing pass. batch 0 in the backward selects the pair-parallel kernel, a negative
@@ -566,14 +582,14 @@ sgad_status sgad_backward(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
     if (s) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     mark(ctx, 5, st);
-    cudaError_t e = cudaMemsetAsync(ws.gacc(), 0, (size_t)sc.n_gauss * 32, st);
+    cudaError_t e = clear_accumulators(sc, ws, st);
     for (int i = 0; i < n_views && e == cudaSuccess; ++i)
         if (sc.view[i].d_pose) e = cudaMemsetAsync(sc.view[i].d_pose, 0, 12 * sizeof(float), st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     s = run_composite(ctx, false, bwd_batch_of(ctx->opt), ctx->opt.bwd_schedule, sc, ws, st);
     if (s) return s;
     mark(ctx, 6, st);
-    launch_finalize(sc, ws.world(), ws.gacc(), st);
+    launch_finalize(sc, ws.gacc(), st);
     mark(ctx, 7, st);
     ctx->bwd_recorded = ctx->profile;
     return last_launch("sgad_backward");
@@ -810,7 +826,7 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
             for (int sched : kScheds) {
                 float ms = 0.f;
                 auto run = [&] {
-                    const cudaError_t e = cudaMemsetAsync(ws.gacc(), 0, (size_t)sc.n_gauss * 32, st);
+                    const cudaError_t e = clear_accumulators(sc, ws, st);
                     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
                     return run_composite(&trial, false, batch, sched, sc, ws, st);
                 };

@@ -324,15 +324,22 @@ struct Staged {
     float4 a, b, c;
 };
 
-// Conic, opacity and culling box of a projected Gaussian. hx < 0 marks a Gaussian that
-// cannot reach alpha >= 1/255 anywhere (opacity below the floor).
-__device__ __forceinline__ void stage(const Proj &p, const float4 w1, float z, Staged &s)
+// Mean, conic, opacity, colour and depth of a projected Gaussian, without its box.
+__device__ __forceinline__ void stage_conic(const Proj &p, const float4 w1, float z, Staged &s)
 {
     const float det = __fsub_rn(__fmul_rn(p.cxx, p.cyy), __fmul_rn(p.cxy, p.cxy));
     const float id = __fdiv_rn(1.0f, det);
-    const float o = w1.x;
-    s.b = make_float4(__fmul_rn(p.cyy, id), -__fmul_rn(p.cxy, id), __fmul_rn(p.cxx, id), o);
+    s.a = make_float4(p.px, p.py, 0.0f, 0.0f);
+    s.b = make_float4(__fmul_rn(p.cyy, id), -__fmul_rn(p.cxy, id), __fmul_rn(p.cxx, id), w1.x);
     s.c = make_float4(w1.y, w1.z, w1.w, z);
+}
+
+// The same with the culling box. hx < 0 marks a Gaussian that cannot reach alpha >= 1/255
+// anywhere (opacity below the floor).
+__device__ __forceinline__ void stage(const Proj &p, const float4 w1, float z, Staged &s)
+{
+    stage_conic(p, w1, z, s);
+    const float o = w1.x;
     // alpha >= 1/255 needs d^T Sigma^-1 d <= 2 ln(255 o); its bounding box has half
     // extents sqrt(2 ln(255 o) Sigma_ii). The box only prunes evaluations (the alpha test
     // decides), so it may be larger than needed but never smaller: the fast logarithm is

@@ -1,10 +1,12 @@
 """The warp-local pair of compositing passes against the block-staged forward and the
 warp-reduced backward on the same inputs, where its own parts can go wrong: sets of more
 than 2^24 Gaussians (whose list entries carry no block masks), Gaussians whose rectangles
-span more than 32 pixel blocks (all blocks marked), lists of one entry, and the smallest
-views. Both forwards walk every pixel's list in the same order with the same arithmetic, so
-images and pixel state are equal bit for bit; the gradients differ by the order of FP32
-additions alone (bounds of tests/test_gpu_batching.py)."""
+span more than 32 pixel blocks (all blocks marked), lists of one entry, blocks that most of
+their tile's entries reach (whose lists carry no pixel masks) and the smallest views; and
+image gradients that are not finite. Every keyframe but the first is fixed. Both forwards
+walk every pixel's list in the same order with the same arithmetic, so images and pixel
+state are equal bit for bit; the gradients differ by the order of FP32 additions alone
+(bounds of tests/test_gpu_batching.py)."""
 import numpy as np
 import pytest
 
@@ -80,3 +82,26 @@ def test_warp_local_passes_match_block_staged(name, n, w, h, f, scale, logit, vi
         assert np.all(np.isfinite(x)), q
         assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y) + 1e-30, q
         assert np.abs(x - y).max() <= 1e-4 * np.abs(y).max() + 1e-30, q
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan"), -3e38])
+def test_gradients_that_are_not_finite_stay_with_their_pixels(value):
+    """An infinite, undefined or huge image gradient at single pixels reaches the Gaussians
+    that contribute there and no others."""
+    import torch
+    kfs = _keyframes(2, 40, 30, 40.0, 1.5, 0.0, seed=8)
+    views = [_cam(40, 30, 40.0, 20.0, 15.0, (0.01, -0.02, 0.0))]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rgb, depth = torch.randn(3, 30, 40, generator=g, device="cuda"), torch.randn(30, 40, generator=g, device="cuda")
+    rgb[1, 7, 9] = value
+    rgb[0, 22, 31] = value
+    depth[13, 20] = value
+    gin = [dict(rgb=rgb, depth=depth)]
+    a = _run(kfs, views, gin, bwd_algorithm="warp_local")[2]
+    b = _run(kfs, views, gin, bwd_algorithm="warp_reduce")[2]
+    for q in ("d_offset", "d_rgb", "d_logit", "d_scale"):
+        x, y = a[q].double().cpu().numpy(), b[q].double().cpu().numpy()
+        ok = np.isfinite(y) & (np.abs(y) < 1e30)
+        assert np.array_equal(ok, np.isfinite(x) & (np.abs(x) < 1e30)), q
+        assert 0 < (~ok).sum() < ok.size // 4
+        assert np.abs(x[ok] - y[ok]).max() <= 1e-4 * np.abs(y[ok]).max(), q
