@@ -8,20 +8,21 @@
 // chunk over a row reads whole sectors).
 //
 // Forward and input gradient (k_conv3x3_tma): a tile is 128 consecutive output pixels of
-// one image row (the MMA's M), all output channels (N = 16 or 32) and K = 9 taps x C_in.
-// The three input rows arrive by TMA as one box per (row, chunk) of 130 pixels, which in
-// shared memory is the K-major canonical layout; the tap (dy, dx) is a descriptor start
-// offset of dx units into row dy, so no im2col copy is made. Weights are staged once per
-// block in the B layout [tap][channel chunk][c_out]. A producer lane, an MMA lane and
-// four epilogue warps overlap loads, MMAs (double TMEM accumulator) and the epilogue
-// (bias + ReLU + bf16; or the ReLU-masked input gradient; or the two f32 outputs).
+// one image row (the MMA's M), all output channels and K = 9 taps x C_in. The input rows
+// arrive by TMA, 130 pixels of a (row, chunk), which in shared memory is the K-major
+// canonical layout; the tap column dx is a descriptor start offset of dx units, so no im2col
+// copy is made, and one MMA covers the taps of a column: the output rows above, at and below
+// the input row side by side as N. Weights are staged once per block in the B layout [dx]
+// [channel chunk][dy = 2, 1, 0][c_out]. A producer lane, an MMA lane and four epilogue warps
+// overlap loads, MMAs (a ring of TMEM accumulators) and the epilogue (bias + ReLU + bf16; or
+// the ReLU-masked input gradient; or the two f32 outputs).
 //
 // Weight gradient (k_conv3x3_wgrad_tma): dW[t][i][o] = sum_p x[p + d_t][i] dy[p][o] is a
 // GEMM with the pixels as K; the same TMA boxes, read with the channels as M (x) or N
 // (dy), are the MN-major canonical layout, so three taps share one M = 128 MMA (below)
 // and no shared-memory transpose is needed; the accumulators stay in tensor memory for
-// the whole persistent block and are added to the output with one atomic per (row,
-// column) at the end.
+// the whole persistent block and are added to the output with one 16-byte atomic per (row,
+// 4 columns) at the end.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -70,17 +71,21 @@ __global__ void k_pack_input(const float *__restrict__ rgb, const float *__restr
     }
 }
 
-// f32 master weights W[9][ci_p][co_p] -> forward B units [9][ci_p/8][co_p] (unit = 8
-// consecutive input channels of one output channel) and, when bwd != nullptr, the
-// input-gradient B units [9][co_p/8][ci_p] of the flipped taps (unit = 8 consecutive
-// output channels of one input channel).
-__global__ void k_prep_weights(const float *__restrict__ w, uint4 *__restrict__ fwd, uint4 *__restrict__ bwd, int ci_p,
-                               int co_p)
+// f32 master weights W[9][ci_p][co_p] (tap 3 dy + dx) -> forward B units [dx][ci_p/8][dy =
+// 2, 1, 0][co_p] (unit = 8 consecutive input channels of one output channel) and, when bwd
+// != nullptr, the input-gradient B units [dx][co_p/8][dy = 2, 1, 0][ci_p] of the flipped
+// taps (unit = 8 consecutive output channels of one input channel). blockIdx.y: layer.
+__global__ void k_prep_weights(const PrepArgs a)
 {
-    const int nf = 9 * (ci_p / 8) * co_p, nb = 9 * (co_p / 8) * ci_p;
+    const float *w = a.w[blockIdx.y];
+    uint4 *fwd = a.fwd[blockIdx.y], *bwd = a.bwd[blockIdx.y];
+    const int ci_p = a.ci_p[blockIdx.y], co_p = a.co_p[blockIdx.y];
+    const int n = 9 * ci_p * co_p / 8;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nf) {
-        const int co = i % co_p, kc = (i / co_p) % (ci_p / 8), t = i / (co_p * (ci_p / 8));
+    if (i >= n) return;
+    {
+        const int co = i % co_p, dy = 2 - i / co_p % 3, kc = i / (3 * co_p) % (ci_p / 8);
+        const int t = 3 * dy + i / (3 * co_p * (ci_p / 8));
         uint32_t u[4];
         for (int j = 0; j < 4; ++j) {
             __nv_bfloat162 v = __floats2bfloat162_rn(w[((size_t)t * ci_p + 8 * kc + 2 * j) * co_p + co],
@@ -89,8 +94,9 @@ __global__ void k_prep_weights(const float *__restrict__ w, uint4 *__restrict__ 
         }
         fwd[i] = make_uint4(u[0], u[1], u[2], u[3]);
     }
-    if (bwd && i < nb) {
-        const int ci = i % ci_p, kc = (i / ci_p) % (co_p / 8), t = i / (ci_p * (co_p / 8));
+    if (bwd) {
+        const int ci = i % ci_p, dy = 2 - i / ci_p % 3, kc = i / (3 * ci_p) % (co_p / 8);
+        const int t = 3 * dy + i / (3 * ci_p * (co_p / 8));
         const int tf = 8 - t;     // (ky, kx) -> (2 - ky, 2 - kx)
         uint32_t u[4];
         for (int j = 0; j < 4; ++j) {
@@ -100,6 +106,14 @@ __global__ void k_prep_weights(const float *__restrict__ w, uint4 *__restrict__ 
         }
         bwd[i] = make_uint4(u[0], u[1], u[2], u[3]);
     }
+}
+
+// Zeroes the parameter gradients of all layers. blockIdx.y: layer.
+__global__ void k_zero_grads(const ZeroArgs a)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < a.n_w[blockIdx.y]) a.dw[blockIdx.y][i] = 0.f;
+    if (i < a.n_b[blockIdx.y]) a.db[blockIdx.y][i] = 0.f;
 }
 
 // Training loss mean_p (y0 - delta_t / 0.01)^2 + lw (y1 - logit_t)^2 and its gradient,
@@ -118,37 +132,53 @@ __global__ void k_loss(const float2 *__restrict__ y4, const float *__restrict__ 
         dy4[planar_unit(p, 0, 2, w)] = v;
         dy4[planar_unit(p, 1, 2, w)] = make_uint4(0u, 0u, 0u, 0u);
     }
+    // one addition per block: one per warp (7000 on one address at 3 x 315x237) took 9 of the
+    // kernel's 12 us
+    __shared__ float part[32];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (loss && (threadIdx.x & 31) == 0) atomicAdd(loss, acc * inv);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (loss && threadIdx.x < 32) {
+        acc = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.f;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (threadIdx.x == 0) atomicAdd(loss, acc * inv);
+    }
 }
 
 // ------------------------------------------------------------------ conv (forward / input gradient)
 
 __device__ __forceinline__ bool bf16_positive(uint32_t half_bits) { return (half_bits & 0x8000u) == 0 && (half_bits & 0x7FFFu) != 0; }
 
-// Epilogue of one output pixel p from its accumulator row r (CO f32 values).
+// Epilogue of output pixel x of image row `row` (frame * H + y) from its accumulator row r
+// (CO f32 values); bias: this layer's, in shared memory.
 template <int CO, int MODE>
-__device__ __forceinline__ void conv_epilogue(const ConvArgs &a, size_t p, const uint32_t (&r)[32])
+__device__ __forceinline__ void conv_epilogue(const ConvArgs &a, const float *bias, size_t row, int x,
+                                              const uint32_t (&r)[32])
 {
     if (MODE == kModeOut) {
-        const float y0 = __uint_as_float(r[0]) + a.bias[0], y1 = __uint_as_float(r[1]) + a.bias[1];
+        const size_t p = row * (size_t)a.W + x;
+        const float y0 = __uint_as_float(r[0]) + bias[0], y1 = __uint_as_float(r[1]) + bias[1];
         a.y4[p] = make_float2(y0, y1);
         if (a.delta) a.delta[p] = 0.01f * y0;
         if (a.logit) a.logit[p] = y1;
     } else {
+        const size_t unit = row * (CO / 8) * (size_t)a.W + x;      // of chunk 0
         uint32_t packed[CO / 2];
         if (MODE == kModeRelu) {
 #pragma unroll
-            for (int c = 0; c < CO; c += 2) {
-                const float v0 = fmaxf(__uint_as_float(r[c]) + a.bias[c], 0.0f);
-                const float v1 = fmaxf(__uint_as_float(r[c + 1]) + a.bias[c + 1], 0.0f);
-                __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
-                packed[c / 2] = *reinterpret_cast<uint32_t *>(&h);
+            for (int c = 0; c < CO; c += 4) {
+                const float4 bb = *reinterpret_cast<const float4 *>(bias + c);
+                __nv_bfloat162 h0 = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[c]) + bb.x, 0.0f),
+                                                          fmaxf(__uint_as_float(r[c + 1]) + bb.y, 0.0f));
+                __nv_bfloat162 h1 = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[c + 2]) + bb.z, 0.0f),
+                                                          fmaxf(__uint_as_float(r[c + 3]) + bb.w, 0.0f));
+                packed[c / 2] = *reinterpret_cast<uint32_t *>(&h0);
+                packed[c / 2 + 1] = *reinterpret_cast<uint32_t *>(&h1);
             }
         } else {     // kModeMask: input gradient times [activation > 0]
 #pragma unroll
             for (int u = 0; u < CO / 8; ++u) {
-                const uint4 mm = __ldg(&a.mask[planar_unit(p, u, CO / 8, a.W)]);
+                const uint4 mm = __ldg(&a.mask[unit + (size_t)u * a.W]);
                 const uint32_t mw[4] = {mm.x, mm.y, mm.z, mm.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -162,38 +192,100 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs &a, size_t p, const
         }
 #pragma unroll
         for (int u = 0; u < CO / 8; ++u)
-            a.out[planar_unit(p, u, CO / 8, a.W)] = make_uint4(packed[4 * u], packed[4 * u + 1], packed[4 * u + 2],
-                                                              packed[4 * u + 3]);
+            a.out[unit + (size_t)u * a.W] = make_uint4(packed[4 * u], packed[4 * u + 1], packed[4 * u + 2],
+                                                       packed[4 * u + 3]);
     }
 }
 
 // ------------------------------------------------------------------ conv, TMA-fed pipeline
 //
-// The same tiles, operands and epilogues as k_conv3x3, with the work split between warps
-// so that loads, MMAs and epilogues of consecutive tiles overlap:
-//   warp 0 (one lane)  TMA producer: the three input rows of a tile arrive as 3 x CI/8
-//                      boxes (8 channels x 130 pixels, zero-filled outside the image)
-//                      into one of kStages shared-memory stages; an mbarrier counts the
-//                      bytes;
-//   warp 1 (one lane)  MMA issuer: waits for a full stage and a free accumulator, issues
-//                      the 9 x CI/16 MMAs into one of two TMEM accumulators, and commits
-//                      to the stage's "empty" and the accumulator's "full" barriers;
+// A block owns a run of output tiles that follow one another down the image columns of 128
+// pixels (tile order: frame, column, row with the rows fastest; the runs of two blocks
+// differ by one tile at most) and streams the input rows of the run, each loaded once (and
+// one above and one below every column part). Input row r takes part in the output rows
+// r - 1, r and r + 1, whose accumulators lie side by side in tensor memory: one MMA of N =
+// 3 C_out columns (the taps dy = 2, 1, 0 of one dx) adds to all three, so the 128 pixels are
+// read from shared memory once per (dx, 16 input channels) and not once per tap. The
+// accumulators are a ring of kAcc; where three of them cross its end the MMA is two.
+//   warp 0 (one lane)  TMA producer: an input row arrives as CI/8 slabs [pixel][8 channels],
+//                      each two boxes of consecutive 16-byte units (128, and the 2 of the
+//                      halo), zero-filled outside the image, in one of kRing slots; an
+//                      mbarrier per slot counts the bytes;
+//   warp 1 (one lane)  MMA issuer: waits for the row and for the accumulator of the output
+//                      row that starts with it, issues the MMAs (the new accumulator's
+//                      first one by itself: it overwrites), and commits to the slot's
+//                      "empty" barrier and the finished accumulator's "full" barrier;
 //   warps 2-5          epilogue: wait for a full accumulator, read their 32 rows (warp
 //                      w reads lanes 32 (w % 4) ...), release the accumulator, store.
 // Every wait is bounded; a wait that gives up records a status and ends the block's loop.
-constexpr int kStages = 3;
+//
+// Bound by memory and the latency of a row's steps. 8 x 640x480: 32 -> 32 channels (315 MB
+// in and out) 59 us, 16 -> 32 43, 32 -> 16 43. With every tap an MMA of its own on a row
+// window of the ring: 69, 46 and 59 (48 cycles per MMA, 2/3 of them spent re-reading the
+// pixels); with three rows loaded per tile as rows of 16 bytes: 129, 112 and 76. Fewer slots
+// and more blocks per SM win: 2 slots 65 us, 3: 59, 4: 61, 6: 63; 8 accumulators (2 blocks) 98.
+#ifndef SGAD_CONV_RING
+#define SGAD_CONV_RING 3
+#endif
+#ifndef SGAD_CONV_ACC
+#define SGAD_CONV_ACC 4
+#endif
+constexpr int kRing = SGAD_CONV_RING;  // input row slots
+constexpr int kAcc = SGAD_CONV_ACC;    // accumulators (C_out tensor memory columns each): three in work, the rest in the epilogue
+static_assert(kAcc >= 4 && (kAcc & (kAcc - 1)) == 0 && kRing >= 2, "ring sizes");
 constexpr int kSlabUnits = 136;        // 16-byte units per staged (row, chunk) slab: 130 used, 128-byte aligned
 
 template <int CI, int CO>
 struct TmaConvSmem {
     static constexpr int kB = 9 * (CI / 8) * CO * 16;                 // weights (bytes)
-    static constexpr int kStage = 3 * (CI / 8) * kSlabUnits * 16;     // one stage of input rows
-    static constexpr int kStageTx = 3 * (CI / 8) * kRowUnits * 16;    // bytes the TMA boxes deliver
-    static constexpr size_t bytes = (size_t)kB + (size_t)kStages * kStage + 1024;   // + alignment slack
+    static constexpr int kRow = (CI / 8) * kSlabUnits * 16;           // one slot
+    static constexpr uint32_t kRowTx = (CI / 8) * kRowUnits * 16;     // bytes the TMA boxes deliver
+    static constexpr size_t bytes = (size_t)kB + (size_t)kRing * kRow + 1024;   // + alignment slack
+};
+
+// The units x0 - 1 .. x0 + 128 of chunk slabs of image row y into consecutive slabs at dst.
+template <int KC>
+__device__ __forceinline__ void load_row(uint32_t dst, const CUtensorMap &wide, const CUtensorMap &halo, int x0, int y,
+                                         int n, uint64_t *bar)
+{
+#pragma unroll
+    for (int kc = 0; kc < KC; ++kc) {
+        const uint32_t d = dst + (uint32_t)(kc * kSlabUnits * 16);
+        tc::tma_load_4d(d, &wide, 2 * (x0 - 1), kc, y, n, bar);
+        tc::tma_load_4d(d + kTileM * 16, &halo, 2 * (x0 - 1 + kTileM), kc, y, n, bar);
+    }
+}
+
+// Walks a block's run of tiles, one column part (output rows y0 .. y1 of one column of 128
+// pixels of one frame) at a time.
+struct TileRun {
+    int y0, y1, xs, n, left;     // left: tiles of the run from y0 on
+    int H, segs;
+    __device__ __forceinline__ TileRun(const ConvArgs &a)
+    {
+        H = a.H;
+        segs = (a.W + kTileM - 1) / kTileM;
+        const long long total = (long long)a.N * segs * a.H;
+        const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
+        left = (int)(t1 - t0);
+        const long long col = t0 / a.H;
+        y0 = (int)(t0 - col * a.H);
+        n = (int)(col / segs);
+        xs = (int)(col - (long long)n * segs);
+        y1 = min(H - 1, y0 + left - 1);
+    }
+    __device__ __forceinline__ void next()
+    {
+        left -= y1 - y0 + 1;
+        y0 = 0;
+        y1 = min(H - 1, left - 1);
+        if (++xs == segs) xs = 0, ++n;
+    }
 };
 
 template <int CI, int CO, int MODE>
-__global__ void __launch_bounds__(192) k_conv3x3_tma(const __grid_constant__ CUtensorMap tmap, const ConvArgs a)
+__global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ CUtensorMap wide,
+                                                     const __grid_constant__ CUtensorMap halo, const ConvArgs a)
 {
     static_assert(CI % 16 == 0 && (CO == 16 || CO == 32), "channel counts");
     using S = TmaConvSmem<CI, CO>;
@@ -202,95 +294,128 @@ __global__ void __launch_bounds__(192) k_conv3x3_tma(const __grid_constant__ CUt
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint4 *sB = reinterpret_cast<uint4 *>(base);
     uint8_t *sA = base + S::kB;
-    __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2];
+    __shared__ uint64_t full[kRing], empty[kRing], tfull[kAcc], tempty[kAcc], drain;
     __shared__ uint32_t taddr_s;
+    __shared__ __align__(16) float bias[CO];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int segs = (a.W + kTileM - 1) / kTileM;
-    const long long n_tiles = (long long)a.N * a.H * segs;
 
-    if (warp == 0) tc::tmem_alloc(&taddr_s, 64);
+    if (warp == 0) tc::tmem_alloc(&taddr_s, kAcc * CO);
     if (threadIdx.x == 32) {
-        for (int i = 0; i < kStages; ++i) {
+        tc::mbar_init(&drain, 1);
+        for (int i = 0; i < kRing; ++i) {
             tc::mbar_init(&full[i], 1);
             tc::mbar_init(&empty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kAcc; ++i) {
             tc::mbar_init(&tfull[i], 1);
             tc::mbar_init(&tempty[i], 4);
         }
     }
-    for (int i = threadIdx.x; i < S::kB / 16; i += blockDim.x) sB[i] = a.wB[i];
+    if (MODE != kModeMask && threadIdx.x >= 64 && threadIdx.x < 64 + CO) bias[threadIdx.x - 64] = a.bias[threadIdx.x - 64];
+#pragma unroll 6
+    for (int i = threadIdx.x; i < S::kB / 16; i += 192) sB[i] = a.wB[i];
     tc::fence_proxy_async();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = taddr_s;
-    constexpr uint32_t idesc = tc::idesc_bf16(kTileM, CO);
 
     if (warp == 0) {
         if (lane == 0) {                                       // TMA producer
-            int k = 0;
-            for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++k) {
-                // (the stage's previous box landed before the MMA that freed it ran)
-                const int st = k % kStages;
-                if (!tc::mbar_wait_bounded(&empty[st], ((k / kStages) & 1) ^ 1, kSpinLimit)) {
-                    set_status(a.status, 3u);
-                    break;
+            uint32_t slot = 0, turn = 0, loads = 0;
+            const uint32_t s0 = tc::smem_u32(sA);
+            bool ok = true;
+            for (TileRun t(a); t.left > 0 && ok; t.next())
+                for (int r = t.y0 - 1; r <= t.y1 + 1; ++r) {
+                    // (the slot's previous row landed before the MMAs that freed it ran)
+                    if (!tc::mbar_wait_bounded(&empty[slot], (turn & 1) ^ 1, kSpinLimit)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::mbar_arrive_expect_tx(&full[slot], S::kRowTx);
+                    load_row<kcn>(s0 + slot * (uint32_t)S::kRow, wide, halo, t.xs * kTileM, r, t.n, &full[slot]);
+                    ++loads;
+                    if (++slot == kRing) slot = 0, ++turn;
                 }
-                const int xs = (int)(tile % segs);
-                const long long ry = tile / segs;
-                const int y = (int)(ry % a.H), n = (int)(ry / a.H);
-                tc::mbar_arrive_expect_tx(&full[st], (uint32_t)S::kStageTx);
-                const uint32_t dst0 = tc::smem_u32(sA + (size_t)st * S::kStage);
-                for (int dy = 0; dy < 3; ++dy)
-                    for (int kc = 0; kc < kcn; ++kc)
-                        tc::tma_load_4d(dst0 + (uint32_t)((dy * kcn + kc) * kSlabUnits * 16), &tmap, 0,
-                                        xs * kTileM - 1, (y + dy - 1) * kcn + kc, n, &full[st]);
-            }
-            // drain: the last boxes have landed before the block may exit
-            if (k > 0) tc::mbar_wait_bounded(&full[(k - 1) % kStages], ((k - 1) / kStages) & 1, kSpinLimit);
+            // drain: the last rows have landed before the block may exit
+            for (uint32_t q = loads < (uint32_t)kRing ? 0u : loads - kRing; q < loads; ++q)
+                if (!tc::mbar_wait_bounded(&full[q % kRing], (q / kRing) & 1, kSpinLimit)) ok = false;
+            if (!ok) set_status(a.status, 3u);
         }
     } else if (warp == 1) {
         if (lane == 0) {                                       // MMA issuer
-            int k = 0;
-            for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++k) {
-                const int st = k % kStages, acc = k & 1;
-                if (!tc::mbar_wait_bounded(&full[st], (k / kStages) & 1, kSpinLimit) ||
-                    !tc::mbar_wait_bounded(&tempty[acc], ((k >> 1) & 1) ^ 1, kSpinLimit)) {
-                    set_status(a.status, 3u);
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t a_base = tc::smem_u32(sA + (size_t)st * S::kStage), b_base = tc::smem_u32(sB);
-                const uint32_t d = tmem + (uint32_t)(acc * 32);
-#pragma unroll
-                for (int t = 0; t < 9; ++t) {
-                    const int dy = t / 3, dx = t % 3;
-#pragma unroll
-                    for (int sk = 0; sk < CI / 16; ++sk) {
-                        const uint32_t aa = a_base + (uint32_t)(((dy * kcn + 2 * sk) * kSlabUnits + dx) * 16);
-                        const uint32_t bb = b_base + (uint32_t)(((t * kcn + 2 * sk) * CO) * 16);
-                        tc::mma_bf16(d, tc::sdesc(aa, kSlabUnits * 16, 128), tc::sdesc(bb, CO * 16, 128), idesc,
-                                     (t | sk) != 0);
+            const uint64_t a0 = tc::sdesc(tc::smem_u32(sA), kSlabUnits * 16, 128);
+            const uint64_t b0 = tc::sdesc(tc::smem_u32(sB), 3 * CO * 16, 128);
+            uint32_t slot = 0, turn = 0;
+            int k = 0;                                         // tiles before this column part
+            bool ok = true;
+            for (TileRun t(a); t.left > 0 && ok; k += t.y1 - t.y0 + 1, t.next())
+                for (int r = t.y0 - 1; r <= t.y1 + 1; ++r) {
+                    const int lo = max(r - 1, t.y0), hi = min(r + 1, t.y1);     // output rows
+                    const int k_lo = k + lo - t.y0, k_hi = k + hi - t.y0;
+                    const bool fresh = hi == r + 1;            // row hi starts
+                    if (!tc::mbar_wait_bounded(&full[slot], turn & 1, kSpinLimit) ||
+                        (fresh && !tc::mbar_wait_bounded(&tempty[k_hi % kAcc], ((k_hi / kAcc) & 1) ^ 1, kSpinLimit))) {
+                        set_status(a.status, 3u);
+                        ok = false;
+                        break;
                     }
+                    tc::fence_after_sync();
+                    // rows lo .. lo + n0 - 1 in accumulators up to the ring's end, then n1 from its start
+                    const int rows = hi - lo + 1, n0 = min(rows, kAcc - k_lo % kAcc), n1 = rows - n0;
+                    const uint32_t d0 = tmem + (uint32_t)(k_lo % kAcc * CO), d1 = tmem;
+                    const uint64_t ad = a0 + (uint64_t)(slot * (uint32_t)(S::kRow / 16));
+                    // taps dy = 2, 1, 0 for the output rows r - 1, r, r + 1
+                    const uint64_t bd = b0 + (uint64_t)((lo - (r - 1)) * CO);
+                    const uint32_t i0 = tc::idesc_bf16(kTileM, 0) + ((uint32_t)(n0 * CO / 8) << 17);
+                    const uint32_t i1 = tc::idesc_bf16(kTileM, 0) + ((uint32_t)(n1 * CO / 8) << 17);
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                        for (int sk = 0; sk < CI / 16; ++sk) {
+                            const uint64_t aa = ad + (uint64_t)(2 * sk * kSlabUnits + dx);
+                            const uint64_t bb = bd + (uint64_t)((dx * kcn + 2 * sk) * 3 * CO);
+                            if ((dx | sk) == 0 && fresh) {
+                                // the new row's accumulator is overwritten, the others added to
+                                constexpr uint32_t one = tc::idesc_bf16(kTileM, CO);
+                                const uint32_t dn = tmem + (uint32_t)(k_hi % kAcc * CO);
+                                const int m0 = min(rows - 1, n0), m1 = rows - 1 - m0;
+                                if (m0) tc::mma_bf16(d0, aa, bb, i0 - ((uint32_t)((n0 - m0) * CO / 8) << 17), true);
+                                if (m1) tc::mma_bf16(d1, aa, bb + (uint64_t)(m0 * CO),
+                                                     i1 - ((uint32_t)((n1 - m1) * CO / 8) << 17), true);
+                                tc::mma_bf16(dn, aa, bb + (uint64_t)((rows - 1) * CO), one, false);
+                            } else {
+                                tc::mma_bf16(d0, aa, bb, i0, true);
+                                if (n1) tc::mma_bf16(d1, aa, bb + (uint64_t)(n0 * CO), i1, true);
+                            }
+                        }
+                    tc::mma_commit(&empty[slot]);
+                    if (r > t.y0) tc::mma_commit(&tfull[(k + r - 1 - t.y0) % kAcc]);    // row r - 1 is done
+                    if (++slot == kRing) slot = 0, ++turn;
                 }
-                tc::mma_commit(&empty[st]);
-                tc::mma_commit(&tfull[acc]);
+            // drain: the last committed MMAs finish before the accumulators are freed (an
+            // output row's last MMAs are the last ones of a run)
+            if (ok) {
+                if (k > 0) tc::mbar_wait_bounded(&tfull[(k - 1) % kAcc], ((k - 1) / kAcc) & 1, kSpinLimit);
+            } else {
+                tc::mma_commit(&drain);
+                tc::mbar_wait_bounded(&drain, 0, kSpinLimit);
             }
-            // drain: the last committed MMAs finish before the accumulators are freed
-            if (k > 0) tc::mbar_wait_bounded(&tfull[(k - 1) & 1], ((k - 1) >> 1) & 1, kSpinLimit);
         }
     } else {                                                   // epilogue warps 2..5
         const int quarter = warp & 3;
         int k = 0;
-        for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++k) {
-            const int acc = k & 1;
-            if (!tc::mbar_wait_bounded(&tfull[acc], (k >> 1) & 1, kSpinLimit)) {
+        bool ok = true;
+        for (TileRun t(a); t.left > 0 && ok; t.next())
+        for (int y = t.y0; y <= t.y1; ++y, ++k) {
+            const int acc = k % kAcc;
+            if (!tc::mbar_wait_bounded(&tfull[acc], (k / kAcc) & 1, kSpinLimit)) {
                 if (lane == 0) set_status(a.status, 3u);
+                ok = false;
                 break;
             }
             tc::fence_after_sync();
-            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 32);
+            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * CO);
             uint32_t r[32];
             {
                 uint32_t q[16];
@@ -307,49 +432,59 @@ __global__ void __launch_bounds__(192) k_conv3x3_tma(const __grid_constant__ CUt
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&tempty[acc]);
-            const int xs = (int)(tile % segs);
-            const long long ry = tile / segs;
-            const int y = (int)(ry % a.H), n = (int)(ry / a.H);
-            const int x = xs * kTileM + quarter * 32 + lane;
-            if (x < a.W) conv_epilogue<CO, MODE>(a, ((size_t)n * a.H + y) * a.W + x, r);
+            const int x = t.xs * kTileM + quarter * 32 + lane;
+            if (x < a.W) conv_epilogue<CO, MODE>(a, bias, (size_t)t.n * a.H + y, x, r);
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, 64);
+    if (warp == 0) tc::tmem_dealloc(tmem, kAcc * CO);
 }
 
 // ------------------------------------------------------------------ weight gradient, TMA-fed
 //
 // The same sums, with the operands read in the layout the TMA boxes land in, so that no
-// shared-memory transpose is needed: a K block is 128 pixels of one output row; its three
-// input rows (pixels x0 - 1 .. x0 + 128) arrive as 3 x CI/8 slabs [pixel][8 channels] of
-// kSlabUnits units and the output-gradient row as CO/8 slabs of 128 units. Read with the
-// pixels as K and the channels as M (x) or N (dy), a slab is the MN-major canonical
-// layout: a core matrix is 8 pixels x 8 channels, 128 contiguous bytes; the next 8
-// channels are one slab further, the next 8 pixels 128 bytes further. For a fixed dx the
-// (dy, channel group) rows of the three input rows form one uniformly strided M
-// dimension of 3 CI rows that starts dx pixels into the slabs, so one M = 128 MMA per
-// (dx, 16-pixel K step) covers the three taps (dy, dx); the M rows after 3 CI read a slab
-// of ones (row 3 CI: the bias gradient, taken from dx = 0) and then whatever follows it
-// in the stage, rows whose products are not used. Accumulators: three TMEM blocks of CO columns (one per dx) for the whole
-// persistent block, added to dW with one atomic per (row, column) at the end.
+// shared-memory transpose is needed. A K block is 128 consecutive pixels q of one image row
+// y: the input's rows y - 1, y, y + 1 at q (one box of 3 x CI/8 slabs [pixel][8 channels] of
+// 128 units) and the output gradient's row y at x0 - 1 .. x0 + 128 (CO/8 slabs of kSlabUnits
+// units, two boxes each: only this operand needs the halo, which makes 9 copies per K block
+// of 32 -> 32 channels instead of 28). Read with the pixels as K and the channels as M (x)
+// or N (dy), a slab is the MN-major canonical layout: a core matrix is 8 pixels x 8
+// channels, 128 contiguous bytes; the next 8 channels are one slab further, the next 8
+// pixels 128 bytes further. The (dy, channel group) rows of the three input rows form one
+// uniformly strided M dimension of 3 CI rows; tap dx pairs the input pixel q with the
+// gradient pixel q + 1 - dx, a start offset of 2 - dx units, so one M = 128 MMA per (dx,
+// 16-pixel K step) covers the three taps (dy, dx). The M rows after 3 CI read a slab of ones
+// (row 3 CI: the bias gradient, taken from dx = 1) and then whatever follows it in the
+// stage, rows whose products are not used. Accumulators: three TMEM blocks of CO columns
+// (one per dx) for the whole persistent block, added to dW at the end with 16-byte atomics.
 // One thread of warp 0 issues the TMA loads into kWgStages stages, one thread of warp 1
 // the MMAs (its descriptors precomputed: an offset adds to the address field); the four
 // warps run the epilogue. Every wait is bounded.
+//
+// The final additions of all blocks meet on the same 3 CI CO addresses, so a small problem
+// takes fewer blocks: kWgTiles K blocks each, at least one block per SM (4: 55 us
+// for the two 32 -> 32 layers of 3 x 315x237, 8: 50, 32: 57).
+// 3 x 315x237, 32 -> 32 channels (28 MB in): 24 us, of which the additions 8 and the launch,
+// setup and drain 8; 94 us with single-float atomics from every resident block (4.2 M onto
+// 9216 addresses) and 28 copies of 16-byte rows per K block.
+#ifndef SGAD_WG_TILES
+#define SGAD_WG_TILES 8
+#endif
+constexpr int kWgTiles = SGAD_WG_TILES;
 constexpr int kWgPix = 128;                // pixels per K block
 constexpr int kWgGroups = 16;              // M groups read by an M = 128 MMA
 constexpr int kWgStages = 3;               // shared-memory stages of the load pipeline
 
 template <int CI, int CO>
 struct WgradTmaSmem {
-    static constexpr int kXBytes = (3 * (CI / 8) + 1) * kSlabUnits * 16;   // slabs of x, then the ones slab
-    static constexpr int kYBytes = (CO / 8) * kWgPix * 16;                 // slabs of dy
+    static constexpr int kXBytes = (3 * (CI / 8) + 1) * kWgPix * 16;       // slabs of x, then the ones slab
+    static constexpr int kYBytes = (CO / 8) * kSlabUnits * 16;             // slabs of dy
     // an M = 128 MMA reads kWgGroups slabs from the x base: past the ones slab it reads
     // the dy slabs (or padding), rows whose products are not used
-    static constexpr int kStage = kXBytes + kYBytes > kWgGroups * kSlabUnits * 16 ? kXBytes + kYBytes
-                                                                                 : kWgGroups * kSlabUnits * 16;
-    static constexpr uint32_t kTx = (uint32_t)(3 * (CI / 8) * kRowUnits * 16 + (CO / 8) * kWgPix * 16);
+    static constexpr int kStage = kXBytes + kYBytes > kWgGroups * kWgPix * 16 ? kXBytes + kYBytes
+                                                                             : kWgGroups * kWgPix * 16;
+    static constexpr uint32_t kTx = (uint32_t)(3 * (CI / 8) * kWgPix * 16 + (CO / 8) * kRowUnits * 16);
     static constexpr size_t bytes = (size_t)kWgStages * kStage + 1024;   // + alignment slack
     static constexpr int kCols = 3 * CO <= 32 ? 32 : (3 * CO <= 64 ? 64 : 128);
     static_assert(3 * (CI / 8) + 1 <= kWgGroups, "the three rows and the ones slab fit one M = 128 MMA");
@@ -373,7 +508,8 @@ __device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t mn_stride,
 
 template <int CI, int CO>
 __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant__ CUtensorMap xmap,
-                                                           const __grid_constant__ CUtensorMap ymap,
+                                                           const __grid_constant__ CUtensorMap ywide,
+                                                           const __grid_constant__ CUtensorMap yhalo,
                                                            const WgradArgs a)
 {
     static_assert(CI % 16 == 0 && (CO == 16 || CO == 32), "channel counts");
@@ -398,8 +534,8 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     }
     // the slab after the three input rows: ones (first element of each unit)
     for (int st = 0; st < kWgStages; ++st) {
-        uint4 *x = reinterpret_cast<uint4 *>(base + (size_t)st * S::kStage) + 3 * kcx * kSlabUnits;
-        for (int i = threadIdx.x; i < kSlabUnits; i += blockDim.x) x[i] = make_uint4(0x3F80u, 0u, 0u, 0u);
+        uint4 *x = reinterpret_cast<uint4 *>(base + (size_t)st * S::kStage) + 3 * kcx * kWgPix;
+        for (int i = threadIdx.x; i < kWgPix; i += blockDim.x) x[i] = make_uint4(0x3F80u, 0u, 0u, 0u);
     }
     tc::fence_proxy_async();
     tc::fence_before_sync();
@@ -421,15 +557,8 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
             const int y = ry % a.H, n = ry / a.H;
             const uint32_t xb = tc::smem_u32(base + (size_t)st * S::kStage), yb = xb + (uint32_t)S::kXBytes;
             tc::mbar_arrive_expect_tx(&full[st], S::kTx);
-#pragma unroll
-            for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-                for (int kc = 0; kc < kcx; ++kc)
-                    tc::tma_load_4d(xb + (uint32_t)((dy * kcx + kc) * kSlabUnits * 16), &xmap, 0,
-                                    xs * kWgPix - 1, (y + dy - 1) * kcx + kc, n, &full[st]);
-#pragma unroll
-            for (int kc = 0; kc < kcy; ++kc)
-                tc::tma_load_4d(yb + (uint32_t)(kc * kWgPix * 16), &ymap, 0, xs * kWgPix, y * kcy + kc, n, &full[st]);
+            tc::tma_load_4d(xb, &xmap, 2 * xs * kWgPix, 0, y - 1, n, &full[st]);
+            load_row<kcy>(yb, ywide, yhalo, xs * kWgPix, y, n, &full[st]);
         }
         // drain: the last boxes have landed before the block may exit
         if (k > 0 && !tc::mbar_wait_bounded(&full[(k - 1) % kWgStages], (uint32_t)(((k - 1) / kWgStages) & 1), kSpinLimit))
@@ -441,7 +570,7 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     } else if (threadIdx.x == 32) {                           // MMA issuer
         // descriptors of stage 0 at offset 0; an offset of o bytes adds o / 16
         const uint32_t x0 = tc::smem_u32(base), y0 = x0 + (uint32_t)S::kXBytes;
-        const uint64_t ad0 = sdesc_mn(x0, kSlabUnits * 16, 128), bd0 = sdesc_mn(y0, kWgPix * 16, 128);
+        const uint64_t ad0 = sdesc_mn(x0, kWgPix * 16, 128), bd0 = sdesc_mn(y0, kSlabUnits * 16, 128);
         int k = 0;
         bool ok = true;
         for (int kb = blockIdx.x; kb < n_kb; kb += gridDim.x, ++k) {
@@ -456,8 +585,8 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
             for (int s = 0; s < kWgPix / 16; ++s)
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx)
-                    tc::mma_bf16(tmem + (uint32_t)(dx * CO), ad0 + so + (uint64_t)(dx + s * 16),
-                                 bd0 + so + (uint64_t)(s * 16), idesc, (k | s) != 0);
+                    tc::mma_bf16(tmem + (uint32_t)(dx * CO), ad0 + so + (uint64_t)(s * 16),
+                                 bd0 + so + (uint64_t)(2 - dx + s * 16), idesc, (k | s) != 0);
             tc::mma_commit(&empty[st]);
         }
         // drain: the last MMAs have completed before the accumulators are read
@@ -474,23 +603,31 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     tc::fence_after_sync();
     if (failed_s == 0) {
         const int row = 32 * warp + lane;
+        constexpr int kParts = 3 * (CO / 16);          // of 16 columns; blocks start at different ones
+#pragma unroll 1
+        for (int i = 0; i < kParts; ++i) {
+            const int part = (i + (int)blockIdx.x) % kParts, dx = part / (CO / 16), c0 = part % (CO / 16) * 16;
+            uint32_t q[16];
+            tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(dx * CO + c0), q);
+            tc::tmem_wait_ld();
+            if (row < 3 * CI) {
+                const int tap = 3 * (row / CI) + dx, ci = row % CI;
+                float *dst = a.dw + ((size_t)tap * CI + ci) * CO + c0;
+                if (a.vec) {
 #pragma unroll
-        for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-            for (int c0 = 0; c0 < CO; c0 += 16) {
-                uint32_t q[16];
-                tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(dx * CO + c0), q);
-                tc::tmem_wait_ld();
-                if (row < 3 * CI) {
-                    const int tap = 3 * (row / CI) + dx, ci = row % CI;
-                    float *dst = a.dw + ((size_t)tap * CI + ci) * CO + c0;
+                    for (int c = 0; c < 16; c += 4)
+                        atomicAdd(reinterpret_cast<float4 *>(dst + c),
+                                  make_float4(__uint_as_float(q[c]), __uint_as_float(q[c + 1]),
+                                              __uint_as_float(q[c + 2]), __uint_as_float(q[c + 3])));
+                } else {
 #pragma unroll
                     for (int c = 0; c < 16; ++c) atomicAdd(dst + c, __uint_as_float(q[c]));
-                } else if (row == 3 * CI && dx == 0) {
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) atomicAdd(a.db + c0 + c, __uint_as_float(q[c]));
                 }
+            } else if (row == 3 * CI && dx == 1) {
+#pragma unroll
+                for (int c = 0; c < 16; ++c) atomicAdd(a.db + c0 + c, __uint_as_float(q[c]));
             }
+        }
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -558,21 +695,24 @@ cudaError_t encode_tiled(EncodeTiledFn *out)
     return cudaSuccess;
 }
 
-// Tensor map of a chunk-planar bf16 activation with ci channels, as dims (8 channels, W,
-// H x ci/8 (row, chunk), N), boxes of 8 channels x box_px pixels of one (row, chunk) of
-// one frame, zero fill outside: the (row, chunk) coordinate of row y and chunk c is
-// y ci/8 + c, so rows -1 and H fall outside the tensor.
-cudaError_t input_map(const void *base, int ci, int n, int h, int w, CUtensorMap *m, int box_px = kTileM + 2)
+// Tensor map of a chunk-planar bf16 activation with ci channels, with the W 16-byte units
+// (8 channels of a pixel) of a chunk of an image row as 2 W 8-byte elements in a row: dims
+// (2 W, ci/8, H, N), boxes of box_px consecutive units of box_kc chunks of box_rows rows, zero
+// fill outside. (With the 8
+// channels as the inner dimension a box is box_px rows of 16 bytes, and the copy engine's
+// rate in rows bounded every convolution: 129 us for 32 -> 32 channels at 8 x 640x480.)
+cudaError_t input_map(const void *base, int ci, int n, int h, int w, CUtensorMap *m, int box_px, int box_kc = 1,
+                      int box_rows = 1)
 {
     EncodeTiledFn fn = nullptr;
     cudaError_t e = encode_tiled(&fn);
     if (e != cudaSuccess) return e;
     const cuuint64_t kc = (cuuint64_t)(ci / 8);
-    const cuuint64_t dims[4] = {8, (cuuint64_t)w, (cuuint64_t)h * kc, (cuuint64_t)n};
-    const cuuint64_t strides[3] = {16, (cuuint64_t)w * 16, (cuuint64_t)h * kc * w * 16};
-    const cuuint32_t box[4] = {8, (cuuint32_t)box_px, 1, 1};
+    const cuuint64_t dims[4] = {2 * (cuuint64_t)w, kc, (cuuint64_t)h, (cuuint64_t)n};
+    const cuuint64_t strides[3] = {(cuuint64_t)w * 16, kc * w * 16, (cuuint64_t)h * kc * w * 16};
+    const cuuint32_t box[4] = {2 * (cuuint32_t)box_px, (cuuint32_t)box_kc, (cuuint32_t)box_rows, 1};
     const cuuint32_t elem[4] = {1, 1, 1, 1};
-    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, elem,
+    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_INT64, 4, const_cast<void *>(base), dims, strides, box, elem,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
@@ -586,12 +726,17 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st)
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)a.N * a.H * ((a.W + kTileM - 1) / kTileM);
     if (tiles <= 0) return cudaSuccess;
-    CUtensorMap m;
-    e = input_map(a.in, CI, a.N, a.H, a.W, &m);
+    CUtensorMap wide, halo;
+    e = input_map(a.in, CI, a.N, a.H, a.W, &wide, kTileM);
+    if (e == cudaSuccess) e = input_map(a.in, CI, a.N, a.H, a.W, &halo, 2);
     if (e != cudaSuccess) return e;
-    // TMEM: 64 columns per block, at most 8 blocks of 512 columns per SM
-    const int grid = resident_grid((const void *)k_conv3x3_tma<CI, CO, MODE>, smem, tiles, 192);
-    k_conv3x3_tma<CI, CO, MODE><<<grid, 192, smem, st>>>(m, a);
+    int grid = resident_grid((const void *)k_conv3x3_tma<CI, CO, MODE>, smem, tiles, 192);
+    // tensor memory: 512 columns per SM
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (grid > sms * (512 / (kAcc * CO))) grid = sms * (512 / (kAcc * CO));
+    k_conv3x3_tma<CI, CO, MODE><<<grid, 192, smem, st>>>(wide, halo, a);
     return cudaGetLastError();
 }
 
@@ -604,9 +749,10 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
     const long long blocks = (long long)a.N * a.H * ((a.W + kWgPix - 1) / kWgPix);
     if (blocks <= 0) return cudaSuccess;
     if (blocks >= (1ll << 31)) return cudaErrorInvalidValue;
-    CUtensorMap xm, ym;
-    e = input_map(a.x, CI, a.N, a.H, a.W, &xm);
-    if (e == cudaSuccess) e = input_map(a.dy, CO, a.N, a.H, a.W, &ym, kWgPix);
+    CUtensorMap xm, wide, halo;
+    e = input_map(a.x, CI, a.N, a.H, a.W, &xm, kWgPix, CI / 8, 3);
+    if (e == cudaSuccess) e = input_map(a.dy, CO, a.N, a.H, a.W, &wide, kTileM);
+    if (e == cudaSuccess) e = input_map(a.dy, CO, a.N, a.H, a.W, &halo, 2);
     if (e != cudaSuccess) return e;
     // keep (resident blocks x TMEM columns) within the 512 columns of an SM
     int grid = resident_grid((const void *)k_conv3x3_wgrad_tma<CI, CO>, S::bytes, blocks);
@@ -615,7 +761,9 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long cap = (long long)sms * (512 / S::kCols);
     if (grid > cap) grid = (int)cap;
-    k_conv3x3_wgrad_tma<CI, CO><<<grid, 128, S::bytes, st>>>(xm, ym, a);
+    const long long by_work = blocks / kWgTiles;
+    if (grid > by_work) grid = (int)(by_work > sms ? by_work : (grid < sms ? grid : sms));
+    k_conv3x3_wgrad_tma<CI, CO><<<grid, 128, S::bytes, st>>>(xm, wide, halo, a);
     return cudaGetLastError();
 }
 
@@ -637,10 +785,19 @@ cudaError_t launch_pack_input(const float *rgb, const float *depth, uint4 *x0, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_prep_weights(const float *w, uint4 *fwd, uint4 *bwd, int ci_p, int co_p, cudaStream_t st)
+cudaError_t launch_prep_weights(const PrepArgs &a, cudaStream_t st)
 {
-    const int n = 9 * ci_p * co_p / 8;
-    k_prep_weights<<<(n + 127) / 128, 128, 0, st>>>(w, fwd, bwd, ci_p, co_p);
+    int n = 0;
+    for (int l = 0; l < kLayers; ++l) n = max(n, 9 * a.ci_p[l] * a.co_p[l] / 8);
+    k_prep_weights<<<dim3((n + 127) / 128, kLayers), 128, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_zero_grads(const ZeroArgs &a, cudaStream_t st)
+{
+    int n = 0;
+    for (int l = 0; l < kLayers; ++l) n = max(n, max(a.n_w[l], a.n_b[l]));
+    k_zero_grads<<<dim3((n + 255) / 256, kLayers), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -115,10 +115,16 @@ sgad_status sgad_net_forward(const sgad_net_params *params, int32_t n_frames, in
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const NetLayout &L = ws.L;
     s = launched(launch_pack_input(rgb, depth, ws.at(L.x[0]), n_frames, height, width, st), "pack input");
-    for (int l = 0; l < 4 && !s; ++l)
-        s = launched(launch_prep_weights(params->w[l], ws.at(L.wf[l]), l > 0 ? ws.at(L.wb[l]) : nullptr, kCinP[l],
-                                         kCoutP[l], st),
-                     "weight conversion");
+    if (s) return s;
+    PrepArgs prep;
+    for (int l = 0; l < kLayers; ++l) {
+        prep.w[l] = params->w[l];
+        prep.fwd[l] = ws.at(L.wf[l]);
+        prep.bwd[l] = l > 0 ? ws.at(L.wb[l]) : nullptr;
+        prep.ci_p[l] = kCinP[l];
+        prep.co_p[l] = kCoutP[l];
+    }
+    s = launched(launch_prep_weights(prep, st), "weight conversion");
     if (s) return s;
     ConvArgs a = {};
     a.N = n_frames;
@@ -174,11 +180,15 @@ sgad_status sgad_net_backward(const sgad_net_params *params, sgad_net_grads *gra
         if (!grads->dw[l] || !grads->db[l]) return err(SGAD_ERR_INVALID_ARG, "sgad_net_backward: a gradient is NULL");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const NetLayout &L = ws.L;
-    for (int l = 0; l < 4; ++l) {
-        cudaError_t e = cudaMemsetAsync(grads->dw[l], 0, (size_t)9 * kCinP[l] * kCoutP[l] * 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(grads->db[l], 0, (size_t)kCoutP[l] * 4, st);
-        if (e != cudaSuccess) return cuda_err(e, "cudaMemsetAsync");
+    ZeroArgs z;
+    for (int l = 0; l < kLayers; ++l) {
+        z.dw[l] = grads->dw[l];
+        z.db[l] = grads->db[l];
+        z.n_w[l] = 9 * kCinP[l] * kCoutP[l];
+        z.n_b[l] = kCoutP[l];
     }
+    s = launched(launch_zero_grads(z, st), "gradient zeroing");
+    if (s) return s;
     // layer l's output gradient (pre-activation): dy4 for l = 3, d[l] below
     ConvArgs a = {};
     a.N = n_frames;
@@ -205,6 +215,7 @@ sgad_status sgad_net_backward(const sgad_net_params *params, sgad_net_grads *gra
         g.dy = dout;
         g.dw = grads->dw[l];
         g.db = grads->db[l];
+        g.vec = (reinterpret_cast<uintptr_t>(g.dw) & 15) == 0;
         cudaError_t e;
         if (l == 0)
             e = launch_wgrad<16, 32>(g, st);
