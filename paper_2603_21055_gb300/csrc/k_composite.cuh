@@ -399,12 +399,19 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks<B>())
 // from one to a quarter. Without masks (more than 2^24 Gaussians) step 1 projects every
 // entry for each block: the L1 wavefronts of those gathers (16 B and 4 B from 32 lines per
 // chunk) were then as many as all others of the kernel (L1 at 80 %).
+// A lane takes two candidates at once: the box covers a pixel that the entry's alpha then
+// misses as often as not, so a step was a chain of shared-memory loads, exponential and test
+// (about 150 cycles) for half an addition, and its branches cost as much issue as its sums.
+// Two alphas side by side and predicated sums: 32 warps per SM 1.05 -> 0.93 ms, a lone warp
+// per SM sub-core (2 views of 160x120) 129 -> 96 us; three or four at once 0.99 ms and 90 us.
 // Measured on the room workload (8 keyframes of 640x480 into 8 views, 34 M entries, 130 M
-// contributing pairs): 1.08 ms in tile order, 1.01 ms heaviest first, against 1.85 and
-// 1.68 ms for the block-staged forward and 1.41 and 1.33 ms without masks; the masks cost
-// the count and the emission 0.08 ms. 4 blocks per SM (59 registers): 5 (48 registers)
-// take 1.14 and 1.07 ms. The two packed multiplies and adds, the exact halves and the
-// flushed exponential take the walk's step from about 60 to 48 instructions.
+// contributing pairs), with one candidate at a time and without the pixel masks for the
+// backward (+0.03 ms): 1.08 ms in tile order, 1.01 ms heaviest first, against 1.85 and
+// 1.68 ms for the block-staged forward and 1.41 and 1.33 ms without block masks; the block
+// masks cost the count and the emission 0.08 ms. 4 blocks per SM (62 registers); 5 (48)
+// took 1.14 and 1.07 ms, 3 takes 1.01 heaviest first. A round's entries and records loaded
+// during the round before it: 1.15 against 1.05 ms. The two packed multiplies and adds, the
+// exact halves and the flushed exponential take a candidate from about 60 to 48 instructions.
 constexpr int kFwdlThreads = 256;           // 8 independent warps per block
 #ifndef SGAD_FWDL_MINBLOCKS
 #define SGAD_FWDL_MINBLOCKS 4
@@ -604,27 +611,40 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
         uint32_t bits = 0u;
         while (__any_sync(kFull, mine != 0u)) {
             if (mine) {
-                const uint32_t low = mine & (0u - mine);
-                mine ^= low;
-                const WalkEntry &g = S.e[31 - __clz(low)];
-                const float4 ga = g.a, gc = g.c;
-                const float2 gb = g.b;
-                float alpha, raw;
-                if (walk_alpha(ga, gb, nq, alpha, raw)) {
-                    const float test = __fmul_rn(T, __fsub_rn(1.0f, alpha));
-                    if (test < kTStop) {
-                        done = true;
-                        n_evals -= __popc(mine);
-                        mine = 0u;
-                    } else {
-                        bits |= low;
-                        const float w = __fmul_rn(alpha, T);
-                        const float2x ww = pack2(w, w);
-                        acc_rg = fma2(ww, pack2(gc.x, gc.y), acc_rg);
-                        acc_bd = fma2(ww, pack2(gc.z, gc.w), acc_bd);
-                        aa = __fadd_rn(aa, w);
-                        T = test;
-                    }
+                // two candidates: their alphas are independent of one another
+                const uint32_t low0 = mine & (0u - mine), rest = mine ^ low0, low1 = rest & (0u - rest);
+                mine = rest ^ low1;
+                const WalkEntry &g0 = S.e[31 - __clz(low0)], &g1 = S.e[31 - __clz(low1 ? low1 : low0)];
+                float alpha0, alpha1, raw;
+                const bool ok0 = walk_alpha(g0.a, g0.b, nq, alpha0, raw);
+                const bool ok1 = walk_alpha(g1.a, g1.b, nq, alpha1, raw) && low1;
+                const float4 c0 = g0.c, c1 = g1.c;
+                const float t0 = __fmul_rn(T, __fsub_rn(1.0f, alpha0));
+                const bool stop0 = ok0 && t0 < kTStop, take0 = ok0 && !stop0;
+                if (take0) {
+                    const float w = __fmul_rn(alpha0, T);
+                    const float2x ww = pack2(w, w);
+                    acc_rg = fma2(ww, pack2(c0.x, c0.y), acc_rg);
+                    acc_bd = fma2(ww, pack2(c0.z, c0.w), acc_bd);
+                    aa = __fadd_rn(aa, w);
+                    T = t0;
+                    bits |= low0;
+                }
+                const float t1 = __fmul_rn(T, __fsub_rn(1.0f, alpha1));
+                const bool stop1 = ok1 && !stop0 && t1 < kTStop, take1 = ok1 && !stop0 && !stop1;
+                if (take1) {
+                    const float w = __fmul_rn(alpha1, T);
+                    const float2x ww = pack2(w, w);
+                    acc_rg = fma2(ww, pack2(c1.x, c1.y), acc_rg);
+                    acc_bd = fma2(ww, pack2(c1.z, c1.w), acc_bd);
+                    aa = __fadd_rn(aa, w);
+                    T = t1;
+                    bits |= low1;
+                }
+                if (stop0 || stop1) {
+                    done = true;
+                    n_evals -= __popc(stop0 ? rest : mine);
+                    mine = 0u;
                 }
             }
         }
@@ -1296,10 +1316,14 @@ __global__ void __launch_bounds__(kPairThreads, 4) k_composite_bwdp(const __grid
 //      depth along the keyframe's ray and adds the result with two vector atomics.
 // A round's list words, entries and world records are loaded during the round before it.
 // Bound by issue (68 % of the slots at 24 warps per SM) and L1 wavefronts (70 %) together.
-// Room workload (8 x 640x480, 130 M contributing pairs): 1.34 ms against 1.56 ms with box
+// A lane takes three entries at once (two with fixed keyframes, whose rounds are one walk):
+// the alphas, reciprocals and colour products of a step do not depend on one another.
+// Room workload (8 x 640x480, 130 M contributing pairs): 1.29 ms (one entry at once 1.34, two
+// 1.33, four 1.35; 5 x 1200x680 with four of five keyframes fixed: 1.48, 1.38 and with three
+// 1.41) against 1.56 ms with box
 // masks, candidates that miss and one lane per entry summing its pixels (a loop as long as
-// the entry with the most, 21.5 against a mean of 7.5). Of it (parts left out in copies) the
-// walk takes 0.56, the moments 0.41, the chain rule 0.12 and staging, masks and loads 0.35.
+// the entry with the most, 21.5 against a mean of 7.5). Of the 1.34 (parts left out in copies)
+// the walk takes 0.56, the moments 0.41, the chain rule 0.12 and staging, masks and loads 0.35.
 // 4 blocks per SM (64 registers): 1.37 ms, 2: 1.64; the rounds loaded when needed: +0.04.
 constexpr int kLocalThreads = 256;          // 8 independent warps per block
 constexpr int kHalf = 16;                   // entries per walk and product
@@ -1416,7 +1440,7 @@ static __device__ __noinline__ void add_not_finite(BwdlWarpSmem &S, int h, int s
 // FIXED: some keyframe is fixed. Its entries are walked (they take part in the pixels'
 // transmittance and suffix sums) but have no moments, unless the view's pose wants them: a
 // round whose other entries are at most 16 is one walk and one product, and nothing is added
-// for the fixed ones. 5 x 1200x680 with four of five keyframes fixed: 1.48 ms against 1.92
+// for the fixed ones. 5 x 1200x680 with four of five keyframes fixed: 1.38 ms against 1.92
 // with all entries' moments (2.23 before the products). Without a fixed keyframe its checks
 // cost 45 us of 1.34 ms, so that case has its own instance.
 template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED>
@@ -1544,6 +1568,7 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
         const uint32_t with = FIXED ? __ballot_sync(kFull, own) : 0u;
         const int span = FIXED && __popc(with) <= kHalf ? 32 : kHalf;
         int my_row = lane;                             // this lane's entry's row of S.mom
+        constexpr int kWide = FIXED ? 2 : 3;           // entries of a lane taken at once
 #pragma unroll 1
         for (int h = 0; h < n; h += span) {
             // 2. walk the entries h .. h + span - 1
@@ -1557,31 +1582,42 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
             uint32_t todo = mine & range;
             while (__any_sync(kFull, todo != 0u)) {
                 if (todo) {
-                    const uint32_t low = todo & (0u - todo);
-                    todo ^= low;
-                    const int j = 31 - __clz(low);
-                    const WalkEntry &e = S.e[j];
-                    const float4 ea = e.a, ec = e.c;
-                    const float2 eb = e.b;
-                    float alpha, raw;
-                    walk_alpha(ea, eb, nq, alpha, raw);
-                    const float om = __fsub_rn(1.0f, alpha);
-                    const float rom = reciprocal_walk(om);
-                    const float Ti = T * rom;
-                    float ca, cb;
-                    unpack2(fma2(pack2(ec.z, ec.w), g_bd, mul2(pack2(ec.x, ec.y), g_rg)), ca, cb);
-                    const float cg = ca + cb;
-                    // PLAIN: no alpha gradient and no background (the terms are zero)
-                    const float dal = PLAIN ? Ti * (cg - Sg)
-                                            : Ti * ((cg - Sg) + (1.0f - SA) * gA) - (Tf * rom) * bgdot;
-                    Sg = alpha * cg + om * Sg;
-                    if (!PLAIN) SA = alpha + om * SA;
-                    const float2 pair = make_float2(raw > kAlphaCap ? 0.f : dal * alpha, alpha * Ti);
-                    if (!FIXED)
-                        S.pairs[j - h][lane] = pair;
-                    else if (with & low)
-                        S.pairs[__popc(with & range & (low - 1u))][lane] = pair;
-                    T = Ti;
+                    // kWide entries: what does not depend on the others first
+                    uint32_t low[kWide];
+                    int j[kWide];
+                    float alpha[kWide], raw[kWide], om[kWide], rom[kWide], cg[kWide];
+#pragma unroll
+                    for (int q = 0; q < kWide; ++q) {
+                        low[q] = todo & (0u - todo);
+                        todo ^= low[q];
+                        j[q] = 31 - __clz(q > 0 && low[q] == 0u ? low[0] : low[q]);
+                        const WalkEntry &e = S.e[j[q]];
+                        const float4 ea = e.a, ec = e.c;
+                        const float2 eb = e.b;
+                        walk_alpha(ea, eb, nq, alpha[q], raw[q]);
+                        om[q] = __fsub_rn(1.0f, alpha[q]);
+                        rom[q] = reciprocal_walk(om[q]);
+                        float ca, cb;
+                        unpack2(fma2(pack2(ec.z, ec.w), g_bd, mul2(pack2(ec.x, ec.y), g_rg)), ca, cb);
+                        cg[q] = ca + cb;
+                    }
+#pragma unroll
+                    for (int q = 0; q < kWide; ++q) {
+                        const bool on = q == 0 || low[q] != 0u;
+                        const float Ti = T * rom[q];
+                        const float dal = PLAIN ? Ti * (cg[q] - Sg)
+                                                : Ti * ((cg[q] - Sg) + (1.0f - SA) * gA) - (Tf * rom[q]) * bgdot;
+                        const float2 pair = make_float2(raw[q] > kAlphaCap ? 0.f : dal * alpha[q], alpha[q] * Ti);
+                        if (on) {
+                            Sg = alpha[q] * cg[q] + om[q] * Sg;
+                            if (!PLAIN) SA = alpha[q] + om[q] * SA;
+                            T = Ti;
+                        }
+                        if (!FIXED) {
+                            if (on) S.pairs[j[q] - h][lane] = pair;
+                        } else if (with & low[q])
+                            S.pairs[__popc(with & range & (low[q] - 1u))][lane] = pair;
+                    }
                 }
             }
             __syncwarp();
