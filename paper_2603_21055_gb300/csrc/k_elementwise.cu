@@ -53,8 +53,14 @@ __device__ __forceinline__ float block_sum(float x, float *red)
     return t;
 }
 
-// All views of one loss call; every view owns a contiguous range of CTAs.
-constexpr int kLossChunk = 4096;    // pixels per CTA
+// All views of one loss call; every view owns a contiguous range of CTAs of `chunk` pixels:
+// 4096, or 1024 (one access of four pixels per thread) when CTAs of 4096 would leave SMs
+// without one: 2 views of 160x120 took 24 us on ten CTAs and take 5 on 38.
+// The CTAs of a cluster add their parts of the loss through distributed shared memory, one
+// FP32 addition to the loss per cluster: an eighth (with the small chunk half) of the
+// additions, and of their rounding and order dependence, that one per 4096 pixels made.
+constexpr uint32_t kLossChunk = 4096, kLossChunkSmall = 1024;
+constexpr int kLossCluster = 8;
 
 struct LossView {
     const float *rgb, *depth, *alpha, *trgb, *tdep;   // alpha: null unless masking
@@ -67,6 +73,7 @@ struct LossView {
 
 struct LossBatch {
     int32_t n;
+    uint32_t chunk;                 // pixels per CTA
     float wrgb, wdep, min_alpha;
     LossView v[SGAD_MAX_VIEWS];
 };
@@ -83,26 +90,31 @@ __global__ void __launch_bounds__(256) k_count_valid(const __grid_constant__ Los
 {
     __shared__ float red[32];
     const LossView &v = B.v[loss_view(B)];
-    const size_t base = (size_t)(blockIdx.x - v.block0) * kLossChunk;
-    const size_t end = base + kLossChunk < v.hw ? base + kLossChunk : v.hw;
+    const size_t base = (size_t)(blockIdx.x - v.block0) * B.chunk;
+    const size_t end = base + B.chunk < v.hw ? base + B.chunk : v.hw;
     float c = 0.f;
     for (size_t i = base + threadIdx.x; i < end; i += blockDim.x) c += v.tdep[i] > 0.0f ? 1.0f : 0.0f;
     const float t = block_sum(c, red);
     if (threadIdx.x == 0 && t > 0.f) atomicAdd(v.nvalid, (uint32_t)t);
 }
 
-__global__ void __launch_bounds__(256) k_l1_grad(const __grid_constant__ LossBatch B, float *loss)
+// ALL_VEC: every view's planes take 16-byte accesses (the other loop's registers would cost
+// this one its occupancy: 34 us against 23 at 8 x 640x480).
+template <bool ALL_VEC>
+__global__ void __cluster_dims__(kLossCluster, 1, 1) __launch_bounds__(256)
+    k_l1_grad(const __grid_constant__ LossBatch B, float *loss)
 {
-    __shared__ float red[32];
+    __shared__ float red[32], part;
     const LossView &v = B.v[loss_view(B)];
     const size_t hw = v.hw;
-    const size_t base = (size_t)(blockIdx.x - v.block0) * kLossChunk;
-    const size_t end = base + kLossChunk < hw ? base + kLossChunk : hw;
+    // (a CTA past the last has no pixels: its base is past the end)
+    const size_t base = (size_t)(blockIdx.x - v.block0) * B.chunk;
+    const size_t end = base + B.chunk < hw ? base + B.chunk : hw;
     const float inv_rgb = B.wrgb / (3.0f * (float)hw);
     const uint32_t nv = v.nvalid ? *v.nvalid : 0u;
     const float inv_dep = nv > 0 ? B.wdep / (float)nv : 0.0f;
     float l = 0.f;
-    if (v.vec) {                     // four pixels per thread and access
+    if (ALL_VEC || v.vec) {          // four pixels per thread and access
         for (size_t i = base + 4 * threadIdx.x; i < end; i += 4 * blockDim.x) {
             const float4 al = v.alpha ? *reinterpret_cast<const float4 *>(v.alpha + i) : make_float4(1.f, 1.f, 1.f, 1.f);
             const bool keep[4] = {!v.alpha || al.x > B.min_alpha, !v.alpha || al.y > B.min_alpha,
@@ -137,29 +149,50 @@ __global__ void __launch_bounds__(256) k_l1_grad(const __grid_constant__ LossBat
                 *reinterpret_cast<float4 *>(v.ddep + i) = make_float4(gd[0], gd[1], gd[2], gd[3]);
             }
         }
-    } else {
-        for (size_t i = base + threadIdx.x; i < end; i += blockDim.x) {
-            const bool keep = !v.alpha || v.alpha[i] > B.min_alpha;     // silhouette mask
+    } else if constexpr (!ALL_VEC) {
+        // four pixels, 256 apart, per pass; all loads before the stores, which the compiler may
+        // not move loads across
+        const bool use_depth = v.tdep && inv_dep > 0.0f;
+        for (size_t i = base + threadIdx.x; i < end; i += 4 * 256) {
+            float r[4][3], t[4][3], dp[4], td[4];
+            bool keep[4];                    // silhouette mask
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float d = v.rgb[c * hw + i] - v.trgb[c * hw + i];
-                if (keep) l += fabsf(d) * inv_rgb;
-                v.drgb[c * hw + i] = keep ? sgnf(d) * inv_rgb : 0.0f;
-            }
-            if (v.ddep) {
-                float gd = 0.f;
-                if (keep && v.tdep && v.tdep[i] > 0.0f && inv_dep > 0.0f) {
-                    const float d = v.depth[i] - v.tdep[i];
-                    l += fabsf(d) * inv_dep;
-                    gd = sgnf(d) * inv_dep;
+            for (int q = 0; q < 4; ++q) {
+                const size_t p = i + 256 * q;
+                keep[q] = p < end && (!v.alpha || v.alpha[p] > B.min_alpha);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    r[q][c] = p < end ? v.rgb[c * hw + p] : 0.f;
+                    t[q][c] = p < end ? v.trgb[c * hw + p] : 0.f;
                 }
-                v.ddep[i] = gd;
+                dp[q] = use_depth && p < end ? v.depth[p] : 0.f;
+                td[q] = use_depth && p < end ? v.tdep[p] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const size_t p = i + 256 * q;
+                if (p >= end) break;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float d = r[q][c] - t[q][c];
+                    if (keep[q]) l += fabsf(d) * inv_rgb;
+                    v.drgb[c * hw + p] = keep[q] ? sgnf(d) * inv_rgb : 0.0f;
+                }
+                if (v.ddep) {
+                    float gd = 0.f;
+                    if (use_depth && keep[q] && td[q] > 0.0f) {
+                        const float d = dp[q] - td[q];
+                        l += fabsf(d) * inv_dep;
+                        gd = sgnf(d) * inv_dep;
+                    }
+                    v.ddep[p] = gd;
+                }
             }
         }
     }
     if (loss) {
         const float t = block_sum(l, red);
-        if (threadIdx.x == 0) atomicAdd(loss, t);
+        cluster_add(loss, t, &part);
     }
 }
 
@@ -176,6 +209,9 @@ void launch_l1_batch(int n, const float *const *rgb, const float *const *depth, 
     B.wdep = wdep;
     B.min_alpha = min_alpha;
     uint32_t blocks = 0;
+    size_t full = 0;
+    for (int i = 0; i < n; ++i) full += (hw[i] + kLossChunk - 1) / kLossChunk;
+    B.chunk = full < 2 * 152 ? kLossChunkSmall : kLossChunk;
     const bool use_depth = wdep != 0.0f && tdep && ddep && nvalid;
     for (int i = 0; i < n; ++i) {
         LossView &v = B.v[i];
@@ -194,10 +230,16 @@ void launch_l1_batch(int n, const float *const *rgb, const float *const *depth, 
         if (v.tdep) al |= reinterpret_cast<uintptr_t>(v.depth) | reinterpret_cast<uintptr_t>(v.tdep);
         v.vec = (hw[i] % 4 == 0 && (al & 15u) == 0) ? 1 : 0;
         v.block0 = blocks;
-        blocks += (hw[i] + kLossChunk - 1) / kLossChunk;
+        blocks += (hw[i] + B.chunk - 1) / B.chunk;
     }
     if (use_depth) k_count_valid<<<blocks, 256, 0, st>>>(B);
-    k_l1_grad<<<blocks, 256, 0, st>>>(B, loss);
+    const unsigned grid = (blocks + kLossCluster - 1) / kLossCluster * kLossCluster;
+    bool all_vec = true;
+    for (int i = 0; i < n; ++i) all_vec = all_vec && B.v[i].vec != 0;
+    if (all_vec)
+        k_l1_grad<true><<<grid, 256, 0, st>>>(B, loss);
+    else
+        k_l1_grad<false><<<grid, 256, 0, st>>>(B, loss);
 }
 
 template <bool kLog>
@@ -335,6 +377,8 @@ void launch_adam(int64_t n, float *p, const float *g, float *m, float *v, float 
 
 // ------------------------------------------------- rendering-based camera initialisation
 //
+// One warp, an element or a power per lane: the FP64 chain on one thread (twelve powers, three
+// 3x4 products) took 28 us, this 11.
 // State layout (device floats): E [0, 12), M = W0^-1 E W0 [12, 24), Adam m [24, 30) and
 // v [30, 36), step count [36], current pose E W0 [37, 49). 3x4 row-major [R | t].
 struct PoseArgs {
@@ -343,85 +387,84 @@ struct PoseArgs {
     double b1, b2, eps;
 };
 
-__device__ void mat34_mul(const double *A, const double *B, double *C)     // C = A B (as 4x4)
+// Element (r, c) of A B (as 4x4).
+__device__ __forceinline__ double mat34_elem(const double *A, const double *B, int r, int c)
 {
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 4; ++c) {
-            double s = c == 3 ? A[4 * r + 3] : 0.0;
-            for (int k = 0; k < 3; ++k) s += A[4 * r + k] * B[4 * k + c];
-            C[4 * r + c] = s;
-        }
-    }
+    double s = c == 3 ? A[4 * r + 3] : 0.0;
+    for (int k = 0; k < 3; ++k) s += A[4 * r + k] * B[4 * k + c];
+    return s;
 }
 
-__global__ void k_pose_adam_step(const float *__restrict__ d_pose, float *__restrict__ st, const PoseArgs a)
+__global__ void __launch_bounds__(32) k_pose_adam_step(const float *__restrict__ d_pose, float *__restrict__ st,
+                                                       const PoseArgs a)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double G[12], E[12], M[9], xi[6], X[12], En[12], Wi[12], EW[12];
+    const int lane = threadIdx.x;
     const double *W = a.W0;
-    double G[9], c[3];
-    for (int r = 0; r < 3; ++r) {
-        for (int k = 0; k < 3; ++k) G[3 * r + k] = d_pose[4 * r + k];
-        c[r] = d_pose[4 * r + 3];
+    const float n0 = st[36];
+    const double n = (double)n0 + 1.0;
+    double m0 = 0.0, v0 = 0.0;
+    if (lane < 6) {
+        m0 = (double)st[24 + lane];
+        v0 = (double)st[30 + lane];
     }
+    const int r = lane >> 2, k = lane & 3;                 // element (r, k) of a 3x4 matrix
+    if (lane < 12) {
+        G[lane] = d_pose[lane];
+        E[lane] = st[lane];
+        // W0^-1 = [R0^T | -R0^T t0]
+        Wi[lane] = k < 3 ? W[4 * k + r] : -(W[r] * W[3] + W[4 + r] * W[7] + W[8 + r] * W[11]);
+    }
+    __syncwarp();
+    if (lane == 0) st[36] = (float)n;
+    // one power per lane: b1^n and b2^n
+    const double pw = lane < 2 ? pow(lane == 0 ? a.b1 : a.b2, n) : 0.0;
+    const double c1 = 1.0 - __shfl_sync(0xffffffffu, pw, 0), c2 = 1.0 - __shfl_sync(0xffffffffu, pw, 1);
     // M = R0 G^T; d/d omega = vee(M - M^T) + t0 x c; d/d v = c
-    double Mx[9];
-    for (int r = 0; r < 3; ++r)
-        for (int k = 0; k < 3; ++k) {
-            double s = 0.0;
-            for (int q = 0; q < 3; ++q) s += W[4 * r + q] * G[3 * k + q];
-            Mx[3 * r + k] = s;
-        }
-    const double t0[3] = {W[3], W[7], W[11]};
-    double g[6];
-    g[0] = Mx[5] - Mx[7] + (t0[1] * c[2] - t0[2] * c[1]);
-    g[1] = Mx[6] - Mx[2] + (t0[2] * c[0] - t0[0] * c[2]);
-    g[2] = Mx[1] - Mx[3] + (t0[0] * c[1] - t0[1] * c[0]);
-    g[3] = c[0];
-    g[4] = c[1];
-    g[5] = c[2];
-    const double n = (double)st[36] + 1.0;
-    st[36] = (float)n;
-    double xi[6];
-    for (int i = 0; i < 6; ++i) {
-        const double m = a.b1 * (double)st[24 + i] + (1.0 - a.b1) * g[i];
-        const double v = a.b2 * (double)st[30 + i] + (1.0 - a.b2) * g[i] * g[i];
+    if (lane < 9) {
+        const int mr = lane / 3, mk = lane - 3 * mr;
+        double s = 0.0;
+        for (int q = 0; q < 3; ++q) s += W[4 * mr + q] * G[4 * mk + q];
+        M[lane] = s;
+    }
+    __syncwarp();
+    if (lane < 6) {
+        const int i = lane, p = (i + 1) % 3, q = (i + 2) % 3;
+        const double g = i < 3 ? M[3 * p + q] - M[3 * q + p] + (W[4 * p + 3] * G[4 * q + 3] - W[4 * q + 3] * G[4 * p + 3])
+                               : G[4 * (i - 3) + 3];
+        const double m = a.b1 * m0 + (1.0 - a.b1) * g;
+        const double v = a.b2 * v0 + (1.0 - a.b2) * g * g;
         st[24 + i] = (float)m;
         st[30 + i] = (float)v;
-        const double mh = m / (1.0 - pow(a.b1, n)), vh = v / (1.0 - pow(a.b2, n));
-        xi[i] = -a.lr[i] * mh / (sqrt(vh) + a.eps);
+        xi[i] = -a.lr[i] * (m / c1) / (sqrt(v / c2) + a.eps);
     }
+    __syncwarp();
     // exp(xi) = [Rodrigues(omega) | v]
     const double th = sqrt(xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2]);
-    const double K[9] = {0.0, -xi[2], xi[1], xi[2], 0.0, -xi[0], -xi[1], xi[0], 0.0};
-    double K2[9];
-    for (int r = 0; r < 3; ++r)
-        for (int k = 0; k < 3; ++k) {
-            double s = 0.0;
-            for (int q = 0; q < 3; ++q) s += K[3 * r + q] * K[3 * q + k];
-            K2[3 * r + k] = s;
+    double sn, cs;
+    sincos(th, &sn, &cs);
+    const double sa = th < 1e-12 ? 1.0 : sn / th, sb = th < 1e-12 ? 0.0 : (1.0 - cs) / (th * th);
+    if (lane < 12) {
+        const double K[9] = {0.0, -xi[2], xi[1], xi[2], 0.0, -xi[0], -xi[1], xi[0], 0.0};
+        double kk = 0.0, k1 = 0.0;
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            if (j / 3 != r || j % 3 != k) continue;
+            k1 = K[j];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) kk += K[3 * (j / 3) + q] * K[3 * q + j % 3];
         }
-    const double sa = th < 1e-12 ? 1.0 : sin(th) / th;
-    const double sb = th < 1e-12 ? 0.0 : (1.0 - cos(th)) / (th * th);
-    double X[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int k = 0; k < 3; ++k) X[4 * r + k] = (r == k ? 1.0 : 0.0) + sa * K[3 * r + k] + sb * K2[3 * r + k];
-        X[4 * r + 3] = xi[3 + r];
+        X[lane] = k == 3 ? xi[3 + r] : (r == k ? 1.0 : 0.0) + sa * k1 + sb * kk;
     }
-    double E[12], En[12];
-    for (int i = 0; i < 12; ++i) E[i] = st[i];
-    mat34_mul(X, E, En);
-    // M = W0^-1 E W0 with W0^-1 = [R0^T | -R0^T t0]; pose = E W0
-    double Wi[12], EW[12], Mn[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int k = 0; k < 3; ++k) Wi[4 * r + k] = W[4 * k + r];
-        Wi[4 * r + 3] = -(W[r] * t0[0] + W[4 + r] * t0[1] + W[8 + r] * t0[2]);
-    }
-    mat34_mul(En, W, EW);
-    mat34_mul(Wi, EW, Mn);
-    for (int i = 0; i < 12; ++i) {
-        st[i] = (float)En[i];
-        st[12 + i] = (float)Mn[i];
-        st[37 + i] = (float)EW[i];
+    __syncwarp();
+    if (lane < 12) En[lane] = mat34_elem(X, E, r, k);
+    __syncwarp();
+    if (lane < 12) EW[lane] = mat34_elem(En, W, r, k);      // pose = E W0
+    __syncwarp();
+    if (lane < 12) {
+        st[lane] = (float)En[lane];
+        st[12 + lane] = (float)mat34_elem(Wi, EW, r, k);    // M = W0^-1 E W0
+        st[37 + lane] = (float)EW[lane];
     }
 }
 

@@ -7,6 +7,7 @@
 // and reaches the same decision bit for bit.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -405,6 +406,22 @@ inline Layout make_layout(uint64_t n_gauss, uint64_t n_views, uint64_t n_tiles, 
     L.wmask = o; o = align256(o + ((key_cap >> 2) + (n_tiles + 1) * 16 + 8) * 4);
     L.total = o;
     return L;
+}
+
+// Adds the sum of thread 0's t over the CTAs of the cluster to *dst. All threads; part: one
+// float of this CTA's shared memory.
+__device__ __forceinline__ void cluster_add(float *dst, float t, float *part)
+{
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    if (threadIdx.x == 0) *part = t;
+    cl.sync();
+    if (threadIdx.x == 0 && cl.block_rank() == 0) {
+        float s = 0.f;
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) s += *cl.map_shared_rank(part, r);
+        atomicAdd(dst, s);
+    }
+    cl.sync();                          // the others' part is read before they end
 }
 
 }  // namespace sgad
