@@ -15,6 +15,7 @@
 //                     pixel blocks the Gaussian's alpha >= 1/255 box may touch (the sort
 //                     keeps its order and separates the two).
 #include "sgad_device.cuh"
+#include "sgad_launch.cuh"
 
 namespace sgad {
 
@@ -39,6 +40,7 @@ template <bool TRIM>
 __global__ void __launch_bounds__(256) k_project_count(const __grid_constant__ Scene sc, World *__restrict__ world,
                                                        uint32_t *__restrict__ tile_cnt, uint2 *__restrict__ rects)
 {
+    dependency_wait();
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = g < sc.n_gauss;
     float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -132,6 +134,7 @@ __device__ __forceinline__ int order_class(uint32_t len)
 __global__ void __launch_bounds__(1024) k_scan_tiles(uint32_t *__restrict__ cnt, uint32_t *__restrict__ off, int n_tiles,
                                                      uint64_t key_cap, WsHeader *hdr, uint32_t *__restrict__ order)
 {
+    dependency_wait();
     __shared__ uint32_t warp_sums[32];
     __shared__ uint64_t carry_s;
     __shared__ uint32_t cls_cnt[kOrderClasses];
@@ -243,6 +246,7 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Scene sc, 
                                               const uint32_t *__restrict__ off, uint32_t *__restrict__ cursor,
                                               uint64_t *__restrict__ entries, WsHeader *hdr)
 {
+    dependency_wait(rects, off);
     if (hdr->overflow) return;
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = g < sc.n_gauss;
@@ -337,15 +341,15 @@ void launch_project_count(const Scene &sc, World *world, uint32_t *tile_cnt, uin
     const unsigned blocks = (sc.n_gauss + 255) / 256;
     if (!blocks) return;
     if (trim)
-        k_project_count<true><<<blocks, 256, 0, st>>>(sc, world, tile_cnt, rects);
+        launch_after(k_project_count<true>, blocks, 256, 0, st, sc, world, tile_cnt, rects);
     else
-        k_project_count<false><<<blocks, 256, 0, st>>>(sc, world, tile_cnt, rects);
+        launch_after(k_project_count<false>, blocks, 256, 0, st, sc, world, tile_cnt, rects);
 }
 
 void launch_scan_tiles(uint32_t *cnt, uint32_t *off, int n_tiles, uint64_t key_cap, WsHeader *hdr, uint32_t *order,
                        cudaStream_t st)
 {
-    k_scan_tiles<<<1, 1024, 0, st>>>(cnt, off, n_tiles, key_cap, hdr, order);
+    launch_after(k_scan_tiles, 1, 1024, 0, st, cnt, off, n_tiles, key_cap, hdr, order);
 }
 
 // pack: entries with block masks (n_gauss <= 2^24, rectangles with trims).
@@ -355,9 +359,9 @@ void launch_emit(const Scene &sc, const uint2 *rects, const uint32_t *off, uint3
     const unsigned blocks = (sc.n_gauss + 255) / 256;
     if (!blocks) return;
     if (pack)
-        k_emit<true><<<blocks, 256, 0, st>>>(sc, rects, off, cursor, entries, hdr);
+        launch_after(k_emit<true>, blocks, 256, 0, st, sc, rects, off, cursor, entries, hdr);
     else
-        k_emit<false><<<blocks, 256, 0, st>>>(sc, rects, off, cursor, entries, hdr);
+        launch_after(k_emit<false>, blocks, 256, 0, st, sc, rects, off, cursor, entries, hdr);
 }
 
 }  // namespace sgad

@@ -50,10 +50,11 @@ cudaError_t persistent_blocks(bool fwd, int batch, const Scene &sc, int max_bloc
     return cudaSuccess;
 }
 
+// queue_clear: the pass's work queue is at its start (cleared with the pass's other state).
 cudaError_t launch_composite(bool fwd, int batch, int schedule, int max_blocks, const Scene &sc, const World *world,
                              const uint32_t *off, const uint64_t *entries, float *pix_t, uint32_t *pix_n, float4 *gacc,
                              WsHeader *hdr, const uint32_t *order, uint32_t *contrib, uint32_t *wmask,
-                             const uint8_t *bmask, cudaStream_t st)
+                             const uint8_t *bmask, bool queue_clear, cudaStream_t st)
 {
     if (sc.n_tiles <= 0) return cudaSuccess;
     CompositeArgs a = {};
@@ -80,8 +81,11 @@ cudaError_t launch_composite(bool fwd, int batch, int schedule, int max_blocks, 
             a.tile0 = tile0;
             a.n_launch_tiles = n_tiles;
             a.order = ord;
-            cudaError_t r = cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), st);
-            if (r != cudaSuccess) return r;
+            if (!queue_clear) {
+                const cudaError_t r = cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), st);
+                if (r != cudaSuccess) return r;
+            }
+            queue_clear = false;
             return dispatch(fwd, batch, sc, a, blocks < n_tiles ? blocks : n_tiles, nullptr, st);
         };
         if (schedule == SGAD_SCHEDULE_PER_VIEW) {
@@ -100,7 +104,7 @@ cudaError_t launch_composite(bool fwd, int batch, int schedule, int max_blocks, 
         if (e != cudaSuccess) return e;
         a.order = order;
         a.queue = fwd ? &hdr->queue_fwd : &hdr->queue_bwd;
-        e = cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), st);
+        if (!queue_clear) e = cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) return e;
         return dispatch(fwd, batch, sc, a, blocks, nullptr, st);
     }

@@ -50,6 +50,7 @@
 #pragma once
 
 #include "sgad_device.cuh"
+#include "sgad_launch.cuh"
 
 namespace sgad {
 
@@ -686,6 +687,7 @@ template <int TW, int TH, bool MASKS>
 __global__ void __launch_bounds__(kFwdlThreads, SGAD_FWDL_MINBLOCKS)
     k_composite_fwdl(const __grid_constant__ Scene sc, const CompositeArgs a)
 {
+    dependency_wait();
     static_assert(TW * TH == 256 && TW % 8 == 0 && TH % 4 == 0, "tile must hold eight 8x4 blocks");
     __shared__ FwdlWarpSmem smem[kFwdlThreads / 32];
     FwdlWarpSmem &S = smem[threadIdx.x >> 5];
@@ -1679,6 +1681,7 @@ template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED>
 __global__ void __launch_bounds__(kLocalThreads, SGAD_BWDL_MINBLOCKS)
     k_composite_bwdl(const __grid_constant__ Scene sc, const CompositeArgs a)
 {
+    dependency_wait();
     static_assert(TW * TH == 256 && TW % 8 == 0 && TH % 4 == 0, "tile must hold eight 8x4 blocks");
     extern __shared__ float4 bwdl_smem[];
     BwdlWarpSmem &S = reinterpret_cast<BwdlWarpSmem *>(bwdl_smem)[threadIdx.x >> 5];
@@ -1811,13 +1814,13 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
     for (int i = 0; i < sc.n_views && plain; ++i) plain = sc.view[i].g_alpha == nullptr;
     for (int i = 0; i < sc.n_kf && !fixed; ++i) fixed = sc.kf[i].learnable == 0;
     if (a.pose)
-        k_composite_bwdl<TW, TH, true, false, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+        launch_after(k_composite_bwdl<TW, TH, true, false, true>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
     else if (!plain)
-        k_composite_bwdl<TW, TH, false, false, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+        launch_after(k_composite_bwdl<TW, TH, false, false, true>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
     else if (fixed)
-        k_composite_bwdl<TW, TH, false, true, true><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+        launch_after(k_composite_bwdl<TW, TH, false, true, true>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
     else
-        k_composite_bwdl<TW, TH, false, true, false><<<grid_blocks, kLocalThreads, kLocalSmemBytes, st>>>(sc, a);
+        launch_after(k_composite_bwdl<TW, TH, false, true, false>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
     return cudaGetLastError();
 }
 
@@ -1828,9 +1831,9 @@ cudaError_t launch_fwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_fwdl<TW, TH, true>, kFwdlThreads, 0);
     if (grid_blocks <= 0) return cudaSuccess;
     if (a.bmask)
-        k_composite_fwdl<TW, TH, true><<<grid_blocks, kFwdlThreads, 0, st>>>(sc, a);
+        launch_after(k_composite_fwdl<TW, TH, true>, grid_blocks, kFwdlThreads, 0, st, sc, a);
     else
-        k_composite_fwdl<TW, TH, false><<<grid_blocks, kFwdlThreads, 0, st>>>(sc, a);
+        launch_after(k_composite_fwdl<TW, TH, false>, grid_blocks, kFwdlThreads, 0, st, sc, a);
     return cudaGetLastError();
 }
 

@@ -5,11 +5,36 @@
 //   k_l1_grad    : L1 terms of Eq. 1 and their image gradients (a8).
 //   k_adam       : bias-corrected Adam step (a11).
 #include "sgad_device.cuh"
+#include "sgad_launch.cuh"
 
 namespace sgad {
 
+// Zeroes all ranges of a list: one launch where one memset each (and its gap) cost about 2 us.
+__global__ void __launch_bounds__(256) k_clear(const __grid_constant__ ClearList c)
+{
+    dependency_wait();
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    for (int r = 0; r < c.n; ++r) {
+        uint32_t *const p = c.at[r];
+        const size_t n = c.words[r];
+        const size_t vec = (reinterpret_cast<uintptr_t>(p) & 15) == 0 ? n / 4 : 0;
+        for (size_t i = first; i < vec; i += step) reinterpret_cast<uint4 *>(p)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (size_t i = 4 * vec + first; i < n; i += step) p[i] = 0u;
+    }
+}
+
+cudaError_t launch_clear(const ClearList &c, cudaStream_t st)
+{
+    size_t most = 0;
+    for (int r = 0; r < c.n; ++r) most = most > c.words[r] ? most : c.words[r];
+    if (!most) return cudaSuccess;
+    const size_t blocks = (most + 1023) / 1024;
+    return launch_after(k_clear, (unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, st, c);
+}
+
 __global__ void __launch_bounds__(256) k_finalize(const __grid_constant__ Scene sc, const float4 *__restrict__ gacc)
 {
+    dependency_wait(gacc);
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= sc.n_gauss) return;
     const KfDev &k = sc.kf[find_kf(sc, g)];
@@ -35,7 +60,7 @@ __global__ void __launch_bounds__(256) k_finalize(const __grid_constant__ Scene 
 void launch_finalize(const Scene &sc, const float4 *gacc, cudaStream_t st)
 {
     const unsigned blocks = (sc.n_gauss + 255) / 256;
-    if (blocks) k_finalize<<<blocks, 256, 0, st>>>(sc, gacc);
+    if (blocks) launch_after(k_finalize, blocks, 256, 0, st, sc, gacc);
 }
 
 __device__ __forceinline__ float sgnf(float x) { return x > 0.0f ? 1.0f : (x < 0.0f ? -1.0f : 0.0f); }
@@ -88,6 +113,7 @@ __device__ __forceinline__ int loss_view(const LossBatch &B)
 
 __global__ void __launch_bounds__(256) k_count_valid(const __grid_constant__ LossBatch B)
 {
+    dependency_wait();
     __shared__ float red[32];
     const LossView &v = B.v[loss_view(B)];
     const size_t base = (size_t)(blockIdx.x - v.block0) * B.chunk;
@@ -104,6 +130,7 @@ template <bool ALL_VEC>
 __global__ void __cluster_dims__(kLossCluster, 1, 1) __launch_bounds__(256)
     k_l1_grad(const __grid_constant__ LossBatch B, float *loss)
 {
+    dependency_wait();
     __shared__ float red[32], part;
     const LossView &v = B.v[loss_view(B)];
     const size_t hw = v.hw;
@@ -232,20 +259,21 @@ void launch_l1_batch(int n, const float *const *rgb, const float *const *depth, 
         v.block0 = blocks;
         blocks += (hw[i] + B.chunk - 1) / B.chunk;
     }
-    if (use_depth) k_count_valid<<<blocks, 256, 0, st>>>(B);
+    if (use_depth) launch_after(k_count_valid, blocks, 256, 0, st, B);
     const unsigned grid = (blocks + kLossCluster - 1) / kLossCluster * kLossCluster;
     bool all_vec = true;
     for (int i = 0; i < n; ++i) all_vec = all_vec && B.v[i].vec != 0;
     if (all_vec)
-        k_l1_grad<true><<<grid, 256, 0, st>>>(B, loss);
+        launch_after(k_l1_grad<true>, grid, 256, 0, st, B, loss);
     else
-        k_l1_grad<false><<<grid, 256, 0, st>>>(B, loss);
+        launch_after(k_l1_grad<false>, grid, 256, 0, st, B, loss);
 }
 
 template <bool kLog>
 __global__ void k_adam(int64_t n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
                        float *__restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2)
 {
+    dependency_wait(g);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float pi = p[i];
         const float gi = kLog ? g[i] * pi : g[i];     // d/d(log s) = s d/ds
@@ -292,6 +320,7 @@ __device__ __forceinline__ void adam_one(float &p, float g, float &m, float &v, 
 
 __global__ void __launch_bounds__(256) k_adam_multi(const __grid_constant__ AdamBatch B, const int32_t *step)
 {
+    dependency_wait();
     int lo = 0, hi = B.n - 1;
     while (lo < hi) {                 // last tensor whose first CTA <= blockIdx.x
         const int mid = (lo + hi + 1) >> 1;
@@ -331,7 +360,11 @@ __global__ void __launch_bounds__(256) k_adam_multi(const __grid_constant__ Adam
     }
 }
 
-__global__ void k_increment(int32_t *c) { *c += 1; }
+__global__ void k_increment(int32_t *c)
+{
+    dependency_wait();
+    *c += 1;
+}
 
 cudaError_t launch_adam_multi(int n_t, const sgad_adam_tensor *t, float b1, float b2, float eps, int32_t *step,
                               cudaStream_t st)
@@ -358,8 +391,8 @@ cudaError_t launch_adam_multi(int n_t, const sgad_adam_tensor *t, float b1, floa
         blocks += (t[i].n + kAdamChunk - 1) / kAdamChunk;
     }
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    if (blocks > 0) k_adam_multi<<<(unsigned)blocks, 256, 0, st>>>(B, step);
-    k_increment<<<1, 1, 0, st>>>(step);
+    if (blocks > 0) launch_after(k_adam_multi, (unsigned)blocks, 256, 0, st, B, step);
+    launch_after(k_increment, 1, 1, 0, st, step);
     return cudaGetLastError();
 }
 
@@ -370,9 +403,9 @@ void launch_adam(int64_t n, float *p, const float *g, float *m, float *v, float 
     if (blocks > 152 * 8) blocks = 152 * 8;
     if (blocks <= 0) return;
     if (log_mode)
-        k_adam<true><<<(unsigned)blocks, 256, 0, st>>>(n, p, g, m, v, lr, b1, b2, eps, c1, c2);
+        launch_after(k_adam<true>, (unsigned)blocks, 256, 0, st, n, p, g, m, v, lr, b1, b2, eps, c1, c2);
     else
-        k_adam<false><<<(unsigned)blocks, 256, 0, st>>>(n, p, g, m, v, lr, b1, b2, eps, c1, c2);
+        launch_after(k_adam<false>, (unsigned)blocks, 256, 0, st, n, p, g, m, v, lr, b1, b2, eps, c1, c2);
 }
 
 // ------------------------------------------------- rendering-based camera initialisation
@@ -398,6 +431,7 @@ __device__ __forceinline__ double mat34_elem(const double *A, const double *B, i
 __global__ void __launch_bounds__(32) k_pose_adam_step(const float *__restrict__ d_pose, float *__restrict__ st,
                                                        const PoseArgs a)
 {
+    dependency_wait(d_pose);
     __shared__ double G[12], E[12], M[9], xi[6], X[12], En[12], Wi[12], EW[12];
     const int lane = threadIdx.x;
     const double *W = a.W0;
@@ -480,7 +514,7 @@ cudaError_t launch_pose_adam_step(const float *d_pose, const float *W0, float *s
     a.b1 = b1;
     a.b2 = b2;
     a.eps = eps;
-    k_pose_adam_step<<<1, 32, 0, st>>>(d_pose, state, a);
+    launch_after(k_pose_adam_step, 1, 32, 0, st, d_pose, state, a);
     return cudaGetLastError();
 }
 

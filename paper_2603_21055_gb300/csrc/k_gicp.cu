@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "sgad_gicp.h"
+#include "sgad_launch.cuh"
 
 namespace sgad {
 sgad_status report_error(sgad_status code, const char *msg);
@@ -268,6 +269,7 @@ __device__ __forceinline__ bool cell_valid(const SelArgs &a, int c, int *u, int 
 
 __global__ void __launch_bounds__(256) k_select_count(const __grid_constant__ SelArgs a)
 {
+    sgad::dependency_wait();
     __shared__ int red[8];
     if (blockIdx.x == 0 && threadIdx.x == 0) a.state->status = 0;   // a new frame: fresh flags
     int n = 0;
@@ -284,6 +286,7 @@ __global__ void __launch_bounds__(256) k_select_count(const __grid_constant__ Se
 
 __global__ void __launch_bounds__(256) k_select_write(const __grid_constant__ SelArgs a)
 {
+    sgad::dependency_wait();
     __shared__ int red[8];
     const int prefix = block_prefix(a.blk, blockIdx.x, red);
     int u[4], v[4];
@@ -611,6 +614,7 @@ __device__ __forceinline__ uint64_t hash_nearest(const ShapeArgs &a, float4 me, 
 template <bool WINDOW>
 __global__ void __launch_bounds__(kShapeThreads) k_shape(const __grid_constant__ ShapeArgs a)
 {
+    sgad::dependency_wait();
     __shared__ float s_cov[kShapePts][7];
     __shared__ uint64_t s_buf[WINDOW ? 1 : kShapeThreads / 32][64];
     const int n = *a.count;
@@ -699,6 +703,7 @@ __global__ void __launch_bounds__(256) k_hash_link(const float4 *pos, int32_t *c
                                                    uint32_t mask, int32_t *head, float4 *pts,
                                                    const GicpState *commit)
 {
+    sgad::dependency_wait();
     const int n = min(commit ? commit->map_old + commit->ins_total : *count, cap);
     if (commit && blockIdx.x == 0 && threadIdx.x == 0) *count = n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1194,6 +1199,7 @@ __device__ bool solve_state(GicpState *st, const double *sys, double &step2)
 
 __global__ void k_gicp_init(GicpState *st, PoseD p0, int keep_pose, int max_iters, float tol, int done)
 {
+    sgad::dependency_wait();
     if (!keep_pose)
         for (int k = 0; k < 12; ++k) st->pose[k] = p0.p[k];
     for (int k = 0; k < 12; ++k) st->posef[k] = (float)st->pose[k];
@@ -1243,6 +1249,7 @@ __device__ __forceinline__ bool overlaps(float3 x, const Grid &g, float d_ov)
 // loads, so it takes a warp's lanes for the 27 nearest cells at once.
 __global__ void __launch_bounds__(1024) k_insert_flag(const __grid_constant__ InsArgs a)
 {
+    sgad::dependency_wait();
     __shared__ int s_keep[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n = *a.scount;
@@ -1266,6 +1273,7 @@ __global__ void __launch_bounds__(1024) k_insert_flag(const __grid_constant__ In
 
 __global__ void __launch_bounds__(256) k_insert_write(const __grid_constant__ InsArgs a)
 {
+    sgad::dependency_wait();
     __shared__ int red[8];
     const int prefix = block_prefix(a.blk, blockIdx.x * (256 / kInsPts), red);
     const int i = blockIdx.x * 256 + threadIdx.x;
@@ -1378,7 +1386,8 @@ sgad_status hash_build(const float4 *pos, int32_t *count, int32_t capacity, floa
     if (cudaMemsetAsync(head, 0, (size_t)table * sizeof(int32_t), st) != cudaSuccess)
         return report_error(SGAD_ERR_CUDA, "sgad_gicp: memset failed");
     const int blocks = std::min((capacity + 255) / 256, 4 * 152);
-    k_hash_link<<<blocks, 256, 0, st>>>(pos, count, capacity, inv_cell, (uint32_t)table - 1u, head, pts, commit);
+    sgad::launch_after(k_hash_link, blocks, 256, 0, st, pos, count, capacity, inv_cell, (uint32_t)table - 1u, head, pts,
+                       commit);
     return launched("sgad_gicp: index launch failed");
 }
 
@@ -1475,8 +1484,8 @@ extern "C" sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_cam
     a.cell_point = window ? a.point_cell + p->src_capacity : nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nb = (int)((ncells + kSelBlock - 1) / kSelBlock);
-    k_select_count<<<nb, 256, 0, st>>>(a);
-    k_select_write<<<nb, 256, 0, st>>>(a);
+    sgad::launch_after(k_select_count, nb, 256, 0, st, a);
+    sgad::launch_after(k_select_write, nb, 256, 0, st, a);
     ShapeArgs sa;
     std::memset(&sa, 0, sizeof(sa));
     sa.pos = reinterpret_cast<const float4 *>(out->pos);
@@ -1496,7 +1505,7 @@ extern "C" sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_cam
         sa.w.step_y = (float)p->stride / cam->fy;
         sa.w.x0 = -cam->cx / cam->fx;
         sa.w.y0 = -cam->cy / cam->fy;
-        k_shape<true><<<sb, kShapeThreads, 0, st>>>(sa);
+        sgad::launch_after(k_shape<true>, sb, kShapeThreads, 0, st, sa);
     } else {
         // cells of about twice the selection spacing at 2 m (a performance choice only: the
         // search proves its result)
@@ -1510,7 +1519,7 @@ extern "C" sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_cam
         if ((s = hash_build(sa.pos, out->count, out->capacity, g.inv_cell, L.knn_table,
                             at<int32_t>(workspace, L.knn_head), at<float4>(workspace, L.knn_pts), nullptr, st)))
             return s;
-        k_shape<false><<<sb, kShapeThreads, 0, st>>>(sa);
+        sgad::launch_after(k_shape<false>, sb, kShapeThreads, 0, st, sa);
     }
     return launched("sgad_gicp_frame: launch failed");
 }
@@ -1587,7 +1596,8 @@ extern "C" sgad_status sgad_gicp_set_pose(const double pose[12], void *workspace
     if (s) return s;
     PoseD p0;
     std::memcpy(p0.p, pose, sizeof(p0.p));
-    k_gicp_init<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(at<GicpState>(workspace, 0), p0, 0, 0, 0.f, 1);
+    sgad::launch_after(k_gicp_init, 1, 1, 0, static_cast<cudaStream_t>(stream), at<GicpState>(workspace, 0), p0, 0, 0,
+                       0.f, 1);
     return launched("sgad_gicp_set_pose: launch failed");
 }
 
@@ -1625,7 +1635,7 @@ extern "C" sgad_status sgad_gicp_track(const sgad_gicp_params *p, const sgad_gau
         if (e == cudaSuccess && dev >= 0 && dev < 64) resident[dev] = blocks;
     }
     if (e != cudaSuccess || blocks < 1) return report_error(SGAD_ERR_CUDA, "sgad_gicp_track: no resident blocks");
-    k_gicp_init<<<1, 1, 0, st>>>(a.state, p0, pose0 ? 0 : 1, p->max_iters, p->tol, 0);
+    sgad::launch_after(k_gicp_init, 1, 1, 0, st, a.state, p0, pose0 ? 0 : 1, p->max_iters, p->tol, 0);
     void *args[] = {&a};
     e = cudaLaunchCooperativeKernel((const void *)k_gicp_step<true>, dim3(std::min(blocks, L.rows)),
                                     dim3(kStepThreads), args, smem, st);
@@ -1655,8 +1665,8 @@ extern "C" sgad_status sgad_gicp_insert(const sgad_gicp_params *p, const sgad_ga
     a.state = at<GicpState>(workspace, L.state);
     a.flags = at<int32_t>(workspace, L.ins_flags);
     a.blk = at<int32_t>(workspace, L.ins_counts);
-    k_insert_flag<<<(p->src_capacity + kInsPts - 1) / kInsPts, 1024, 0, st>>>(a);
-    k_insert_write<<<L.max_blocks, 256, 0, st>>>(a);
+    sgad::launch_after(k_insert_flag, (p->src_capacity + kInsPts - 1) / kInsPts, 1024, 0, st, a);
+    sgad::launch_after(k_insert_write, L.max_blocks, 256, 0, st, a);
     if ((s = launched("sgad_gicp_insert: launch failed"))) return s;
     return build_index(p, map, workspace, L, a.state, st);
 }

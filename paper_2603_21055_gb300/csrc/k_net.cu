@@ -26,6 +26,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include "sgad_launch.cuh"
 #include "sgad_net_device.cuh"
 #include "tc5.cuh"
 
@@ -55,6 +56,7 @@ __device__ __forceinline__ size_t planar_unit(size_t p, int c, int kc, int w)
 __global__ void k_pack_input(const float *__restrict__ rgb, const float *__restrict__ depth, uint4 *__restrict__ x0,
                              int n, int h, int w)
 {
+    dependency_wait(rgb, depth);
     const size_t hw = (size_t)h * w, total = (size_t)n * hw;
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
         const size_t f = p / hw, q = p - f * hw;
@@ -77,6 +79,7 @@ __global__ void k_pack_input(const float *__restrict__ rgb, const float *__restr
 // taps (unit = 8 consecutive output channels of one input channel). blockIdx.y: layer.
 __global__ void k_prep_weights(const PrepArgs a)
 {
+    dependency_wait();
     const float *w = a.w[blockIdx.y];
     uint4 *fwd = a.fwd[blockIdx.y], *bwd = a.bwd[blockIdx.y];
     const int ci_p = a.ci_p[blockIdx.y], co_p = a.co_p[blockIdx.y];
@@ -111,6 +114,7 @@ __global__ void k_prep_weights(const PrepArgs a)
 // Zeroes the parameter gradients of all layers. blockIdx.y: layer.
 __global__ void k_zero_grads(const ZeroArgs a)
 {
+    dependency_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.n_w[blockIdx.y]) a.dw[blockIdx.y][i] = 0.f;
     if (i < a.n_b[blockIdx.y]) a.db[blockIdx.y][i] = 0.f;
@@ -121,6 +125,7 @@ __global__ void k_zero_grads(const ZeroArgs a)
 __global__ void k_loss(const float2 *__restrict__ y4, const float *__restrict__ td, const float *__restrict__ tl,
                        float lw, uint4 *__restrict__ dy4, float *loss, size_t total, int w)
 {
+    dependency_wait(y4, td, tl);
     const float inv = 1.0f / (float)total;
     float acc = 0.f;
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
@@ -311,6 +316,7 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
             tc::mbar_init(&tempty[i], 4);
         }
     }
+    dependency_wait();
     if (MODE != kModeMask && threadIdx.x >= 64 && threadIdx.x < 64 + CO) bias[threadIdx.x - 64] = a.bias[threadIdx.x - 64];
 #pragma unroll 6
     for (int i = threadIdx.x; i < S::kB / 16; i += 192) sB[i] = a.wB[i];
@@ -541,6 +547,7 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    dependency_wait();
     const uint32_t tmem = taddr_s;
     constexpr uint32_t idesc = idesc_bf16_mn(128, CO);
 
@@ -736,8 +743,7 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (grid > sms * (512 / (kAcc * CO))) grid = sms * (512 / (kAcc * CO));
-    k_conv3x3_tma<CI, CO, MODE><<<grid, 192, smem, st>>>(wide, halo, a);
-    return cudaGetLastError();
+    return launch_after(k_conv3x3_tma<CI, CO, MODE>, grid, 192, smem, st, wide, halo, a);
 }
 
 template <int CI, int CO>
@@ -763,8 +769,7 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
     if (grid > cap) grid = (int)cap;
     const long long by_work = blocks / kWgTiles;
     if (grid > by_work) grid = (int)(by_work > sms ? by_work : (grid < sms ? grid : sms));
-    k_conv3x3_wgrad_tma<CI, CO><<<grid, 128, S::bytes, st>>>(xm, wide, halo, a);
-    return cudaGetLastError();
+    return launch_after(k_conv3x3_wgrad_tma<CI, CO>, grid, 128, S::bytes, st, xm, wide, halo, a);
 }
 
 template cudaError_t launch_conv<16, 32, kModeRelu>(const ConvArgs &, cudaStream_t);
@@ -781,24 +786,21 @@ cudaError_t launch_pack_input(const float *rgb, const float *depth, uint4 *x0, i
     const size_t total = (size_t)n * h * w;
     if (!total) return cudaSuccess;
     const int grid = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-    k_pack_input<<<grid, 256, 0, st>>>(rgb, depth, x0, n, h, w);
-    return cudaGetLastError();
+    return launch_after(k_pack_input, grid, 256, 0, st, rgb, depth, x0, n, h, w);
 }
 
 cudaError_t launch_prep_weights(const PrepArgs &a, cudaStream_t st)
 {
     int n = 0;
     for (int l = 0; l < kLayers; ++l) n = max(n, 9 * a.ci_p[l] * a.co_p[l] / 8);
-    k_prep_weights<<<dim3((n + 127) / 128, kLayers), 128, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(k_prep_weights, dim3((n + 127) / 128, kLayers), 128, 0, st, a);
 }
 
 cudaError_t launch_zero_grads(const ZeroArgs &a, cudaStream_t st)
 {
     int n = 0;
     for (int l = 0; l < kLayers; ++l) n = max(n, max(a.n_w[l], a.n_b[l]));
-    k_zero_grads<<<dim3((n + 255) / 256, kLayers), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(k_zero_grads, dim3((n + 255) / 256, kLayers), 256, 0, st, a);
 }
 
 cudaError_t launch_loss(const float2 *y4, const float *td, const float *tl, float lw, uint4 *dy4, float *loss,
@@ -806,8 +808,7 @@ cudaError_t launch_loss(const float2 *y4, const float *td, const float *tl, floa
 {
     if (!total) return cudaSuccess;
     const int grid = (int)((total + 255) / 256 < 2048 ? (total + 255) / 256 : 2048);
-    k_loss<<<grid, 256, 0, st>>>(y4, td, tl, lw, dy4, loss, total, w);
-    return cudaGetLastError();
+    return launch_after(k_loss, grid, 256, 0, st, y4, td, tl, lw, dy4, loss, total, w);
 }
 
 }  // namespace net

@@ -34,6 +34,7 @@
 // block mask in the low 8: the order is the same (a Gaussian is listed once per tile), and
 // the last write separates the plain entry from the mask, kept as one byte per entry.
 #include "sgad_device.cuh"
+#include "sgad_launch.cuh"
 
 namespace sgad {
 
@@ -298,6 +299,7 @@ __global__ void __launch_bounds__(kSortThreads, kPer <= 12 ? 2 : 1)
     k_sort_tiles(const uint32_t *__restrict__ off, uint64_t *__restrict__ entries, uint64_t *__restrict__ alt, int cap,
                  const WsHeader *hdr, const uint32_t *__restrict__ list, uint8_t *__restrict__ masks)
 {
+    dependency_wait(off, list);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem &s = *reinterpret_cast<SortSmem *>(smem_raw);
     uint64_t *ks = reinterpret_cast<uint64_t *>(smem_raw + ((sizeof(SortSmem) + 15) & ~size_t(15)));
@@ -369,6 +371,7 @@ __global__ void __launch_bounds__(kBucketThreads, 3)
     k_sort_tiles_bucket(const uint32_t *__restrict__ off, uint64_t *__restrict__ entries, int cap, WsHeader *hdr,
                         uint32_t *__restrict__ list, uint8_t *__restrict__ masks)
 {
+    dependency_wait(off);
     __shared__ __align__(16) uint32_t start[1 << kBucketBinsLog2];    // bucket counts, then bucket starts
     __shared__ uint32_t red[2][kBucketThreads / 32];
     __shared__ int heavy;
@@ -536,13 +539,14 @@ static cudaError_t launch_sort(const uint32_t *off, uint64_t *entries, uint64_t 
         if (dev >= 0 && dev < 64) bucket_configured[dev] = 1;
     }
     if (n_tiles <= 0) return cudaSuccess;
-    k_sort_tiles_bucket<PACK><<<n_tiles, kBucketThreads, bucket_smem, st>>>(off, entries, cap, hdr, list, masks);
+    launch_after(k_sort_tiles_bucket<PACK>, n_tiles, kBucketThreads, bucket_smem, st, off, entries, cap, hdr, list,
+                 masks);
     // the listed tiles: a fixed grid (two blocks per SM) so the launch can be captured
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int grid = n_tiles < 2 * sms ? n_tiles : 2 * sms;
-    k_sort_tiles<kPer, PACK><<<grid, kSortThreads, smem, st>>>(off, entries, alt, cap, hdr, list, masks);
+    launch_after(k_sort_tiles<kPer, PACK>, grid, kSortThreads, smem, st, off, entries, alt, cap, hdr, list, masks);
     return cudaSuccess;
 }
 

@@ -28,6 +28,7 @@
 #include <cstring>
 
 #include "sgad_device.cuh"
+#include "sgad_launch.cuh"
 
 namespace sgad {
 sgad_status report_error(sgad_status code, const char *msg);
@@ -168,6 +169,7 @@ __device__ __forceinline__ void load_strip(const float *row, int c0, float (&v)[
 
 __global__ void __launch_bounds__(kThreads, 4) k_ssim_maps(const __grid_constant__ SsimBatch b)
 {
+    dependency_wait();
     __shared__ __align__(16) float sxy[2][kExt][kPitch];       // x, y
     __shared__ __align__(16) float h[5][kExt][kTile];          // m1, my, m2, myy, m12 (horizontal)
     __shared__ float red[kThreads / 32];
@@ -264,6 +266,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_ssim_maps(const __grid_constant
 
 __global__ void __launch_bounds__(kThreads, 4) k_ssim_grad(const __grid_constant__ SsimBatch b)
 {
+    dependency_wait();
     __shared__ __align__(16) float sd[3][kExt][kPitch];
     __shared__ __align__(16) float h[3][kExt][kTile];
     const TileAt t = tile_at(b);
@@ -413,8 +416,8 @@ extern "C" sgad_status sgad_ssim_loss_grad(int32_t n_views, const sgad_camera *v
             return fail(SGAD_ERR_CUDA, "sgad_ssim_loss_grad: cannot set the shared-memory carveout");
         if (dev >= 0 && dev < 64) configured[dev] = 1;
     }
-    k_ssim_maps<<<blocks, kThreads, 0, st>>>(b);
-    k_ssim_grad<<<blocks, kThreads, 0, st>>>(b);
+    launch_after(k_ssim_maps, blocks, kThreads, 0, st, b);
+    launch_after(k_ssim_grad, blocks, kThreads, 0, st, b);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SGAD_OK : fail(SGAD_ERR_CUDA, "sgad_ssim_loss_grad: launch failed");
 }

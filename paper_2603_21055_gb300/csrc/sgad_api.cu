@@ -16,9 +16,10 @@ cudaError_t launch_sort_tiles(const uint32_t *, uint64_t *, uint64_t *, int, int
                               cudaStream_t);
 cudaError_t launch_composite(bool, int, int, int, const Scene &, const World *, const uint32_t *, const uint64_t *,
                              float *, uint32_t *, float4 *, WsHeader *, const uint32_t *, uint32_t *, uint32_t *,
-                             const uint8_t *, cudaStream_t);
+                             const uint8_t *, bool, cudaStream_t);
 bool valid_batch(int, bool);
 void launch_finalize(const Scene &, const float4 *, cudaStream_t);
+cudaError_t launch_clear(const ClearList &, cudaStream_t);
 void launch_l1_batch(int, const float *const *, const float *const *, const float *const *, const float *const *,
                      const float *const *, float *const *, float *const *, uint32_t *, const uint32_t *, float, float,
                      float, float *, cudaStream_t);
@@ -233,9 +234,11 @@ bool uses_masks(const sgad_options &o, const Scene &sc)
 sgad_status run_binning_count(const sgad_options &o, const Scene &sc, const Ws &ws, int64_t key_cap,
                               bool clear_sticky, cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(ws.hdr(), 0, clear_sticky ? sizeof(WsHeader) : kHeaderPerCall, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws.tile_cnt(), 0, ((size_t)sc.n_tiles + 1) * 4, st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    ClearList c = {};
+    c.add(ws.hdr(), clear_sticky ? sizeof(WsHeader) : kHeaderPerCall);
+    c.add(ws.tile_cnt(), ((size_t)sc.n_tiles + 1) * 4);
+    const cudaError_t e = launch_clear(c, st);
+    if (e != cudaSuccess) return cuda_fail(e, "clear");
     launch_project_count(sc, ws.world(), ws.tile_cnt(), ws.rects(), uses_masks(o, sc), st);
     launch_scan_tiles(ws.tile_cnt(), ws.tile_off(), sc.n_tiles, (uint64_t)key_cap, ws.hdr(),
                       uses_order(o) ? ws.tile_order() : nullptr, st);
@@ -259,32 +262,35 @@ sgad_status run_forward_prep(sgad_ctx *ctx, const Scene &sc, const Ws &ws, int64
     return last_launch("binning / emission / sort");
 }
 
-// Zeroes the gradient accumulators of the learnable keyframes (the others' are not used),
-// neighbours in one call.
-cudaError_t clear_accumulators(const Scene &sc, const Ws &ws, cudaStream_t st)
+// Zeroes what a backward accumulates into: the accumulators of the learnable keyframes (the
+// others' are not used), neighbours as one range, the pose gradients, and the work queue.
+cudaError_t clear_gradients(const Scene &sc, const Ws &ws, bool poses, cudaStream_t st)
 {
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; i < sc.n_kf && e == cudaSuccess;) {
+    ClearList c = {};
+    for (int i = 0; i < sc.n_kf;) {
         int j = i;
         while (j < sc.n_kf && (sc.kf[j].learnable != 0) == (sc.kf[i].learnable != 0)) ++j;
         const uint32_t from = sc.kf[i].gbase, to = j < sc.n_kf ? sc.kf[j].gbase : sc.n_gauss;
-        if (sc.kf[i].learnable)
-            e = cudaMemsetAsync(ws.gacc() + 2 * (size_t)from, 0, (size_t)(to - from) * 32, st);
+        if (sc.kf[i].learnable) c.add(ws.gacc() + 2 * (size_t)from, (size_t)(to - from) * 32);
         i = j;
     }
-    return e;
+    for (int i = 0; i < sc.n_views && poses; ++i)
+        if (sc.view[i].d_pose) c.add(sc.view[i].d_pose, 12 * sizeof(float));
+    c.add(&ws.hdr()->queue_bwd, sizeof(uint32_t));
+    return launch_clear(c, st);
 }
 
 // One compositing pass. batch 0 in the backward selects the pair-parallel kernel, a negative
 // batch the warp-local kernel of either pass; the block-staged forward records contribution
 // words when the context's backward is pair-parallel.
 sgad_status run_composite(const sgad_ctx *ctx, bool fwd, int batch, int schedule, const Scene &sc, const Ws &ws,
-                          cudaStream_t st)
+                          bool queue_clear, cudaStream_t st)
 {
     uint32_t *contrib = (!fwd || batch < 0 || ctx->opt.bwd_algorithm == SGAD_BWD_PAIRS) ? ws.contrib() : nullptr;
     const cudaError_t e = launch_composite(fwd, batch, schedule, ctx->opt.max_blocks, sc, ws.world(), ws.tile_off(), ws.keys(), ws.pix_t(),
                                            ws.pix_n(), fwd ? nullptr : ws.gacc(), ws.hdr(), ws.tile_order(), contrib,
-                                           ws.wmask(), batch < 0 && uses_masks(ctx->opt, sc) ? ws.bmask() : nullptr, st);
+                                           ws.wmask(), batch < 0 && uses_masks(ctx->opt, sc) ? ws.bmask() : nullptr,
+                                           queue_clear, st);
     return e == cudaSuccess ? SGAD_OK : cuda_fail(e, fwd ? "forward compositing launch" : "backward compositing launch");
 }
 
@@ -561,7 +567,7 @@ sgad_status sgad_forward(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf, 
     if (s) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     s = run_forward_prep(ctx, sc, ws, key_capacity, st);
-    if (!s) s = run_composite(ctx, true, fwd_batch_of(ctx->opt), ctx->opt.fwd_schedule, sc, ws, st);
+    if (!s) s = run_composite(ctx, true, fwd_batch_of(ctx->opt), ctx->opt.fwd_schedule, sc, ws, true, st);
     if (s) return s;
     mark(ctx, 4, st);
     ctx->fwd_recorded = ctx->profile;
@@ -582,11 +588,9 @@ sgad_status sgad_backward(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
     if (s) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     mark(ctx, 5, st);
-    cudaError_t e = clear_accumulators(sc, ws, st);
-    for (int i = 0; i < n_views && e == cudaSuccess; ++i)
-        if (sc.view[i].d_pose) e = cudaMemsetAsync(sc.view[i].d_pose, 0, 12 * sizeof(float), st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-    s = run_composite(ctx, false, bwd_batch_of(ctx->opt), ctx->opt.bwd_schedule, sc, ws, st);
+    const cudaError_t e = clear_gradients(sc, ws, true, st);
+    if (e != cudaSuccess) return cuda_fail(e, "clear");
+    s = run_composite(ctx, false, bwd_batch_of(ctx->opt), ctx->opt.bwd_schedule, sc, ws, true, st);
     if (s) return s;
     mark(ctx, 6, st);
     launch_finalize(sc, ws.gacc(), st);
@@ -668,8 +672,10 @@ sgad_status sgad_l1_loss_grad(int32_t n_views, const sgad_camera *views, const s
         hw[i] = (uint32_t)views[i].width * (uint32_t)views[i].height;
     }
     if (use_depth) {
-        cudaError_t e = cudaMemsetAsync(valid_count, 0, sizeof(uint32_t) * (size_t)n_views, st);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+        ClearList c = {};
+        c.add(valid_count, sizeof(uint32_t) * (size_t)n_views);
+        const cudaError_t e = launch_clear(c, st);
+        if (e != cudaSuccess) return cuda_fail(e, "clear");
     }
     launch_l1_batch(n_views, rgb, dep, mask ? alp : nullptr, target_rgb, use_depth ? target_depth : nullptr, d_rgb,
                     d_depth, use_depth ? valid_count : nullptr, hw, rgb_weight, depth_weight, min_alpha, loss_accum,
@@ -788,7 +794,7 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
         for (int sched : kScheds)
             for (int batch : kBatches) {
                 float ms = 0.f;
-                s = timer.median(reps, st, [&] { return run_composite(&trial, true, batch, sched, sc, ws, st); }, &ms);
+                s = timer.median(reps, st, [&] { return run_composite(&trial, true, batch, sched, sc, ws, false, st); }, &ms);
                 if (s) return s;
                 log.add(shape[0], shape[1], SGAD_TUNE_FWD, batch, sched, ms);
                 if (best_f < 0.f || ms < best_f) {
@@ -814,7 +820,7 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
                     if (batch == 0 && sched != fs) continue;
                     float ms = 0.f;
                     s = timer.median(reps, st, [&] {
-                        return run_composite(&trial, true, batch < 0 ? -1 : fb, sched, sc, ws, st);
+                        return run_composite(&trial, true, batch < 0 ? -1 : fb, sched, sc, ws, false, st);
                     }, &ms);
                     if (s) return s;
                     if (fwd_ms < 0.f || ms < fwd_ms) {
@@ -826,9 +832,9 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
             for (int sched : kScheds) {
                 float ms = 0.f;
                 auto run = [&] {
-                    const cudaError_t e = clear_accumulators(sc, ws, st);
-                    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-                    return run_composite(&trial, false, batch, sched, sc, ws, st);
+                    const cudaError_t e = clear_gradients(sc, ws, false, st);
+                    if (e != cudaSuccess) return cuda_fail(e, "clear");
+                    return run_composite(&trial, false, batch, sched, sc, ws, true, st);
                 };
                 s = timer.median(reps, st, run, &ms);
                 if (s) return s;

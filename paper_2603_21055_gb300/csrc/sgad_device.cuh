@@ -85,6 +85,19 @@ struct WsHeader {
 static_assert(sizeof(WsHeader) == 256, "header is one 256-byte block");
 constexpr size_t kHeaderPerCall = 128;   // bytes cleared by every forward
 
+// Ranges of 32-bit words that one launch zeroes: the accumulators of every keyframe, a pose
+// gradient per view, and the header, tile counts and queues of the pass.
+struct ClearList {
+    uint32_t *at[SGAD_MAX_KEYFRAMES + SGAD_MAX_VIEWS + 4];
+    size_t words[SGAD_MAX_KEYFRAMES + SGAD_MAX_VIEWS + 4];
+    int32_t n;
+    __host__ void add(void *p, size_t bytes)
+    {
+        at[n] = static_cast<uint32_t *>(p);
+        words[n++] = bytes / 4;
+    }
+};
+
 // Per-Gaussian record computed once per forward (view independent):
 //   w0 = (mu_x, mu_y, mu_z, s), w1 = (opacity, r, g, b)
 struct __align__(16) World {

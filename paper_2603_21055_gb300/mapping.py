@@ -131,7 +131,8 @@ class Mapper:
         """Library kernels per iteration: projection+count, scan, emission, sort, forward
         compositing (one launch per view with the per-view schedule); valid-depth count and
         L1 gradient; the two SSIM passes when that term is on; backward compositing,
-        finalisation; multi-tensor Adam and its step counter."""
+        finalisation; multi-tensor Adam and its step counter (launches that only zero the
+        accumulators of a pass are not counted)."""
         o = self.sp.options
         per = lambda sched: len(self.views) if sched == B.SGAD_SCHEDULE_PER_VIEW else 1
         n = 4 + per(o.fwd_schedule) + (2 if self.scene.depth_weight != 0 else 1) + per(o.bwd_schedule) + 1
