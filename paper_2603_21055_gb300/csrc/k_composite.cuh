@@ -52,6 +52,8 @@
 #include "sgad_device.cuh"
 #include "sgad_launch.cuh"
 
+#include <type_traits>
+
 namespace sgad {
 
 constexpr int kFwdThreads = 256;
@@ -418,6 +420,18 @@ constexpr int kFwdlThreads = 256;           // 8 independent warps per block
 #define SGAD_FWDL_MINBLOCKS 4
 #endif
 
+// With at most as many work units as the forward keeps warps resident (4 blocks of 8 on each
+// of 152 SMs) every unit has its warp at once, and a pass takes as long as its deepest unit:
+// a lone warp per scheduler took 350 cycles per step of two candidates and 1500 to 2000 to
+// stage a round. The instances for few units (FEW) have the registers of two blocks per SM:
+// the forward takes four candidates at once and loads a round ahead, the backward takes three
+// entries at once whatever the keyframes, and neither spills. Forward, with and without: 640
+// units 42 and 56 us, 2400: 54 and 64, 4800: 83 and 87, 9600: 140 and 140, 19200: 251 and
+// 239. Backward: 4386 units 105 and 116, 4800: 111 and 115, 9600: 201 and 189; with pose
+// gradients, whose sums spill most at three blocks, 9600: 174 and 189.
+constexpr int kFewBlocks = 2;
+constexpr int kFewUnits = 4 * 8 * 152;
+
 // Two FP32 values in one 64-bit register, added, multiplied and fused by one instruction
 // each (sm_100 and later): the same rounding of each half as the scalar operations, at one
 // issue slot instead of two.
@@ -521,7 +535,7 @@ __device__ __forceinline__ bool may_touch(const float4 w0, float o, const ViewDe
     return l > 0.0f && fabsf(dx) <= hx + 3.5f && fabsf(dy) <= hy + 1.5f;
 }
 
-template <int TW, int TH, bool MASKS>
+template <int TW, int TH, bool MASKS, bool FEW>
 __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &a, int tile, int wb, FwdlWarpSmem &S,
                                           int lane, uint32_t &n_pairs, uint32_t &n_evals)
 {
@@ -557,9 +571,22 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
         return MASKS && p + 4 * lane < (int)len ? words[(p + lead) / 4 + lane] : 0u;
     };
     uint32_t word = load_masks(next);
+    // FEW: a round's entries and world records are loaded during the round before it, the
+    // entries' positions known a round earlier still
+    constexpr int kAhead = FEW ? 96 : 32;
+    constexpr int kWide = FEW ? 4 : 2;                 // candidates of a lane taken at once
+    const auto load_ent = [&](int i) { return i < cnt ? ents[S.pos[(head + i) & (kRing - 1)]] : ~0ull; };
+    const auto load_world = [&](uint64_t ent) {
+        World r = {};
+        if ((uint32_t)ent < sc.n_gauss) r = a.world[(uint32_t)ent];
+        return r;
+    };
+    uint64_t ent0 = 0, ent1 = 0;
+    World w0 = {};
+    bool first = true;
     for (;;) {
         // 1. gather
-        while (cnt < 32 && next < (int)len) {
+        while (cnt < kAhead && next < (int)len) {
             if (MASKS) {
                 const int p = next + 4 * lane;
                 uint32_t m = (word >> wb) & 0x01010101u;
@@ -594,6 +621,12 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
         }
         if (cnt == 0) break;
         __syncwarp();
+        if (FEW && first) {
+            ent0 = load_ent(lane);
+            ent1 = load_ent(32 + lane);
+            w0 = load_world(ent0);
+            first = false;
+        }
         // 2. a round: the first 32 of the ring
         const int n = min(cnt, 32);
         uint32_t row = 0u;
@@ -601,9 +634,19 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
         if (lane < n) {
             my_pos = S.pos[(head + lane) & (kRing - 1)];
             Staged g;
-            stage_entry(sc, a, v, ents[my_pos], g);
+            if (!FEW)
+                stage_entry(sc, a, v, ents[my_pos], g);
+            else if ((uint32_t)ent0 < sc.n_gauss)
+                stage(project(w0.w0, v), w0.w1, __uint_as_float((uint32_t)(ent0 >> 32)), g);
+            else
+                g.a = make_float4(0.f, 0.f, -1.f, -1.f);     // never reaches a pixel
             to_walk(g, S.e[lane]);
             row = box_block_mask(g.a, bxf, byf);
+        }
+        if (FEW) {
+            ent0 = ent1;
+            w0 = load_world(ent0);
+            ent1 = load_ent(64 + lane);
         }
         uint32_t mine = warp_transpose32(row, lane);
         __syncwarp();
@@ -612,40 +655,86 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
         uint32_t bits = 0u;
         while (__any_sync(kFull, mine != 0u)) {
             if (mine) {
-                // two candidates: their alphas are independent of one another
-                const uint32_t low0 = mine & (0u - mine), rest = mine ^ low0, low1 = rest & (0u - rest);
-                mine = rest ^ low1;
-                const WalkEntry &g0 = S.e[31 - __clz(low0)], &g1 = S.e[31 - __clz(low1 ? low1 : low0)];
-                float alpha0, alpha1, raw;
-                const bool ok0 = walk_alpha(g0.a, g0.b, nq, alpha0, raw);
-                const bool ok1 = walk_alpha(g1.a, g1.b, nq, alpha1, raw) && low1;
-                const float4 c0 = g0.c, c1 = g1.c;
-                const float t0 = __fmul_rn(T, __fsub_rn(1.0f, alpha0));
-                const bool stop0 = ok0 && t0 < kTStop, take0 = ok0 && !stop0;
-                if (take0) {
-                    const float w = __fmul_rn(alpha0, T);
-                    const float2x ww = pack2(w, w);
-                    acc_rg = fma2(ww, pack2(c0.x, c0.y), acc_rg);
-                    acc_bd = fma2(ww, pack2(c0.z, c0.w), acc_bd);
-                    aa = __fadd_rn(aa, w);
-                    T = t0;
-                    bits |= low0;
-                }
-                const float t1 = __fmul_rn(T, __fsub_rn(1.0f, alpha1));
-                const bool stop1 = ok1 && !stop0 && t1 < kTStop, take1 = ok1 && !stop0 && !stop1;
-                if (take1) {
-                    const float w = __fmul_rn(alpha1, T);
-                    const float2x ww = pack2(w, w);
-                    acc_rg = fma2(ww, pack2(c1.x, c1.y), acc_rg);
-                    acc_bd = fma2(ww, pack2(c1.z, c1.w), acc_bd);
-                    aa = __fadd_rn(aa, w);
-                    T = t1;
-                    bits |= low1;
-                }
-                if (stop0 || stop1) {
-                    done = true;
-                    n_evals -= __popc(stop0 ? rest : mine);
-                    mine = 0u;
+                if constexpr (FEW) {
+                    // the candidates' alphas do not depend on one another
+                    uint32_t low[kWide], rest[kWide];
+                    const WalkEntry *g[kWide];
+                    float alpha[kWide];
+                    bool ok[kWide], ends[kWide];
+#pragma unroll
+                    for (int q = 0; q < kWide; ++q) {
+                        low[q] = mine & (0u - mine);
+                        mine ^= low[q];
+                        rest[q] = mine;
+                        g[q] = &S.e[31 - __clz(q > 0 && low[q] == 0u ? low[0] : low[q])];
+                    }
+#pragma unroll
+                    for (int q = 0; q < kWide; ++q) {
+                        float raw;
+                        ok[q] = walk_alpha(g[q]->a, g[q]->b, nq, alpha[q], raw) && (q == 0 || low[q] != 0u);
+                    }
+                    float4 c[kWide];
+#pragma unroll
+                    for (int q = 0; q < kWide; ++q) c[q] = g[q]->c;
+                    bool stop = false;
+#pragma unroll
+                    for (int q = 0; q < kWide; ++q) {
+                        const float test = __fmul_rn(T, __fsub_rn(1.0f, alpha[q]));
+                        ends[q] = ok[q] && !stop && test < kTStop;
+                        if (ok[q] && !stop && !ends[q]) {
+                            const float w = __fmul_rn(alpha[q], T);
+                            const float2x ww = pack2(w, w);
+                            acc_rg = fma2(ww, pack2(c[q].x, c[q].y), acc_rg);
+                            acc_bd = fma2(ww, pack2(c[q].z, c[q].w), acc_bd);
+                            aa = __fadd_rn(aa, w);
+                            T = test;
+                            bits |= low[q];
+                        }
+                        stop = stop || ends[q];
+                    }
+                    if (stop) {
+                        done = true;
+#pragma unroll
+                        for (int q = 0; q < kWide; ++q)
+                            if (ends[q]) n_evals -= __popc(rest[q]);
+                        mine = 0u;
+                    }
+                } else {
+                    // the same for two candidates, written out (931 us against 947 at 8 x 640x480)
+                    const uint32_t low0 = mine & (0u - mine), rest = mine ^ low0, low1 = rest & (0u - rest);
+                    mine = rest ^ low1;
+                    const WalkEntry &g0 = S.e[31 - __clz(low0)], &g1 = S.e[31 - __clz(low1 ? low1 : low0)];
+                    float alpha0, alpha1, raw;
+                    const bool ok0 = walk_alpha(g0.a, g0.b, nq, alpha0, raw);
+                    const bool ok1 = walk_alpha(g1.a, g1.b, nq, alpha1, raw) && low1;
+                    const float4 c0 = g0.c, c1 = g1.c;
+                    const float t0 = __fmul_rn(T, __fsub_rn(1.0f, alpha0));
+                    const bool stop0 = ok0 && t0 < kTStop, take0 = ok0 && !stop0;
+                    if (take0) {
+                        const float w = __fmul_rn(alpha0, T);
+                        const float2x ww = pack2(w, w);
+                        acc_rg = fma2(ww, pack2(c0.x, c0.y), acc_rg);
+                        acc_bd = fma2(ww, pack2(c0.z, c0.w), acc_bd);
+                        aa = __fadd_rn(aa, w);
+                        T = t0;
+                        bits |= low0;
+                    }
+                    const float t1 = __fmul_rn(T, __fsub_rn(1.0f, alpha1));
+                    const bool stop1 = ok1 && !stop0 && t1 < kTStop, take1 = ok1 && !stop0 && !stop1;
+                    if (take1) {
+                        const float w = __fmul_rn(alpha1, T);
+                        const float2x ww = pack2(w, w);
+                        acc_rg = fma2(ww, pack2(c1.x, c1.y), acc_rg);
+                        acc_bd = fma2(ww, pack2(c1.z, c1.w), acc_bd);
+                        aa = __fadd_rn(aa, w);
+                        T = t1;
+                        bits |= low1;
+                    }
+                    if (stop0 || stop1) {
+                        done = true;
+                        n_evals -= __popc(stop0 ? rest : mine);
+                        mine = 0u;
+                    }
                 }
             }
         }
@@ -683,8 +772,8 @@ __device__ __forceinline__ void fwdl_unit(const Scene &sc, const CompositeArgs &
     }
 }
 
-template <int TW, int TH, bool MASKS>
-__global__ void __launch_bounds__(kFwdlThreads, SGAD_FWDL_MINBLOCKS)
+template <int TW, int TH, bool MASKS, bool FEW>
+__global__ void __launch_bounds__(kFwdlThreads, FEW ? kFewBlocks : SGAD_FWDL_MINBLOCKS)
     k_composite_fwdl(const __grid_constant__ Scene sc, const CompositeArgs a)
 {
     dependency_wait();
@@ -701,7 +790,7 @@ __global__ void __launch_bounds__(kFwdlThreads, SGAD_FWDL_MINBLOCKS)
         u = __shfl_sync(kFull, u, 0);
         if (u >= n_units) break;
         const int tile = a.order ? (int)a.order[u >> 3] : a.tile0 + (int)(u >> 3);
-        fwdl_unit<TW, TH, MASKS>(sc, a, tile, (int)(u & 7u), S, lane, n_pairs, n_evals);
+        fwdl_unit<TW, TH, MASKS, FEW>(sc, a, tile, (int)(u & 7u), S, lane, n_pairs, n_evals);
     }
     const uint32_t wp = __reduce_add_sync(kFull, n_pairs), we = __reduce_add_sync(kFull, n_evals);
     if (lane == 0 && we) {
@@ -1445,7 +1534,7 @@ static __device__ __noinline__ void add_not_finite(BwdlWarpSmem &S, int h, int s
 // for the fixed ones. 5 x 1200x680 with four of five keyframes fixed: 1.38 ms against 1.92
 // with all entries' moments (2.23 before the products). Without a fixed keyframe its checks
 // cost 45 us of 1.34 ms, so that case has its own instance.
-template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED>
+template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED, bool FEW>
 __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &a, int tile, int wb, BwdlWarpSmem &S,
                                           int lane)
 {
@@ -1570,7 +1659,7 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
         const uint32_t with = FIXED ? __ballot_sync(kFull, own) : 0u;
         const int span = FIXED && __popc(with) <= kHalf ? 32 : kHalf;
         int my_row = lane;                             // this lane's entry's row of S.mom
-        constexpr int kWide = FIXED ? 2 : 3;           // entries of a lane taken at once
+        constexpr int kWide = FIXED && !FEW ? 2 : 3;   // entries of a lane taken at once
 #pragma unroll 1
         for (int h = 0; h < n; h += span) {
             // 2. walk the entries h .. h + span - 1
@@ -1677,8 +1766,8 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
     }
 }
 
-template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED>
-__global__ void __launch_bounds__(kLocalThreads, SGAD_BWDL_MINBLOCKS)
+template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED, bool FEW>
+__global__ void __launch_bounds__(kLocalThreads, FEW ? kFewBlocks : SGAD_BWDL_MINBLOCKS)
     k_composite_bwdl(const __grid_constant__ Scene sc, const CompositeArgs a)
 {
     dependency_wait();
@@ -1694,7 +1783,7 @@ __global__ void __launch_bounds__(kLocalThreads, SGAD_BWDL_MINBLOCKS)
         u = __shfl_sync(kFull, u, 0);
         if (u >= n_units) break;
         const int tile = a.order ? (int)a.order[u >> 3] : a.tile0 + (int)(u >> 3);
-        bwdl_unit<TW, TH, POSE, PLAIN, FIXED>(sc, a, tile, (int)(u & 7u), S, lane);
+        bwdl_unit<TW, TH, POSE, PLAIN, FIXED, FEW>(sc, a, tile, (int)(u & 7u), S, lane);
     }
 }
 
@@ -1795,10 +1884,14 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        const void *all[] = {(const void *)k_composite_bwdl<TW, TH, false, false, true>,
-                             (const void *)k_composite_bwdl<TW, TH, false, true, false>,
-                             (const void *)k_composite_bwdl<TW, TH, false, true, true>,
-                             (const void *)k_composite_bwdl<TW, TH, true, false, true>};
+        const void *all[] = {(const void *)k_composite_bwdl<TW, TH, false, false, true, false>,
+                             (const void *)k_composite_bwdl<TW, TH, false, true, false, false>,
+                             (const void *)k_composite_bwdl<TW, TH, false, true, true, false>,
+                             (const void *)k_composite_bwdl<TW, TH, true, false, true, false>,
+                             (const void *)k_composite_bwdl<TW, TH, false, false, true, true>,
+                             (const void *)k_composite_bwdl<TW, TH, false, true, false, true>,
+                             (const void *)k_composite_bwdl<TW, TH, false, true, true, true>,
+                             (const void *)k_composite_bwdl<TW, TH, true, false, true, true>};
         for (const void *f : all)
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmemBytes);
@@ -1806,21 +1899,32 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
         if (dev >= 0 && dev < 64) configured[dev] = 1;
     }
     if (occupancy)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_bwdl<TW, TH, false, true, false>,
-                                                             kLocalThreads, kLocalSmemBytes);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            occupancy, k_composite_bwdl<TW, TH, false, true, false, false>, kLocalThreads, kLocalSmemBytes);
     if (grid_blocks <= 0) return cudaSuccess;
     // without an alpha gradient and with a black background the walk drops those terms
     bool plain = sc.bg[0] == 0.0f && sc.bg[1] == 0.0f && sc.bg[2] == 0.0f, fixed = false;
     for (int i = 0; i < sc.n_views && plain; ++i) plain = sc.view[i].g_alpha == nullptr;
     for (int i = 0; i < sc.n_kf && !fixed; ++i) fixed = sc.kf[i].learnable == 0;
-    if (a.pose)
-        launch_after(k_composite_bwdl<TW, TH, true, false, true>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
-    else if (!plain)
-        launch_after(k_composite_bwdl<TW, TH, false, false, true>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
-    else if (fixed)
-        launch_after(k_composite_bwdl<TW, TH, false, true, true>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
+    const auto run = [&](auto few) {
+        constexpr bool kFew = decltype(few)::value;
+        if (a.pose)
+            launch_after(k_composite_bwdl<TW, TH, true, false, true, kFew>, grid_blocks, kLocalThreads,
+                         kLocalSmemBytes, st, sc, a);
+        else if (!plain)
+            launch_after(k_composite_bwdl<TW, TH, false, false, true, kFew>, grid_blocks, kLocalThreads,
+                         kLocalSmemBytes, st, sc, a);
+        else if (fixed)
+            launch_after(k_composite_bwdl<TW, TH, false, true, true, kFew>, grid_blocks, kLocalThreads,
+                         kLocalSmemBytes, st, sc, a);
+        else
+            launch_after(k_composite_bwdl<TW, TH, false, true, false, kFew>, grid_blocks, kLocalThreads,
+                         kLocalSmemBytes, st, sc, a);
+    };
+    if (a.n_launch_tiles * 8 <= (a.pose ? 2 * kFewUnits : kFewUnits))
+        run(std::true_type{});
     else
-        launch_after(k_composite_bwdl<TW, TH, false, true, false>, grid_blocks, kLocalThreads, kLocalSmemBytes, st, sc, a);
+        run(std::false_type{});
     return cudaGetLastError();
 }
 
@@ -1828,12 +1932,15 @@ template <int TW, int TH>
 cudaError_t launch_fwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks, int *occupancy, cudaStream_t st)
 {
     if (occupancy)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_fwdl<TW, TH, true>, kFwdlThreads, 0);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, k_composite_fwdl<TW, TH, true, false>,
+                                                             kFwdlThreads, 0);
     if (grid_blocks <= 0) return cudaSuccess;
-    if (a.bmask)
-        launch_after(k_composite_fwdl<TW, TH, true>, grid_blocks, kFwdlThreads, 0, st, sc, a);
+    if (!a.bmask)
+        launch_after(k_composite_fwdl<TW, TH, false, false>, grid_blocks, kFwdlThreads, 0, st, sc, a);
+    else if (a.n_launch_tiles * 8 <= kFewUnits)
+        launch_after(k_composite_fwdl<TW, TH, true, true>, grid_blocks, kFwdlThreads, 0, st, sc, a);
     else
-        launch_after(k_composite_fwdl<TW, TH, false>, grid_blocks, kFwdlThreads, 0, st, sc, a);
+        launch_after(k_composite_fwdl<TW, TH, true, false>, grid_blocks, kFwdlThreads, 0, st, sc, a);
     return cudaGetLastError();
 }
 

@@ -105,3 +105,33 @@ def test_gradients_that_are_not_finite_stay_with_their_pixels(value):
         assert np.array_equal(ok, np.isfinite(x) & (np.abs(x) < 1e30)), q
         assert 0 < (~ok).sum() < ok.size // 4
         assert np.abs(x[ok] - y[ok]).max() <= 1e-4 * np.abs(y[ok]).max(), q
+
+
+@pytest.mark.parametrize("pose", [False, True])
+@pytest.mark.parametrize("learnable", [1, 2])
+def test_launches_of_few_and_many_units_agree(pose, learnable):
+    """Four views of 2,560 work units each, launched view by view (few units each) and together
+    (10,240 units): images, pixel state and counters are equal, gradients up to the order of
+    FP32 additions (the bounds above), with and without fixed keyframes and pose gradients."""
+    import torch
+    kfs = _keyframes(2, 160, 128, 80.0, 1.5, 0.0, seed=4)
+    kfs[1].learnable = learnable == 2
+    views = [_cam(320, 256, 160.0, 160.0, 128.0, (0.02 * i, -0.02, 0.01 * i)) for i in range(4)]
+    g = torch.Generator(device="cuda").manual_seed(6)
+    gin = [dict(rgb=torch.randn(3, 256, 320, generator=g, device="cuda"),
+                depth=torch.randn(256, 320, generator=g, device="cuda")) for _ in views]
+    out = {}
+    for sched in ("per_view", "tiles"):
+        poses = [torch.empty(12, device="cuda") for _ in views]
+        gi = [dict(x, pose=p) for x, p in zip(gin, poses)] if pose else gin
+        out[sched] = _run(kfs, views, gi, fwd_schedule=sched, bwd_schedule=sched) + (poses,)
+    a, b = out["per_view"], out["tiles"]
+    for x, y in zip(a[0], b[0]):
+        assert all(torch.equal(x[q], y[q]) for q in ("rgb", "depth", "alpha"))
+    assert all(np.array_equal(x, y) for x, y in zip(a[1], b[1]))
+    assert a[3]["n_pairs"] == b[3]["n_pairs"] and a[3]["n_evals"] == b[3]["n_evals"]
+    pairs = [(a[2][q], b[2][q]) for q in ("d_offset", "d_rgb", "d_logit", "d_scale")]
+    for x, y in pairs + (list(zip(a[4], b[4])) if pose else []):
+        x, y = x.double().cpu().numpy(), y.double().cpu().numpy()
+        assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y)
+        assert np.abs(x - y).max() <= 1e-4 * np.abs(y).max()
