@@ -7,7 +7,7 @@
 // chunk][pixel], so the units of one chunk of one image row are contiguous (a TMA box of a
 // chunk over a row reads whole sectors).
 //
-// Forward and input gradient (k_conv3x3_tma): a tile is 128 consecutive output pixels of
+// Forward and input gradient (conv_block): a tile is 128 consecutive output pixels of
 // one image row (the MMA's M), all output channels and K = 9 taps x C_in. The input rows
 // arrive by TMA, 130 pixels of a (row, chunk), which in shared memory is the K-major
 // canonical layout; the tap column dx is a descriptor start offset of dx units, so no im2col
@@ -17,7 +17,7 @@
 // overlap loads, MMAs (a ring of TMEM accumulators) and the epilogue (bias + ReLU + bf16; or
 // the ReLU-masked input gradient; or the two f32 outputs).
 //
-// Weight gradient (k_conv3x3_wgrad_tma): dW[t][i][o] = sum_p x[p + d_t][i] dy[p][o] is a
+// Weight gradient (wgrad_block): dW[t][i][o] = sum_p x[p + d_t][i] dy[p][o] is a
 // GEMM with the pixels as K; the same TMA boxes, read with the channels as M (x) or N
 // (dy), are the MN-major canonical layout, so three taps share one M = 128 MMA (below)
 // and no shared-memory transpose is needed; the accumulators stay in tensor memory for
@@ -25,6 +25,8 @@
 // 4 columns) at the end.
 #include <cuda.h>
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "sgad_launch.cuh"
 #include "sgad_net_device.cuh"
@@ -266,12 +268,12 @@ __device__ __forceinline__ void load_row(uint32_t dst, const CUtensorMap &wide, 
 struct TileRun {
     int y0, y1, xs, n, left;     // left: tiles of the run from y0 on
     int H, segs;
-    __device__ __forceinline__ TileRun(const ConvArgs &a)
+    __device__ __forceinline__ TileRun(const ConvArgs &a, int block, int blocks)
     {
         H = a.H;
         segs = (a.W + kTileM - 1) / kTileM;
         const long long total = (long long)a.N * segs * a.H;
-        const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
+        const long long t0 = total * block / blocks, t1 = total * (block + 1) / blocks;
         left = (int)(t1 - t0);
         const long long col = t0 / a.H;
         y0 = (int)(t0 - col * a.H);
@@ -288,9 +290,10 @@ struct TileRun {
     }
 };
 
+// Block `block` of `blocks` of a convolution; 192 threads.
 template <int CI, int CO, int MODE>
-__global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ CUtensorMap wide,
-                                                     const __grid_constant__ CUtensorMap halo, const ConvArgs a)
+__device__ __forceinline__ void conv_block(const CUtensorMap &wide, const CUtensorMap &halo, const ConvArgs &a, int block,
+                                           int blocks)
 {
     static_assert(CI % 16 == 0 && (CO == 16 || CO == 32), "channel counts");
     using S = TmaConvSmem<CI, CO>;
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
             uint32_t slot = 0, turn = 0, loads = 0;
             const uint32_t s0 = tc::smem_u32(sA);
             bool ok = true;
-            for (TileRun t(a); t.left > 0 && ok; t.next())
+            for (TileRun t(a, block, blocks); t.left > 0 && ok; t.next())
                 for (int r = t.y0 - 1; r <= t.y1 + 1; ++r) {
                     // (the slot's previous row landed before the MMAs that freed it ran)
                     if (!tc::mbar_wait_bounded(&empty[slot], (turn & 1) ^ 1, kSpinLimit)) {
@@ -355,7 +358,7 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
             uint32_t slot = 0, turn = 0;
             int k = 0;                                         // tiles before this column part
             bool ok = true;
-            for (TileRun t(a); t.left > 0 && ok; k += t.y1 - t.y0 + 1, t.next())
+            for (TileRun t(a, block, blocks); t.left > 0 && ok; k += t.y1 - t.y0 + 1, t.next())
                 for (int r = t.y0 - 1; r <= t.y1 + 1; ++r) {
                     const int lo = max(r - 1, t.y0), hi = min(r + 1, t.y1);     // output rows
                     const int k_lo = k + lo - t.y0, k_hi = k + hi - t.y0;
@@ -412,7 +415,7 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
         const int quarter = warp & 3;
         int k = 0;
         bool ok = true;
-        for (TileRun t(a); t.left > 0 && ok; t.next())
+        for (TileRun t(a, block, blocks); t.left > 0 && ok; t.next())
         for (int y = t.y0; y <= t.y1; ++y, ++k) {
             const int acc = k % kAcc;
             if (!tc::mbar_wait_bounded(&tfull[acc], (k / kAcc) & 1, kSpinLimit)) {
@@ -447,6 +450,13 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
     if (warp == 0) tc::tmem_dealloc(tmem, kAcc * CO);
 }
 
+template <int CI, int CO, int MODE>
+__global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ CUtensorMap wide,
+                                                        const __grid_constant__ CUtensorMap halo, const ConvArgs a)
+{
+    conv_block<CI, CO, MODE>(wide, halo, a, (int)blockIdx.x, (int)gridDim.x);
+}
+
 // ------------------------------------------------------------------ weight gradient, TMA-fed
 //
 // The same sums, with the operands read in the layout the TMA boxes land in, so that no
@@ -470,10 +480,10 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
 //
 // The final additions of all blocks meet on the same 3 CI CO addresses, so a small problem
 // takes fewer blocks: kWgTiles K blocks each, at least one block per SM (4: 55 us
-// for the two 32 -> 32 layers of 3 x 315x237, 8: 50, 32: 57).
-// 3 x 315x237, 32 -> 32 channels (28 MB in): 24 us, of which the additions 8 and the launch,
-// setup and drain 8; 94 us with single-float atomics from every resident block (4.2 M onto
-// 9216 addresses) and 28 copies of 16-byte rows per K block.
+// for two 32 -> 32 layers of 3 x 315x237 in launches of their own, 8: 50, 32: 57).
+// 3 x 315x237, 32 -> 32 channels (28 MB in) in a launch of its own: 24 us, of which the
+// additions 8 and the launch, setup and drain 8; 94 us with single-float atomics from every
+// resident block (4.2 M onto 9216 addresses) and 28 copies of 16-byte rows per K block.
 #ifndef SGAD_WG_TILES
 #define SGAD_WG_TILES 8
 #endif
@@ -482,7 +492,7 @@ constexpr int kWgPix = 128;                // pixels per K block
 constexpr int kWgGroups = 16;              // M groups read by an M = 128 MMA
 constexpr int kWgStages = 3;               // shared-memory stages of the load pipeline
 
-template <int CI, int CO>
+template <int CI, int CO, int STAGES = kWgStages>
 struct WgradTmaSmem {
     static constexpr int kXBytes = (3 * (CI / 8) + 1) * kWgPix * 16;       // slabs of x, then the ones slab
     static constexpr int kYBytes = (CO / 8) * kSlabUnits * 16;             // slabs of dy
@@ -491,7 +501,7 @@ struct WgradTmaSmem {
     static constexpr int kStage = kXBytes + kYBytes > kWgGroups * kWgPix * 16 ? kXBytes + kYBytes
                                                                              : kWgGroups * kWgPix * 16;
     static constexpr uint32_t kTx = (uint32_t)(3 * (CI / 8) * kWgPix * 16 + (CO / 8) * kRowUnits * 16);
-    static constexpr size_t bytes = (size_t)kWgStages * kStage + 1024;   // + alignment slack
+    static constexpr size_t bytes = (size_t)STAGES * kStage + 1024;   // + alignment slack
     static constexpr int kCols = 3 * CO <= 32 ? 32 : (3 * CO <= 64 ? 64 : 128);
     static_assert(3 * (CI / 8) + 1 <= kWgGroups, "the three rows and the ones slab fit one M = 128 MMA");
 };
@@ -512,18 +522,18 @@ __device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t mn_stride,
     return tc::sdesc(saddr, k_stride, mn_stride);
 }
 
-template <int CI, int CO>
-__global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant__ CUtensorMap xmap,
-                                                           const __grid_constant__ CUtensorMap ywide,
-                                                           const __grid_constant__ CUtensorMap yhalo,
-                                                           const WgradArgs a)
+// Block `block` of `blocks` of a weight gradient; 128 threads or more, of which the first
+// four warps read the accumulators.
+template <int CI, int CO, int STAGES>
+__device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUtensorMap &ywide, const CUtensorMap &yhalo,
+                                            const WgradArgs &a, int block, int blocks)
 {
     static_assert(CI % 16 == 0 && (CO == 16 || CO == 32), "channel counts");
-    using S = WgradTmaSmem<CI, CO>;
+    using S = WgradTmaSmem<CI, CO, STAGES>;
     constexpr int kcx = CI / 8, kcy = CO / 8;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ uint64_t full[kWgStages], empty[kWgStages];
+    __shared__ uint64_t full[STAGES], empty[STAGES];
     __shared__ uint32_t taddr_s;
     __shared__ int failed_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -532,14 +542,14 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
 
     if (warp == 0) tc::tmem_alloc(&taddr_s, S::kCols);
     if (threadIdx.x == 32) {
-        for (int i = 0; i < kWgStages; ++i) {
+        for (int i = 0; i < STAGES; ++i) {
             tc::mbar_init(&full[i], 1);
             tc::mbar_init(&empty[i], 1);
         }
         failed_s = 0;
     }
     // the slab after the three input rows: ones (first element of each unit)
-    for (int st = 0; st < kWgStages; ++st) {
+    for (int st = 0; st < STAGES; ++st) {
         uint4 *x = reinterpret_cast<uint4 *>(base + (size_t)st * S::kStage) + 3 * kcx * kWgPix;
         for (int i = threadIdx.x; i < kWgPix; i += blockDim.x) x[i] = make_uint4(0x3F80u, 0u, 0u, 0u);
     }
@@ -554,9 +564,9 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     if (threadIdx.x == 0) {                                    // TMA producer
         int k = 0;
         bool ok = true;
-        for (int kb = blockIdx.x; kb < n_kb; kb += gridDim.x, ++k) {
-            const int st = k % kWgStages;
-            if (!tc::mbar_wait_bounded(&empty[st], (uint32_t)(((k / kWgStages) & 1) ^ 1), kSpinLimit)) {
+        for (int kb = block; kb < n_kb; kb += blocks, ++k) {
+            const int st = k % STAGES;
+            if (!tc::mbar_wait_bounded(&empty[st], (uint32_t)(((k / STAGES) & 1) ^ 1), kSpinLimit)) {
                 ok = false;
                 break;
             }
@@ -568,7 +578,7 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
             load_row<kcy>(yb, ywide, yhalo, xs * kWgPix, y, n, &full[st]);
         }
         // drain: the last boxes have landed before the block may exit
-        if (k > 0 && !tc::mbar_wait_bounded(&full[(k - 1) % kWgStages], (uint32_t)(((k - 1) / kWgStages) & 1), kSpinLimit))
+        if (k > 0 && !tc::mbar_wait_bounded(&full[(k - 1) % STAGES], (uint32_t)(((k - 1) / STAGES) & 1), kSpinLimit))
             ok = false;
         if (!ok) {
             set_status(a.status, 3u);
@@ -580,9 +590,9 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
         const uint64_t ad0 = sdesc_mn(x0, kWgPix * 16, 128), bd0 = sdesc_mn(y0, kSlabUnits * 16, 128);
         int k = 0;
         bool ok = true;
-        for (int kb = blockIdx.x; kb < n_kb; kb += gridDim.x, ++k) {
-            const int st = k % kWgStages;
-            if (!tc::mbar_wait_bounded(&full[st], (uint32_t)((k / kWgStages) & 1), kSpinLimit)) {
+        for (int kb = block; kb < n_kb; kb += blocks, ++k) {
+            const int st = k % STAGES;
+            if (!tc::mbar_wait_bounded(&full[st], (uint32_t)((k / STAGES) & 1), kSpinLimit)) {
                 ok = false;
                 break;
             }
@@ -597,7 +607,7 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
             tc::mma_commit(&empty[st]);
         }
         // drain: the last MMAs have completed before the accumulators are read
-        if (k > 0 && !tc::mbar_wait_bounded(&empty[(k - 1) % kWgStages], (uint32_t)(((k - 1) / kWgStages) & 1), kSpinLimit))
+        if (k > 0 && !tc::mbar_wait_bounded(&empty[(k - 1) % STAGES], (uint32_t)(((k - 1) / STAGES) & 1), kSpinLimit))
             ok = false;
         if (!ok) {
             set_status(a.status, 2u);
@@ -608,12 +618,12 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    if (failed_s == 0) {
+    if (failed_s == 0 && warp < 4) {
         const int row = 32 * warp + lane;
         constexpr int kParts = 3 * (CO / 16);          // of 16 columns; blocks start at different ones
 #pragma unroll 1
         for (int i = 0; i < kParts; ++i) {
-            const int part = (i + (int)blockIdx.x) % kParts, dx = part / (CO / 16), c0 = part % (CO / 16) * 16;
+            const int part = (i + block) % kParts, dx = part / (CO / 16), c0 = part % (CO / 16) * 16;
             uint32_t q[16];
             tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(dx * CO + c0), q);
             tc::tmem_wait_ld();
@@ -639,6 +649,37 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem, S::kCols);
+}
+
+template <int CI, int CO>
+__global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant__ CUtensorMap xmap,
+                                                           const __grid_constant__ CUtensorMap ywide,
+                                                           const __grid_constant__ CUtensorMap yhalo,
+                                                           const WgradArgs a)
+{
+    wgrad_block<CI, CO, kWgStages>(xmap, ywide, yhalo, a, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// Both gradients of a layer (CI channels in, CO out) side by side: the first n_conv blocks the
+// input gradient, the others the weight gradient. Each is a chain of latencies at small sizes
+// and leaves bandwidth at large ones: the net's backward of 3 x 315x237 takes 90 us against 126
+// with a launch each, of 8 x 640x480 459 against 522. Half of the blocks each: three or five
+// eighths for the weight gradient 514 and 531 us at 8 x 640x480. Small problems give the weight
+// gradient a block per 8 to 12 K blocks (8 with few: 54 us against 61 at 1 x 315x237, 12 at
+// 3 x 315x237: 90 against 95), whose final additions meet on the same addresses.
+constexpr int kPairStages = 2;             // load stages of the weight gradient: three blocks fit an SM
+constexpr int kPairBlocks = 3;
+template <int CI, int CO>
+__global__ void __launch_bounds__(192, kPairBlocks) k_conv3x3_grads(const __grid_constant__ CUtensorMap xmap,
+                                                                    const __grid_constant__ CUtensorMap ywide,
+                                                                    const __grid_constant__ CUtensorMap yhalo,
+                                                                    const ConvArgs c, const WgradArgs w, int n_conv)
+{
+    const int b = (int)blockIdx.x;
+    if (b < n_conv)
+        conv_block<CO, CI, kModeMask>(ywide, yhalo, c, b, n_conv);
+    else
+        wgrad_block<CI, CO, kPairStages>(xmap, ywide, yhalo, w, b - n_conv, (int)gridDim.x - n_conv);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -772,14 +813,37 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
     return launch_after(k_conv3x3_wgrad_tma<CI, CO>, grid, 128, S::bytes, st, xm, wide, halo, a);
 }
 
+template <int CI, int CO>
+cudaError_t launch_grads(const ConvArgs &c, const WgradArgs &w, cudaStream_t st)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long tiles = (long long)c.N * c.H * ((c.W + kTileM - 1) / kTileM);
+    constexpr size_t smem = WgradTmaSmem<CI, CO, kPairStages>::bytes > TmaConvSmem<CO, CI>::bytes
+                                ? WgradTmaSmem<CI, CO, kPairStages>::bytes
+                                : TmaConvSmem<CO, CI>::bytes;
+    cudaError_t e = set_smem(k_conv3x3_grads<CI, CO>, smem);
+    if (e != cudaSuccess || tiles <= 0) return e;
+    CUtensorMap xm, wide, halo;
+    e = input_map(w.x, CI, w.N, w.H, w.W, &xm, kWgPix, CI / 8, 3);
+    if (e == cudaSuccess) e = input_map(w.dy, CO, w.N, w.H, w.W, &wide, kTileM);
+    if (e == cudaSuccess) e = input_map(w.dy, CO, w.N, w.H, w.W, &halo, 2);
+    if (e != cudaSuccess) return e;
+    // (tiles and K blocks are the same in number)
+    const int room = kPairBlocks * sms;
+    const int n_wgrad = (int)std::min<long long>({std::max<long long>(1, tiles / kWgTiles),
+                                                  std::max<long long>(128, tiles / 12), room / 2});
+    const int n_conv = (int)std::min<long long>(tiles, room - n_wgrad);
+    return launch_after(k_conv3x3_grads<CI, CO>, n_conv + n_wgrad, 192, smem, st, xm, wide, halo, c, w, n_conv);
+}
+
 template cudaError_t launch_conv<16, 32, kModeRelu>(const ConvArgs &, cudaStream_t);
 template cudaError_t launch_conv<32, 32, kModeRelu>(const ConvArgs &, cudaStream_t);
 template cudaError_t launch_conv<32, 16, kModeOut>(const ConvArgs &, cudaStream_t);
-template cudaError_t launch_conv<16, 32, kModeMask>(const ConvArgs &, cudaStream_t);
-template cudaError_t launch_conv<32, 32, kModeMask>(const ConvArgs &, cudaStream_t);
 template cudaError_t launch_wgrad<16, 32>(const WgradArgs &, cudaStream_t);
-template cudaError_t launch_wgrad<32, 32>(const WgradArgs &, cudaStream_t);
-template cudaError_t launch_wgrad<32, 16>(const WgradArgs &, cudaStream_t);
+template cudaError_t launch_grads<32, 32>(const ConvArgs &, const WgradArgs &, cudaStream_t);
+template cudaError_t launch_grads<32, 16>(const ConvArgs &, const WgradArgs &, cudaStream_t);
 
 cudaError_t launch_pack_input(const float *rgb, const float *depth, uint4 *x0, int n, int h, int w, cudaStream_t st)
 {

@@ -202,28 +202,21 @@ sgad_status sgad_net_backward(const sgad_net_params *params, sgad_net_grads *gra
     g.status = ws.status();
     for (int l = 3; l >= 0 && !s; --l) {
         const uint4 *dout = l == 3 ? ws.at(L.dy4) : ws.at(L.d[l]);
-        if (l > 0) {     // input gradient of layer l = output gradient of layer l - 1, through its ReLU
-            a.in = dout;
-            a.wB = ws.at(L.wb[l]);
-            a.out = ws.at(L.d[l - 1]);
-            a.mask = ws.at(L.x[l]);
-            s = launched(l == 3 ? launch_conv<16, 32, kModeMask>(a, st) : launch_conv<32, 32, kModeMask>(a, st),
-                         "conv input gradient");
-            if (s) break;
-        }
         g.x = ws.at(L.x[l]);
         g.dy = dout;
         g.dw = grads->dw[l];
         g.db = grads->db[l];
         g.vec = (reinterpret_cast<uintptr_t>(g.dw) & 15) == 0;
-        cudaError_t e;
-        if (l == 0)
-            e = launch_wgrad<16, 32>(g, st);
-        else if (l < 3)
-            e = launch_wgrad<32, 32>(g, st);
-        else
-            e = launch_wgrad<32, 16>(g, st);
-        s = launched(e, "conv weight gradient");
+        if (l == 0) {
+            s = launched(launch_wgrad<16, 32>(g, st), "conv weight gradient");
+            break;
+        }
+        // input gradient of layer l = output gradient of layer l - 1, through its ReLU
+        a.in = dout;
+        a.wB = ws.at(L.wb[l]);
+        a.out = ws.at(L.d[l - 1]);
+        a.mask = ws.at(L.x[l]);
+        s = launched(l == 3 ? launch_grads<32, 16>(a, g, st) : launch_grads<32, 32>(a, g, st), "conv gradients");
     }
     return s;
 }

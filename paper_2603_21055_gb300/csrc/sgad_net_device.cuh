@@ -52,6 +52,9 @@ template <int CI, int CO, int MODE>
 cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st);
 template <int CI, int CO>
 cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st);
+// Input and weight gradient of a layer of CI channels in and CO out.
+template <int CI, int CO>
+cudaError_t launch_grads(const ConvArgs &c, const WgradArgs &w, cudaStream_t st);
 cudaError_t launch_pack_input(const float *rgb, const float *depth, uint4 *x0, int n, int h, int w, cudaStream_t st);
 cudaError_t launch_prep_weights(const PrepArgs &a, cudaStream_t st);
 cudaError_t launch_zero_grads(const ZeroArgs &a, cudaStream_t st);
