@@ -1676,11 +1676,14 @@ extern "C" sgad_status sgad_gicp_result(void *workspace, size_t ws_bytes, double
 {
     sgad_status s = check_ws(workspace, ws_bytes, sizeof(GicpState));
     if (s) return s;
-    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess)
-        return report_error(SGAD_ERR_CUDA, "sgad_gicp_result: stream failed");
+    // on the caller's stream alone: a plain copy would wait for the work of the default stream
+    // too
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
     GicpState h;
-    if (cudaMemcpy(&h, workspace, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (cudaMemcpyAsync(&h, workspace, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return report_error(SGAD_ERR_CUDA, "sgad_gicp_result: copy failed");
+    if (cudaStreamSynchronize(st) != cudaSuccess)
+        return report_error(SGAD_ERR_CUDA, "sgad_gicp_result: stream failed");
     if (pose) std::memcpy(pose, h.pose, sizeof(h.pose));
     if (stats) {
         stats->iterations = h.iters;

@@ -150,15 +150,28 @@ class GicpTracker:
         self.frame(cam, depths[0])
         self.set_pose(poses[0])
         self.insert()
+        if len(depths) > 1:
+            self.frame(cam, depths[1])
+        # The host needs a frame's pose for the next guess only: it reads it on a stream of its
+        # own as soon as the track is over, while the map update and the next frame's Gaussians,
+        # which need no guess, run (about 60 us of host time a frame otherwise).
+        side, tracked = torch.cuda.Stream(), torch.cuda.Event()
         for i in range(1, len(depths)):
             if i >= 2:
                 T1, T0 = pose44(poses[-1]), pose44(poses[-2])
                 guess = (T1 @ np.linalg.inv(T0) @ T1)[:3]
             else:
                 guess = poses[-1]
-            self.frame(cam, depths[i])
             self.track(guess)
-            self.insert()
-            pose, _ = self.result()
+            if i + 1 < len(depths):
+                tracked.record()
+                self.insert()
+                self.frame(cam, depths[i + 1])
+                side.wait_event(tracked)
+                with torch.cuda.stream(side):
+                    pose, _ = self.result()
+            else:
+                self.insert()
+                pose, _ = self.result()
             poses.append(pose)
         return poses
