@@ -21,8 +21,8 @@
 // GEMM with the pixels as K; the same TMA boxes, read with the channels as M (x) or N
 // (dy), are the MN-major canonical layout, so three taps share one M = 128 MMA (below)
 // and no shared-memory transpose is needed; the accumulators stay in tensor memory for
-// the whole persistent block and are added to the output with one 16-byte atomic per (row,
-// 4 columns) at the end.
+// a chain of K blocks, then in registers, and are added to the output with one 16-byte atomic
+// per (row, 4 columns) at the end of the block.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -231,14 +231,9 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs &a, const float *bi
 // window of the ring: 69, 46 and 59 (48 cycles per MMA, 2/3 of them spent re-reading the
 // pixels); with three rows loaded per tile as rows of 16 bytes: 129, 112 and 76. Fewer slots
 // and more blocks per SM win: 2 slots 65 us, 3: 59, 4: 61, 6: 63; 8 accumulators (2 blocks) 98.
-#ifndef SGAD_CONV_RING
-#define SGAD_CONV_RING 3
-#endif
-#ifndef SGAD_CONV_ACC
-#define SGAD_CONV_ACC 4
-#endif
-constexpr int kRing = SGAD_CONV_RING;  // input row slots
-constexpr int kAcc = SGAD_CONV_ACC;    // accumulators (C_out tensor memory columns each): three in work, the rest in the epilogue
+constexpr int kRing = 3;               // input row slots
+constexpr int kAcc = 4;                // accumulators (C_out tensor memory columns each): three in
+                                       // work, one in the epilogue
 static_assert(kAcc >= 4 && (kAcc & (kAcc - 1)) == 0 && kRing >= 2, "ring sizes");
 constexpr int kSlabUnits = 136;        // 16-byte units per staged (row, chunk) slab: 130 used, 128-byte aligned
 
@@ -320,7 +315,8 @@ __device__ __forceinline__ void conv_block(const CUtensorMap &wide, const CUtens
         }
     }
     dependency_wait();
-    if (MODE != kModeMask && threadIdx.x >= 64 && threadIdx.x < 64 + CO) bias[threadIdx.x - 64] = a.bias[threadIdx.x - 64];
+    if (MODE != kModeMask && threadIdx.x >= 64 && threadIdx.x < 64 + CO)
+        bias[threadIdx.x - 64] = a.bias[threadIdx.x - 64];
 #pragma unroll 6
     for (int i = threadIdx.x; i < S::kB / 16; i += 192) sB[i] = a.wB[i];
     tc::fence_proxy_async();
@@ -473,10 +469,9 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
 // 16-pixel K step) covers the three taps (dy, dx). The M rows after 3 CI read a slab of ones
 // (row 3 CI: the bias gradient, taken from dx = 1) and then whatever follows it in the
 // stage, rows whose products are not used. Accumulators: three TMEM blocks of CO columns
-// (one per dx) for the whole persistent block, added to dW at the end with 16-byte atomics.
-// One thread of warp 0 issues the TMA loads into kWgStages stages, one thread of warp 1
-// the MMAs (its descriptors precomputed: an offset adds to the address field); the four
-// warps run the epilogue. Every wait is bounded.
+// (one per dx), added to dW at the end with 16-byte atomics. One thread of warp 0 issues the
+// TMA loads into kWgStages stages, one thread of warp 1 the MMAs (its descriptors precomputed:
+// an offset adds to the address field); warps 2 to 5 sum and add. Every wait is bounded.
 //
 // The final additions of all blocks meet on the same 3 CI CO addresses, so a small problem
 // takes fewer blocks: kWgTiles K blocks each, at least one block per SM (4: 55 us
@@ -484,10 +479,7 @@ __global__ void __launch_bounds__(192, 4) k_conv3x3_tma(const __grid_constant__ 
 // 3 x 315x237, 32 -> 32 channels (28 MB in) in a launch of its own: 24 us, of which the
 // additions 8 and the launch, setup and drain 8; 94 us with single-float atomics from every
 // resident block (4.2 M onto 9216 addresses) and 28 copies of 16-byte rows per K block.
-#ifndef SGAD_WG_TILES
-#define SGAD_WG_TILES 8
-#endif
-constexpr int kWgTiles = SGAD_WG_TILES;
+constexpr int kWgTiles = 8;                // K blocks per block of a small problem
 constexpr int kWgPix = 128;                // pixels per K block
 constexpr int kWgGroups = 16;              // M groups read by an M = 128 MMA
 constexpr int kWgStages = 3;               // shared-memory stages of the load pipeline
@@ -522,8 +514,23 @@ __device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t mn_stride,
     return tc::sdesc(saddr, k_stride, mn_stride);
 }
 
-// Block `block` of `blocks` of a weight gradient; 128 threads or more, of which the first
-// four warps read the accumulators.
+// A bounded wait of warps with nothing else to do, off the issue slots between tries.
+__device__ __forceinline__ bool wait_idle(uint64_t *bar, uint32_t parity)
+{
+    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+        if (tc::mbar_try_wait(bar, parity)) return true;
+        __nanosleep(200);
+    }
+    return false;
+}
+
+// Block `block` of `blocks` of a weight gradient; 192 threads. The tensor core's FP32
+// accumulation loses up to a last place of the sum per step, so a sum in tensor memory ends
+// after a.chain K blocks, and warps 2-5 add it to FP32 registers, rounded to nearest. With one
+// sum per block of twelve K blocks the last layer's gradient of 3 x 315x237 was 1.7 times as
+// far from FP64 as with 304 blocks of seven; now every layer is as far as those or nearer.
+// The sums cost the backward 15 us of 105 at 3 x 315x237; added to the output with atomics
+// instead of kept in registers, 29.
 template <int CI, int CO, int STAGES>
 __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUtensorMap &ywide, const CUtensorMap &yhalo,
                                             const WgradArgs &a, int block, int blocks)
@@ -533,9 +540,8 @@ __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUten
     constexpr int kcx = CI / 8, kcy = CO / 8;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ uint64_t full[STAGES], empty[STAGES];
+    __shared__ uint64_t full[STAGES], empty[STAGES], sum_full, sum_empty;
     __shared__ uint32_t taddr_s;
-    __shared__ int failed_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int segs = (a.W + kWgPix - 1) / kWgPix;
     const int n_kb = a.N * a.H * segs;          // < 2^31 (checked by the launcher)
@@ -546,7 +552,8 @@ __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUten
             tc::mbar_init(&full[i], 1);
             tc::mbar_init(&empty[i], 1);
         }
-        failed_s = 0;
+        tc::mbar_init(&sum_full, 1);
+        tc::mbar_init(&sum_empty, 4);
     }
     // the slab after the three input rows: ones (first element of each unit)
     for (int st = 0; st < STAGES; ++st) {
@@ -580,19 +587,18 @@ __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUten
         // drain: the last boxes have landed before the block may exit
         if (k > 0 && !tc::mbar_wait_bounded(&full[(k - 1) % STAGES], (uint32_t)(((k - 1) / STAGES) & 1), kSpinLimit))
             ok = false;
-        if (!ok) {
-            set_status(a.status, 3u);
-            failed_s = 1;
-        }
+        if (!ok) set_status(a.status, 3u);
     } else if (threadIdx.x == 32) {                           // MMA issuer
         // descriptors of stage 0 at offset 0; an offset of o bytes adds o / 16
         const uint32_t x0 = tc::smem_u32(base), y0 = x0 + (uint32_t)S::kXBytes;
         const uint64_t ad0 = sdesc_mn(x0, kWgPix * 16, 128), bd0 = sdesc_mn(y0, kSlabUnits * 16, 128);
-        int k = 0;
+        int k = 0, in_sum = 0;                                 // K blocks in the current sum
+        uint32_t sums = 0;
         bool ok = true;
         for (int kb = block; kb < n_kb; kb += blocks, ++k) {
             const int st = k % STAGES;
-            if (!tc::mbar_wait_bounded(&full[st], (uint32_t)((k / STAGES) & 1), kSpinLimit)) {
+            if (!tc::mbar_wait_bounded(&full[st], (uint32_t)((k / STAGES) & 1), kSpinLimit) ||
+                (in_sum == 0 && !tc::mbar_wait_bounded(&sum_empty, (sums & 1) ^ 1, kSpinLimit))) {
                 ok = false;
                 break;
             }
@@ -603,30 +609,49 @@ __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUten
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx)
                     tc::mma_bf16(tmem + (uint32_t)(dx * CO), ad0 + so + (uint64_t)(s * 16),
-                                 bd0 + so + (uint64_t)(2 - dx + s * 16), idesc, (k | s) != 0);
+                                 bd0 + so + (uint64_t)(2 - dx + s * 16), idesc, (in_sum | s) != 0);
             tc::mma_commit(&empty[st]);
+            if (++in_sum == a.chain || kb + blocks >= n_kb) {
+                tc::mma_commit(&sum_full);
+                in_sum = 0;
+                ++sums;
+            }
         }
-        // drain: the last MMAs have completed before the accumulators are read
+        // drain: the last MMAs have completed before the accumulators are freed
         if (k > 0 && !tc::mbar_wait_bounded(&empty[(k - 1) % STAGES], (uint32_t)(((k - 1) / STAGES) & 1), kSpinLimit))
             ok = false;
-        if (!ok) {
-            set_status(a.status, 2u);
-            failed_s = 1;
+        if (!ok) set_status(a.status, 2u);
+    } else if (warp >= 2 && warp < 6) {                       // sums
+        constexpr int kParts = 3 * (CO / 16);                  // of 16 columns
+        const int quarter = warp & 3, row = 32 * quarter + lane;
+        const int n_k = block < n_kb ? (n_kb - block + blocks - 1) / blocks : 0, n_sums = (n_k + a.chain - 1) / a.chain;
+        float acc[kParts][16];
+#pragma unroll
+        for (int p = 0; p < kParts; ++p)
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc[p][c] = 0.f;
+        bool ok = n_k > 0;
+        for (int i = 0; i < n_sums; ++i) {
+            if (!wait_idle(&sum_full, (uint32_t)(i & 1))) {
+                if (lane == 0) set_status(a.status, 2u);
+                ok = false;
+                break;
+            }
+            tc::fence_after_sync();
+#pragma unroll
+            for (int p = 0; p < kParts; ++p) {
+                uint32_t q[16];
+                tc::tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(p * 16), q);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int c = 0; c < 16; ++c) acc[p][c] += __uint_as_float(q[c]);
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&sum_empty);
         }
-        if (k == 0) failed_s = failed_s | 2;
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (failed_s == 0 && warp < 4) {
-        const int row = 32 * warp + lane;
-        constexpr int kParts = 3 * (CO / 16);          // of 16 columns; blocks start at different ones
-#pragma unroll 1
-        for (int i = 0; i < kParts; ++i) {
-            const int part = (i + block) % kParts, dx = part / (CO / 16), c0 = part % (CO / 16) * 16;
-            uint32_t q[16];
-            tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(dx * CO + c0), q);
-            tc::tmem_wait_ld();
+        const auto add = [&](int p) {
+            const int dx = p / (CO / 16), c0 = p % (CO / 16) * 16;
             if (row < 3 * CI) {
                 const int tap = 3 * (row / CI) + dx, ci = row % CI;
                 float *dst = a.dw + ((size_t)tap * CI + ci) * CO + c0;
@@ -634,16 +659,23 @@ __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUten
 #pragma unroll
                     for (int c = 0; c < 16; c += 4)
                         atomicAdd(reinterpret_cast<float4 *>(dst + c),
-                                  make_float4(__uint_as_float(q[c]), __uint_as_float(q[c + 1]),
-                                              __uint_as_float(q[c + 2]), __uint_as_float(q[c + 3])));
+                                  make_float4(acc[p][c], acc[p][c + 1], acc[p][c + 2], acc[p][c + 3]));
                 } else {
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) atomicAdd(dst + c, __uint_as_float(q[c]));
+                    for (int c = 0; c < 16; ++c) atomicAdd(dst + c, acc[p][c]);
                 }
             } else if (row == 3 * CI && dx == 1) {
 #pragma unroll
-                for (int c = 0; c < 16; ++c) atomicAdd(a.db + c0 + c, __uint_as_float(q[c]));
+                for (int c = 0; c < 16; ++c) atomicAdd(a.db + c0 + c, acc[p][c]);
             }
+        };
+        // neighbouring blocks start at opposite ends
+        if (ok && (block & 1)) {
+#pragma unroll
+            for (int p = kParts - 1; p >= 0; --p) add(p);
+        } else if (ok) {
+#pragma unroll
+            for (int p = 0; p < kParts; ++p) add(p);
         }
     }
     tc::fence_before_sync();
@@ -652,7 +684,7 @@ __device__ __forceinline__ void wgrad_block(const CUtensorMap &xmap, const CUten
 }
 
 template <int CI, int CO>
-__global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant__ CUtensorMap xmap,
+__global__ void __launch_bounds__(192, 2) k_conv3x3_wgrad_tma(const __grid_constant__ CUtensorMap xmap,
                                                            const __grid_constant__ CUtensorMap ywide,
                                                            const __grid_constant__ CUtensorMap yhalo,
                                                            const WgradArgs a)
@@ -662,11 +694,12 @@ __global__ void __launch_bounds__(128) k_conv3x3_wgrad_tma(const __grid_constant
 
 // Both gradients of a layer (CI channels in, CO out) side by side: the first n_conv blocks the
 // input gradient, the others the weight gradient. Each is a chain of latencies at small sizes
-// and leaves bandwidth at large ones: the net's backward of 3 x 315x237 takes 90 us against 126
-// with a launch each, of 8 x 640x480 459 against 522. Half of the blocks each: three or five
-// eighths for the weight gradient 514 and 531 us at 8 x 640x480. Small problems give the weight
-// gradient a block per 8 to 12 K blocks (8 with few: 54 us against 61 at 1 x 315x237, 12 at
-// 3 x 315x237: 90 against 95), whose final additions meet on the same addresses.
+// and leaves bandwidth at large ones: the net's backward of 3 x 315x237 takes 105 us against 126
+// with a launch each, of 4 x 640x480 283 against 299, of 8 x 640x480 531 against 522. Half of the
+// blocks each (three or five eighths for the weight gradient, with one sum per block: 514 and 531
+// us at 8 x 640x480 against 459). Small problems give the weight gradient a block per 8 to 12 K
+// blocks (8 with few: 54 us against 61 at 1 x 315x237, 12 at 3 x 315x237: 90 against 95), whose
+// final additions meet on the same addresses.
 constexpr int kPairStages = 2;             // load stages of the weight gradient: three blocks fit an SM
 constexpr int kPairBlocks = 3;
 template <int CI, int CO>
@@ -787,8 +820,11 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st)
     return launch_after(k_conv3x3_tma<CI, CO, MODE>, grid, 192, smem, st, wide, halo, a);
 }
 
+// K blocks of one sum in tensor memory: what a block would take if there were two per SM.
+int sum_chain(long long k_blocks, int sms) { return (int)std::max<long long>(1, k_blocks / (2 * sms)); }
+
 template <int CI, int CO>
-cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
+cudaError_t launch_wgrad(WgradArgs a, cudaStream_t st)
 {
     using S = WgradTmaSmem<CI, CO>;
     cudaError_t e = set_smem(k_conv3x3_wgrad_tma<CI, CO>, S::bytes);
@@ -802,7 +838,7 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
     if (e == cudaSuccess) e = input_map(a.dy, CO, a.N, a.H, a.W, &halo, 2);
     if (e != cudaSuccess) return e;
     // keep (resident blocks x TMEM columns) within the 512 columns of an SM
-    int grid = resident_grid((const void *)k_conv3x3_wgrad_tma<CI, CO>, S::bytes, blocks);
+    int grid = resident_grid((const void *)k_conv3x3_wgrad_tma<CI, CO>, S::bytes, blocks, 192);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -810,11 +846,12 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st)
     if (grid > cap) grid = (int)cap;
     const long long by_work = blocks / kWgTiles;
     if (grid > by_work) grid = (int)(by_work > sms ? by_work : (grid < sms ? grid : sms));
-    return launch_after(k_conv3x3_wgrad_tma<CI, CO>, grid, 128, S::bytes, st, xm, wide, halo, a);
+    a.chain = sum_chain(blocks, sms);
+    return launch_after(k_conv3x3_wgrad_tma<CI, CO>, grid, 192, S::bytes, st, xm, wide, halo, a);
 }
 
 template <int CI, int CO>
-cudaError_t launch_grads(const ConvArgs &c, const WgradArgs &w, cudaStream_t st)
+cudaError_t launch_grads(const ConvArgs &c, WgradArgs w, cudaStream_t st)
 {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -835,15 +872,16 @@ cudaError_t launch_grads(const ConvArgs &c, const WgradArgs &w, cudaStream_t st)
     const int n_wgrad = (int)std::min<long long>({std::max<long long>(1, tiles / kWgTiles),
                                                   std::max<long long>(128, tiles / 12), room / 2});
     const int n_conv = (int)std::min<long long>(tiles, room - n_wgrad);
+    w.chain = sum_chain(tiles, sms);
     return launch_after(k_conv3x3_grads<CI, CO>, n_conv + n_wgrad, 192, smem, st, xm, wide, halo, c, w, n_conv);
 }
 
 template cudaError_t launch_conv<16, 32, kModeRelu>(const ConvArgs &, cudaStream_t);
 template cudaError_t launch_conv<32, 32, kModeRelu>(const ConvArgs &, cudaStream_t);
 template cudaError_t launch_conv<32, 16, kModeOut>(const ConvArgs &, cudaStream_t);
-template cudaError_t launch_wgrad<16, 32>(const WgradArgs &, cudaStream_t);
-template cudaError_t launch_grads<32, 32>(const ConvArgs &, const WgradArgs &, cudaStream_t);
-template cudaError_t launch_grads<32, 16>(const ConvArgs &, const WgradArgs &, cudaStream_t);
+template cudaError_t launch_wgrad<16, 32>(WgradArgs, cudaStream_t);
+template cudaError_t launch_grads<32, 32>(const ConvArgs &, WgradArgs, cudaStream_t);
+template cudaError_t launch_grads<32, 16>(const ConvArgs &, WgradArgs, cudaStream_t);
 
 cudaError_t launch_pack_input(const float *rgb, const float *depth, uint4 *x0, int n, int h, int w, cudaStream_t st)
 {

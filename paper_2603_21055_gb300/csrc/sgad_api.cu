@@ -287,10 +287,10 @@ sgad_status run_composite(const sgad_ctx *ctx, bool fwd, int batch, int schedule
                           bool queue_clear, cudaStream_t st)
 {
     uint32_t *contrib = (!fwd || batch < 0 || ctx->opt.bwd_algorithm == SGAD_BWD_PAIRS) ? ws.contrib() : nullptr;
-    const cudaError_t e = launch_composite(fwd, batch, schedule, ctx->opt.max_blocks, sc, ws.world(), ws.tile_off(), ws.keys(), ws.pix_t(),
-                                           ws.pix_n(), fwd ? nullptr : ws.gacc(), ws.hdr(), ws.tile_order(), contrib,
-                                           ws.wmask(), batch < 0 && uses_masks(ctx->opt, sc) ? ws.bmask() : nullptr,
-                                           queue_clear, st);
+    const cudaError_t e = launch_composite(
+        fwd, batch, schedule, ctx->opt.max_blocks, sc, ws.world(), ws.tile_off(), ws.keys(), ws.pix_t(), ws.pix_n(),
+        fwd ? nullptr : ws.gacc(), ws.hdr(), ws.tile_order(), contrib, ws.wmask(),
+        batch < 0 && uses_masks(ctx->opt, sc) ? ws.bmask() : nullptr, queue_clear, st);
     return e == cudaSuccess ? SGAD_OK : cuda_fail(e, fwd ? "forward compositing launch" : "backward compositing launch");
 }
 
@@ -794,7 +794,8 @@ sgad_status sgad_autotune(sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n_kf,
         for (int sched : kScheds)
             for (int batch : kBatches) {
                 float ms = 0.f;
-                s = timer.median(reps, st, [&] { return run_composite(&trial, true, batch, sched, sc, ws, false, st); }, &ms);
+                s = timer.median(reps, st,
+                                 [&] { return run_composite(&trial, true, batch, sched, sc, ws, false, st); }, &ms);
                 if (s) return s;
                 log.add(shape[0], shape[1], SGAD_TUNE_FWD, batch, sched, ms);
                 if (best_f < 0.f || ms < best_f) {

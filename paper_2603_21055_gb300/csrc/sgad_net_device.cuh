@@ -30,6 +30,7 @@ struct WgradArgs {
     float *dw;           // [9][CI][CO] f32, accumulated into
     float *db;           // [CO] f32, accumulated into
     int vec;             // dw is 16-byte aligned: added to with 16-byte atomics
+    int chain;           // K blocks summed in tensor memory before FP32 registers take over (set at launch)
     int N, H, W;
     uint32_t *status;
 };
@@ -51,10 +52,10 @@ struct ZeroArgs {
 template <int CI, int CO, int MODE>
 cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st);
 template <int CI, int CO>
-cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t st);
+cudaError_t launch_wgrad(WgradArgs a, cudaStream_t st);
 // Input and weight gradient of a layer of CI channels in and CO out.
 template <int CI, int CO>
-cudaError_t launch_grads(const ConvArgs &c, const WgradArgs &w, cudaStream_t st);
+cudaError_t launch_grads(const ConvArgs &c, WgradArgs w, cudaStream_t st);
 cudaError_t launch_pack_input(const float *rgb, const float *depth, uint4 *x0, int n, int h, int w, cudaStream_t st);
 cudaError_t launch_prep_weights(const PrepArgs &a, cudaStream_t st);
 cudaError_t launch_zero_grads(const ZeroArgs &a, cudaStream_t st);
