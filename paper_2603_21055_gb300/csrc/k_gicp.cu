@@ -731,8 +731,10 @@ struct StepArgs {
     float *partial;          // [rows][32]
 };
 
-// Rows of partial sums that hold points: row v sums points 16 (v + k rows) .. + 15.
-__device__ __forceinline__ int rows_used(int n, int rows) { return max(1, min(rows, (n + kRowPts - 1) / kRowPts)); }
+// Rows of partial sums that hold points: row v sums points 16 (v + k rows) .. + 15. Every such
+// row has points (the barriers between zeroing its terms and summing them are in the loop over
+// them); an empty set has no row, and its sums are zero.
+__device__ __forceinline__ int rows_used(int n, int rows) { return min(rows, (n + kRowPts - 1) / kRowPts); }
 
 // The contribution of one correspondence to the Gauss-Newton system (H upper triangle,
 // g = J^T M e, cost, count) in FP32.
