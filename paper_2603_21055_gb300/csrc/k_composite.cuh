@@ -1595,6 +1595,7 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
             gf.b[k][0] = __float_as_uint(S.mom[8 * k + (lane & 3)][lane >> 2]);
             gf.b[k][1] = __float_as_uint(S.mom[8 * k + (lane & 3) + 4][lane >> 2]);
         }
+        __syncwarp();                   // read before a first round without masks stores positions there
     }
     const float bgdot = sc.bg[0] * gr + sc.bg[1] * gg + sc.bg[2] * gb;
     // Reverse-walk state: transmittance, and the suffix sums of colour and depth behind
