@@ -70,7 +70,9 @@ typedef struct {
                              sgad_gicp_frame, set by it or by sgad_gicp_insert);
                              bit 1: fewer than 6 correspondences or a singular system
                              ended the last sgad_gicp_track; bit 2: a wait between the
-                             tracking kernel's blocks gave up */
+                             tracking kernel's blocks gave up in the last sgad_gicp_track,
+                             whose pose is not its result (kept until the next
+                             sgad_gicp_track or sgad_gicp_set_pose) */
     double cost;          /* Eq. 2 at the start of the last iteration */
     double step;          /* |xi| of the last iteration */
 } sgad_gicp_stats;

@@ -44,6 +44,9 @@ struct GicpState {
     int32_t map_old, ins_total;
     int32_t blocks_done;     // step blocks finished in the current iteration
     uint32_t sync;           // grid-wide steps completed (the tracking kernel waits on it)
+    int32_t gave_up;         // 1: a wait of the last track ended without the others. A word of its own,
+                             // which the next frame does not clear: a caller may read the state of a
+                             // track while the next frame is selected
 };
 
 struct GLayout {
@@ -1024,7 +1027,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_gicp_step(const __grid_cons
             while (ld_acquire(&a.state->sync) != epoch + it + 1u && ++t < kSyncSpins) {
             }
             if (t >= kSyncSpins) {                             // recorded; the block ends
-                atomicOr(&a.state->status, 4);
+                a.state->gave_up = 1;
                 s_done = 1;
             } else {
                 s_done = __ldcg(&a.state->done);
@@ -1214,6 +1217,7 @@ __global__ void k_gicp_init(GicpState *st, PoseD p0, int keep_pose, int max_iter
     st->max_iters = max_iters;
     st->tol = tol;
     st->status &= 1;                 // keep the source's overflow flag, clear the rest
+    st->gave_up = 0;
     st->blocks_done = 0;
 }
 
@@ -1691,7 +1695,7 @@ extern "C" sgad_status sgad_gicp_result(void *workspace, size_t ws_bytes, double
         stats->iterations = h.iters;
         stats->converged = h.converged;
         stats->n_matches = h.n;
-        stats->status = h.status;
+        stats->status = (h.status & 3) | (h.gave_up == 1 ? 4 : 0);
         stats->cost = h.cost;
         stats->step = h.step;
     }

@@ -145,7 +145,8 @@ class GicpTracker:
     def track_sequence(self, cam, depths: List[torch.Tensor], first_pose) -> List[np.ndarray]:
         """Cam -> world poses of a depth sequence: frame 0 at `first_pose` seeds the map;
         every later frame starts from the constant-speed guess, is tracked by GICP and
-        then adds its non-overlapping Gaussians to the map."""
+        then adds its non-overlapping Gaussians to the map. Raises SgadError if a track ends
+        before its last iteration because its blocks did not meet in time."""
         poses = [np.asarray(first_pose, np.float64).reshape(3, 4)]
         self.frame(cam, depths[0])
         self.set_pose(poses[0])
@@ -169,9 +170,11 @@ class GicpTracker:
                 self.frame(cam, depths[i + 1])
                 side.wait_event(tracked)
                 with torch.cuda.stream(side):
-                    pose, _ = self.result()
+                    pose, st = self.result()
             else:
                 self.insert()
-                pose, _ = self.result()
+                pose, st = self.result()
+            if st.status & 4:                       # the track was left unfinished
+                raise B.SgadError(B.SGAD_ERR_TIMEOUT, "track_sequence: frame %d: a wait of the track gave up" % i)
             poses.append(pose)
         return poses
