@@ -1097,23 +1097,13 @@ __global__ void __launch_bounds__(kStepThreads) k_gicp_sum(const float *partial,
     if (threadIdx.x < kSys) out[threadIdx.x] = sys[threadIdx.x];
 }
 
-// Reciprocal of a positive, normal d: the hardware's approximation (error e0 ~ 2^-20) and one
-// step of the third-order Newton iteration r (1 + e + e^2), e = 1 - d r, which leaves e0^3.
-__device__ __forceinline__ double reciprocal(double d)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    const double e = fma(-d, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // One warp: from the summed system, an L D L^T solve of H xi = -g in FP64 and the pose
 // update (R, t) <- (Exp(omega) R, Exp(omega) t + v); returns whether the track is over, and
 // |xi|^2 (-1: no step) in step2.
 // Lane r < 6 holds row r of H and lane 6 the row -g, whose factor is the forward
 // substitution; FP64 operations are slow and dependent here, so the rows go side by side,
-// with reciprocals instead of square roots (one thread with a Cholesky factor took ~20 us,
-// this ~3 us).
+// with one rounded reciprocal per column instead of square roots and a division per element
+// (one thread with a Cholesky factor took ~20 us, this ~3 us).
 __device__ bool solve_state(GicpState *st, const double *sys, double &step2)
 {
     const int lane = threadIdx.x & 31;
@@ -1142,7 +1132,7 @@ __device__ bool solve_state(GicpState *st, const double *sys, double &step2)
         const double d = __shfl_sync(kFull, A[j], j);
         good = good && d > 0.0;
         const double u = A[j];
-        A[j] = u * reciprocal(d);
+        A[j] = u * __drcp_rn(d);
 #pragma unroll
         for (int c = j + 1; c < 6; ++c) A[c] -= A[j] * __shfl_sync(kFull, u, c);
     }
