@@ -51,6 +51,7 @@
 
 #include "sgad_device.cuh"
 #include "sgad_launch.cuh"
+#include "sgad_ray.cuh"
 
 #include <type_traits>
 
@@ -932,13 +933,6 @@ __device__ __forceinline__ Proj project_chain(const float4 w0, const ViewDev &v)
     return p;
 }
 
-// a / b to within an ulp, b not subnormal: the approximate reciprocal and one correction.
-__device__ __forceinline__ float quotient(float a, float b)
-{
-    const float r = __fdividef(1.0f, b), q = a * r;
-    return fmaf(fmaf(-q, b, a), r, q);
-}
-
 // Chain rule of one staged Gaussian from its ten accumulated pair moments (colour (3),
 // depth, G, G dx, G dy, G dx^2, G dx dy, G dy^2 with G = dL/dpower) down to the depth
 // |D + delta| along its keyframe ray, s, opacity and colour, added to its accumulator when
@@ -982,7 +976,8 @@ __device__ __forceinline__ float3 chain_and_accumulate(const float *A, const Sta
         int row = (int)__fdividef((float)j, (float)k.W), col = j - row * k.W;   // one off at most
         if (col < 0) --row, col += k.W;
         if (col >= k.W) ++row, col -= k.W;
-        const float rx = quotient((float)col - k.cx, k.fx), ry = quotient((float)row - k.cy, k.fy);
+        const float rx = ray_slope((float)col - k.cx, k.fx, k.inv_fx);
+        const float ry = ray_slope((float)row - k.cy, k.fy, k.inv_fy);
         const float ex = k.R[0] * rx + k.R[1] * ry + k.R[2], ey = k.R[3] * rx + k.R[4] * ry + k.R[5];
         const float ez = k.R[6] * rx + k.R[7] * ry + k.R[8];
         const float d_ray = gtx * (v.R[0] * ex + v.R[1] * ey + v.R[2] * ez) +

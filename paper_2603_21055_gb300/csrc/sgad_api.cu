@@ -1,5 +1,6 @@
 // C ABI entry points (include/sgad.h): argument checks, the workspace layout, and the
 // launch sequence of each call. No device memory is allocated here.
+#include <cfloat>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -141,6 +142,8 @@ sgad_status build_scene(const sgad_ctx *ctx, const sgad_keyframe *kfs, int32_t n
         if (k.world_transform && k.learnable)
             return fail(SGAD_ERR_INVALID_ARG, "keyframe %d: a world transform is only allowed on a fixed keyframe", i);
         set_cam(k.cam, d.fx, d.fy, d.cx, d.cy, d.R, d.t);
+        d.inv_fx = std::fmin(1.0f / d.fx, FLT_MAX);
+        d.inv_fy = std::fmin(1.0f / d.fy, FLT_MAX);
         d.W = k.cam.width;
         d.H = k.cam.height;
         d.gbase = (uint32_t)ng;

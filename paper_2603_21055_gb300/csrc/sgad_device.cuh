@@ -32,6 +32,7 @@ struct KfDev {
     const float *xform;          // optional world transform of the centres (device 3x4), or null
     float *d_offset, *d_rgb, *d_logit, *d_scale;
     float fx, fy, cx, cy;
+    float inv_fx, inv_fy;        // rounded reciprocals (ray_slope)
     float R[9], t[3];            // cam -> world
     int32_t W, H;
     uint32_t gbase;              // global index of this keyframe's first Gaussian
