@@ -140,7 +140,7 @@ typedef struct {
  *     barrier. The forward walks only the entries whose alpha >= 1/255 box may touch the
  *     block (up to 2^24 Gaussians the lists carry that as a mask) and lists the ones that
  *     reached one of its pixels; the backward walks those, 32 per round; per (entry, pixel)
- *     pair it keeps two numbers in shared memory, and one lane per entry sums them
+ *     pair it keeps two numbers in shared memory, and two lanes per entry sum them
  *     (fwd_batch and bwd_batch do not apply).
  *   WARP_REDUCE: thread blocks walk the masked entries of a tile in batches of bwd_batch
  *     staged entries per block-wide barrier, evaluate each at all 32 pixels of a warp's

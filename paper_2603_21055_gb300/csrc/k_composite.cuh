@@ -26,22 +26,21 @@
 // is stable because alpha <= 0.99. Per (pixel, entry) it forms the gradient of the
 // colour, depth and alpha terms; the moments of the lane's pixels are summed in
 // registers, reduced over the warp with a reduce-scatter (two entries at a time) and
-// accumulated per staged Gaussian in shared memory. At the end of the batch each staging thread turns them into d mu, d s,
-// d opacity and d colour and adds them to the per-Gaussian accumulator with two 16-byte
-// vector atomics.
+// accumulated per staged Gaussian in shared memory. At the end of the batch each staging thread
+// turns them into d |D + delta| along the keyframe's ray, d s, d opacity and d colour and adds
+// them to the per-Gaussian accumulator with a 16-byte and an 8-byte vector atomic.
 //
 // A second backward, the pair-parallel variant further below (k_composite_bwdp), walks
 // only the pairs the forward marked as contributing and sums them with shared-memory
 // atomics; it is selectable (SGAD_BWD_PAIRS) but slower on the room workloads (same-
-// Gaussian atomic conflicts between neighbouring pixels), so the warp-reduced one above
-// is the default.
+// Gaussian atomic conflicts between neighbouring pixels) than the warp-reduced one above.
 //
 // A third backward, the warp-local one (k_composite_bwdl, the default) with a forward of its
 // own (k_composite_fwdl), has no block-wide barrier at all: every warp takes (tile, 8x4 pixel block) units from a queue and walks
 // only the entries its forward listed, 32 at a time. Each lane keeps its pixel's
 // reverse-walk state; per (entry, contributing pixel) it leaves two numbers in the warp's
-// shared memory (dL/dpower and the blend weight), and then one lane per entry sums its
-// pixels' moments and applies the chain rule. No (entry, lane) slot of a warp-wide
+// shared memory (dL/dpower and the blend weight), and then two lanes per entry sum its
+// pixels' moments and one applies the chain rule. No (entry, lane) slot of a warp-wide
 // reduction is spent on a pixel the entry does not reach.
 //
 // Work split (CompositeArgs): either one block per tile (blockIdx.x + tile0), or a
@@ -89,7 +88,7 @@ struct CompositeArgs {
     const uint32_t *order;        // persistent: heavy-first tile order; nullptr: one block per tile
     uint32_t *queue;              // persistent: next position in `order` (starts at 0)
     int32_t tile0;                // one block per tile: tile of block 0
-    int32_t n_launch_tiles;       // warp-local backward: tiles this launch covers (from
+    int32_t n_launch_tiles;       // warp-local passes: tiles this launch covers (from
                                   // tile0, or through `order` when it is set)
     // Contribution words (forward writes, pair-parallel backward reads; may be null):
     // for tile t, list chunk c (entries 32c .. 32c + 31) and forward thread i (its
@@ -421,15 +420,21 @@ constexpr int kFwdlThreads = 256;           // 8 independent warps per block
 #define SGAD_FWDL_MINBLOCKS 4
 #endif
 
-// With at most as many work units as the forward keeps warps resident (4 blocks of 8 on each
-// of 152 SMs) every unit has its warp at once, and a pass takes as long as its deepest unit:
-// a lone warp per scheduler took 350 cycles per step of two candidates and 1500 to 2000 to
-// stage a round. The instances for few units (FEW) have the registers of two blocks per SM:
-// the forward takes four candidates at once and loads a round ahead, the backward takes three
-// entries at once whatever the keyframes, and neither spills. Forward, with and without: 640
-// units 42 and 56 us, 2400: 54 and 64, 4800: 83 and 87, 9600: 140 and 140, 19200: 251 and
-// 239. Backward: 4386 units 105 and 116, 4800: 111 and 115, 9600: 201 and 189; with pose
-// gradients, whose sums spill most at three blocks, 9600: 174 and 189.
+// With few work units a pass takes as long as its deepest units: a lone warp per scheduler took
+// 350 cycles per step of two candidates and 1500 to 2000 to stage a round. The instances for few
+// units (FEW) have the registers of two blocks per SM: the forward takes four candidates at once
+// and loads a round ahead. Where the line lies is measured (the two blocks hold 2,432 warps, half
+// of it): what the lists are like matters as much as the number of units.
+// Forward with FEW and without, us: one 640x480 keyframe in its own view scaled to 640 units 22
+// and 26, 2400: 30 and 32, 3800: 44 and 44, 4704: 46 and 46, 6144: 58 and 54, 9600: 79 and 75;
+// deep lists (2 to 8 keyframes in smaller views) 640: 98 and 137, 2880: 175 and 228, 3800: 148
+// and 176, 4160: 190 and 227, 4520: 77 and 96, 8320: 316 and 316, 9600: 175 and 175.
+// Backward: 640: 43 and 43, 2400: 47 and 45, 3800: 68 and 61, 4704: 70 and 70, 6144: 93 and 82;
+// deep lists 640: 92 and 97, 2880: 184 and 199 (three of four keyframes fixed: 142 and 161),
+// 3800: 179 and 177 (121 and 127), 4160: 207 and 187 (144 and 145), 4520: 97 and 105.
+// Pose gradients, whose sums spill at three blocks per SM, take FEW up to twice the line: 640:
+// 44 and 47, 4704: 109 and 120, 6144: 136 and 130, 7776: 153 and 159, 9600: 184 and 192, 15200:
+// 257 and 262, 21600: 349 and 355; of two keyframes 6400: 151 and 152, 17328: 317 and 301.
 constexpr int kFewBlocks = 2;
 constexpr int kFewUnits = 4 * 8 * 152;
 
@@ -1392,58 +1397,41 @@ __global__ void __launch_bounds__(kPairThreads, 4) k_composite_bwdp(const __grid
 //   2. walk, 16 entries at a time: each lane visits its own entries, in order, recovers the
 //      transmittance by division, forms dL/dalpha from its suffix sums and stores
 //      (G = alpha dL/dalpha, zero at the alpha cap; w = alpha T) at [entry][pixel] of a
-//      zeroed 16 x 32 buffer;
-//   3. moments: the ten sums of an entry over the pixels (colour and depth: w times the
-//      pixel's image gradients; G times 1, x, y, x^2, xy, y^2 of the pixel relative to the
-//      block's centre) are two 16 x 32 by 32 x 8 products on the tensor cores. Each FP32
-//      operand enters as the sum of two TF32 numbers (split_tf32), the coordinates' monomials
-//      are exact, and the products accumulate in FP32;
-//   4. chain: lane j moves entry j's moments to its mean, applies the chain rule down to the
-//      depth along the keyframe's ray and adds the result with two vector atomics.
+//      16 x 32 buffer;
+//   3. moments: two lanes per entry, with half of the block's pixels each, sum over the pixels
+//      the entry reached, in FP32 (colour and depth: w times the pixel's image gradients; G
+//      times 1, dx, dy, dx^2, dx dy, dy^2 of the pixel's offset from the mean);
+//   4. chain: lane j applies the chain rule to entry j's moments down to the depth along the
+//      keyframe's ray and adds the result with a 16-byte and an 8-byte vector atomic.
 // A round's list words, entries and world records are loaded during the round before it.
-// Bound by issue (68 % of the slots at 24 warps per SM) and L1 wavefronts (70 %) together.
-// A lane takes three entries at once (two with fixed keyframes, whose rounds are one walk):
-// the alphas, reciprocals and colour products of a step do not depend on one another.
-// Room workload (8 x 640x480, 130 M contributing pairs): 1.29 ms (one entry at once 1.34, two
-// 1.33, four 1.35; 5 x 1200x680 with four of five keyframes fixed: 1.48, 1.38 and with three
-// 1.41) against 1.56 ms with box
-// masks, candidates that miss and one lane per entry summing its pixels (a loop as long as
-// the entry with the most, 21.5 against a mean of 7.5). Of the 1.34 (parts left out in copies)
-// the walk takes 0.56, the moments 0.41, the chain rule 0.12 and staging, masks and loads 0.35.
-// 4 blocks per SM (64 registers): 1.37 ms, 2: 1.64; the rounds loaded when needed: +0.04.
+// A lane takes three entries at once (two with fixed keyframes, whose rounds are one walk): the
+// alphas, reciprocals and colour products of a step do not depend on one another (5 x 1200x680
+// with four of five keyframes fixed: three 1.285 ms, two 1.275).
+// Room workload (8 x 640x480, 130 M contributing pairs): 1.28 ms, against 1.56 with box masks,
+// candidates that miss and one lane per entry summing its pixels (a loop as long as the entry
+// with the most, 21.5 against a mean of 7.5). The moments as products on the tensor cores:
+// operands as two TF32 numbers 1.29 ms (22 bits: the sums were 2.5 to 5 times as far from 64
+// bits as FP32's), as three BF16 numbers (exact) 1.49. Where one keyframe fills its own view and
+// entries reach many pixels, the TF32 products took 5 to 10 % less (111 us against 117 at one
+// 640x480 view), elsewhere up to 11 % more.
+// 8,000 bytes of shared memory per warp leave the L1 60 KB beside three blocks; rows of pairs of
+// 36 instead of 34 entries cross the next step of the split (+4 us).
 constexpr int kLocalThreads = 256;          // 8 independent warps per block
-constexpr int kHalf = 16;                   // entries per walk and product
-constexpr int kPairStride = 36;             // float2 per entry row: 32 pixels, conflict-free fragments
+constexpr int kHalf = 16;                   // entries per walk, two lanes each for their moments
+constexpr int kPairStride = 34;             // float2 per entry row: 32 pixels, and two for the banks
 #ifndef SGAD_BWDL_MINBLOCKS
 #define SGAD_BWDL_MINBLOCKS 3
 #endif
 
 struct BwdlWarpSmem {
     WalkEntry e[32];                        // the round's entries
-    float2 pairs[kHalf][kPairStride];       // (G, w) per entry and pixel
-    float mom[32][12];                      // ten moments per entry
+    float2 pairs[kHalf][kPairStride];       // (G, w) per entry and pixel it reached
+    float mom[32][10];                      // moments per entry
+    float4 grad[32];                        // image gradients (colour, depth) of the block's pixels
+    float2 at[32];                          // their coordinates
+    uint32_t src[kHalf];                    // FIXED: lane of the entry of a row of pairs
 };
 constexpr size_t kLocalSmemBytes = (kLocalThreads / 32) * sizeof(BwdlWarpSmem);
-
-// x as the sum of two TF32 operands: x itself, of which the product takes the leading 11
-// bits, and the rest (13 bits, of which it takes 11). Rounding both (two integer operations
-// more) measured the same gradient errors against FP64 (median 1.3e-5 relative on three
-// windows, from the FP32 means, as without tensor cores) and 2 % of the kernel's time; the
-// conversion instruction, at a fraction of the others' rate, 8 %.
-__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo)
-{
-    hi = __float_as_uint(x);
-    lo = __float_as_uint(x - __uint_as_float(hi & 0xffffe000u));
-}
-
-// D += A B for a 16 x 8 (row-major) and an 8 x 8 (column-major) TF32 fragment.
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 __device__ __forceinline__ float reciprocal_walk(float x)     // x in [0.01, 1]
 {
@@ -1452,83 +1440,48 @@ __device__ __forceinline__ float reciprocal_walk(float x)     // x in [0.01, 1]
     return r;
 }
 
-// Fragment B of the colour and depth product: rows (pixels) 8 s + t and 8 s + t + 4, column
-// g = lane / 4 (t = lane % 4): the image gradients' high parts in columns 0 .. 3, their low
-// parts in 4 .. 7.
-struct GradFrags {
-    uint32_t b[4][2];
-};
-
-// Moments of the sixteen rows of S.pairs into rows h .. h + 15 of S.mom. Whole warp.
-__device__ __forceinline__ void bwdl_moments(BwdlWarpSmem &S, int h, int lane, const GradFrags &gf)
+// Moments of the entries of the rows of S.pairs into rows h .. h + 15 of S.mom, in FP32 about the
+// entry's mean. Two lanes per entry, with half of the block's pixels each: mean is the entry's
+// mean, reached the pixels it reached. Whole warp.
+__device__ __forceinline__ void bwdl_moments(BwdlWarpSmem &S, int h, int lane, float2 mean, uint32_t reached)
 {
-    const int g = lane >> 2, t = lane & 3;
-    float dw[4] = {0.f, 0.f, 0.f, 0.f}, dg[4] = {0.f, 0.f, 0.f, 0.f};
-    // column g of the monomials 1, x, y, x^2, x y, y^2 is al + be y + ga y^2 at the pixels
-    // x = t - 3.5 (row t) and x = t + 0.5 (row t + 4); y = s - 1.5
-    const float x0 = (float)t - 3.5f, x1 = (float)t + 0.5f;
-    const float ga = g == 5 ? 1.f : 0.f;
-    const float al0 = g == 0 ? 1.f : (g == 1 ? x0 : (g == 3 ? x0 * x0 : 0.f));
-    const float al1 = g == 0 ? 1.f : (g == 1 ? x1 : (g == 3 ? x1 * x1 : 0.f));
-    const float be0 = g == 2 ? 1.f : (g == 4 ? x0 : 0.f), be1 = g == 2 ? 1.f : (g == 4 ? x1 : 0.f);
+    const int e = lane & (kHalf - 1);
+    reached &= lane < kHalf ? 0xffffu : 0xffff0000u;
+    float A[10];
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const float y = (float)s - 1.5f;
-        const float2 v[4] = {S.pairs[g][8 * s + t], S.pairs[g + 8][8 * s + t], S.pairs[g][8 * s + t + 4],
-                             S.pairs[g + 8][8 * s + t + 4]};
-        uint32_t hi[4], lo[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) split_tf32(v[q].y, hi[q], lo[q]);
-        mma_tf32(dw, hi, gf.b[s][0], gf.b[s][1]);
-        mma_tf32(dw, lo, gf.b[s][0], gf.b[s][1]);
-        const uint32_t m0 = __float_as_uint(fmaf(y, fmaf(y, ga, be0), al0));
-        const uint32_t m1 = __float_as_uint(fmaf(y, fmaf(y, ga, be1), al1));
-#pragma unroll
-        for (int q = 0; q < 4; ++q) split_tf32(v[q].x, hi[q], lo[q]);
-        mma_tf32(dg, hi, m0, m1);
-        mma_tf32(dg, lo, m0, m1);
+    for (int q = 0; q < 10; ++q) A[q] = 0.f;
+    while (reached) {
+        const int p = 31 - __clz(reached);
+        reached ^= 1u << p;
+        const float2 gw = S.pairs[e][p];
+        const float4 pg = S.grad[p];
+        const float2 pq = S.at[p];
+        const float dx = __fsub_rn(mean.x, pq.x), dy = __fsub_rn(mean.y, pq.y);
+        A[0] += gw.y * pg.x;
+        A[1] += gw.y * pg.y;
+        A[2] += gw.y * pg.z;
+        A[3] += gw.y * pg.w;
+        const float G = gw.x;
+        A[4] += G;
+        A[5] += G * dx;
+        A[6] += G * dy;
+        A[7] += G * dx * dx;
+        A[8] += G * dx * dy;
+        A[9] += G * dy * dy;
     }
-    // columns 2 t, 2 t + 1 of rows g and g + 8; the low parts' columns join the high parts'
 #pragma unroll
-    for (int q = 0; q < 4; ++q) dw[q] += __shfl_xor_sync(kFull, dw[q], 2);
-    float *r0 = S.mom[h + g], *r1 = S.mom[h + g + 8];
-    if (t < 2) {
-        *reinterpret_cast<float2 *>(r0 + 2 * t) = make_float2(dw[0], dw[1]);
-        *reinterpret_cast<float2 *>(r1 + 2 * t) = make_float2(dw[2], dw[3]);
-    }
-    if (t < 3) {
-        *reinterpret_cast<float2 *>(r0 + 4 + 2 * t) = make_float2(dg[0], dg[1]);
-        *reinterpret_cast<float2 *>(r1 + 4 + 2 * t) = make_float2(dg[2], dg[3]);
-    }
-}
-
-// Colour and depth moments of the pixels left out of the product: w times the gradients for
-// the entries that contributed there (mine: the lane's own), in FP32. Whole warp; slot: the
-// lane's entry's row of S.pairs, -1 for none in this product.
-static __device__ __noinline__ void add_not_finite(BwdlWarpSmem &S, int h, int slot, uint32_t bad, uint32_t mine,
-                                                   float gr, float gg, float gb, float gD)
-{
-    const int lane = threadIdx.x & 31;
-    while (bad) {
-        const int p = __ffs(bad) - 1;
-        bad &= bad - 1u;
-        const uint32_t theirs = __shfl_sync(kFull, mine, p);
-        const float g[4] = {__shfl_sync(kFull, gr, p), __shfl_sync(kFull, gg, p), __shfl_sync(kFull, gb, p),
-                            __shfl_sync(kFull, gD, p)};
-        if (slot >= 0 && (theirs >> lane & 1u)) {
+    for (int q = 0; q < 10; ++q) A[q] += __shfl_xor_sync(kFull, A[q], kHalf);
+    if (lane < kHalf) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) S.mom[h + slot][c] += S.pairs[slot][p].y * g[c];
-        }
+        for (int q = 0; q < 10; q += 2) *reinterpret_cast<float2 *>(&S.mom[h + e][q]) = make_float2(A[q], A[q + 1]);
     }
-    __syncwarp();
 }
 
 // FIXED: some keyframe is fixed. Its entries are walked (they take part in the pixels'
-// transmittance and suffix sums) but have no moments, unless the view's pose wants them: a
-// round whose other entries are at most 16 is one walk and one product, and nothing is added
-// for the fixed ones. 5 x 1200x680 with four of five keyframes fixed: 1.38 ms against 1.92
-// with all entries' moments (2.23 before the products). Without a fixed keyframe its checks
-// cost 45 us of 1.34 ms, so that case has its own instance.
+// transmittance and suffix sums) but have no moments: a round whose other entries are at most 16
+// is one walk, and nothing is added for the fixed ones. 5 x 1200x680 with four of five keyframes
+// fixed: 1.28 ms (all entries' moments, when those were products: 1.92 against 1.38). Pose
+// gradients need every entry's moments, so POSE takes the instances without FIXED.
 template <int TW, int TH, bool POSE, bool PLAIN, bool FIXED, bool FEW>
 __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &a, int tile, int wb, BwdlWarpSmem &S,
                                           int lane)
@@ -1565,33 +1518,9 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
         if (v.g_depth) gD = v.g_depth[q];
         if (v.g_alpha) gA = v.g_alpha[q];
     }
-    // the image gradients as fragments, through the moment rows
-    // (a pixel with a gradient that is not finite stays out of the product, where it would
-    // reach every entry of a round as 0 x inf; see add_not_finite)
-    GradFrags gf;
-    const bool fine = fabsf(gr) < 1e38f && fabsf(gg) < 1e38f && fabsf(gb) < 1e38f && fabsf(gD) < 1e38f;
-    const uint32_t bad = ~__ballot_sync(kFull, fine);
     __syncwarp();                       // the previous unit's readers of S are done
-    {
-        uint32_t hi[4], lo[4];
-        split_tf32(fine ? gr : 0.f, hi[0], lo[0]);
-        split_tf32(fine ? gg : 0.f, hi[1], lo[1]);
-        split_tf32(fine ? gb : 0.f, hi[2], lo[2]);
-        split_tf32(fine ? gD : 0.f, hi[3], lo[3]);
-        uint32_t *row = reinterpret_cast<uint32_t *>(S.mom[lane]);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            row[c] = hi[c];
-            row[4 + c] = lo[c];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            gf.b[k][0] = __float_as_uint(S.mom[8 * k + (lane & 3)][lane >> 2]);
-            gf.b[k][1] = __float_as_uint(S.mom[8 * k + (lane & 3) + 4][lane >> 2]);
-        }
-        __syncwarp();                   // read before a first round without masks stores positions there
-    }
+    S.grad[lane] = make_float4(gr, gg, gb, gD);
+    S.at[lane] = make_float2(qx, qy);
     const float bgdot = sc.bg[0] * gr + sc.bg[1] * gg + sc.bg[2] * gb;
     // Reverse-walk state: transmittance, and the suffix sums of colour and depth behind
     // the current entry already dotted with this pixel's image gradients (Sg = S_C . g_C
@@ -1649,9 +1578,10 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
             }
             __syncwarp();
         }
+        const uint32_t reached = masked ? my_mask : warp_transpose32(mine, lane);   // by the lane's entry
         // the entries with moments, and the walks: 16 entries, or all with at most 16 moments
         const int kf = FIXED ? find_kf(sc, my_g) : 0;
-        const bool own = lane < n && (!FIXED || POSE || sc.kf[kf].learnable);
+        const bool own = lane < n && (!FIXED || sc.kf[kf].learnable);
         const uint32_t with = FIXED ? __ballot_sync(kFull, own) : 0u;
         const int span = FIXED && __popc(with) <= kHalf ? 32 : kHalf;
         int my_row = lane;                             // this lane's entry's row of S.mom
@@ -1659,12 +1589,6 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
 #pragma unroll 1
         for (int h = 0; h < n; h += span) {
             // 2. walk the entries h .. h + span - 1
-#pragma unroll
-            for (int k = 0; k < kHalf * 32 / 64; ++k) {
-                const int q = lane + 32 * k;             // 16 float4 per row
-                *reinterpret_cast<float4 *>(&S.pairs[q >> 4][2 * (q & 15)]) = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            __syncwarp();
             const uint32_t range = span == 32 ? kFull : 0xffffu << h;
             uint32_t todo = mine & range;
             while (__any_sync(kFull, todo != 0u)) {
@@ -1710,12 +1634,23 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
             __syncwarp();
             // 3. their moments
             if (!FIXED || (with & range)) {
-                bwdl_moments(S, h, lane, gf);
+                int from = h + (lane & (kHalf - 1));
+                uint32_t on = kFull;
+                if (FIXED) {
+                    const int slot = __popc(with & range & lane_mask_lt(lane));
+                    if (own && (range >> lane & 1u)) {
+                        S.src[slot] = (uint32_t)lane;
+                        my_row = h + slot;
+                    }
+                    __syncwarp();
+                    const bool some = (lane & (kHalf - 1)) < __popc(with & range);
+                    from = some ? (int)S.src[lane & (kHalf - 1)] : 0;
+                    on = some ? kFull : 0u;
+                }
+                const float4 ea = S.e[from].a;
+                const uint32_t theirs = __shfl_sync(kFull, reached, from) & on;
+                bwdl_moments(S, h, lane, make_float2(ea.x, ea.y), theirs);
                 __syncwarp();
-                const bool here = FIXED ? own && (range >> lane & 1u) : lane >= h && lane < h + kHalf;
-                const int slot = FIXED ? __popc(with & range & lane_mask_lt(lane)) : lane - h;
-                if (FIXED && here) my_row = h + slot;
-                if (bad) add_not_finite(S, h, here ? slot : -1, bad, mine, gr, gg, gb, gD);
             }
             if (h == 0) ent = left - 1 - lane >= 0 ? ents[pos] : 0ull;
         }
@@ -1728,16 +1663,10 @@ __device__ __forceinline__ void bwdl_unit(const Scene &sc, const CompositeArgs &
             st.b = make_float4(-2.f * ea.z, eb.x, -2.f * ea.w, eb.y);
             float A[10];
 #pragma unroll
-            for (int q = 0; q < 10; ++q) A[q] = S.mom[my_row][q];
-            // sums over the offsets (dx, dy) = (X, Y) - (x, y) of the pixels from the mean
-            const float X = ea.x - (bxf + 3.5f), Y = ea.y - (byf + 1.5f);
-            const float S0 = A[4], Sx = A[5], Sy = A[6];
-            const float Gx = fmaf(X, S0, -Sx), Gy = fmaf(Y, S0, -Sy);
-            A[7] = fmaf(X, Gx - Sx, A[7]);                               // X^2 S0 - 2 X Sx + Sxx
-            A[8] = fmaf(X, Gy, fmaf(-Y, Sx, A[8]));                      // X Y S0 - X Sy - Y Sx + Sxy
-            A[9] = fmaf(Y, Gy - Sy, A[9]);
-            A[5] = Gx;
-            A[6] = Gy;
+            for (int q = 0; q < 10; q += 2) {
+                const float2 m = *reinterpret_cast<const float2 *>(&S.mom[my_row][q]);
+                A[q] = m.x, A[q + 1] = m.y;
+            }
             const float3 gt = chain_and_accumulate(A, st, project_chain(my_w0, v), my_w0.w, sc.kf[FIXED ? kf : find_kf(sc, my_g)], v, a.gacc,
                                                    my_g);
             if (POSE) {
@@ -1883,11 +1812,11 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
         const void *all[] = {(const void *)k_composite_bwdl<TW, TH, false, false, true, false>,
                              (const void *)k_composite_bwdl<TW, TH, false, true, false, false>,
                              (const void *)k_composite_bwdl<TW, TH, false, true, true, false>,
-                             (const void *)k_composite_bwdl<TW, TH, true, false, true, false>,
+                             (const void *)k_composite_bwdl<TW, TH, true, false, false, false>,
                              (const void *)k_composite_bwdl<TW, TH, false, false, true, true>,
                              (const void *)k_composite_bwdl<TW, TH, false, true, false, true>,
                              (const void *)k_composite_bwdl<TW, TH, false, true, true, true>,
-                             (const void *)k_composite_bwdl<TW, TH, true, false, true, true>};
+                             (const void *)k_composite_bwdl<TW, TH, true, false, false, true>};
         for (const void *f : all)
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmemBytes);
@@ -1905,7 +1834,7 @@ cudaError_t launch_bwdl(const Scene &sc, const CompositeArgs &a, int grid_blocks
     const auto run = [&](auto few) {
         constexpr bool kFew = decltype(few)::value;
         if (a.pose)
-            launch_after(k_composite_bwdl<TW, TH, true, false, true, kFew>, grid_blocks, kLocalThreads,
+            launch_after(k_composite_bwdl<TW, TH, true, false, false, kFew>, grid_blocks, kLocalThreads,
                          kLocalSmemBytes, st, sc, a);
         else if (!plain)
             launch_after(k_composite_bwdl<TW, TH, false, false, true, kFew>, grid_blocks, kLocalThreads,
