@@ -694,12 +694,11 @@ __global__ void __launch_bounds__(192, 2) k_conv3x3_wgrad_tma(const __grid_const
 
 // Both gradients of a layer (CI channels in, CO out) side by side: the first n_conv blocks the
 // input gradient, the others the weight gradient. Each is a chain of latencies at small sizes
-// and leaves bandwidth at large ones: the net's backward of 3 x 315x237 takes 105 us against 126
-// with a launch each, of 4 x 640x480 283 against 299, of 8 x 640x480 531 against 522. Half of the
-// blocks each (three or five eighths for the weight gradient, with one sum per block: 514 and 531
-// us at 8 x 640x480 against 459). Small problems give the weight gradient a block per 8 to 12 K
-// blocks (8 with few: 54 us against 61 at 1 x 315x237, 12 at 3 x 315x237: 90 against 95), whose
-// final additions meet on the same addresses.
+// and leaves bandwidth at large ones: the net's backward of 1 x 315x237 takes 71 us against 76
+// with a launch each, of 3 x 315x237 106 against 131, of 2 x 640x480 162 against 183, of 4 x
+// 640x480 284 against 309, of 8 x 640x480 533 against 545, of 8 x 1200x680 1455 against 1445. At
+// most half of the blocks for the weight gradient (three eighths 314 us at 4 x 640x480 and 588 at
+// 8, five eighths 291 and 542), and one per 8 K blocks (one per 12: 81 us at 1 x 315x237).
 constexpr int kPairStages = 2;             // load stages of the weight gradient: three blocks fit an SM
 constexpr int kPairBlocks = 3;
 template <int CI, int CO>
@@ -869,8 +868,7 @@ cudaError_t launch_grads(const ConvArgs &c, WgradArgs w, cudaStream_t st)
     if (e != cudaSuccess) return e;
     // (tiles and K blocks are the same in number)
     const int room = kPairBlocks * sms;
-    const int n_wgrad = (int)std::min<long long>({std::max<long long>(1, tiles / kWgTiles),
-                                                  std::max<long long>(128, tiles / 12), room / 2});
+    const int n_wgrad = (int)std::min<long long>(std::max<long long>(1, tiles / kWgTiles), room / 2);
     const int n_conv = (int)std::min<long long>(tiles, room - n_wgrad);
     w.chain = sum_chain(tiles, sms);
     return launch_after(k_conv3x3_grads<CI, CO>, n_conv + n_wgrad, 192, smem, st, xm, wide, halo, c, w, n_conv);
