@@ -516,7 +516,6 @@ struct FwdlWarpSmem {
     WalkEntry e[32];                // the round's entries
     uint32_t pos[kRing];            // ring: list positions of entries that may touch the block
 };
-constexpr size_t kFwdlSmemBytes = (kFwdlThreads / 32) * sizeof(FwdlWarpSmem);
 
 // Whether the alpha >= 1/255 box of a Gaussian (world record w0, opacity o) may touch the
 // pixels [bx, bx + 7] x [by, by + 3]. Never false when the exact box (stage()) does: the

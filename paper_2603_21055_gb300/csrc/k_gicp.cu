@@ -722,7 +722,6 @@ struct StepArgs {
     const float4 *spos, *scov;
     const int32_t *scount;
     const float4 *mpos, *mcov, *mnorm;
-    const int32_t *mcount;
     Grid grid;
     float r_max;
     int32_t kmatch;
@@ -1405,7 +1404,6 @@ StepArgs step_args(const sgad_gicp_params *p, const sgad_gaussian_set *src, cons
     a.mpos = reinterpret_cast<const float4 *>(map->pos);
     a.mcov = reinterpret_cast<const float4 *>(map->cov);
     a.mnorm = reinterpret_cast<const float4 *>(map->normal);
-    a.mcount = map->count;
     a.grid = grid_of(p, ws, L);
     a.r_max = p->r_max;
     a.kmatch = p->k_match;
