@@ -96,8 +96,8 @@ sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_camera *cam, c
                             const sgad_gaussian_set *out, int32_t *pix_out, int32_t *knn_out, void *workspace,
                             size_t ws_bytes, void *stream);
 
-/* The map's spatial hash grid (cells of max(r_max, d_overlap) / 2; searches visit rings
- * of cells until their result is proven). Required after the caller changes the map;
+/* The map's spatial hash grid (cells of a half to a sixth of max(r_max, d_overlap), by the
+ * map's density; searches visit rings of cells until their result is proven). Required after the caller changes the map;
  * sgad_gicp_insert rebuilds it itself. */
 sgad_status sgad_gicp_index(const sgad_gicp_params *p, const sgad_gaussian_set *map, void *workspace,
                             size_t ws_bytes, void *stream);

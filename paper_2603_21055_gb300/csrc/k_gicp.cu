@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstring>
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "sgad_gicp.h"
@@ -47,6 +48,7 @@ struct GicpState {
     int32_t gave_up;         // 1: a wait of the last track ended without the others. A word of its own,
                              // which the next frame does not clear: a caller may read the state of a
                              // track while the next frame is selected
+    int32_t level;           // cell size of the map's index (see kLevels); the next build starts with it
 };
 
 struct GLayout {
@@ -81,7 +83,7 @@ GLayout glayout(const sgad_gicp_params &p)
     };
     L.state = take(sizeof(GicpState));
     L.sel_counts = take((size_t)kMaxSelBlocks * sizeof(int32_t));
-    L.hash_head = take((size_t)L.table * sizeof(int32_t));
+    L.hash_head = take(((size_t)L.table + 1) * sizeof(int32_t));      // and the occupied buckets
     L.hash_pts = take((size_t)p.map_capacity * sizeof(float4));
     L.knn_head = take((size_t)L.knn_table * sizeof(int32_t));
     L.knn_pts = take((size_t)p.src_capacity * sizeof(float4));
@@ -336,13 +338,47 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr uint64_t kNone = ~0ull;
 constexpr int kRings = 6;                // rings searched before the exhaustive pass
 
+// Cell sizes of the map's index: half to a sixth of the larger search radius R, so that as many
+// rings of cells as kDivisor prove a search of that radius. Half of it where a cell holds few
+// points (cells of a third took 343 to reach as far, most of them empty at the 2-8 cm spacing of
+// most maps' points). A chain is walked by one lane, so of a dense map, whose searches end in
+// the first ring, smaller cells are linked (k_hash_relink). 640x480 frames at R = 0.1 m, a
+// sequence's time per frame with cells of R / 2 alone and with these: stride 1 (307,200 points,
+// 190 in a cell of R / 2) 64 and 24 ms, stride 2 at R = 0.3 23.6 and 4.7, stride 3 at 0.3 3.5 and
+// 1.6, stride 5 at 0.6 1.20 and 0.50, stride 10 0.28 and 0.27.
+constexpr int kLevels = 4;
+__device__ constexpr int kDivisor[kLevels] = {2, 3, 4, 6};
+constexpr int kMaxRings = 6;
+
 struct Grid {
     const int32_t *head;      // [table] first point of a bucket's chain + 1, 0: empty
     const float4 *pts;        // [cap] x, y, z, next point of the chain + 1 (bits)
     float inv_cell, cell;
     uint32_t mask;
     int32_t cap;
+    int32_t divisor;          // of the map's index
 };
+
+// The map's index as the last build left it: level 0's grid and the cells of every level.
+struct MapGrid {
+    Grid g;
+    float cell[kLevels], inv_cell[kLevels];
+};
+
+__device__ __forceinline__ int valid_level(int l) { return l >= 0 && l < kLevels ? l : 0; }
+
+__device__ __forceinline__ Grid grid_at(const MapGrid &m, int level)
+{
+    Grid g = m.g;
+#pragma unroll
+    for (int l = 1; l < kLevels; ++l)
+        if (level == l) {
+            g.cell = m.cell[l];
+            g.inv_cell = m.inv_cell[l];
+            g.divisor = kDivisor[l];
+        }
+    return g;
+}
 
 __device__ __forceinline__ uint64_t pack_key(float d, int j)
 {
@@ -698,23 +734,65 @@ __global__ void __launch_bounds__(kShapeThreads) k_shape(const __grid_constant__
 }
 
 // ------------------------------------------------------------------ hash grid
-// Links every point into its bucket's chain (any order: a search's result does not depend
-// on it). The chains replace a counting sort of the buckets (a count, three scans and a
-// fill). `commit`: the points are the map after an update, whose count becomes
-// min(old + inserted, capacity).
-__global__ void __launch_bounds__(256) k_hash_link(const float4 *pos, int32_t *count, int32_t cap, float inv_cell,
-                                                   uint32_t mask, int32_t *head, float4 *pts,
-                                                   const GicpState *commit)
+// Links points into their buckets' chains (any order: a search's result does not depend on it).
+// The chains replace a counting sort of the buckets (a count, three scans and a fill). Returns
+// how many buckets the thread was the first of.
+__device__ __forceinline__ int link_points(const float4 *pos, int n, const Grid &g, int32_t *head, float4 *pts, int first,
+                                           int step)
 {
-    sgad::dependency_wait();
-    const int n = min(commit ? commit->map_old + commit->ins_total : *count, cap);
-    if (commit && blockIdx.x == 0 && threadIdx.x == 0) *count = n;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    int fresh = 0;
+    for (int i = first; i < n; i += step) {
         const float4 p = pos[i];
-        const uint32_t h = cell_hash(cell_of(p.x, inv_cell), cell_of(p.y, inv_cell), cell_of(p.z, inv_cell), mask);
+        const uint32_t h = cell_hash(cell_of(p.x, g.inv_cell), cell_of(p.y, g.inv_cell), cell_of(p.z, g.inv_cell), g.mask);
         const int next = atomicExch(&head[h], i + 1);
         pts[i] = make_float4(p.x, p.y, p.z, __int_as_float(next));
+        fresh += next == 0 ? 1 : 0;
     }
+    return fresh;
+}
+
+// state: the points are the map, linked at the level of its last build, and the occupied buckets
+// are counted after the last head; commit: the map after an update, whose count becomes
+// min(old + inserted, capacity).
+__global__ void __launch_bounds__(256) k_hash_link(const float4 *pos, int32_t *count, int32_t cap,
+                                                   const __grid_constant__ MapGrid m, int32_t *head, float4 *pts,
+                                                   const GicpState *state, int commit)
+{
+    sgad::dependency_wait();
+    const int n = min(commit ? state->map_old + state->ins_total : *count, cap);
+    if (commit && blockIdx.x == 0 && threadIdx.x == 0) *count = n;
+    const Grid g = grid_at(m, state ? valid_level(state->level) : 0);
+    const int fresh = __reduce_add_sync(
+        kFull, link_points(pos, n, g, head, pts, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x));
+    if (state && fresh && (threadIdx.x & 31) == 0) atomicAdd(&head[g.mask + 1u], fresh);
+}
+
+// Links the map again where its density does not suit the level: longer chains than kLongChain
+// points, or shorter than kShortChain at a small cell. One cluster, which has nothing to do
+// otherwise (a surface's points per cell go with the square of the cell's size, so a new level's
+// chains lie between the two and it stays).
+constexpr int kLongChain = 24, kShortChain = 4;
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(1024)
+    k_hash_relink(const float4 *pos, const int32_t *count, int32_t cap, const __grid_constant__ MapGrid m, int32_t *head,
+                  float4 *pts, GicpState *state)
+{
+    sgad::dependency_wait();
+    const int n = min(*count, cap), level = valid_level(state->level);
+    const float chain = (float)n / (float)max(head[m.g.mask + 1u], 1);
+    if (!(chain > (float)kLongChain && level < kLevels - 1) && !(chain < (float)kShortChain && level > 0)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) state->level = level;
+        return;
+    }
+    const float d = 0.5f * (float)kDivisor[level], coarse = chain * d * d;    // points per cell of half the radius
+    const int want = coarse < 16.f ? 0 : (coarse < 32.f ? 1 : (coarse < 64.f ? 2 : 3));
+    const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();                                            // every block has read the level and the counts
+    if (first == 0) state->level = want;
+    for (uint32_t i = first; i <= m.g.mask; i += step) head[i] = 0;
+    __threadfence();
+    cluster.sync();
+    link_points(pos, n, grid_at(m, want), head, pts, first, step);
 }
 
 // ------------------------------------------------------------------ Gauss-Newton step
@@ -722,7 +800,7 @@ struct StepArgs {
     const float4 *spos, *scov;
     const int32_t *scount;
     const float4 *mpos, *mcov, *mnorm;
-    Grid grid;
+    MapGrid grid;
     float r_max;
     int32_t kmatch;
     int32_t system;          // accumulate the Gauss-Newton system
@@ -807,7 +885,8 @@ constexpr float kMargin = 1.f - 1e-4f;
 // move of `slack` (0.3 of a cell, 1.5 cm at the default radius: with half of that, single
 // points outran theirs in each of the next ten iterations, and one search delays the
 // iteration of all by 10-15 us).
-__device__ __forceinline__ int match_point(const StepArgs &a, float3 x, Kept *kept, bool first, uint64_t *buf)
+__device__ __forceinline__ int match_point(const StepArgs &a, const Grid &grid, float3 x, Kept *kept, bool first,
+                                           uint64_t *buf)
 {
     const int lane = threadIdx.x & 31;
     const int K = a.kmatch;
@@ -837,14 +916,14 @@ __device__ __forceinline__ int match_point(const StepArgs &a, float3 x, Kept *ke
     }
     if (!ok) {
         const bool keep = kept && !first;
-        const float slack = 0.3f * a.grid.cell;
+        const float slack = 0.3f * a.grid.cell[0];
         uint64_t best = kNone;
         float rho = 0.f;
-        // rings of cells of half of r_max or more: two prove any result
+        // as many rings as the cells' divisor prove any result
 #pragma unroll 1
-        for (int r = 1; r <= 3; ++r) {
-            search_ring(a.grid, x, r, keep ? 32 : K, best, buf);
-            const float reach = (float)r * a.grid.cell * (1.f - 1e-4f);
+        for (int r = 1; r <= min(grid.divisor + 1, kMaxRings); ++r) {
+            search_ring(grid, x, r, keep ? 32 : K, best, buf);
+            const float reach = (float)r * grid.cell * (1.f - 1e-4f);
             const uint64_t kth = __shfl_sync(kFull, best, K - 1), end = __shfl_sync(kFull, best, 31);
             const bool have = kth != kNone && key_dist(kth) <= r2;
             const bool proven = reach >= a.r_max || (kth != kNone && key_dist(kth) < reach * reach);
@@ -857,7 +936,7 @@ __device__ __forceinline__ int match_point(const StepArgs &a, float3 x, Kept *ke
         j = best != kNone ? (int)(uint32_t)best : -1;
         member = lane < K && j >= 0 && d <= r2;
         if (keep ? j >= 0 : member) {
-            q = a.grid.pts[j];
+            q = grid.pts[j];
             const float4 nr = a.mnorm[j];
             nx = nr.x;
             ny = nr.y;
@@ -939,6 +1018,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_gicp_step(const __grid_cons
     const int n = *a.scount;
     const int used = rows_used(n, a.rows);
     const uint32_t epoch = TRACK && threadIdx.x == 0 ? ld_acquire(&a.state->sync) : 0u;
+    const Grid grid = grid_at(a.grid, valid_level(a.state->level));
 #pragma unroll 1
     for (uint32_t it = 0;; ++it) {
         if (threadIdx.x < 12) s_pose[threadIdx.x] = TRACK ? __ldcg(&a.state->posef[threadIdx.x]) : a.pose.p[threadIdx.x];
@@ -966,7 +1046,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_gicp_step(const __grid_cons
                                 kept->x0 = make_float4(0.f, 0.f, 0.f, 0.f);
                             }
                         }
-                        j = match_point(a, transform(s_pose, src), kept, it == 0, s_buf[warp]);
+                        j = match_point(a, grid, transform(s_pose, src), kept, it == 0, s_buf[warp]);
                         if (!TRACK && a.idx_out && lane == 0) a.idx_out[i] = j;
                     }
                     if (lane == 0) s_match[b][warp] = j;
@@ -1217,7 +1297,7 @@ struct InsArgs {
     float4 *mpos, *mcov, *mnorm;
     int32_t *mcount;
     int32_t mcap;
-    Grid grid;
+    MapGrid grid;
     float d_ov;
     GicpState *state;
     int32_t *flags;
@@ -1232,12 +1312,21 @@ __device__ __forceinline__ bool overlaps(float3 x, const Grid &g, float d_ov)
     const auto near = [&](float4 b) {
         if (sqdist(b.x, b.y, b.z, x.x, x.y, x.z) <= d2ov) hit = true;
     };
-    // cells of half of max(r_max, d_ov) >= d_ov / 2: two rings reach d_ov
-    ring_cells<1, true>(g, x, near);
-    if (__any_sync(kFull, hit)) return true;
-    if (g.cell * (1.f - 1e-4f) >= d_ov) return false;
-    ring_cells<2, false>(g, x, near);
-    return __any_sync(kFull, hit);
+    // (as many rings as the cells' divisor reach d_ov)
+#pragma unroll 1
+    for (int r = 1; r <= kMaxRings; ++r) {
+        switch (r) {
+        case 1: ring_cells<1, true>(g, x, near); break;
+        case 2: ring_cells<2, false>(g, x, near); break;
+        case 3: ring_cells<3, false>(g, x, near); break;
+        case 4: ring_cells<4, false>(g, x, near); break;
+        case 5: ring_cells<5, false>(g, x, near); break;
+        default: ring_cells<6, false>(g, x, near); break;
+        }
+        if (__any_sync(kFull, hit)) return true;
+        if ((float)r * g.cell * (1.f - 1e-4f) >= d_ov) break;
+    }
+    return false;
 }
 
 // One warp per source point, kInsPts points per block: the search is a chain of dependent
@@ -1248,13 +1337,18 @@ __global__ void __launch_bounds__(1024) k_insert_flag(const __grid_constant__ In
     __shared__ int s_keep[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n = *a.scount;
+    if ((int)blockIdx.x * kInsPts >= n) {
+        if (threadIdx.x == 0) a.blk[blockIdx.x] = 0;
+        return;
+    }
     const bool empty = *a.mcount == 0;
+    const Grid grid = grid_at(a.grid, valid_level(a.state->level));
     int kept = 0;
 #pragma unroll 1
     for (int k = 0; k < kInsPts / 32; ++k) {
         const int i = blockIdx.x * kInsPts + k * 32 + warp;
         if (i >= n) break;
-        const bool keep = empty || !overlaps(transform(a.state->posef, a.spos[i]), a.grid, a.d_ov);
+        const bool keep = empty || !overlaps(transform(a.state->posef, a.spos[i]), grid, a.d_ov);
         if (lane == 0) a.flags[i] = keep ? 1 : 0;
         kept += keep ? 1 : 0;
     }
@@ -1349,22 +1443,22 @@ sgad_status check_ws(void *ws, size_t bytes, size_t need)
 template <typename T>
 T *at(void *ws, size_t off) { return reinterpret_cast<T *>(static_cast<char *>(ws) + off); }
 
-// Map grid cells of half the larger search radius: correspondence and overlap searches
-// visit rings of cells until their result is proven (at most 2 rings, 125 cells; cells of a
-// third took 343 to reach as far, most of them empty at the 2-8 cm spacing of a map's
-// points).
-float cell_size(const sgad_gicp_params *p) { return fmaxf(p->r_max, p->d_overlap) * (1.001f / 2.f); }
-
-Grid grid_of(const sgad_gicp_params *p, void *ws, const GLayout &L)
+MapGrid grid_of(const sgad_gicp_params *p, void *ws, const GLayout &L)
 {
-    Grid g;
-    g.head = at<int32_t>(ws, L.hash_head);
-    g.pts = at<float4>(ws, L.hash_pts);
-    g.cap = p->map_capacity;
-    g.cell = cell_size(p);
-    g.inv_cell = 1.f / g.cell;
-    g.mask = (uint32_t)L.table - 1u;
-    return g;
+    MapGrid m;
+    m.g.head = at<int32_t>(ws, L.hash_head);
+    m.g.pts = at<float4>(ws, L.hash_pts);
+    m.g.cap = p->map_capacity;
+    m.g.mask = (uint32_t)L.table - 1u;
+    m.g.divisor = 2;
+    const int divisor[kLevels] = {2, 3, 4, 6};
+    for (int l = 0; l < kLevels; ++l) {
+        m.cell[l] = fmaxf(p->r_max, p->d_overlap) * (1.001f / (float)divisor[l]);
+        m.inv_cell[l] = 1.f / m.cell[l];
+    }
+    m.g.cell = m.cell[0];
+    m.g.inv_cell = m.inv_cell[0];
+    return m;
 }
 
 sgad_status launched(const char *what)
@@ -1373,24 +1467,24 @@ sgad_status launched(const char *what)
     return e == cudaSuccess ? SGAD_OK : report_error(SGAD_ERR_CUDA, what);
 }
 
-// Index of a set: empty chains, then every point linked into its cell's chain. `commit`:
-// the map update's state, whose new count is written to *count (see k_hash_link).
-sgad_status hash_build(const float4 *pos, int32_t *count, int32_t capacity, float inv_cell, int32_t table,
-                       int32_t *head, float4 *pts, const GicpState *commit, cudaStream_t st)
+// Index of a set: empty chains, then every point linked into its cell's chain. state, commit:
+// the map's (see k_hash_link).
+sgad_status hash_build(const float4 *pos, int32_t *count, int32_t capacity, const MapGrid &m, int32_t *head,
+                       float4 *pts, GicpState *state, int commit, cudaStream_t st)
 {
-    if (cudaMemsetAsync(head, 0, (size_t)table * sizeof(int32_t), st) != cudaSuccess)
+    if (cudaMemsetAsync(head, 0, ((size_t)m.g.mask + (state ? 2 : 1)) * sizeof(int32_t), st) != cudaSuccess)
         return report_error(SGAD_ERR_CUDA, "sgad_gicp: memset failed");
     const int blocks = std::min((capacity + 255) / 256, 4 * 152);
-    sgad::launch_after(k_hash_link, blocks, 256, 0, st, pos, count, capacity, inv_cell, (uint32_t)table - 1u, head, pts,
-                       commit);
+    sgad::launch_after(k_hash_link, blocks, 256, 0, st, pos, count, capacity, m, head, pts, state, commit);
+    if (state) sgad::launch_after(k_hash_relink, 8, 1024, 0, st, pos, count, capacity, m, head, pts, state);
     return launched("sgad_gicp: index launch failed");
 }
 
 sgad_status build_index(const sgad_gicp_params *p, const sgad_gaussian_set *map, void *ws, const GLayout &L,
-                        const GicpState *commit, cudaStream_t st)
+                        int commit, cudaStream_t st)
 {
-    return hash_build(reinterpret_cast<const float4 *>(map->pos), map->count, map->capacity, 1.f / cell_size(p),
-                      L.table, at<int32_t>(ws, L.hash_head), at<float4>(ws, L.hash_pts), commit, st);
+    return hash_build(reinterpret_cast<const float4 *>(map->pos), map->count, map->capacity, grid_of(p, ws, L),
+                      at<int32_t>(ws, L.hash_head), at<float4>(ws, L.hash_pts), at<GicpState>(ws, L.state), commit, st);
 }
 
 StepArgs step_args(const sgad_gicp_params *p, const sgad_gaussian_set *src, const sgad_gaussian_set *map, void *ws,
@@ -1510,8 +1604,10 @@ extern "C" sgad_status sgad_gicp_frame(const sgad_gicp_params *p, const sgad_cam
         g.inv_cell = 1.f / g.cell;
         g.mask = (uint32_t)L.knn_table - 1u;
         g.cap = p->src_capacity;
-        if ((s = hash_build(sa.pos, out->count, out->capacity, g.inv_cell, L.knn_table,
-                            at<int32_t>(workspace, L.knn_head), at<float4>(workspace, L.knn_pts), nullptr, st)))
+        MapGrid m = {};
+        m.g = g;
+        if ((s = hash_build(sa.pos, out->count, out->capacity, m, at<int32_t>(workspace, L.knn_head),
+                            at<float4>(workspace, L.knn_pts), nullptr, 0, st)))
             return s;
         sgad::launch_after(k_shape<false>, sb, kShapeThreads, 0, st, sa);
     }
@@ -1526,7 +1622,7 @@ extern "C" sgad_status sgad_gicp_index(const sgad_gicp_params *p, const sgad_gau
     if ((s = check_set(map, p->map_capacity, "sgad_gicp_index: bad map set"))) return s;
     const GLayout L = glayout(*p);
     if ((s = check_ws(workspace, ws_bytes, L.total))) return s;
-    return build_index(p, map, workspace, L, nullptr, static_cast<cudaStream_t>(stream));
+    return build_index(p, map, workspace, L, 0, static_cast<cudaStream_t>(stream));
 }
 
 namespace {
@@ -1662,7 +1758,7 @@ extern "C" sgad_status sgad_gicp_insert(const sgad_gicp_params *p, const sgad_ga
     sgad::launch_after(k_insert_flag, (p->src_capacity + kInsPts - 1) / kInsPts, 1024, 0, st, a);
     sgad::launch_after(k_insert_write, L.max_blocks, 256, 0, st, a);
     if ((s = launched("sgad_gicp_insert: launch failed"))) return s;
-    return build_index(p, map, workspace, L, a.state, st);
+    return build_index(p, map, workspace, L, 1, st);
 }
 
 extern "C" sgad_status sgad_gicp_result(void *workspace, size_t ws_bytes, double pose[12], sgad_gicp_stats *stats,
