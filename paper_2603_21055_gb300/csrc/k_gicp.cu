@@ -800,6 +800,7 @@ struct StepArgs {
     const float4 *spos, *scov;
     const int32_t *scount;
     const float4 *mpos, *mcov, *mnorm;
+    const int32_t *mcount;
     MapGrid grid;
     float r_max;
     int32_t kmatch;
@@ -992,7 +993,16 @@ __device__ __forceinline__ void st_release(uint32_t *p, uint32_t v)
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-constexpr uint32_t kSyncSpins = 1u << 22;   // a wait on the other blocks gives up after a few seconds
+// A wait on the other blocks gives up after about a second, and later where a block's searches
+// may take longer: after four times as many tries more as a warp's searches may visit points (a
+// point of a chain takes 0.3 us, about a try). 16 points in a map of 4.2 M points in one cell take
+// 1.3 s an iteration.
+constexpr uint32_t kSyncSpins = 1u << 22;
+__device__ __forceinline__ uint32_t spin_limit(int n, int map, int blocks)
+{
+    const unsigned long long per_warp = ((unsigned)n + (unsigned)(blocks * kRowPts) - 1u) / (unsigned)(blocks * kRowPts);
+    return kSyncSpins + (uint32_t)min(4ull * per_warp * (unsigned)max(map, 0), 1ull << 31);
+}
 
 // Correspondences and partial sums of the Gauss-Newton system. A block takes rows of 16
 // points, one warp per point. TRACK: the whole of a track in one cooperative launch: after
@@ -1102,10 +1112,11 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_gicp_step(const __grid_cons
                 }
             }
         } else if (threadIdx.x == 0) {
+            const uint32_t limit = spin_limit(n, *a.mcount, (int)gridDim.x);
             uint32_t t = 0;
-            while (ld_acquire(&a.state->sync) != epoch + it + 1u && ++t < kSyncSpins) {
+            while (ld_acquire(&a.state->sync) != epoch + it + 1u && ++t < limit) {
             }
-            if (t >= kSyncSpins) {                             // recorded; the block ends
+            if (t >= limit) {                             // recorded; the block ends
                 a.state->gave_up = 1;
                 s_done = 1;
             } else {
@@ -1498,6 +1509,7 @@ StepArgs step_args(const sgad_gicp_params *p, const sgad_gaussian_set *src, cons
     a.mpos = reinterpret_cast<const float4 *>(map->pos);
     a.mcov = reinterpret_cast<const float4 *>(map->cov);
     a.mnorm = reinterpret_cast<const float4 *>(map->normal);
+    a.mcount = map->count;
     a.grid = grid_of(p, ws, L);
     a.r_max = p->r_max;
     a.kmatch = p->k_match;
