@@ -569,11 +569,39 @@ __device__ __forceinline__ float slope_gap(float d, float r, float a, float b)
     return d * fminf(fabsf(a) * rsqrtf(1.f + (r + a) * (r + a)), fabsf(b) * rsqrtf(1.f + (r + b) * (r + b)));
 }
 
+// Every point.
+__device__ __forceinline__ uint64_t all_nearest(const ShapeArgs &a, float4 me, int n, int K)
+{
+    const int lane = threadIdx.x & 31;
+    uint64_t best = kNone;
+    float4 next = lane < n ? a.pos[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int j = lane; j - lane < n; j += 32) {
+        const float4 q = next;
+        if (j + 32 < n) next = a.pos[j + 32];
+        uint64_t k = kNone;
+        if (j < n) {
+            const float d = sqdist(q.x, q.y, q.z, me.x, me.y, me.z);
+            if (d <= FLT_MAX) k = pack_key(d, j);
+        }
+        warp_insert(best, k, K);
+    }
+    return best;
+}
+
 // K nearest points by windows of the selection grid around the point's cell: the points
 // outside the window lie on rays at least one window edge away, so the search ends once the
 // K-th distance is below the smallest distance to such a ray. No hash grid is built (its
-// build was 6 launches) and a window's 25 cells are one step of the warp.
-__device__ __forceinline__ uint64_t window_nearest(const ShapeArgs &a, int i, float4 me, int K)
+// build was 6 launches) and a window's 25 cells are one step of the warp. A window that has grown
+// to twice as many cells as there are points gives way to a pass over the points, and where the
+// cells are so sparsely filled that it would (K points take K ncells / n cells of an even spread,
+// and two to three times as many to prove it) the pass is taken at once. 1 % of 640x480 pixels at
+// stride 1 valid, K = 10: 135 us (443 by windows alone, 728 by the hash grid of all points), 0.1 %
+// with K = 32: 42 (16,850 and 416); 10 % of 1200x680: 2.8 ms (4.2, 5.4; giving way at as many
+// cells as points 1.9, but at 3 % of 640x480 280 us instead of 183).
+constexpr float kSparse = 4.f;
+constexpr int kWindowMost = 2;
+__device__ __forceinline__ uint64_t window_nearest(const ShapeArgs &a, int i, float4 me, int n, int K)
 {
     const Window &w = a.w;
     const int lane = threadIdx.x & 31;
@@ -608,6 +636,7 @@ __device__ __forceinline__ uint64_t window_nearest(const ShapeArgs &a, int i, fl
         const uint64_t kth = __shfl_sync(kFull, best, K - 1);
         gap = gap * (1.f - 1e-4f) - off_ray;
         if (gap > 0.f && kth != kNone && key_dist(kth) < gap * gap) break;
+        if ((2 * m + 1) * (2 * m + 1) >= kWindowMost * n) return all_nearest(a, me, n, K);
         // the next frame of cells: 8 (m + 1) of them, side by side
         const int m1 = m + 1, edge = 2 * m1;
 #pragma unroll 1
@@ -625,7 +654,6 @@ __device__ __forceinline__ uint64_t window_nearest(const ShapeArgs &a, int i, fl
 // searched radius, else every point.
 __device__ __forceinline__ uint64_t hash_nearest(const ShapeArgs &a, float4 me, int n, int K, uint64_t *buf)
 {
-    const int lane = threadIdx.x & 31;
     const float3 x = make_float3(me.x, me.y, me.z);
     uint64_t best = kNone;
 #pragma unroll 1
@@ -635,19 +663,7 @@ __device__ __forceinline__ uint64_t hash_nearest(const ShapeArgs &a, float4 me, 
         const uint64_t kth = __shfl_sync(kFull, best, K - 1);
         if (kth != kNone && key_dist(kth) < reach * reach) return best;
     }
-    best = kNone;
-#pragma unroll 1
-    for (int j0 = 0; j0 < n; j0 += 32) {
-        const int j = j0 + lane;
-        uint64_t k = kNone;
-        if (j < n) {
-            const float4 q = a.pos[j];
-            const float d = sqdist(q.x, q.y, q.z, x.x, x.y, x.z);
-            if (d <= FLT_MAX) k = pack_key(d, j);
-        }
-        warp_insert(best, k, K);
-    }
-    return best;
+    return all_nearest(a, me, n, K);
 }
 
 template <bool WINDOW>
@@ -661,12 +677,15 @@ __global__ void __launch_bounds__(kShapeThreads) k_shape(const __grid_constant__
     if (i0 >= n) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int K = min(a.K, n);                                // fewer points than K_c: all of them
+    const bool sparse = WINDOW && (float)n * (float)n < kSparse * (float)K * (float)a.w.ncx * (float)a.w.ncy;
 #pragma unroll 1
     for (int t = 0; t < kShapeRounds; ++t) {
         const int slot = t * (kShapeThreads / 32) + warp, i = i0 + slot;
         if (i >= n) break;
         const float4 me = a.pos[i];
-        const uint64_t best = WINDOW ? window_nearest(a, i, me, K) : hash_nearest(a, me, n, K, s_buf[WINDOW ? 0 : warp]);
+        const uint64_t best = sparse   ? all_nearest(a, me, n, K)
+                              : WINDOW ? window_nearest(a, i, me, n, K)
+                                       : hash_nearest(a, me, n, K, s_buf[WINDOW ? 0 : warp]);
         const int nb = best != kNone ? (int)(uint32_t)best : -1;
         if (a.knn_out && lane < a.K) a.knn_out[(size_t)i * a.K + lane] = lane < K ? nb : -1;
         const float4 q = lane < K && nb >= 0 ? a.pos[nb] : me;
