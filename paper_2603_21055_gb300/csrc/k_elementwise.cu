@@ -80,7 +80,8 @@ __device__ __forceinline__ float block_sum(float x, float *red)
 
 // All views of one loss call; every view owns a contiguous range of CTAs of `chunk` pixels:
 // 4096, or 1024 (one access of four pixels per thread) when CTAs of 4096 would leave SMs
-// without one: 2 views of 160x120 took 24 us on ten CTAs and take 5 on 38.
+// without one: 2 views of 160x120 took 24 us on ten CTAs and take 5 on 38; one of 1200x680 (200
+// of 4096) takes 10.0 us with depth and 5.8 without in the large chunk, 10.9 and 6.7 in the small.
 // The CTAs of a cluster add their parts of the loss through distributed shared memory, one
 // FP32 addition to the loss per cluster: an eighth (with the small chunk half) of the
 // additions, and of their rounding and order dependence, that one per 4096 pixels made.
@@ -130,8 +131,9 @@ template <bool ALL_VEC>
 __global__ void __cluster_dims__(kLossCluster, 1, 1) __launch_bounds__(256)
     k_l1_grad(const __grid_constant__ LossBatch B, float *loss)
 {
+    cluster_begin();
     dependency_wait();
-    __shared__ float red[32], part;
+    __shared__ float red[32], part[kLossCluster];
     const LossView &v = B.v[loss_view(B)];
     const size_t hw = v.hw;
     // (a CTA past the last has no pixels: its base is past the end)
@@ -219,7 +221,7 @@ __global__ void __cluster_dims__(kLossCluster, 1, 1) __launch_bounds__(256)
     }
     if (loss) {
         const float t = block_sum(l, red);
-        cluster_add(loss, t, &part);
+        cluster_add(loss, t, part);
     }
 }
 
@@ -238,7 +240,7 @@ void launch_l1_batch(int n, const float *const *rgb, const float *const *depth, 
     uint32_t blocks = 0;
     size_t full = 0;
     for (int i = 0; i < n; ++i) full += (hw[i] + kLossChunk - 1) / kLossChunk;
-    B.chunk = full < 2 * 152 ? kLossChunkSmall : kLossChunk;
+    B.chunk = full < 152 ? kLossChunkSmall : kLossChunk;
     const bool use_depth = wdep != 0.0f && tdep && ddep && nvalid;
     for (int i = 0; i < n; ++i) {
         LossView &v = B.v[i];

@@ -422,20 +422,27 @@ inline Layout make_layout(uint64_t n_gauss, uint64_t n_views, uint64_t n_tiles, 
     return L;
 }
 
-// Adds the sum of thread 0's t over the CTAs of the cluster to *dst. All threads; part: one
-// float of this CTA's shared memory.
+// The sum over a cluster of CTAs, in two parts: cluster_begin() by every thread at the start of
+// the kernel, and cluster_add(), which adds thread 0's t of every CTA, in rank order, to *dst
+// (part: as many floats of shared memory as the cluster has CTAs). Only the first CTA waits for
+// the others; they hand it their parts and end.
+__device__ __forceinline__ void cluster_begin() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
+
 __device__ __forceinline__ void cluster_add(float *dst, float t, float *part)
 {
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
-    if (threadIdx.x == 0) *part = t;
-    cl.sync();
-    if (threadIdx.x == 0 && cl.block_rank() == 0) {
+    const unsigned rank = cl.block_rank();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");             // every CTA has started
+    if (threadIdx.x == 0) *cl.map_shared_rank(part + rank, 0) = t;
+    asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");           // (releases the store)
+    if (rank != 0) return;
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (threadIdx.x == 0) {
         float s = 0.f;
-        for (unsigned r = 0; r < cl.num_blocks(); ++r) s += *cl.map_shared_rank(part, r);
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) s += part[r];
         atomicAdd(dst, s);
     }
-    cl.sync();                          // the others' part is read before they end
 }
 
 }  // namespace sgad
