@@ -234,15 +234,17 @@ bool uses_masks(const sgad_options &o, const Scene &sc)
 }
 
 // Projection, binning count and scan: the part shared by sgad_count_keys and sgad_forward.
+// count_only: the keys' number alone is wanted (the rectangles carry no block trims, and the
+// sticky flags start anew).
 sgad_status run_binning_count(const sgad_options &o, const Scene &sc, const Ws &ws, int64_t key_cap,
-                              bool clear_sticky, cudaStream_t st)
+                              bool count_only, cudaStream_t st)
 {
     ClearList c = {};
-    c.add(ws.hdr(), clear_sticky ? sizeof(WsHeader) : kHeaderPerCall);
+    c.add(ws.hdr(), count_only ? sizeof(WsHeader) : kHeaderPerCall);
     c.add(ws.tile_cnt(), ((size_t)sc.n_tiles + 1) * 4);
     const cudaError_t e = launch_clear(c, st);
     if (e != cudaSuccess) return cuda_fail(e, "clear");
-    launch_project_count(sc, ws.world(), ws.tile_cnt(), ws.rects(), uses_masks(o, sc), st);
+    launch_project_count(sc, ws.world(), ws.tile_cnt(), ws.rects(), !count_only && uses_masks(o, sc), st);
     launch_scan_tiles(ws.tile_cnt(), ws.tile_off(), sc.n_tiles, (uint64_t)key_cap, ws.hdr(),
                       uses_order(o) ? ws.tile_order() : nullptr, st);
     return last_launch("binning");
