@@ -415,6 +415,7 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks<B>())
 // took 1.14 and 1.07 ms, 3 takes 1.01 heaviest first. A round's entries and records loaded
 // during the round before it: 1.15 against 1.05 ms. The two packed multiplies and adds, the
 // exact halves and the flushed exponential take a candidate from about 60 to 48 instructions.
+// Bound by issue (85 % of the slots; L1 data pipe 63 %).
 constexpr int kFwdlThreads = 256;           // 8 independent warps per block
 #ifndef SGAD_FWDL_MINBLOCKS
 #define SGAD_FWDL_MINBLOCKS 4
@@ -1413,6 +1414,8 @@ __global__ void __launch_bounds__(kPairThreads, 4) k_composite_bwdp(const __grid
 // bits as FP32's), as three BF16 numbers (exact) 1.49. Where one keyframe fills its own view and
 // entries reach many pixels, the TF32 products took 5 to 10 % less (111 us against 117 at one
 // 640x480 view), elsewhere up to 11 % more.
+// Bound by shared-memory wavefronts (81 % of the L1 data pipe) and issue (78 %) at 24 warps per SM;
+// the pose instance for few units by latency (issue 52 %, 23 % of the warps active).
 // 8,000 bytes of shared memory per warp leave the L1 60 KB beside three blocks; rows of pairs of
 // 36 instead of 34 entries cross the next step of the split (+4 us).
 constexpr int kLocalThreads = 256;          // 8 independent warps per block
